@@ -133,7 +133,9 @@ int rs_create(rs_handle** out, int64_t max_n, int device) {
   // the allocation-free call's static scratch on this device: looked up now, so that calls
   // made later while a stream is captured find it ready
   bool ok = rsk::noalloc_prepare_current_device() == RS_OK;
-  ok &= cudaMalloc(&s.d, sizeof(int32_t) * max_n) == cudaSuccess;
+  // (the claims, or the claimed bits: of a batch, one extra byte per filter)
+  s.max_filters = max_n / 16 > 1024 ? max_n / 16 : 1024;
+  ok &= cudaMalloc(&s.d, sizeof(int32_t) * max_n + s.max_filters) == cudaSuccess;
   ok &= cudaMalloc(&s.a_tmp, sizeof(int32_t) * max_n) == cudaSuccess;
   ok &= cudaMalloc(&s.W, 8 * static_cast<size_t>(max_n)) == cudaSuccess;
   ok &= cudaMalloc(&s.guide, sizeof(int32_t) * (max_n + 1)) == cudaSuccess;
@@ -141,7 +143,6 @@ int rs_create(rs_handle** out, int64_t max_n, int device) {
   ok &= cudaMalloc(&s.blockmax, sizeof(double) * s.max_blocks) == cudaSuccess;
   ok &= cudaMalloc(&s.irec, sizeof(long long) * 2 * (s.max_tiles + 2)) == cudaSuccess;
   ok &= cudaMalloc(&s.glob, sizeof(rsk::ScanGlob)) == cudaSuccess;
-  s.max_filters = max_n / 16 > 1024 ? max_n / 16 : 1024;
   s.batch_tile_cap = max_n / rsk::kTile + s.max_filters + 1;
   const size_t mf = static_cast<size_t>(s.max_filters);
   const size_t tc = static_cast<size_t>(s.batch_tile_cap);

@@ -107,8 +107,15 @@ struct Batch {
   double2* s_rec;        // tile totals, indexed by batch tile
   double2* P_rec;        // tile prefixes, filter f at tile_start[f] + f
   const uint8_t* resample;  // F flags (0: the filter keeps its particles), or null = all
+  uint8_t* cl;           // claimed bits (filter f's bytes at (off[f] >> 3) + f), or null
   int* err;
 };
+
+// The claimed bits of filter f, whose particles start at lo: its bytes end before those of
+// filter f + 1 start, (lo >> 3) + ceil(n / 8) <= ((lo + n) >> 3) + 1.
+__device__ __forceinline__ uint8_t* claimed_bits(const Batch& b, int f, int64_t lo) {
+  return b.cl ? b.cl + (lo >> 3) + f : nullptr;
+}
 
 // Filter f is resampled unless a flag array says otherwise (rs_resample_batched_masked).
 __device__ __forceinline__ bool resampled(const uint8_t* flags, int f) {
@@ -167,6 +174,14 @@ __device__ __forceinline__ bool locate_tile(const Batch& b, int tile, TileLoc& L
   L.hi = __ldg(b.off + L.f + 1);
   L.base = L.lo + static_cast<int64_t>(L.t) * kTile;
   return true;
+}
+
+// Every slot of a tile claimed (cl: the filter's claimed bits, or null).
+__device__ __forceinline__ void claim_all(uint8_t* cl, const TileLoc& L) {
+  if (!cl) return;
+  const int64_t i0 = L.base - L.lo;  // (a multiple of 8)
+  const int64_t i1 = min(i0 + kTile, L.hi - L.lo);
+  for (int64_t k = (i0 >> 3) + threadIdx.x; k < ((i1 + 7) >> 3); k += kBlock) cl[k] = 0xFFu;
 }
 
 template <typename T>
@@ -271,6 +286,7 @@ batch_emit_kernel(const T* __restrict__ lw, Batch b, Keys base_keys,
       if (d) d[e] = static_cast<int32_t>(e - L.lo);
       if (W) W[e] = vzero(V());
     }
+    claim_all(claimed_bits(b, L.f, L.lo), L);
     return;
   }
   const WeightCtx wc = make_ctx<T, V>(M, sh_tab);
@@ -291,7 +307,8 @@ batch_emit_kernel(const T* __restrict__ lw, Batch b, Keys base_keys,
         SCHEME == RS_STRATIFIED ? typename Path<T, V>::U() : cta_uniform0<T, V>(keys);
     emit_seg_cumoff<T, V, SCHEME == RS_STRATIFIED>(
         lw, L.lo, L.hi, base, wc, vec, Ps, Pn, load_v_cg<V>(b.fS + L.f),
-        load_v_cg<V>(b.fscale + L.f), u_sys, keys, a, d, sh.win[warp]);
+        load_v_cg<V>(b.fscale + L.f), u_sys, keys, a, d, sh.win[warp],
+        claimed_bits(b, L.f, L.lo));
   }
 }
 
@@ -435,6 +452,7 @@ batch_coop_kernel(const T* __restrict__ lw, Batch b, Keys base_keys, int32_t* __
         if (d) d[e] = static_cast<int32_t>(e - L.lo);
         if (W) W[e] = vzero(V());
       }
+      claim_all(claimed_bits(b, L.f, L.lo), L);
       continue;
     }
     const WeightCtx wc = ctx_staged<T, V>(M, sh_tab);  // (the table was staged at the start)
@@ -451,7 +469,8 @@ batch_coop_kernel(const T* __restrict__ lw, Batch b, Keys base_keys, int32_t* __
           SCHEME == RS_STRATIFIED ? typename Path<T, V>::U()
                                   : Path<T, V>::draw_u(draw(keys, 0u, 0u));
       emit_seg_cumoff<T, V, SCHEME == RS_STRATIFIED>(lw, L.lo, L.hi, base, wc, vec, Ps, Pn, S,
-                                                      scale, u_sys, keys, a, d, sh.win[warp]);
+                                                      scale, u_sys, keys, a, d, sh.win[warp],
+                                                      claimed_bits(b, L.f, L.lo));
     }
   }
   grid_exit(bar, target);
@@ -625,21 +644,73 @@ batch_rejection_kernel(const T* __restrict__ lw, const int64_t* __restrict__ off
   }
 }
 
-// Permute of every filter (permute.cuh), ipt slots per thread (tunable launch shape).
+// filter_of for one position g, by a whole warp (every lane calls it with the same g): 32
+// offsets are compared at a time, so 4096 filters take three dependent loads instead of twelve.
+__device__ __forceinline__ int filter_of_warp(const int64_t* __restrict__ off, int F, int64_t g) {
+  const int lane = threadIdx.x & 31;
+  int lo = 0, hi = F;  // invariant: off[lo] <= g < off[hi]
+  while (hi - lo > 1) {
+    const int step = (hi - lo + 31) >> 5;
+    const int at = lo + (lane + 1) * step;
+    const bool below = at < hi && __ldg(off + at) <= g;
+    const int cnt = __popc(__ballot_sync(0xffffffffu, below));
+    lo += cnt * step;
+    hi = min(hi, lo + step);
+  }
+  return lo;
+}
+
+// Permute of every filter: each warp takes 128 consecutive slots of the batch (four per lane),
+// ipt times (tunable launch shape). Nearly every warp lies inside one filter: its filter is
+// looked up once per warp and its slots run as in the single-filter kernels (permute4_slots;
+// SORTED: permute_sorted_slots, the non-decreasing ancestries of stratified and systematic from
+// the claimed bits cl of their emission, filter f's bytes at (offsets[f] >> 3) + f). A warp that
+// meets a filter boundary takes its slots one by one. Bound by L2 latency of the claims and
+// walks, as in the single-filter kernels; looking the filter up per slot instead (a binary
+// search of the offsets each) took 350 instructions per slot.
+constexpr int kPermSlots = 4;                         // consecutive slots per lane
+constexpr size_t kPermSmemPerWarp = 128 * (sizeof(int2) + sizeof(int32_t));
+template <bool SORTED>
 __global__ void __launch_bounds__(kMaxTunedBlock)
 batch_permute_kernel(const int64_t* __restrict__ off, int F, int64_t total,
                      const int32_t* __restrict__ a, const int32_t* __restrict__ d,
-                     int32_t* __restrict__ c, int ipt, int* err) {
+                     const uint8_t* __restrict__ cl, int32_t* __restrict__ c, int ipt, int* err) {
   pdl_wait();
+  extern __shared__ __align__(16) unsigned char sh_perm[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int32_t* const cw = reinterpret_cast<int32_t*>(sh_perm + warp * kPermSmemPerWarp);
+  int2* const pend = reinterpret_cast<int2*>(cw + 128);
   const int64_t offF = __ldg(off + F);
-  int f = -1;  // the filter of this thread's previous item (items ascend by blockDim.x)
+  const int64_t end = offF < total ? offF : total;
   for (int q = 0; q < ipt; ++q) {
-    const int64_t g = item_index(ipt, q);
-    if (g >= total || g >= offF) return;
-    f = f < 0 ? filter_of(off, F, g) : advance_filter(off, F, g, f);
+    // first slot of this warp (of this lane: kPermSlots * lane further)
+    const int64_t gw = kPermSlots * ((static_cast<int64_t>(blockIdx.x) * ipt + q) * blockDim.x +
+                                     32 * static_cast<int64_t>(warp));
+    if (gw >= end) return;  // (uniform over the warp)
+    const int f = filter_of_warp(off, F, gw);
+    const int64_t g0 = gw + kPermSlots * lane;
     PartLoc P;
-    if (!locate_in(off, f, total, g, P)) continue;
-    permute_one(a + P.lo, d + P.lo, P.n, c + P.lo, P.i, err);
+    const bool ok = locate_in(off, f, total, gw, P);  // (uniform over the warp)
+    if (ok && P.i + 32 * kPermSlots <= P.n) {
+      if constexpr (SORTED)
+        permute_sorted_slots<kPermSlots>(a + P.lo, cl + (P.lo >> 3) + f, P.n, c + P.lo, g0 - P.lo,
+                                         cw, pend, err);
+      else
+        permute4_slots(a + P.lo, d + P.lo, P.n, c + P.lo, g0 - P.lo, pend, err);
+      __syncwarp();  // (the warp's shared lists are rewritten by its next slots)
+      continue;
+    }
+    int fs = f;
+    for (int k = 0; k < kPermSlots; ++k) {
+      const int64_t g = g0 + k;
+      if (g >= end) break;
+      fs = advance_filter(off, F, g, fs);
+      if (!locate_in(off, fs, total, g, P)) continue;
+      if constexpr (SORTED)
+        permute_sorted_one(a + P.lo, cl + (P.lo >> 3) + fs, P.n, c + P.lo, P.i, err);
+      else
+        permute_one(a + P.lo, d + P.lo, P.n, c + P.lo, P.i, err);
+    }
   }
 }
 
@@ -738,6 +809,12 @@ cudaError_t launch_batched(const Scratch& s, int scheme, Acc acc, const void* lo
                            const uint8_t* flags, int32_t* out, int permute, cudaStream_t st) {
   int32_t* a = permute ? s.a_tmp : out;
   int32_t* d = permute ? s.d : nullptr;
+  // a non-decreasing ancestry (stratified, systematic): claimed bits in the claims' buffer
+  uint8_t* cl = nullptr;
+  if (permute && (scheme == RS_STRATIFIED || scheme == RS_SYSTEMATIC)) {
+    cl = reinterpret_cast<uint8_t*>(s.d);
+    d = nullptr;
+  }
   const bool f64 = acc == Acc::F64 || acc == Acc::F64N;
   const Keys keys = make_keys(seed, step, 0u, static_cast<uint32_t>(scheme));
   // particles are bounded by the capacity; the true total is offsets[F] (checked per filter)
@@ -788,6 +865,7 @@ cudaError_t launch_batched(const Scratch& s, int scheme, Acc acc, const void* lo
     b.s_rec = s.batch_s_rec;
     b.P_rec = s.batch_P_rec;
     b.resample = flags;
+    b.cl = cl;
     b.err = s.err;
     trace_mark(s.trace, "batch_plan", st);
     launch_pdl(batch_plan_kernel, 1, 1024, st, b);
@@ -816,8 +894,10 @@ cudaError_t launch_batched(const Scratch& s, int scheme, Acc acc, const void* lo
   if (e == cudaSuccess && permute) {
     trace_mark(s.trace, "batch_permute", st);
     const LaunchCfg& c = s.batch_cfg[kCfgPermute];
-    launch_pdl(batch_permute_kernel, grid_shaped(total, c), c.block, st, offsets, F, total,
-               s.a_tmp, s.d, out, c.ipt, s.err);
+    const int grid = grid_shaped((total + kPermSlots - 1) / kPermSlots, c);
+    const size_t smem = kPermSmemPerWarp * (c.block / 32);
+    launch_pdl_smem(cl ? batch_permute_kernel<true> : batch_permute_kernel<false>, grid, c.block,
+                    smem, st, offsets, F, total, s.a_tmp, s.d, cl, out, c.ipt, s.err);
     e = cudaGetLastError();
   }
   return e;

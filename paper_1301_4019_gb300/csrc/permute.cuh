@@ -112,5 +112,179 @@ __device__ __forceinline__ void walk_queue(const Claim& claim, int32_t sentinel,
   if (bad) flag_error(err, RS_ERR_ARG);
 }
 
+// Four consecutive slots i0 .. i0 + 3 of the Permute of n ancestors a with claims d (any
+// ancestry; the general form of permute_one): 128-bit slot loads where the addresses allow, the
+// four claim checks d[a_i] issued together, and the walks of failed claims run together
+// (walk_queue). Called by all 32 lanes of a warp; slots at n or beyond do nothing. Same reads
+// and writes per slot as permute_one, so c is the same.
+__device__ __forceinline__ void permute4_slots(const int32_t* __restrict__ a,
+                                               const int32_t* __restrict__ d, int64_t n,
+                                               int32_t* __restrict__ c, int64_t i0, int2* pend,
+                                               int* err) {
+  const int32_t sentinel = static_cast<int32_t>(n);
+  int32_t A[4], D[4];
+  const bool vec = i0 + 3 < n && ((reinterpret_cast<uintptr_t>(a + i0) |
+                                   reinterpret_cast<uintptr_t>(d + i0)) & 15u) == 0;
+  if (vec) {
+    const int4 va = *reinterpret_cast<const int4*>(a + i0);
+    const int4 vd = *reinterpret_cast<const int4*>(d + i0);
+    A[0] = va.x; A[1] = va.y; A[2] = va.z; A[3] = va.w;
+    D[0] = vd.x; D[1] = vd.y; D[2] = vd.z; D[3] = vd.w;
+  } else {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      A[q] = i0 + q < n ? a[i0 + q] : 0;
+      D[q] = i0 + q < n ? d[i0 + q] : sentinel;
+    }
+  }
+  bool ok[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    ok[q] = i0 + q < n;
+    if (ok[q] && (A[q] < 0 || A[q] >= n)) {
+      flag_error(err, RS_ERR_ARG);
+      ok[q] = false;
+    }
+  }
+  int32_t claim[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) claim[q] = ok[q] ? d[A[q]] : static_cast<int32_t>(i0 + q);
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+    if (ok[q] && D[q] != sentinel) c[i0 + q] = static_cast<int32_t>(i0 + q);
+  bool fail[4];
+  int32_t x[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    fail[q] = ok[q] && claim[q] != static_cast<int32_t>(i0 + q);
+    x[q] = static_cast<int32_t>(i0 + q);
+  }
+  walk_queue<4>(ClaimsOf{d}, sentinel, c, x, D, A, fail, n, pend, err);
+}
+
+// Permute of a non-decreasing ancestry from a and the claimed bits of its emission (cl: bit
+// i % 8 of cl[i / 8] set when particle i has offspring). For such an ancestry the claims of
+// Prepermute are d_j = the first position of the run of j for every claimed j, so Code 10's
+// walks can be followed from their ends instead of their starts:
+//  - a claimed slot x keeps its particle: c_x = x;
+//  - an unclaimed slot x that is not the first of its run (a_{x-1} = a_x) is a failed claim
+//    whose walk ends at once, at x: c_x = a_x;
+//  - an unclaimed slot x that is the first of its run was reached from z = a_x (d_z = x);
+//    while z is itself the first of its run (z = 0 or a_{z-1} != a_z) it was reached from
+//    a_z in turn, and the first z that is not is the walk's start: c_x = a_z.
+// d is injective on the claimed slots and the walks end (Appendix C), so each backward chain
+// is one walk reversed and c is Code 10's exactly; the claims are never stored.
+//
+// The chain of one unclaimed run head whose ancestor is z, to its start: returns the value
+// that the head receives, or sets bad (only a corrupted a can do that).
+__device__ __forceinline__ int32_t sorted_chain(const int32_t* __restrict__ a, int32_t z,
+                                                int64_t n, bool& bad) {
+  const uint32_t un = static_cast<uint32_t>(n);
+  for (int64_t steps = 0;; ++steps) {
+    const int32_t y = a[z];
+    const bool zhead = z == 0 || a[z - 1] != y;
+    if (static_cast<uint32_t>(y) >= un || steps > n) {
+      bad = true;
+      return 0;
+    }
+    if (!zhead) return y;
+    z = y;
+  }
+}
+
+// One slot i of it (n ancestors, local indices).
+__device__ __forceinline__ void permute_sorted_one(const int32_t* __restrict__ a,
+                                                   const uint8_t* __restrict__ cl, int64_t n,
+                                                   int32_t* __restrict__ c, int64_t i, int* err) {
+  const int32_t ai = a[i];
+  if (ai < 0 || ai >= n) {
+    flag_error(err, RS_ERR_ARG);
+    return;
+  }
+  bool bad = false;
+  int32_t v;
+  if ((cl[i >> 3] >> (i & 7)) & 1) v = static_cast<int32_t>(i);
+  else if (i > 0 && a[i - 1] == ai) v = ai;
+  else v = sorted_chain(a, ai, n, bad);
+  if (bad) flag_error(err, RS_ERR_ARG);
+  else c[i] = v;
+}
+
+// K consecutive slots i0 .. i0 + K - 1 of it per lane (lane l's follow lane l - 1's), called by
+// all 32 lanes of a warp; slots at n or beyond do nothing. The chains that go on past their
+// first step are queued per warp (pend: 32 K entries) and run one per lane; the warp's results
+// are gathered in cw (32 K entries, 16-byte aligned) and stored 128 bits at a time where the
+// addresses allow.
+template <int K>
+__device__ __forceinline__ void permute_sorted_slots(const int32_t* __restrict__ a,
+                                                     const uint8_t* __restrict__ cl, int64_t n,
+                                                     int32_t* __restrict__ c, int64_t i0,
+                                                     int32_t* cw, int2* pend, int* err) {
+  static_assert(K == 1 || K == 4, "one or four slots per thread");
+  const int lane = threadIdx.x & 31;
+  const bool full = i0 + K <= n;
+  int32_t A[K];
+  if (K == 4 && full && (reinterpret_cast<uintptr_t>(a + i0) & 15u) == 0) {
+    const int4 va = *reinterpret_cast<const int4*>(a + i0);
+    A[0] = va.x; A[1] = va.y; A[2] = va.z; A[3] = va.w;
+  } else {
+#pragma unroll
+    for (int q = 0; q < K; ++q) A[q] = i0 + q < n ? a[i0 + q] : 0;
+  }
+  // a_{i0-1}: the previous lane's last slot, loaded by lane 0 only
+  int32_t prev = __shfl_up_sync(0xffffffffu, A[K - 1], 1);
+  if (lane == 0) prev = (i0 > 0 && i0 - 1 < n) ? a[i0 - 1] : -1;
+  uint32_t bits = 0u;
+  if (i0 < n) {
+    const int sh = static_cast<int>(i0 & 7);
+    bits = static_cast<uint32_t>(cl[i0 >> 3]) >> sh;
+    if (K == 4 && sh > 4 && i0 + (8 - sh) < n)  // (the slots reach into the next byte)
+      bits |= static_cast<uint32_t>(cl[(i0 >> 3) + 1]) << (8 - sh);
+  }
+  const unsigned below = (1u << lane) - 1u;
+  int total = 0;
+  bool bad = false;
+  int32_t R[K];
+#pragma unroll
+  for (int q = 0; q < K; ++q) {
+    const int64_t x = i0 + q;
+    bool go = false;
+    R[q] = 0;
+    const int32_t ax = A[q];
+    if (x < n) {
+      if (ax < 0 || ax >= n) bad = true;
+      else if ((bits >> q) & 1u) R[q] = static_cast<int32_t>(x);
+      else if (prev == ax) R[q] = ax;  // not the first of its run
+      else go = true;
+      prev = ax;
+    }
+    const unsigned m = __ballot_sync(0xffffffffu, go);
+    if (go) pend[total + __popc(m & below)] = make_int2(K * lane + q, ax);
+    total += __popc(m);
+  }
+  if (K == 4) {
+    reinterpret_cast<int4*>(cw)[lane] = make_int4(R[0], R[1], R[2], R[3]);
+  } else {
+    cw[lane] = R[0];
+  }
+  __syncwarp();
+  for (int e = lane; e < total; e += 32) {
+    const int2 w = pend[e];
+    bool cbad = false;
+    const int32_t v = sorted_chain(a, w.y, n, cbad);
+    if (cbad) bad = true;
+    else cw[w.x] = v;
+  }
+  __syncwarp();
+  if (K == 4 && full && (reinterpret_cast<uintptr_t>(c + i0) & 15u) == 0) {
+    *reinterpret_cast<int4*>(c + i0) = reinterpret_cast<const int4*>(cw)[lane];
+  } else {
+#pragma unroll
+    for (int q = 0; q < K; ++q)
+      if (i0 + q < n) c[i0 + q] = cw[K * lane + q];
+  }
+  if (bad) flag_error(err, RS_ERR_ARG);
+}
+
 }  // namespace
 }  // namespace rsk

@@ -255,3 +255,33 @@ def test_batched_cooperative_equals_separate_kernels(rs, h, dtype, prec):
             assert np.array_equal(a, b) and np.array_equal(a2, b2), (scheme, permute)
             lo, hi = offsets[6], offsets[7]
             assert np.array_equal(np.sort(a[lo:hi]), np.arange(hi - lo))
+
+
+# sizes whose filters begin at every residue modulo 8 and whose boundaries fall inside, at the
+# ends of and between the 128-slot groups of the batched Permute (1 .. 129, 255 .. 257, a long
+# filter, empty ones, a short tail)
+EDGE_SIZES = [1, 7, 0, 8, 9, 127, 128, 129, 3, 255, 256, 257, 0, 0, 5, 64, 4099, 2, 511, 1]
+
+
+@pytest.mark.parametrize("scheme", range(5))
+@pytest.mark.parametrize("masked", [False, True])
+def test_batched_permute_at_filter_boundaries(rs, scheme, masked):
+    """The batched Permute (claims, and for stratified / systematic the claimed bits) equals
+    Code 10 of the same call's unpermuted ancestors on every filter, whatever its alignment."""
+    offsets, lw = _batch(EDGE_SIZES, np.float32, seed=5)
+    lw[offsets[9]:offsets[10]] = -np.inf
+    lw[offsets[9] + 17] = 0.0  # one particle takes every offspring
+    t = torch.from_numpy(lw).to(DEV)
+    off = torch.from_numpy(offsets).to(DEV)
+    flags = None
+    if masked:
+        flags = torch.tensor([f % 3 != 1 for f in range(len(EDGE_SIZES))], dtype=torch.uint8,
+                             device=DEV)
+    with rs.Handle(int(offsets[-1])) as hh:
+        out = [rs.rs_resample_batched(hh, scheme, t, off, B=8, seed=4, step=2, permute=p,
+                                      resample=flags).cpu().numpy() for p in (False, True)]
+        assert rs.rs_last_error(hh) == rs.RS_OK
+    for f in range(len(EDGE_SIZES)):
+        a, c = (o[offsets[f]:offsets[f + 1]] for o in out)
+        if a.size:
+            assert np.array_equal(c, oracle.permute(a)), (f, a.size)
