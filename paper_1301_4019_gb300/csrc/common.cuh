@@ -75,6 +75,41 @@ __device__ __forceinline__ uint4 draw(const Keys& k, uint32_t index, uint32_t n)
   return c;
 }
 
+// The draws (index, n), n = 0, 1, ..., of one index: the products of the first three rounds that
+// depend on the index alone are formed once (DrawRow), so that a draw takes 16 products instead
+// of 20. Same words as draw(k, index, n).
+struct DrawRow {
+  uint32_t a, b, c, d;
+};
+__device__ __forceinline__ DrawRow draw_row(const Keys& k, uint32_t index) {
+  const uint64_t p0 = static_cast<uint64_t>(0xD2511F53u) * index;
+  const uint64_t p1 = static_cast<uint64_t>(0xCD9E8D57u) * k.step;
+  const uint64_t q1 = static_cast<uint64_t>(0xCD9E8D57u) *
+                      (static_cast<uint32_t>(p0 >> 32) ^ k.tag ^ k.rk1[0]);
+  const uint64_t r0 = static_cast<uint64_t>(0xD2511F53u) *
+                      (static_cast<uint32_t>(q1 >> 32) ^ static_cast<uint32_t>(p1) ^ k.rk0[1]);
+  return DrawRow{static_cast<uint32_t>(p0) ^ k.rk1[1], static_cast<uint32_t>(q1) ^ k.rk0[2],
+                 static_cast<uint32_t>(r0 >> 32) ^ k.rk1[2], static_cast<uint32_t>(r0)};
+}
+__device__ __forceinline__ uint4 draw(const Keys& k, const DrawRow& row, uint32_t n) {
+  const uint64_t p1 = static_cast<uint64_t>(0xCD9E8D57u) * k.step;
+  const uint64_t U = static_cast<uint64_t>(0xD2511F53u) *
+                     (static_cast<uint32_t>(p1 >> 32) ^ n ^ k.rk0[0]);
+  const uint64_t V = static_cast<uint64_t>(0xCD9E8D57u) * (static_cast<uint32_t>(U >> 32) ^ row.a);
+  uint4 c = make_uint4(static_cast<uint32_t>(V >> 32) ^ row.b, static_cast<uint32_t>(V),
+                       row.c ^ static_cast<uint32_t>(U), row.d);
+#pragma unroll
+  for (int round = 3; round < 10; ++round) {
+    const uint64_t p0 = static_cast<uint64_t>(0xD2511F53u) * c.x;
+    const uint64_t p1r = static_cast<uint64_t>(0xCD9E8D57u) * c.z;
+    c = make_uint4(static_cast<uint32_t>(p1r >> 32) ^ c.y ^ k.rk0[round],
+                   static_cast<uint32_t>(p1r),
+                   static_cast<uint32_t>(p0 >> 32) ^ c.w ^ k.rk1[round],
+                   static_cast<uint32_t>(p0));
+  }
+  return c;
+}
+
 // U[0,1) with 24 (binary32) or 53 (binary64) random bits; both conversions are exact.
 __device__ __forceinline__ float u01_f32(uint4 x) {
   return __fmul_rn(__uint2float_rn(x.x >> 8), 0x1p-24f);
@@ -87,29 +122,27 @@ template <typename T> __device__ __forceinline__ T u01(uint4 x);
 template <> __device__ __forceinline__ float u01<float>(uint4 x) { return u01_f32(x); }
 template <> __device__ __forceinline__ double u01<double>(uint4 x) { return u01_f64(x); }
 
-// Uniform index on {0..N-1}: the high 64 bits of V * N, V = words 2,3 as a 64-bit integer.
-// For N < 2^32 this is (x2 N + floor(x3 N / 2^32)) / 2^32 rounded down (the discarded low
-// part cannot carry), two 32x32->64 products with no overflow.
-__device__ __forceinline__ int64_t uniform_index(uint4 x, int64_t N) {
-  const uint64_t n = static_cast<uint64_t>(N);
-  const uint64_t lo = static_cast<uint64_t>(x.w) * n;
-  const uint64_t hi = static_cast<uint64_t>(x.z) * n + (lo >> 32);
-  return static_cast<int64_t>(hi >> 32);
+// Uniform index on {0..n-1}: the high 64 bits of V * n, V = words 2,3 as a 64-bit integer. For
+// n < 2^32 this is (x2 n + floor(x3 n / 2^32)) / 2^32 rounded down (the discarded low part
+// cannot carry), two 32x32->64 products with no overflow.
+__device__ __forceinline__ uint32_t uniform_index(uint4 x, uint32_t n) {
+  return static_cast<uint32_t>((static_cast<uint64_t>(x.z) * n + __umulhi(x.w, n)) >> 32);
 }
 
 // The two step halves of a binary32 Metropolis block (h = 0: words 0, 1; h = 1: words 2, 3):
-// the uniform is the top 24 bits of the first word times 2^-24, the proposal floor(V N / 2^40)
-// with V = (the first word's low byte) 2^32 + the second word. With Q = (V >> 32) N and
-// P = (V mod 2^32) N, V N = (Q + floor(P / 2^32)) 2^32 + (P mod 2^32) and the last term
-// cannot carry past bit 40, so the index is (Q + floor(P / 2^32)) / 2^8 rounded down.
+// the uniform is the top 24 bits of the first word times 2^-24 (half_u24: those bits as a
+// binary32 integer, exact), the proposal floor(V n / 2^40) with V = (the first word's low
+// byte) 2^32 + the second word, for n < 2^31. With V = 256 T + r (r the low byte) the proposal
+// is floor((T n + floor(r n / 256)) / 2^32), and with n = 256 n1 + n0 the inner quotient is
+// r n1 + floor(r n0 / 256): one 32x32->64 product instead of two 64-bit ones.
+__device__ __forceinline__ float half_u24(uint32_t w0) { return __uint2float_rn(w0 >> 8); }
 __device__ __forceinline__ float half_u01_f32(uint32_t w0) {
-  return __fmul_rn(__uint2float_rn(w0 >> 8), 0x1p-24f);
+  return __fmul_rn(half_u24(w0), 0x1p-24f);
 }
-__device__ __forceinline__ int64_t half_index(uint32_t w0, uint32_t w1, int64_t N) {
-  const uint64_t n = static_cast<uint64_t>(N);
-  const uint64_t P = static_cast<uint64_t>(w1) * n;
-  const uint64_t Q = static_cast<uint64_t>(w0 & 0xffu) * n;
-  return static_cast<int64_t>((Q + (P >> 32)) >> 8);
+__device__ __forceinline__ uint32_t half_index(uint32_t w0, uint32_t w1, uint32_t n) {
+  const uint32_t T = __funnelshift_r(w1, w0, 8), r = w1 & 0xffu;
+  const uint32_t x = r * (n >> 8) + ((r * (n & 0xffu)) >> 8);
+  return static_cast<uint32_t>((static_cast<uint64_t>(T) * n + x) >> 32);
 }
 
 // ---------------------------------------------------------------------------------------

@@ -197,7 +197,7 @@ estimate_bound_kernel(const T* __restrict__ lw, int64_t N, int64_t sample, Keys 
   double m = -INFINITY;
   for (int64_t k = threadIdx.x; k < sample; k += kEstBlock) {
     const uint4 x = draw(keys, static_cast<uint32_t>(k), 0u);
-    const double v = static_cast<double>(__ldg(lw + uniform_index(x, N)));
+    const double v = static_cast<double>(__ldg(lw + uniform_index(x, static_cast<uint32_t>(N))));
     if (v > m) m = v;  // (NaN never compares)
   }
 #pragma unroll
@@ -255,9 +255,10 @@ __device__ __forceinline__ void count_add(unsigned long long* out, unsigned long
   if ((threadIdx.x & 31) == 0 && v) atomicAdd(out, v);
 }
 
-// Every binary32 delta with bit pattern first + k (k < count): the binary32 test decides
-// from the band [RD(e (1 - 2^-15)), RU(e (1 + 2^-15))] around e = exp_band_estimate(delta),
-// which is right exactly when exp_pinned(delta) lies inside it.
+// Every binary32 delta with bit pattern first + k (k < count): the tests decide from the band
+// [RD(e (1 - 2^-15)), RU(e (1 + 2^-15))] around e = exp_band_estimate(delta) (the binary64
+// filter) or exp_band_estimate24(delta) 2^-24 (the binary32 steps), which is right exactly when
+// exp_pinned(delta) lies inside it.
 __global__ void __launch_bounds__(kBlock)
 check_band_f32_kernel(uint32_t first, uint32_t count, unsigned long long* out) {
   unsigned long long bad = 0;
@@ -267,7 +268,11 @@ check_band_f32_kernel(uint32_t first, uint32_t count, unsigned long long* out) {
     const float e = exp_band_estimate(delta);
     const float lo = __fmul_rd(e, 1.0f - kExpBand), hi = __fmul_ru(e, 1.0f + kExpBand);
     const float p = exp_pinned(delta);
+    const float e24 = exp_band_estimate24(delta), p24 = __fmul_rn(p, 0x1p24f);  // (exact)
     if (!(lo <= p && p <= hi)) ++bad;
+    else if (!(__fmaf_rd(e24, 1.0f - kExpBand, -0x1p-36f) <= p24 &&
+               p24 <= __fmul_ru(e24, 1.0f + kExpBand)))
+      ++bad;
   }
   count_add(out, bad);
 }

@@ -31,27 +31,48 @@ __device__ __forceinline__ float exp_band_estimate(float delta) {
   return e;
 }
 
-__device__ __forceinline__ bool u_below_exp(float u, float delta) {
-  if (!(delta >= -86.5f)) return false;
-  const float e = exp_band_estimate(delta);
-  if (u < __fmul_rd(e, 1.0f - kExpBand)) return true;
-  if (u >= __fmul_ru(e, 1.0f + kExpBand)) return false;
-  return u < exp_pinned(delta);
+// 2^24 exp(delta), the scaling by one exponent addition inside the product (an FMA: one rounding
+// of delta log2 e + 24, whose magnitude is below 2^7: 2^-18, so still within a relative 1e-5).
+__device__ __forceinline__ float exp_band_estimate24(float delta) {
+  float e;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(__fmaf_rn(delta, 0x1.715476p+0f, 24.0f)));
+  return e;
+}
+
+// u < exp_pinned(delta) for u = u24 2^-24 (u24 an integer), by definition.
+__device__ __forceinline__ bool u24_below_exp_exact(float u24, float delta) {
+  return delta >= -86.5f && __fmul_rn(u24, 0x1p-24f) < exp_pinned(delta);
 }
 
 // u < w^j / w^k from log-weights: a ratio >= 1 or a zero-weight current state accepts.
-template <typename T>
-__device__ __forceinline__ bool metropolis_accept(T lwk, T lwj, T u) {
-  if (lwk == neg_inf<T>()) return true;
-  const T delta = lwj - lwk;
-  if (delta >= T(0)) return true;
-  return u < exp_pinned(delta);
-}
-__device__ __forceinline__ bool metropolis_accept(float lwk, float lwj, float u) {
+__device__ __noinline__ bool metropolis_accept_exact(float lwk, float lwj, float u24) {
   if (lwk == neg_inf<float>()) return true;
   const float delta = lwj - lwk;
-  if (delta >= 0.0f) return true;
-  return u_below_exp(u, delta);
+  return delta >= 0.0f || u24_below_exp_exact(u24, delta);
+}
+
+// The same for binary32, u24 the 24 uniform bits as an integer, decided by the band alone in
+// almost every case, whatever delta is: e = exp_band_estimate24(delta) is +inf, or at least
+// 2^24 (1 - 1e-5) > u24 (1 - 2^-15), for a ratio >= 1 and for a zero-weight current state with a
+// proposal of non-zero weight, 0 for a zero-weight proposal, and NaN (neither comparison holds)
+// for two zero weights or a NaN. u24 = 0 accepts only where e is above 2^-36 (delta > -42); a
+// smaller e leaves it to the definition unless e is 0 (delta < -86.5: rejected, as there).
+// Seven instructions a step where the chain of tests took about twenty.
+__device__ __forceinline__ bool metropolis_accept24(float lwk, float lwj, float u24) {
+  const float e = exp_band_estimate24(__fsub_rn(lwj, lwk));
+  const bool yes = u24 < __fmaf_rd(e, 1.0f - kExpBand, -0x1p-36f);
+  const bool no = u24 >= __fmul_ru(e, 1.0f + kExpBand);
+  if (yes || no) return yes;
+  return metropolis_accept_exact(lwk, lwj, u24);
+}
+
+// u < exp_pinned(delta) for delta < 0, u = u24 2^-24.
+__device__ __forceinline__ bool u24_below_exp(float u24, float delta) {
+  const float e = exp_band_estimate24(delta);
+  const bool yes = u24 < __fmaf_rd(e, 1.0f - kExpBand, -0x1p-36f);
+  const bool no = u24 >= __fmul_ru(e, 1.0f + kExpBand);
+  if (yes || no) return yes;
+  return u24_below_exp_exact(u24, delta);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -144,57 +165,66 @@ __device__ __forceinline__ float f64_sidecar(double x) {
 constexpr int kUnroll = 4;    // binary32 chains: proposals issued together
 constexpr int kUnroll64 = 4;  // binary64 chains (2 measured slower)
 
-// Metropolis chain of particle i over n binary32 log-weights lw (Code 2): B steps; steps 2m
-// and 2m + 1 take the two halves of the block of counter (i, m) (half_u01_f32, half_index),
-// so a chain draws ceil(B / 2) blocks. Returns the ancestor.
-__device__ __forceinline__ int32_t metropolis_one(const float* __restrict__ lw, int64_t n,
-                                                  int32_t B, const Keys& keys, int64_t i,
-                                                  int* err) {
+// Metropolis chain of particle i over n < 2^31 binary32 log-weights (Code 2), from the state i
+// with log-weight lwk; gather(j) reads the log-weight of proposal j. B steps; steps 2m and
+// 2m + 1 take the two halves of the block of counter (i, m) (half_u24, half_index), so a chain
+// draws ceil(B / 2) blocks. Returns the ancestor.
+template <typename Gather>
+__device__ __forceinline__ int32_t metropolis_chain(float lwk, const Gather& gather, uint32_t n,
+                                                    int32_t B, const Keys& keys, uint32_t i) {
   static_assert(kUnroll % 2 == 0, "whole blocks per round");
-  float lwk = __ldg(lw + i);
-  if (nonfinite_logw(lwk)) flag_error(err, RS_ERR_NONFINITE);
-  int64_t k = i;
-  const uint32_t ii = static_cast<uint32_t>(i);
+  uint32_t k = i;
+  const DrawRow row = draw_row(keys, i);
   int32_t s = 0;
   for (; s + kUnroll <= B; s += kUnroll) {  // (s even)
     float u[kUnroll], lwj[kUnroll];
-    int64_t j[kUnroll];
+    uint32_t j[kUnroll];
 #pragma unroll
     for (int p = 0; p < kUnroll / 2; ++p) {
-      const uint4 x = draw(keys, ii, static_cast<uint32_t>(s / 2 + p));
+      const uint4 x = draw(keys, row, static_cast<uint32_t>(s / 2 + p));
       j[2 * p] = half_index(x.x, x.y, n);
-      u[2 * p] = half_u01_f32(x.x);
+      u[2 * p] = half_u24(x.x);
       j[2 * p + 1] = half_index(x.z, x.w, n);
-      u[2 * p + 1] = half_u01_f32(x.z);
-      lwj[2 * p] = __ldg(lw + j[2 * p]);
-      lwj[2 * p + 1] = __ldg(lw + j[2 * p + 1]);
+      u[2 * p + 1] = half_u24(x.z);
+      lwj[2 * p] = gather(j[2 * p]);
+      lwj[2 * p + 1] = gather(j[2 * p + 1]);
     }
 #pragma unroll
     for (int q = 0; q < kUnroll; ++q) {
-      if (metropolis_accept(lwk, lwj[q], u[q])) {
+      if (metropolis_accept24(lwk, lwj[q], u[q])) {
         k = j[q];
         lwk = lwj[q];
       }
     }
   }
   for (; s < B; s += 2) {  // the last B mod kUnroll steps, a block per two
-    const uint4 x = draw(keys, ii, static_cast<uint32_t>(s / 2));
-    const int64_t j0 = half_index(x.x, x.y, n);
-    const float lwj0 = __ldg(lw + j0);
-    if (metropolis_accept(lwk, lwj0, half_u01_f32(x.x))) {
+    const uint4 x = draw(keys, row, static_cast<uint32_t>(s / 2));
+    const uint32_t j0 = half_index(x.x, x.y, n);
+    const float lwj0 = gather(j0);
+    if (metropolis_accept24(lwk, lwj0, half_u24(x.x))) {
       k = j0;
       lwk = lwj0;
     }
     if (s + 1 < B) {
-      const int64_t j1 = half_index(x.z, x.w, n);
-      const float lwj1 = __ldg(lw + j1);
-      if (metropolis_accept(lwk, lwj1, half_u01_f32(x.z))) {
+      const uint32_t j1 = half_index(x.z, x.w, n);
+      const float lwj1 = gather(j1);
+      if (metropolis_accept24(lwk, lwj1, half_u24(x.z))) {
         k = j1;
         lwk = lwj1;
       }
     }
   }
   return static_cast<int32_t>(k);
+}
+
+// The chain of particle i with its proposals gathered from the log-weights themselves.
+__device__ __forceinline__ int32_t metropolis_one(const float* __restrict__ lw, int64_t n,
+                                                  int32_t B, const Keys& keys, int64_t i,
+                                                  int* err) {
+  const float lwi = __ldg(lw + i);
+  if (nonfinite_logw(lwi)) flag_error(err, RS_ERR_NONFINITE);
+  return metropolis_chain(lwi, [&](uint32_t j) { return __ldg(lw + j); },
+                          static_cast<uint32_t>(n), B, keys, static_cast<uint32_t>(i));
 }
 
 __device__ __forceinline__ bool f64_step_accept(double lwk, float lwk_f, bool okk, long long kk,
@@ -215,7 +245,7 @@ __device__ __forceinline__ int32_t metropolis_one(const double* __restrict__ lw,
   bool okk = f64_to_f32_trunc(lwk, lwk_f);
   long long kk = f64_key(lwk);
   int64_t k = i;
-  const uint32_t ii = static_cast<uint32_t>(i);
+  const DrawRow row = draw_row(keys, static_cast<uint32_t>(i));
   int32_t s = 0;
   for (; s + kUnroll64 <= B; s += kUnroll64) {
     uint4 x[kUnroll64];
@@ -223,8 +253,8 @@ __device__ __forceinline__ int32_t metropolis_one(const double* __restrict__ lw,
     int64_t j[kUnroll64];
 #pragma unroll
     for (int q = 0; q < kUnroll64; ++q) {
-      x[q] = draw(keys, ii, static_cast<uint32_t>(s + q));
-      j[q] = uniform_index(x[q], n);
+      x[q] = draw(keys, row, static_cast<uint32_t>(s + q));
+      j[q] = uniform_index(x[q], static_cast<uint32_t>(n));
       lwj[q] = __ldg(lw + j[q]);
     }
 #pragma unroll
@@ -242,8 +272,8 @@ __device__ __forceinline__ int32_t metropolis_one(const double* __restrict__ lw,
     }
   }
   for (; s < B; ++s) {
-    const uint4 x = draw(keys, ii, static_cast<uint32_t>(s));
-    const int64_t j = uniform_index(x, n);
+    const uint4 x = draw(keys, row, static_cast<uint32_t>(s));
+    const int64_t j = uniform_index(x, static_cast<uint32_t>(n));
     const double lwj = __ldg(lw + j);
     const long long kj = f64_key(lwj);
     float lwj_f;
@@ -277,27 +307,25 @@ __device__ __forceinline__ bool sc_step_accept(const double* __restrict__ lw, in
                        [&] { return exact_f64_less_exp(__ldg(lw + j), __ldg(lw + k), x); });
 }
 
-// metropolis_one for binary64 log-weights with their sidecars lwf: the proposals gather
-// 4 bytes (lwf[j]) instead of 8; same ancestor as metropolis_one.
-__device__ __forceinline__ int32_t metropolis_one_sc(const double* __restrict__ lw,
-                                                     const float* __restrict__ lwf, int64_t n,
-                                                     int32_t B, const Keys& keys, int64_t i,
-                                                     int* err) {
-  const double lwi = __ldg(lw + i);
-  if (nonfinite_logw(lwi)) flag_error(err, RS_ERR_NONFINITE);
-  int64_t k = i;
-  float tk = f64_sidecar(lwi);
-  const uint32_t ii = static_cast<uint32_t>(i);
+// metropolis_chain for n < 2^31 binary64 log-weights lw from the state i with sidecar tk:
+// gather(j) reads the sidecar of proposal j (4 bytes instead of 8). Same ancestor as
+// metropolis_one on the binary64 values.
+template <typename Gather>
+__device__ __forceinline__ int32_t metropolis_chain_sc(const double* __restrict__ lw, float tk,
+                                                       const Gather& gather, uint32_t n,
+                                                       int32_t B, const Keys& keys, uint32_t i) {
+  uint32_t k = i;
+  const DrawRow row = draw_row(keys, i);
   int32_t s = 0;
   for (; s + kUnroll64 <= B; s += kUnroll64) {
     uint4 x[kUnroll64];
-    int64_t j[kUnroll64];
+    uint32_t j[kUnroll64];
     float tj[kUnroll64];
 #pragma unroll
     for (int q = 0; q < kUnroll64; ++q) {
-      x[q] = draw(keys, ii, static_cast<uint32_t>(s + q));
+      x[q] = draw(keys, row, static_cast<uint32_t>(s + q));
       j[q] = uniform_index(x[q], n);
-      tj[q] = __ldg(lwf + j[q]);
+      tj[q] = gather(j[q]);
     }
 #pragma unroll
     for (int q = 0; q < kUnroll64; ++q) {
@@ -308,15 +336,26 @@ __device__ __forceinline__ int32_t metropolis_one_sc(const double* __restrict__ 
     }
   }
   for (; s < B; ++s) {
-    const uint4 x = draw(keys, ii, static_cast<uint32_t>(s));
-    const int64_t j = uniform_index(x, n);
-    const float tj = __ldg(lwf + j);
+    const uint4 x = draw(keys, row, static_cast<uint32_t>(s));
+    const uint32_t j = uniform_index(x, n);
+    const float tj = gather(j);
     if (sc_step_accept(lw, k, tk, j, tj, x)) {
       k = j;
       tk = tj;
     }
   }
   return static_cast<int32_t>(k);
+}
+
+// The chain of particle i with its proposals gathered from the sidecars lwf in memory.
+__device__ __forceinline__ int32_t metropolis_one_sc(const double* __restrict__ lw,
+                                                     const float* __restrict__ lwf, int64_t n,
+                                                     int32_t B, const Keys& keys, int64_t i,
+                                                     int* err) {
+  const double lwi = __ldg(lw + i);
+  if (nonfinite_logw(lwi)) flag_error(err, RS_ERR_NONFINITE);
+  return metropolis_chain_sc(lw, f64_sidecar(lwi), [&](uint32_t j) { return __ldg(lwf + j); },
+                             static_cast<uint32_t>(n), B, keys, static_cast<uint32_t>(i));
 }
 
 // Rejection loop of particle i (Code 3): attempt 0 proposes j = i, attempt s >= 1 a uniform
@@ -336,7 +375,7 @@ __device__ __forceinline__ int32_t rejection_one(const float* __restrict__ lw, i
   for (int64_t s = 0; s < max_trials; ++s) {
     if ((s & 1) == 0) x = draw(keys, ii, static_cast<uint32_t>(s >> 1));
     const uint32_t w0 = (s & 1) ? x.z : x.x, w1 = (s & 1) ? x.w : x.y;
-    if (s > 0) j = half_index(w0, w1, n);
+    if (s > 0) j = half_index(w0, w1, static_cast<uint32_t>(n));
     const float u = half_u01_f32(w0);
     const float lwj = (s == 0) ? lwi : __ldg(lw + j);
     const float delta = lwj - lwmax;
@@ -363,7 +402,7 @@ __device__ __forceinline__ int32_t rejection_one(const double* __restrict__ lw, 
   int64_t j = i;
   for (int64_t s = 0; s < max_trials; ++s) {
     const uint4 x = draw(keys, ii, static_cast<uint32_t>(s));
-    if (s > 0) j = uniform_index(x, n);
+    if (s > 0) j = uniform_index(x, static_cast<uint32_t>(n));
     const double lwj = (s == 0) ? lwi : __ldg(lw + j);
     const long long kj = f64_key(lwj);
     if (kj > km && !is_nan(lwj)) {  // above the bound (NaN never compares)
@@ -410,17 +449,17 @@ __device__ __forceinline__ RejBound make_bound(double log_wmax, bool clamp = fal
   return r;
 }
 
-// Decision of one rejection attempt with uniform u (binary32) or draw x (binary64) and
+// Decision of one rejection attempt with uniform bits u24 (binary32) or draw x (binary64) and
 // proposal log-weight lwj: accept when u < exp(lw^j - log w_max); a log-weight above the bound
 // is flagged (unless clamped) and accepted.
-__device__ __forceinline__ bool rejection_accept(const RejBound& rb, float u, float lwj,
+__device__ __forceinline__ bool rejection_accept(const RejBound& rb, float u24, float lwj,
                                                  int* err) {
   const float delta = lwj - rb.lwmax_rn;
   if (delta > 0.0f) {
     if (!rb.clamp) flag_error(err, RS_ERR_BOUND_VIOLATED);
     return true;
   }
-  return delta == 0.0f || u_below_exp(u, delta);
+  return delta == 0.0f || u24_below_exp(u24, delta);
 }
 
 __device__ __forceinline__ bool rejection_accept(const RejBound& rb, uint4 x, double lwj,
@@ -473,7 +512,7 @@ __device__ __forceinline__ bool rejection_attempts(const T* __restrict__ lw, int
   for (int q = 0; q < K; ++q) {
     const uint32_t sq = s + static_cast<uint32_t>(q);
     x[q] = draw(keys, static_cast<uint32_t>(i), sq);
-    jq[q] = (sq > 0) ? uniform_index(x[q], n) : i;
+    jq[q] = (sq > 0) ? uniform_index(x[q], static_cast<uint32_t>(n)) : i;
     lwj[q] = (sq > 0) ? __ldg(lw + jq[q]) : lwi;
   }
 #pragma unroll
@@ -501,10 +540,10 @@ __device__ __forceinline__ bool rejection_attempts(const float* __restrict__ lw,
   for (int p = 0; p < K / 2; ++p) {
     const uint4 x = draw(keys, static_cast<uint32_t>(i), s / 2 + static_cast<uint32_t>(p));
     const uint32_t s0 = s + 2 * static_cast<uint32_t>(p);
-    jq[2 * p] = (s0 > 0) ? half_index(x.x, x.y, n) : i;
-    u[2 * p] = half_u01_f32(x.x);
-    jq[2 * p + 1] = half_index(x.z, x.w, n);
-    u[2 * p + 1] = half_u01_f32(x.z);
+    jq[2 * p] = (s0 > 0) ? half_index(x.x, x.y, static_cast<uint32_t>(n)) : i;
+    u[2 * p] = half_u24(x.x);
+    jq[2 * p + 1] = half_index(x.z, x.w, static_cast<uint32_t>(n));
+    u[2 * p + 1] = half_u24(x.z);
     lwj[2 * p] = (s0 > 0) ? __ldg(lw + jq[2 * p]) : lwi;
     lwj[2 * p + 1] = __ldg(lw + jq[2 * p + 1]);
   }
@@ -534,7 +573,7 @@ __device__ __forceinline__ bool rejection_attempts_sc(const double* __restrict__
   for (int q = 0; q < K; ++q) {
     const uint32_t sq = s + static_cast<uint32_t>(q);
     x[q] = draw(keys, static_cast<uint32_t>(i), sq);
-    jq[q] = (sq > 0) ? uniform_index(x[q], n) : i;
+    jq[q] = (sq > 0) ? uniform_index(x[q], static_cast<uint32_t>(n)) : i;
     tj[q] = (sq > 0) ? __ldg(lwf + jq[q]) : ti;
   }
 #pragma unroll
