@@ -21,6 +21,7 @@
 // random-number counter: filter f of a batched call equals rs_resample on that filter's slice
 // with filter = f, bit for bit.
 #include <climits>
+#include <mutex>
 
 #include "common.cuh"
 #include "grid.cuh"
@@ -58,6 +59,23 @@ __device__ __forceinline__ int filter_of(const int64_t* __restrict__ off, int F,
   while (hi - lo > 1) {
     const int mid = (lo + hi) >> 1;
     if (__ldg(off + mid) <= g) lo = mid; else hi = mid;
+  }
+  return lo;
+}
+
+// filter_of for one position g, by a whole warp (every lane calls it with the same g): 32
+// offsets are compared at a time, so 4096 filters take three dependent loads instead of twelve.
+template <typename I>
+__device__ __forceinline__ int filter_of_warp(const I* __restrict__ off, int F, I g) {
+  const int lane = threadIdx.x & 31;
+  int lo = 0, hi = F;  // invariant: off[lo] <= g < off[hi]
+  while (hi - lo > 1) {
+    const int step = (hi - lo + 31) >> 5;
+    const int at = lo + (lane + 1) * step;
+    const bool below = at < hi && __ldg(off + at) <= g;
+    const int cnt = __popc(__ballot_sync(0xffffffffu, below));
+    lo += cnt * step;
+    hi = min(hi, lo + step);
   }
   return lo;
 }
@@ -493,42 +511,252 @@ batch_search_kernel(const V* __restrict__ W, Batch b, int64_t total, Keys base_k
   if (d) atomicMin(d + P.lo + k, static_cast<int32_t>(P.i));
 }
 
-// Claims start from the sentinel n of each particle's filter. Eight consecutive particles per
-// thread: the filter of the first is found by binary search (filter_of) and the others by
-// stepping past the offsets they cross; each particle gets what locate_particle gives it
-// (nothing when it fails), stored 128 bits at a time where all eight are set.
+// The claims' sentinels: d[g] = n of particle g's filter, for the positions [g0, g0 + 256) of one
+// warp (eight consecutive per lane), whose filter is looked up once; across a filter boundary
+// each position's filter is found by stepping past the offsets it crosses. Positions that
+// locate_in rejects get nothing.
 constexpr int kFillPer = 8;
-__global__ void __launch_bounds__(kBlock)
-batch_fill_sentinel_kernel(const int64_t* __restrict__ off, int F, int64_t total,
-                           int32_t* __restrict__ d) {
-  pdl_wait();
-  const int64_t g0 = kFillPer * (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x);
-  const int64_t offF = __ldg(off + F);
-  const int64_t end = offF < total ? offF : total;
-  if (g0 >= end) return;
-  int f = filter_of(off, F, g0);
-  int32_t v[kFillPer];
-  unsigned set = 0;
-#pragma unroll
+__device__ __forceinline__ void fill_sentinels_warp(const int64_t* __restrict__ off, int F,
+                                                    int64_t total, int64_t end, int64_t gw,
+                                                    int32_t* __restrict__ d) {
+  if (gw >= end) return;  // (uniform over the warp)
+  int f = filter_of_warp(off, F, gw);
+  const int64_t g0 = gw + kFillPer * static_cast<int64_t>(threadIdx.x & 31);
+  PartLoc P;
+  if (locate_in(off, f, total, gw, P) && P.i + 32 * kFillPer <= P.n && gw + 32 * kFillPer <= end &&
+      (reinterpret_cast<uintptr_t>(d + g0) & 15u) == 0) {
+    const int32_t n = static_cast<int32_t>(P.n);
+    int4* const p4 = reinterpret_cast<int4*>(d + g0);
+    p4[0] = make_int4(n, n, n, n);
+    p4[1] = make_int4(n, n, n, n);
+    return;
+  }
   for (int q = 0; q < kFillPer; ++q) {
     const int64_t g = g0 + q;
-    v[q] = 0;
-    if (g >= end) continue;
+    if (g >= end) break;
     f = advance_filter(off, F, g, f);
-    PartLoc P;
-    if (locate_in(off, f, total, g, P)) {
-      v[q] = static_cast<int32_t>(P.n);
-      set |= 1u << q;
-    }
+    if (locate_in(off, f, total, g, P)) d[g] = static_cast<int32_t>(P.n);
   }
-  if (set == (1u << kFillPer) - 1u && (reinterpret_cast<uintptr_t>(d + g0) & 15u) == 0) {
-    int4* const p4 = reinterpret_cast<int4*>(d + g0);
-    p4[0] = make_int4(v[0], v[1], v[2], v[3]);
-    p4[1] = make_int4(v[4], v[5], v[6], v[7]);
-  } else {
+}
+
+// Metropolis steps of filter f (a negative B counts as 0; flagged by the plan).
+__device__ __forceinline__ int32_t filter_steps(const int32_t* __restrict__ Bf, int32_t B, int f) {
+  const int32_t v = Bf ? __ldg(Bf + f) : B;
+  return v < 0 ? 0 : v;
+}
+
+// Work of one particle of the batched chains, in units of a chain's step: its B steps and what a
+// particle costs besides (its first draw products, log-weight, result and claim).
+constexpr int kParticleSteps = 8;
+__device__ __forceinline__ unsigned long long particle_work(const uint8_t* flags,
+                                                            const int32_t* __restrict__ Bf,
+                                                            int32_t B, int f) {
+  return resampled(flags, f) ? static_cast<unsigned long long>(filter_steps(Bf, B, f)) + kParticleSteps
+                             : 2ull;
+}
+
+// Plan of the batched chains (CTA 0): the exclusive prefix over the filters of their work,
+// work[0 .. F], and the chunk counter reset; malformed filters and negative B are flagged and
+// get no work. The other CTAs (every CTA when work is null) write the claims' sentinels (d given).
+constexpr int kChainBlock = 1024;
+__global__ void __launch_bounds__(kChainBlock)
+batch_chain_plan_kernel(const int64_t* __restrict__ off, int F, int64_t total,
+                        const int32_t* __restrict__ Bf, int32_t B,
+                        const uint8_t* __restrict__ flags, unsigned long long* work,
+                        unsigned int* counter, int32_t* __restrict__ d, int* err) {
+  pdl_wait();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int planners = work ? 1 : 0;
+  if (static_cast<int>(blockIdx.x) >= planners) {
+    const int64_t offF = __ldg(off + F);
+    const int64_t end = offF < total ? offF : total;
+    const int64_t warps = static_cast<int64_t>(gridDim.x - planners) * (kChainBlock / 32);
+    for (int64_t w = static_cast<int64_t>(blockIdx.x - planners) * (kChainBlock / 32) + warp;
+         w * (32 * kFillPer) < end; w += warps)
+      fill_sentinels_warp(off, F, total, end, w * (32 * kFillPer), d);
+    return;
+  }
+  __shared__ unsigned long long sh[kChainBlock / 32];
+  const int chunk = (F + kChainBlock - 1) / kChainBlock;
+  const int f0 = min(F, static_cast<int>(threadIdx.x) * chunk), f1 = min(F, f0 + chunk);
+  auto filter_work = [&](int f) -> unsigned long long {
+    const int64_t lo = __ldg(off + f), hi = __ldg(off + f + 1), n = hi - lo;
+    if (!(lo >= 0 && n >= 0 && hi <= total && n <= kBatchMaxN)) return ~0ull;
+    return static_cast<unsigned long long>(n) * particle_work(flags, Bf, B, f);
+  };
+  unsigned long long local = 0;
+  for (int f = f0; f < f1; ++f) {
+    const unsigned long long w = filter_work(f);
+    if (w == ~0ull) flag_error(err, RS_ERR_ARG);
+    else local += w;
+    if (resampled(flags, f) && (Bf ? __ldg(Bf + f) : B) < 0 && w != ~0ull && w > 0)
+      flag_error(err, RS_ERR_ARG);
+  }
+  unsigned long long incl = local;
 #pragma unroll
-    for (int q = 0; q < kFillPer; ++q)
-      if ((set >> q) & 1u) d[g0 + q] = v[q];
+  for (int dd = 1; dd < 32; dd <<= 1) {
+    const unsigned long long y = __shfl_up_sync(0xffffffffu, incl, dd);
+    if (lane >= dd) incl += y;
+  }
+  if (lane == 31) sh[warp] = incl;
+  __syncthreads();
+  unsigned long long p = incl - local;
+  for (int k = 0; k < warp; ++k) p += sh[k];
+  for (int f = f0; f < f1; ++f) {
+    work[f] = p;
+    const unsigned long long w = filter_work(f);
+    if (w != ~0ull) p += w;
+  }
+  if (f1 == F && f0 < F) work[F] = p;
+  if (threadIdx.x == 0) *counter = 0u;
+}
+
+// ---------------------------------------------------------------------------------------
+// Metropolis chains of all filters with the log-weights in shared memory.
+//
+// A chain's proposals are random 4-byte reads of its filter's log-weights. With one thread per
+// particle and CTAs of any filter on an SM, half of those reads missed L1 and the kernel ran at
+// the L2's rate of random sectors (4096 filters of 256 .. 65536 particles, 2.5 G steps: 5.3 ms).
+// Here one CTA of 1024 threads per SM stages the log-weights of a window of whole filters (up to
+// kChainCap values, 224 KB; of a longer filter the first kChainCap, the rest is read from
+// memory) and runs the chains of its particles from there (4.05 ms: 42 instructions and 61 cycles
+// a step on each SM quarter, of which the 8 wide products of its half Philox block and the
+// product of its index take about 45 in the multiplier: 5 and 4 cycles each, measured).
+//
+// The particles of the batch are cut into chunks of equal work (steps plus kParticleSteps a
+// particle, batch_chain_plan_kernel), taken in order from a counter: the first half of the
+// chunks covers 9/10 of the work, the second half the rest, so that the last one to end is
+// short. A chunk holds whole turns of the CTA's 1024 chains where it can: the end of a window
+// waits for its slowest warp (32 chunks per CTA instead of 16: 4.65 against 4.51 ms a call). Inside a window every warp takes the next 32 particles from a shared
+// counter (filters of one window may differ in B). Every particle's chain and claim are those of
+// batch_mcmc_kernel.
+// ---------------------------------------------------------------------------------------
+static_assert(kBatchMaxN < (1 << 24), "half_index<true>");
+constexpr int kChainCap = 57344;                            // staged log-weights
+constexpr size_t kChainSmem = sizeof(float) * (kChainCap + 4);  // (+ the alignment shift)
+constexpr int kChainChunks = 16;                            // chunks per CTA, at most
+
+__global__ void __launch_bounds__(kChainBlock, 1)
+batch_chain_kernel(const float* __restrict__ lw, const int64_t* __restrict__ off, int F,
+                   int64_t total, const int32_t* __restrict__ Bf, int32_t B, Keys base_keys,
+                   const uint8_t* __restrict__ flags,
+                   const unsigned long long* __restrict__ work, unsigned int* counter,
+                   int32_t* __restrict__ a, int32_t* __restrict__ d, int* err) {
+  pdl_wait();
+  extern __shared__ __align__(16) float sh_lw[];
+  __shared__ unsigned int sh_chunk, sh_group;
+  __shared__ int sh_f[2], sh_i[2];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const unsigned long long W = __ldg(work + F);
+  if (W == 0) return;
+  // chunks: four turns of the CTA's threads each where there are (one turn: 243 against 175 us for
+  // 150 filters of 256 .. 65536, the chunks of the highest B too few chains for the CTA), at
+  // least one per CTA
+  const int64_t offF = __ldg(off + F);
+  const unsigned long long G = gridDim.x;
+  unsigned long long K = static_cast<unsigned long long>(offF < total ? offF : total) / (4 * kChainBlock);
+  K = K < G ? G : K > kChainChunks * G ? kChainChunks * G : K;
+  const bool tapered = K >= 8 * G;  // (fewer chunks: all alike)
+  const unsigned long long K1 = tapered ? K / 2 : K, W1 = tapered ? W / 10 * 9 : W;
+  for (;;) {
+    __syncthreads();  // (the previous chunk's shared state has been read)
+    if (threadIdx.x == 0) sh_chunk = atomicAdd(counter, 1u);
+    __syncthreads();
+    const unsigned long long c = sh_chunk;
+    if (c >= K) return;
+    if (warp < 2) {  // the chunk's first particle (warp 0) and the next chunk's (warp 1)
+      const unsigned long long b = c + warp;
+      const unsigned long long X = b < K1 ? W1 / K1 * b : b < K ? W1 + (W - W1) / (K - K1) * (b - K1)
+                                                               : W;
+      int f = F, i = 0;
+      if (X < W) {
+        f = filter_of_warp(work, F, X);
+        // whole turns of the CTA's threads where a chunk holds several, else whole warps
+        const unsigned long long per = particle_work(flags, Bf, B, f);
+        const int turn = W / K >= 4 * kChainBlock * per ? kChainBlock : 32;
+        i = static_cast<int>((X - __ldg(work + f)) / per) & -turn;
+      }
+      if (lane == 0) {
+        sh_f[warp] = f;
+        sh_i[warp] = i;
+      }
+    }
+    __syncthreads();
+    int f = sh_f[0], i = sh_i[0];
+    const int fe = sh_f[1], ie = sh_i[1];
+    while (f < fe || (f == fe && i < ie)) {  // one window of filters (uniform over the CTA)
+      const int64_t lo = __ldg(off + f), n = __ldg(off + f + 1) - lo;
+      if (__ldg(work + f + 1) == __ldg(work + f)) {  // empty or malformed: no particles
+        ++f;
+        i = 0;
+        continue;
+      }
+      // the last filter f1 of the window: whole filters while they fit, up to the chunk's end
+      int f1 = f;
+      {
+        int hi = ie > 0 ? fe : fe - 1;  // (the last filter with particles of this chunk)
+        while (f1 < hi) {
+          const int mid = (f1 + hi + 1) >> 1;
+          const int64_t e = __ldg(off + mid + 1), len = e - lo;
+          if (len <= kChainCap && len >= n && e <= total) f1 = mid; else hi = mid - 1;
+        }
+      }
+      const int64_t len = __ldg(off + f1 + 1) - lo;
+      const bool whole = len <= kChainCap;
+      const int staged = static_cast<int>(whole ? len : kChainCap);
+      const int pad = static_cast<int>(lo & 3);  // shared index = particle - lo + pad
+      __syncthreads();  // (the previous window has been read)
+      if (threadIdx.x == 0) sh_group = 0u;
+      if ((reinterpret_cast<uintptr_t>(lw) & 15u) == 0) {  // 128-bit loads of whole quadruples
+        const float4* const src = reinterpret_cast<const float4*>(lw + (lo - pad));
+        const int q1 = (staged + pad) >> 2;  // quadruples that end inside the window
+        float4* const dst = reinterpret_cast<float4*>(sh_lw);
+#pragma unroll 4
+        for (int q = threadIdx.x; q < q1; q += kChainBlock) dst[q] = __ldg(src + q);
+        for (int e = 4 * q1 + threadIdx.x; e < staged + pad; e += kChainBlock)
+          if (e >= pad) sh_lw[e] = __ldg(lw + (lo - pad) + e);
+      } else {
+        for (int e = threadIdx.x; e < staged; e += kChainBlock) sh_lw[e + pad] = __ldg(lw + lo + e);
+      }
+      __syncthreads();
+      const int64_t ps = lo + i, pe = f1 == fe ? __ldg(off + fe) + ie : lo + len;
+      for (;;) {
+        unsigned int grp = 0;
+        if (lane == 0) grp = atomicAdd(&sh_group, 1u);
+        grp = __shfl_sync(0xffffffffu, grp, 0);
+        const int64_t gw = ps + 32 * static_cast<int64_t>(grp);
+        if (gw >= pe) break;
+        const int64_t g = gw + lane;
+        if (g < pe) {
+          int ff = f;
+          if (f1 > f) ff = f + filter_of(off + f, f1 + 1 - f, g);
+          PartLoc P;
+          if (locate_in(off, ff, total, g, P)) {
+            const uint32_t un = static_cast<uint32_t>(P.n), ui = static_cast<uint32_t>(P.i);
+            const float* const sw = sh_lw + (pad + static_cast<int>(P.lo - lo));
+            int32_t k = static_cast<int32_t>(P.i);  // (not resampled: keeps its particle)
+            if (resampled(flags, ff)) {
+              const int32_t Bv = filter_steps(Bf, B, ff);
+              const Keys keys = with_tag(base_keys, static_cast<uint32_t>(ff), RS_METROPOLIS);
+              const float lwi = __ldg(lw + g);
+              if (nonfinite_logw(lwi)) flag_error(err, RS_ERR_NONFINITE);
+              const float* const lf = lw + P.lo;
+              auto all = [&](uint32_t j) { return sw[j]; };
+              auto part = [&](uint32_t j) {
+                return j < static_cast<uint32_t>(kChainCap) ? sw[j] : __ldg(lf + j);
+              };
+              k = whole ? metropolis_chain<true>(lwi, all, un, Bv, keys, ui)
+                        : metropolis_chain<true>(lwi, part, un, Bv, keys, ui);
+            }
+            a[g] = k;
+            if (d) atomicMin(d + P.lo + k, static_cast<int32_t>(P.i));
+          }
+        }
+        __syncwarp();
+      }
+      f = f1 + 1;
+      i = 0;
+    }
   }
 }
 
@@ -538,14 +766,12 @@ __device__ __forceinline__ int64_t item_index(int ipt, int q) {
   return (static_cast<int64_t>(blockIdx.x) * ipt + q) * blockDim.x + threadIdx.x;
 }
 
-// Metropolis (or one-particle-per-thread rejection) over the particles of all filters, ipt
-// particles per thread (the launch shape is tunable; every particle's chain and claim are the
-// same for any shape).
+// Metropolis over the particles of all filters, ipt particles per thread, one thread per particle
+// (the launch shape is tunable; every particle's chain and claim are the same for any shape).
 template <typename T>
 __global__ void __launch_bounds__(kMaxTunedBlock)
 batch_mcmc_kernel(const T* __restrict__ lw, const int64_t* __restrict__ off, int F,
-                  int64_t total, int scheme, const int32_t* __restrict__ Bf, int32_t B,
-                  Keys base_keys, double log_wmax, int64_t max_trials,
+                  int64_t total, const int32_t* __restrict__ Bf, int32_t B, Keys base_keys,
                   const uint8_t* __restrict__ flags, int32_t* __restrict__ a,
                   int32_t* __restrict__ d, int ipt, int* err) {
   pdl_wait();
@@ -560,17 +786,15 @@ batch_mcmc_kernel(const T* __restrict__ lw, const int64_t* __restrict__ off, int
     int32_t k;
     if (!resampled(flags, P.f)) {
       k = static_cast<int32_t>(P.i);  // the filter keeps its particles
-    } else if (scheme == RS_METROPOLIS) {
+    } else {
       int32_t Bv = Bf ? __ldg(Bf + P.f) : B;
       if (Bv < 0) {
         flag_error(err, RS_ERR_ARG);
         Bv = 0;
       }
       const Keys keys = with_tag(base_keys, static_cast<uint32_t>(P.f), RS_METROPOLIS);
-      k = metropolis_one(lw + P.lo, P.n, Bv, keys, P.i, err);
-    } else {
-      const Keys keys = with_tag(base_keys, static_cast<uint32_t>(P.f), RS_REJECTION);
-      k = rejection_one(lw + P.lo, P.n, log_wmax, max_trials, keys, P.i, err);
+      if constexpr (sizeof(T) == 4) k = metropolis_one<true>(lw + P.lo, P.n, Bv, keys, P.i, err);
+      else k = metropolis_one(lw + P.lo, P.n, Bv, keys, P.i, err);
     }
     a[g] = k;
     if (d) atomicMin(d + P.lo + k, static_cast<int32_t>(P.i));
@@ -644,33 +868,24 @@ batch_rejection_kernel(const T* __restrict__ lw, const int64_t* __restrict__ off
   }
 }
 
-// filter_of for one position g, by a whole warp (every lane calls it with the same g): 32
-// offsets are compared at a time, so 4096 filters take three dependent loads instead of twelve.
-__device__ __forceinline__ int filter_of_warp(const int64_t* __restrict__ off, int F, int64_t g) {
-  const int lane = threadIdx.x & 31;
-  int lo = 0, hi = F;  // invariant: off[lo] <= g < off[hi]
-  while (hi - lo > 1) {
-    const int step = (hi - lo + 31) >> 5;
-    const int at = lo + (lane + 1) * step;
-    const bool below = at < hi && __ldg(off + at) <= g;
-    const int cnt = __popc(__ballot_sync(0xffffffffu, below));
-    lo += cnt * step;
-    hi = min(hi, lo + step);
-  }
-  return lo;
-}
-
-// Permute of every filter: each warp takes 128 consecutive slots of the batch (four per lane),
-// ipt times (tunable launch shape). Nearly every warp lies inside one filter: its filter is
+// Permute of every filter: each warp takes 32 K consecutive slots of the batch, ipt times
+// (tunable launch shape). Nearly every warp lies inside one filter: its filter is
 // looked up once per warp and its slots run as in the single-filter kernels (permute4_slots;
 // SORTED: permute_sorted_slots, the non-decreasing ancestries of stratified and systematic from
 // the claimed bits cl of their emission, filter f's bytes at (offsets[f] >> 3) + f). A warp that
 // meets a filter boundary takes its slots one by one. Bound by L2 latency of the claims and
 // walks, as in the single-filter kernels; looking the filter up per slot instead (a binary
 // search of the offsets each) took 350 instructions per slot.
-constexpr int kPermSlots = 4;                         // consecutive slots per lane
-constexpr size_t kPermSmemPerWarp = 128 * (sizeof(int2) + sizeof(int32_t));
-template <bool SORTED>
+//
+// K slots per lane: four for large batches; one for small ones, where it keeps more threads in
+// flight (50 filters of up to 5000: 30.8 against 34.9 us a call).
+constexpr int64_t kBatchSorted4MinN = int64_t{1} << 18;
+constexpr int64_t kBatchPermute4MinN = int64_t{1} << 20;
+template <int K>
+constexpr size_t perm_smem_per_warp() {
+  return 32 * K * (sizeof(int2) + sizeof(int32_t));
+}
+template <bool SORTED, int K>
 __global__ void __launch_bounds__(kMaxTunedBlock)
 batch_permute_kernel(const int64_t* __restrict__ off, int F, int64_t total,
                      const int32_t* __restrict__ a, const int32_t* __restrict__ d,
@@ -678,30 +893,32 @@ batch_permute_kernel(const int64_t* __restrict__ off, int F, int64_t total,
   pdl_wait();
   extern __shared__ __align__(16) unsigned char sh_perm[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  int32_t* const cw = reinterpret_cast<int32_t*>(sh_perm + warp * kPermSmemPerWarp);
-  int2* const pend = reinterpret_cast<int2*>(cw + 128);
+  int32_t* const cw = reinterpret_cast<int32_t*>(sh_perm + warp * perm_smem_per_warp<K>());
+  int2* const pend = reinterpret_cast<int2*>(cw + 32 * K);
   const int64_t offF = __ldg(off + F);
   const int64_t end = offF < total ? offF : total;
   for (int q = 0; q < ipt; ++q) {
-    // first slot of this warp (of this lane: kPermSlots * lane further)
-    const int64_t gw = kPermSlots * ((static_cast<int64_t>(blockIdx.x) * ipt + q) * blockDim.x +
-                                     32 * static_cast<int64_t>(warp));
+    // first slot of this warp (of this lane: K * lane further)
+    const int64_t gw = K * ((static_cast<int64_t>(blockIdx.x) * ipt + q) * blockDim.x +
+                            32 * static_cast<int64_t>(warp));
     if (gw >= end) return;  // (uniform over the warp)
     const int f = filter_of_warp(off, F, gw);
-    const int64_t g0 = gw + kPermSlots * lane;
+    const int64_t g0 = gw + K * lane;
     PartLoc P;
     const bool ok = locate_in(off, f, total, gw, P);  // (uniform over the warp)
-    if (ok && P.i + 32 * kPermSlots <= P.n) {
+    if (ok && P.i + 32 * K <= P.n) {
       if constexpr (SORTED)
-        permute_sorted_slots<kPermSlots>(a + P.lo, cl + (P.lo >> 3) + f, P.n, c + P.lo, g0 - P.lo,
-                                         cw, pend, err);
-      else
+        permute_sorted_slots<K>(a + P.lo, cl + (P.lo >> 3) + f, P.n, c + P.lo, g0 - P.lo, cw, pend,
+                                err);
+      else if constexpr (K == 4)
         permute4_slots(a + P.lo, d + P.lo, P.n, c + P.lo, g0 - P.lo, pend, err);
+      else
+        permute_one(a + P.lo, d + P.lo, P.n, c + P.lo, g0 - P.lo, err);
       __syncwarp();  // (the warp's shared lists are rewritten by its next slots)
       continue;
     }
     int fs = f;
-    for (int k = 0; k < kPermSlots; ++k) {
+    for (int k = 0; k < K; ++k) {
       const int64_t g = g0 + k;
       if (g >= end) break;
       fs = advance_filter(off, F, g, fs);
@@ -720,6 +937,31 @@ inline int grid_particles(int64_t cap) { return static_cast<int>((cap + kBlock -
 inline int grid_shaped(int64_t cap, const LaunchCfg& c) {
   const int64_t per = static_cast<int64_t>(c.block) * c.ipt;
   return static_cast<int>((cap + per - 1) / per);
+}
+
+// CTAs that write the claims' sentinels beside the plan: 32 warps each, 256 positions a warp and
+// turn, two CTAs per SM at most.
+inline int fill_grid(int64_t cap) {
+  const int64_t want = (cap + 32 * kFillPer * (kChainBlock / 32) - 1) /
+                       (32 * kFillPer * (kChainBlock / 32));
+  const int64_t most = 2 * static_cast<int64_t>(device_sm_count());
+  return static_cast<int>(want < most ? want : most);
+}
+
+// Whether the current device grants batch_chain_kernel its shared memory (asked once per device).
+inline bool chain_available() {
+  static std::mutex mu;
+  static int known[64] = {};  // 0: not asked, 1: yes, 2: no
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
+  std::lock_guard<std::mutex> lock(mu);
+  if (known[dev] == 0) {
+    const cudaError_t e = cudaFuncSetAttribute(
+        batch_chain_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kChainSmem));
+    if (e != cudaSuccess) cudaGetLastError();  // (not an error of the call: the other kernel runs)
+    known[dev] = e == cudaSuccess ? 1 : 2;
+  }
+  return known[dev] == 1;
 }
 
 const char* const kLblSum[4] = {"batch_sum_f32", "batch_sum_f32c", "batch_sum_f64", "batch_sum_f64n"};
@@ -821,11 +1063,19 @@ cudaError_t launch_batched(const Scratch& s, int scheme, Acc acc, const void* lo
   const int64_t total = s.max_n;
   cudaError_t e = cudaSuccess;
   if (scheme == RS_METROPOLIS || scheme == RS_REJECTION) {
-    if (d) {
+    const LaunchCfg& mc = s.batch_cfg[f64 ? kCfgMetropolisF64 : kCfgMetropolisF32];
+    // binary32: the staged chains at the default launch shape; another shape (set or tuned), and
+    // binary64, whose chains are bound by their draws (a block a step) and gained nothing from
+    // staged sidecars (1000 filters of 256 .. 65536: 2975 against 2946 us; 64 of 64 .. 8000: 128
+    // against 116), run one thread per particle
+    const bool staged = scheme == RS_METROPOLIS && !f64 && mc.block == kBlock && mc.ipt == 1 &&
+                        chain_available();
+    auto* work = reinterpret_cast<unsigned long long*>(s.batch_fS);  // F + 1 <= 2 max_filters
+    if (d || staged) {
       trace_mark(s.trace, "batch_fill", st);
-      launch_pdl(batch_fill_sentinel_kernel,
-                 static_cast<int>((total + kFillPer * kBlock - 1) / (kFillPer * kBlock)), kBlock, st,
-                 offsets, F, total, d);
+      launch_pdl(batch_chain_plan_kernel, (staged ? 1 : 0) + (d ? fill_grid(total) : 0),
+                 kChainBlock, st, offsets, F, total, Bf, B, flags, staged ? work : nullptr,
+                 &s.glob->batch_next, d, s.err);
     }
     trace_mark(s.trace, scheme == RS_METROPOLIS ? (f64 ? "batch_metropolis_f64" : "batch_metropolis_f32")
                                                 : (f64 ? "batch_rejection_f64" : "batch_rejection_f32"),
@@ -841,16 +1091,18 @@ cudaError_t launch_batched(const Scratch& s, int scheme, Acc acc, const void* lo
         launch_pdl(batch_rejection_kernel<float>, grid_runs, kBlock, st,
             static_cast<const float*>(logw), offsets, F, total, keys, log_wmax, max_trials,
             flags, a, d, s.err);
+    } else if (staged) {
+      launch_pdl_smem(batch_chain_kernel, device_sm_count(), kChainBlock, kChainSmem, st,
+                      static_cast<const float*>(logw), offsets, F, total, Bf, B, keys, flags, work,
+                      &s.glob->batch_next, a, d, s.err);
     } else if (f64) {
-      const LaunchCfg& c = s.batch_cfg[kCfgMetropolisF64];
-      launch_pdl(batch_mcmc_kernel<double>, grid_shaped(total, c), c.block, st,
-          static_cast<const double*>(logw), offsets, F, total, scheme, Bf, B, keys, log_wmax,
-          max_trials, flags, a, d, c.ipt, s.err);
+      launch_pdl(batch_mcmc_kernel<double>, grid_shaped(total, mc), mc.block, st,
+                 static_cast<const double*>(logw), offsets, F, total, Bf, B, keys, flags, a, d,
+                 mc.ipt, s.err);
     } else {
-      const LaunchCfg& c = s.batch_cfg[kCfgMetropolisF32];
-      launch_pdl(batch_mcmc_kernel<float>, grid_shaped(total, c), c.block, st,
-          static_cast<const float*>(logw), offsets, F, total, scheme, Bf, B, keys, log_wmax,
-          max_trials, flags, a, d, c.ipt, s.err);
+      launch_pdl(batch_mcmc_kernel<float>, grid_shaped(total, mc), mc.block, st,
+                 static_cast<const float*>(logw), offsets, F, total, Bf, B, keys, flags, a, d,
+                 mc.ipt, s.err);
     }
   } else {
     Batch b;
@@ -894,10 +1146,12 @@ cudaError_t launch_batched(const Scratch& s, int scheme, Acc acc, const void* lo
   if (e == cudaSuccess && permute) {
     trace_mark(s.trace, "batch_permute", st);
     const LaunchCfg& c = s.batch_cfg[kCfgPermute];
-    const int grid = grid_shaped((total + kPermSlots - 1) / kPermSlots, c);
-    const size_t smem = kPermSmemPerWarp * (c.block / 32);
-    launch_pdl_smem(cl ? batch_permute_kernel<true> : batch_permute_kernel<false>, grid, c.block,
-                    smem, st, offsets, F, total, s.a_tmp, s.d, cl, out, c.ipt, s.err);
+    const bool four = total >= (cl ? kBatchSorted4MinN : kBatchPermute4MinN);
+    const int grid = grid_shaped(four ? (total + 3) / 4 : total, c);
+    const size_t smem = (four ? perm_smem_per_warp<4>() : perm_smem_per_warp<1>()) * (c.block / 32);
+    launch_pdl_smem(cl ? (four ? batch_permute_kernel<true, 4> : batch_permute_kernel<true, 1>)
+                       : (four ? batch_permute_kernel<false, 4> : batch_permute_kernel<false, 1>),
+                    grid, c.block, smem, st, offsets, F, total, s.a_tmp, s.d, cl, out, c.ipt, s.err);
     e = cudaGetLastError();
   }
   return e;

@@ -130,19 +130,19 @@ __device__ __forceinline__ uint32_t uniform_index(uint4 x, uint32_t n) {
 }
 
 // The two step halves of a binary32 Metropolis block (h = 0: words 0, 1; h = 1: words 2, 3):
-// the uniform is the top 24 bits of the first word times 2^-24 (half_u24: those bits as a
-// binary32 integer, exact), the proposal floor(V n / 2^40) with V = (the first word's low
-// byte) 2^32 + the second word, for n < 2^31. With V = 256 T + r (r the low byte) the proposal
-// is floor((T n + floor(r n / 256)) / 2^32), and with n = 256 n1 + n0 the inner quotient is
-// r n1 + floor(r n0 / 256): one 32x32->64 product instead of two 64-bit ones.
-__device__ __forceinline__ float half_u24(uint32_t w0) { return __uint2float_rn(w0 >> 8); }
+// the uniform is the top 24 bits of the first word times 2^-24, the proposal floor(V n / 2^40)
+// with V = b 2^32 + w1, b the first word's low byte and w1 the second word, for n < 2^31. With
+// V n = (b n + floor(w1 n / 2^32)) 2^32 + ... (the rest cannot carry past bit 40) the proposal is
+// (b n + hi(w1 n)) / 2^8 rounded down; the sum is below 2^8 n, so 32 bits hold it for n <= 2^24
+// (SMALL).
 __device__ __forceinline__ float half_u01_f32(uint32_t w0) {
-  return __fmul_rn(half_u24(w0), 0x1p-24f);
+  return __fmul_rn(__uint2float_rn(w0 >> 8), 0x1p-24f);
 }
+template <bool SMALL>
 __device__ __forceinline__ uint32_t half_index(uint32_t w0, uint32_t w1, uint32_t n) {
-  const uint32_t T = __funnelshift_r(w1, w0, 8), r = w1 & 0xffu;
-  const uint32_t x = r * (n >> 8) + ((r * (n & 0xffu)) >> 8);
-  return static_cast<uint32_t>((static_cast<uint64_t>(T) * n + x) >> 32);
+  const uint32_t b = w0 & 0xffu;
+  if constexpr (SMALL) return (b * n + __umulhi(w1, n)) >> 8;
+  return static_cast<uint32_t>((static_cast<uint64_t>(b) * n + __umulhi(w1, n)) >> 8);
 }
 
 // ---------------------------------------------------------------------------------------

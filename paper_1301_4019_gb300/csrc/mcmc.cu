@@ -22,33 +22,21 @@ namespace {
 // slower: their four proposals in flight need them).
 template <typename T> constexpr int metropolis_min_ctas() { return sizeof(T) == 4 ? 6 : 1; }
 
-// One thread per particle. COOP: a persistent cooperative grid that first sets the claims to
-// the sentinel N (the Prepermute initialisation), meets at a grid barrier, then runs the
-// chains over a grid-stride loop -- one launch instead of a fill and the chains.
-// Binary64 log-weights come with their sidecars lwf (f64_sidecar; sidecar_kernel), which the
-// chains gather instead of the binary64 values.
-template <typename T, bool COOP>
+// One thread per particle (the claims d, when given, were set to the sentinel N before). SMALL:
+// N < 2^24. Binary64 log-weights come with their sidecars lwf (f64_sidecar; sidecar_kernel),
+// which the chains gather instead of the binary64 values.
+template <typename T, bool SMALL>
 __global__ void __launch_bounds__(kBlock, metropolis_min_ctas<T>())
 metropolis_kernel(const T* __restrict__ lw, const float* __restrict__ lwf, int64_t N, int32_t B,
-                  Keys keys, int32_t* __restrict__ a, int32_t* __restrict__ d, GridBar* bar,
-                  int* err) {
+                  Keys keys, int32_t* __restrict__ a, int32_t* __restrict__ d, int* err) {
   pdl_wait();
-  const int64_t t0 = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  const int64_t stride = COOP ? static_cast<int64_t>(gridDim.x) * blockDim.x : N;
-  unsigned int target = 0;
-  if constexpr (COOP) {
-    if (d)
-      for (int64_t i = t0; i < N; i += stride) d[i] = static_cast<int32_t>(N);
-    grid_barrier(bar, target, err);
-  }
-  for (int64_t i = t0; i < N; i += stride) {
-    int32_t k;
-    if constexpr (sizeof(T) == 8) k = metropolis_one_sc(lw, lwf, N, B, keys, i, err);
-    else k = metropolis_one(lw, N, B, keys, i, err);
-    a[i] = k;
-    if (d) atomicMin(d + k, static_cast<int32_t>(i));
-  }
-  if constexpr (COOP) grid_exit(bar, target);
+  const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (i >= N) return;
+  int32_t k;
+  if constexpr (sizeof(T) == 8) k = metropolis_one_sc(lw, lwf, N, B, keys, i, err);
+  else k = metropolis_one<SMALL>(lw, N, B, keys, i, err);
+  a[i] = k;
+  if (d) atomicMin(d + k, static_cast<int32_t>(i));
 }
 
 // Rejection with warp refill (mcmc.cuh) over the particles [start, end) of one warp run.
@@ -257,7 +245,7 @@ __device__ __forceinline__ void count_add(unsigned long long* out, unsigned long
 
 // Every binary32 delta with bit pattern first + k (k < count): the tests decide from the band
 // [RD(e (1 - 2^-15)), RU(e (1 + 2^-15))] around e = exp_band_estimate(delta) (the binary64
-// filter) or exp_band_estimate24(delta) 2^-24 (the binary32 steps), which is right exactly when
+// filter) or exp_band_estimate32(delta) 2^-32 (the binary32 steps), which is right exactly when
 // exp_pinned(delta) lies inside it.
 __global__ void __launch_bounds__(kBlock)
 check_band_f32_kernel(uint32_t first, uint32_t count, unsigned long long* out) {
@@ -268,11 +256,9 @@ check_band_f32_kernel(uint32_t first, uint32_t count, unsigned long long* out) {
     const float e = exp_band_estimate(delta);
     const float lo = __fmul_rd(e, 1.0f - kExpBand), hi = __fmul_ru(e, 1.0f + kExpBand);
     const float p = exp_pinned(delta);
-    const float e24 = exp_band_estimate24(delta), p24 = __fmul_rn(p, 0x1p24f);  // (exact)
+    const float e32 = exp_band_estimate32(delta), p32 = __fmul_rn(p, 0x1p32f);  // (exact)
     if (!(lo <= p && p <= hi)) ++bad;
-    else if (!(__fmaf_rd(e24, 1.0f - kExpBand, -0x1p-36f) <= p24 &&
-               p24 <= __fmul_ru(e24, 1.0f + kExpBand)))
-      ++bad;
+    else if (!(fabsf(__fsub_rn(p32, e32)) <= __fmul_rd(e32, 0.99f * kExpBand))) ++bad;
   }
   count_add(out, bad);
 }
@@ -347,9 +333,8 @@ template <typename T>
 cudaError_t launch_metropolis_t(const Scratch& s, const T* lw, int64_t N, int32_t B,
                                 const Keys& keys, int32_t* a_out, int32_t* d, bool f64,
                                 cudaStream_t st) {
-  // (The cooperative form, fill and chains in one launch, measured slower than a fill launch
-  // followed by one thread per particle: the chains hide their gathers better in waves.)
-  GridBar* bar = &s.glob->bar;
+  // (One cooperative launch, fill and chains, measured slower than a fill launch followed by one
+  // thread per particle: the chains hide their gathers better in waves.)
   float* lwf = static_cast<float*>(s.W);  // the sidecars of binary64 log-weights (4 B each)
   if (sizeof(T) == 8) {
     trace_mark(s.trace, "sidecar", st);
@@ -363,8 +348,12 @@ cudaError_t launch_metropolis_t(const Scratch& s, const T* lw, int64_t N, int32_
     if (e != cudaSuccess) return e;
   }
   trace_mark(s.trace, f64 ? "metropolis_f64" : "metropolis_f32", st);
-  launch_pdl(metropolis_kernel<T, false>, static_cast<int>((N + kBlock - 1) / kBlock), kBlock,
-             st, lw, lwf, N, B, keys, a_out, d, bar, s.err);
+  const int grid = static_cast<int>((N + kBlock - 1) / kBlock);
+  if (sizeof(T) == 4 && N < (int64_t{1} << 24))
+    launch_pdl(metropolis_kernel<T, sizeof(T) == 4>, grid, kBlock, st, lw, lwf, N, B, keys, a_out,
+               d, s.err);
+  else
+    launch_pdl(metropolis_kernel<T, false>, grid, kBlock, st, lw, lwf, N, B, keys, a_out, d, s.err);
   return cudaGetLastError();
 }
 

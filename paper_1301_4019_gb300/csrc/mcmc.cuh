@@ -31,48 +31,38 @@ __device__ __forceinline__ float exp_band_estimate(float delta) {
   return e;
 }
 
-// 2^24 exp(delta), the scaling by one exponent addition inside the product (an FMA: one rounding
-// of delta log2 e + 24, whose magnitude is below 2^7: 2^-18, so still within a relative 1e-5).
-__device__ __forceinline__ float exp_band_estimate24(float delta) {
+// 2^32 exp(delta), the scaling an addition inside the product (an FMA: one rounding of
+// delta log2 e + 32, whose magnitude is below 2^7: 2^-18, so still within a relative 1e-5).
+__device__ __forceinline__ float exp_band_estimate32(float delta) {
   float e;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(__fmaf_rn(delta, 0x1.715476p+0f, 24.0f)));
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(__fmaf_rn(delta, 0x1.715476p+0f, 32.0f)));
   return e;
 }
 
-// u < exp_pinned(delta) for u = u24 2^-24 (u24 an integer), by definition.
-__device__ __forceinline__ bool u24_below_exp_exact(float u24, float delta) {
-  return delta >= -86.5f && __fmul_rn(u24, 0x1p-24f) < exp_pinned(delta);
+// The binary32 acceptance test u < exp_pinned(delta), u = (w0 >> 8) 2^-24, from the band: with
+// e = 2^32 exp(delta) and v = w0 rounded towards zero to binary32, which is at most 256 above
+// 2^32 u, the test is v < e wherever |v - e| > e 2^-15 + 256. Where that does not hold `amb` is
+// set (and stays set): probability about 6e-5 e / 2^32 a test, and every test of a NaN, of an
+// infinite e (a ratio above 2^95, or a zero-weight current state) and of u = 0 against
+// exp(delta) < 2^-24. Four operations after the exponential, no branch.
+__device__ __forceinline__ bool band_accept(uint32_t w0, float delta, bool& amb) {
+  const float e = exp_band_estimate32(delta);
+  const float d = __fsub_rn(__uint2float_rz(w0), e);
+  amb |= !(fabsf(d) > __fmaf_rn(e, kExpBand, 256.0f));
+  return d < 0.0f;
 }
 
-// u < w^j / w^k from log-weights: a ratio >= 1 or a zero-weight current state accepts.
-__device__ __noinline__ bool metropolis_accept_exact(float lwk, float lwj, float u24) {
+// The same by definition.
+__device__ __forceinline__ bool u_below_exp_exact(uint32_t w0, float delta) {
+  return delta >= -86.5f && half_u01_f32(w0) < exp_pinned(delta);
+}
+
+// u < w^j / w^k from log-weights, by definition: a ratio >= 1 or a zero-weight current state
+// accepts.
+__device__ __noinline__ bool metropolis_accept_exact(float lwk, float lwj, uint32_t w0) {
   if (lwk == neg_inf<float>()) return true;
   const float delta = lwj - lwk;
-  return delta >= 0.0f || u24_below_exp_exact(u24, delta);
-}
-
-// The same for binary32, u24 the 24 uniform bits as an integer, decided by the band alone in
-// almost every case, whatever delta is: e = exp_band_estimate24(delta) is +inf, or at least
-// 2^24 (1 - 1e-5) > u24 (1 - 2^-15), for a ratio >= 1 and for a zero-weight current state with a
-// proposal of non-zero weight, 0 for a zero-weight proposal, and NaN (neither comparison holds)
-// for two zero weights or a NaN. u24 = 0 accepts only where e is above 2^-36 (delta > -42); a
-// smaller e leaves it to the definition unless e is 0 (delta < -86.5: rejected, as there).
-// Seven instructions a step where the chain of tests took about twenty.
-__device__ __forceinline__ bool metropolis_accept24(float lwk, float lwj, float u24) {
-  const float e = exp_band_estimate24(__fsub_rn(lwj, lwk));
-  const bool yes = u24 < __fmaf_rd(e, 1.0f - kExpBand, -0x1p-36f);
-  const bool no = u24 >= __fmul_ru(e, 1.0f + kExpBand);
-  if (yes || no) return yes;
-  return metropolis_accept_exact(lwk, lwj, u24);
-}
-
-// u < exp_pinned(delta) for delta < 0, u = u24 2^-24.
-__device__ __forceinline__ bool u24_below_exp(float u24, float delta) {
-  const float e = exp_band_estimate24(delta);
-  const bool yes = u24 < __fmaf_rd(e, 1.0f - kExpBand, -0x1p-36f);
-  const bool no = u24 >= __fmul_ru(e, 1.0f + kExpBand);
-  if (yes || no) return yes;
-  return u24_below_exp_exact(u24, delta);
+  return delta >= 0.0f || u_below_exp_exact(w0, delta);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -165,66 +155,82 @@ __device__ __forceinline__ float f64_sidecar(double x) {
 constexpr int kUnroll = 4;    // binary32 chains: proposals issued together
 constexpr int kUnroll64 = 4;  // binary64 chains (2 measured slower)
 
-// Metropolis chain of particle i over n < 2^31 binary32 log-weights (Code 2), from the state i
-// with log-weight lwk; gather(j) reads the log-weight of proposal j. B steps; steps 2m and
-// 2m + 1 take the two halves of the block of counter (i, m) (half_u24, half_index), so a chain
-// draws ceil(B / 2) blocks. Returns the ancestor.
-template <typename Gather>
+// 2 P consecutive steps (s even) of a binary32 chain in state (k, lwk), those below B: the P
+// blocks drawn and their proposals gathered together, then the decisions from the band
+// (band_accept: a ratio >= 1 is e >= 2^32 (1 - 1e-5), never rejected by it). If any of them was
+// undecided the steps are taken again by definition: one branch for 2 P steps.
+template <int P, bool SMALL, typename Gather>
+__device__ __forceinline__ void metropolis_steps(uint32_t& k, float& lwk, const Gather& gather,
+                                                 uint32_t n, int32_t s, int32_t B,
+                                                 const Keys& keys, const DrawRow& row) {
+  uint32_t w[2 * P], j[2 * P];
+  float lwj[2 * P];
+#pragma unroll
+  for (int p = 0; p < P; ++p) {
+    const uint4 x = draw(keys, row, static_cast<uint32_t>(s / 2 + p));
+    w[2 * p] = x.x;
+    w[2 * p + 1] = x.z;
+    j[2 * p] = half_index<SMALL>(x.x, x.y, n);
+    j[2 * p + 1] = half_index<SMALL>(x.z, x.w, n);
+    lwj[2 * p] = gather(j[2 * p]);
+    lwj[2 * p + 1] = gather(j[2 * p + 1]);
+  }
+  const uint32_t k0 = k;
+  const float lwk0 = lwk;
+  bool amb = false;
+#pragma unroll
+  for (int q = 0; q < 2 * P; ++q) {
+    const bool yes = band_accept(w[q], __fsub_rn(lwj[q], lwk), amb);
+    if (yes && (P > 1 || q == 0 || s + 1 < B)) {  // (P > 1: called for whole rounds only)
+      k = j[q];
+      lwk = lwj[q];
+    }
+  }
+  if (amb) {
+    k = k0;
+    lwk = lwk0;
+#pragma unroll 1
+    for (int32_t t = s; t < s + 2 * P && t < B; ++t) {
+      const uint4 x = draw(keys, row, static_cast<uint32_t>(t >> 1));
+      const uint32_t w0 = (t & 1) ? x.z : x.x, w1 = (t & 1) ? x.w : x.y;
+      const uint32_t jt = half_index<SMALL>(w0, w1, n);
+      const float lwt = gather(jt);
+      if (metropolis_accept_exact(lwk, lwt, w0)) {
+        k = jt;
+        lwk = lwt;
+      }
+    }
+  }
+}
+
+// Metropolis chain of particle i over n < 2^31 (SMALL: n < 2^24) binary32 log-weights (Code 2),
+// from the state i with log-weight lwk; gather(j) reads the log-weight of proposal j. B steps;
+// steps 2m and 2m + 1 take the two halves of the block of counter (i, m) (half_u01_f32,
+// half_index), so a chain draws ceil(B / 2) blocks. Returns the ancestor.
+template <bool SMALL, typename Gather>
 __device__ __forceinline__ int32_t metropolis_chain(float lwk, const Gather& gather, uint32_t n,
                                                     int32_t B, const Keys& keys, uint32_t i) {
   static_assert(kUnroll % 2 == 0, "whole blocks per round");
   uint32_t k = i;
   const DrawRow row = draw_row(keys, i);
   int32_t s = 0;
-  for (; s + kUnroll <= B; s += kUnroll) {  // (s even)
-    float u[kUnroll], lwj[kUnroll];
-    uint32_t j[kUnroll];
-#pragma unroll
-    for (int p = 0; p < kUnroll / 2; ++p) {
-      const uint4 x = draw(keys, row, static_cast<uint32_t>(s / 2 + p));
-      j[2 * p] = half_index(x.x, x.y, n);
-      u[2 * p] = half_u24(x.x);
-      j[2 * p + 1] = half_index(x.z, x.w, n);
-      u[2 * p + 1] = half_u24(x.z);
-      lwj[2 * p] = gather(j[2 * p]);
-      lwj[2 * p + 1] = gather(j[2 * p + 1]);
-    }
-#pragma unroll
-    for (int q = 0; q < kUnroll; ++q) {
-      if (metropolis_accept24(lwk, lwj[q], u[q])) {
-        k = j[q];
-        lwk = lwj[q];
-      }
-    }
-  }
-  for (; s < B; s += 2) {  // the last B mod kUnroll steps, a block per two
-    const uint4 x = draw(keys, row, static_cast<uint32_t>(s / 2));
-    const uint32_t j0 = half_index(x.x, x.y, n);
-    const float lwj0 = gather(j0);
-    if (metropolis_accept24(lwk, lwj0, half_u24(x.x))) {
-      k = j0;
-      lwk = lwj0;
-    }
-    if (s + 1 < B) {
-      const uint32_t j1 = half_index(x.z, x.w, n);
-      const float lwj1 = gather(j1);
-      if (metropolis_accept24(lwk, lwj1, half_u24(x.z))) {
-        k = j1;
-        lwk = lwj1;
-      }
-    }
-  }
+  for (; s + kUnroll <= B; s += kUnroll)  // (s even)
+    metropolis_steps<kUnroll / 2, SMALL>(k, lwk, gather, n, s, B, keys, row);
+  for (; s < B; s += 2)  // the last B mod kUnroll steps, a block per two
+    metropolis_steps<1, SMALL>(k, lwk, gather, n, s, B, keys, row);
   return static_cast<int32_t>(k);
 }
 
 // The chain of particle i with its proposals gathered from the log-weights themselves.
+template <bool SMALL>
 __device__ __forceinline__ int32_t metropolis_one(const float* __restrict__ lw, int64_t n,
                                                   int32_t B, const Keys& keys, int64_t i,
                                                   int* err) {
   const float lwi = __ldg(lw + i);
   if (nonfinite_logw(lwi)) flag_error(err, RS_ERR_NONFINITE);
-  return metropolis_chain(lwi, [&](uint32_t j) { return __ldg(lw + j); },
-                          static_cast<uint32_t>(n), B, keys, static_cast<uint32_t>(i));
+  const auto gather = [&](uint32_t j) { return __ldg(lw + j); };
+  return metropolis_chain<SMALL>(lwi, gather, static_cast<uint32_t>(n), B, keys,
+                                 static_cast<uint32_t>(i));
 }
 
 __device__ __forceinline__ bool f64_step_accept(double lwk, float lwk_f, bool okk, long long kk,
@@ -245,7 +251,7 @@ __device__ __forceinline__ int32_t metropolis_one(const double* __restrict__ lw,
   bool okk = f64_to_f32_trunc(lwk, lwk_f);
   long long kk = f64_key(lwk);
   int64_t k = i;
-  const DrawRow row = draw_row(keys, static_cast<uint32_t>(i));
+  const uint32_t ii = static_cast<uint32_t>(i);
   int32_t s = 0;
   for (; s + kUnroll64 <= B; s += kUnroll64) {
     uint4 x[kUnroll64];
@@ -253,7 +259,7 @@ __device__ __forceinline__ int32_t metropolis_one(const double* __restrict__ lw,
     int64_t j[kUnroll64];
 #pragma unroll
     for (int q = 0; q < kUnroll64; ++q) {
-      x[q] = draw(keys, row, static_cast<uint32_t>(s + q));
+      x[q] = draw(keys, ii, static_cast<uint32_t>(s + q));
       j[q] = uniform_index(x[q], static_cast<uint32_t>(n));
       lwj[q] = __ldg(lw + j[q]);
     }
@@ -272,7 +278,7 @@ __device__ __forceinline__ int32_t metropolis_one(const double* __restrict__ lw,
     }
   }
   for (; s < B; ++s) {
-    const uint4 x = draw(keys, row, static_cast<uint32_t>(s));
+    const uint4 x = draw(keys, ii, static_cast<uint32_t>(s));
     const int64_t j = uniform_index(x, static_cast<uint32_t>(n));
     const double lwj = __ldg(lw + j);
     const long long kj = f64_key(lwj);
@@ -375,7 +381,7 @@ __device__ __forceinline__ int32_t rejection_one(const float* __restrict__ lw, i
   for (int64_t s = 0; s < max_trials; ++s) {
     if ((s & 1) == 0) x = draw(keys, ii, static_cast<uint32_t>(s >> 1));
     const uint32_t w0 = (s & 1) ? x.z : x.x, w1 = (s & 1) ? x.w : x.y;
-    if (s > 0) j = half_index(w0, w1, static_cast<uint32_t>(n));
+    if (s > 0) j = half_index<false>(w0, w1, static_cast<uint32_t>(n));
     const float u = half_u01_f32(w0);
     const float lwj = (s == 0) ? lwi : __ldg(lw + j);
     const float delta = lwj - lwmax;
@@ -449,17 +455,20 @@ __device__ __forceinline__ RejBound make_bound(double log_wmax, bool clamp = fal
   return r;
 }
 
-// Decision of one rejection attempt with uniform bits u24 (binary32) or draw x (binary64) and
+// Decision of one rejection attempt with the uniform's word w0 (binary32) or draw x (binary64) and
 // proposal log-weight lwj: accept when u < exp(lw^j - log w_max); a log-weight above the bound
 // is flagged (unless clamped) and accepted.
-__device__ __forceinline__ bool rejection_accept(const RejBound& rb, float u24, float lwj,
+__device__ __forceinline__ bool rejection_accept(const RejBound& rb, uint32_t w0, float lwj,
                                                  int* err) {
   const float delta = lwj - rb.lwmax_rn;
   if (delta > 0.0f) {
     if (!rb.clamp) flag_error(err, RS_ERR_BOUND_VIOLATED);
     return true;
   }
-  return delta == 0.0f || u24_below_exp(u24, delta);
+  if (delta == 0.0f) return true;
+  bool amb = false;
+  const bool yes = band_accept(w0, delta, amb);
+  return amb ? u_below_exp_exact(w0, delta) : yes;
 }
 
 __device__ __forceinline__ bool rejection_accept(const RejBound& rb, uint4 x, double lwj,
@@ -534,23 +543,24 @@ __device__ __forceinline__ bool rejection_attempts(const float* __restrict__ lw,
                                                    int64_t i, uint32_t s, float lwi,
                                                    int64_t max_trials, int64_t& j, int* err) {
   static_assert(K % 2 == 0, "whole blocks");
-  float u[K], lwj[K];
+  uint32_t w[K];
+  float lwj[K];
   int64_t jq[K];
 #pragma unroll
   for (int p = 0; p < K / 2; ++p) {
     const uint4 x = draw(keys, static_cast<uint32_t>(i), s / 2 + static_cast<uint32_t>(p));
     const uint32_t s0 = s + 2 * static_cast<uint32_t>(p);
-    jq[2 * p] = (s0 > 0) ? half_index(x.x, x.y, static_cast<uint32_t>(n)) : i;
-    u[2 * p] = half_u24(x.x);
-    jq[2 * p + 1] = half_index(x.z, x.w, static_cast<uint32_t>(n));
-    u[2 * p + 1] = half_u24(x.z);
+    jq[2 * p] = (s0 > 0) ? half_index<false>(x.x, x.y, static_cast<uint32_t>(n)) : i;
+    w[2 * p] = x.x;
+    jq[2 * p + 1] = half_index<false>(x.z, x.w, static_cast<uint32_t>(n));
+    w[2 * p + 1] = x.z;
     lwj[2 * p] = (s0 > 0) ? __ldg(lw + jq[2 * p]) : lwi;
     lwj[2 * p + 1] = __ldg(lw + jq[2 * p + 1]);
   }
 #pragma unroll
   for (int q = 0; q < K; ++q) {
     if (static_cast<int64_t>(s) + q >= max_trials) return false;
-    if (rejection_accept(rb, u[q], lwj[q], err)) {
+    if (rejection_accept(rb, w[q], lwj[q], err)) {
       j = jq[q];
       return true;
     }

@@ -285,3 +285,50 @@ def test_batched_permute_at_filter_boundaries(rs, scheme, masked):
         a, c = (o[offsets[f]:offsets[f + 1]] for o in out)
         if a.size:
             assert np.array_equal(c, oracle.permute(a)), (f, a.size)
+
+
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+@pytest.mark.parametrize("layout", ["small", "cap", "one", "odd_base"])
+def test_staged_chains_equal_one_thread_per_particle(rs, dtype, layout):
+    """The batched Metropolis chains with the log-weights staged in shared memory (the default
+    launch shape) equal the one-thread-per-particle kernel (any other shape) bit for bit:
+    windows of many small filters, filters at and above the staged capacity (57344), one filter,
+    log-weights that start off a 16-byte boundary; B per filter from 0 to 61 and the uniform B;
+    masked filters; -inf, NaN and zero-weight starts."""
+    sizes = {"small": [1, 2, 0, 33, 31, 1000, 64] * 40 + [1024, 1023, 1025, 0, 5],
+             "cap": [57343, 57344, 57345, 3, 0, 131077, 17],
+             "one": [2047],
+             "odd_base": [511, 4097, 60001, 2]}[layout]
+    F = len(sizes)
+    offsets, lw = _batch(sizes, dtype, seed=17)
+    rng = np.random.default_rng(3)
+    lw[rng.random(lw.size) < 0.05] = -np.inf
+    skip = 1 if layout == "odd_base" else 0
+    buf = torch.empty(lw.size + skip, dtype=torch.from_numpy(lw).dtype, device=DEV)
+    t = buf[skip:]
+    t.copy_(torch.from_numpy(lw))
+    off = torch.from_numpy(offsets).to(DEV)
+    Bs = torch.from_numpy(rng.choice([0, 1, 2, 3, 4, 5, 9, 61], F).astype(np.int32)).to(DEV)
+    flags = torch.from_numpy((rng.random(F) < 0.7).astype(np.uint8)).to(DEV)
+    kernel = rs.BATCHED_METROPOLIS_F64 if dtype == np.float64 else rs.BATCHED_METROPOLIS_F32
+    with rs.Handle(lw.size) as hh:
+        got = {}
+        for shape in ((256, 1), (128, 2)):
+            rs.rs_set_batched_launch(hh, kernel, *shape)
+            for kw in ({"B": 7}, {"B_per_filter": Bs}, {"B_per_filter": Bs, "resample": flags}):
+                for p in (False, True):
+                    a = rs.rs_resample_batched(hh, rs.METROPOLIS, t, off, seed=8, step=1,
+                                               permute=p, **kw).cpu().numpy()
+                    assert rs.rs_last_error(hh) == rs.RS_OK
+                    key = (len(kw), "B" in kw, p)
+                    if key in got:
+                        assert np.array_equal(got[key], a), key
+                    got[key] = a
+            # a NaN among the weights and a negative B are reported by either kernel
+            t[lw.size // 2] = float("nan")
+            rs.rs_resample_batched(hh, rs.METROPOLIS, t, off, B=3)
+            assert rs.rs_last_error(hh) == rs.RS_ERR_NONFINITE
+            t.copy_(torch.from_numpy(lw))
+            rs.rs_resample_batched(hh, rs.METROPOLIS, t, off, B_per_filter=Bs - 1)
+            assert rs.rs_last_error(hh) == (rs.RS_ERR_ARG if int((Bs.cpu() == 0).sum()) and any(
+                s and b == 0 for s, b in zip(sizes, Bs.cpu().tolist())) else rs.RS_OK)
