@@ -146,7 +146,7 @@ int rs_create(rs_handle** out, int64_t max_n, int device) {
   s.batch_tile_cap = max_n / rsk::kTile + s.max_filters + 1;
   const size_t mf = static_cast<size_t>(s.max_filters);
   const size_t tc = static_cast<size_t>(s.batch_tile_cap);
-  ok &= cudaMalloc(&s.batch_tile_start, sizeof(int32_t) * (mf + 1)) == cudaSuccess;
+  ok &= cudaMalloc(&s.batch_tile_start, sizeof(int32_t) * (2 * mf + 3)) == cudaSuccess;
   ok &= cudaMalloc(&s.batch_fmax, sizeof(long long) * mf) == cudaSuccess;
   ok &= cudaMalloc(&s.batch_fS, sizeof(double2) * mf) == cudaSuccess;
   ok &= cudaMalloc(&s.batch_fscale, sizeof(double2) * mf) == cudaSuccess;

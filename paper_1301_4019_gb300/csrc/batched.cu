@@ -117,7 +117,9 @@ struct Batch {
   const int64_t* off;
   int F;
   int64_t max_n;
-  int32_t* tile_start;   // F + 1
+  int32_t* tile_start;   // F + 1: first tile of each filter
+  int32_t* seg_start;    // F + 2: first segment (of kSeg particles) of each filter, and the
+                         // segments of the longest one
   long long* fmax;       // F, keys of the per-filter maxima
   double2* fS;           // F: total (accumulator type)
   double2* fscale;       // F: N / total
@@ -140,42 +142,67 @@ __device__ __forceinline__ bool resampled(const uint8_t* flags, int f) {
   return flags == nullptr || __ldg(flags + f) != 0;
 }
 
-// Plan: tiles per filter and their exclusive prefix; per-filter maxima reset; offsets checked.
+// Plan: tiles and segments per filter and their exclusive prefixes; per-filter maxima reset;
+// offsets checked.
 __global__ void __launch_bounds__(1024) batch_plan_kernel(Batch b) {
   pdl_wait();
-  __shared__ int sh[32];
+  __shared__ int2 sh[32];
   const int F = b.F;
   const int chunk = (F + blockDim.x - 1) / blockDim.x;
   const int f0 = min(F, static_cast<int>(threadIdx.x) * chunk), f1 = min(F, f0 + chunk);
-  int local = 0;
+  auto counts = [&](int f, bool flag) -> int2 {  // (tiles, segments) of filter f
+    const int64_t lo = __ldg(b.off + f), hi = __ldg(b.off + f + 1), n = hi - lo;
+    if (!(lo >= 0 && n >= 0 && hi <= b.max_n && n <= kBatchMaxN)) {
+      if (flag) flag_error(b.err, RS_ERR_ARG);
+      return make_int2(0, 0);
+    }
+    return make_int2(static_cast<int>((n + kTile - 1) / kTile),
+                     static_cast<int>((n + kSeg - 1) / kSeg));
+  };
+  int2 local = make_int2(0, 0);
+  int longest = 0;
   for (int f = f0; f < f1; ++f) {
-    const int64_t lo = b.off[f], hi = b.off[f + 1], n = hi - lo;
-    const bool ok = lo >= 0 && n >= 0 && hi <= b.max_n &&
-                    n <= kBatchMaxN;
-    if (!ok) flag_error(b.err, RS_ERR_ARG);
-    local += ok ? static_cast<int>((n + kTile - 1) / kTile) : 0;
+    const int2 c = counts(f, true);
+    local.x += c.x;
+    local.y += c.y;
+    longest = max(longest, c.y);
     b.fmax[f] = LLONG_MIN;
   }
+  __shared__ int sh_longest;
+  if (threadIdx.x == 0) sh_longest = 0;
+  __syncthreads();
+  longest = __reduce_max_sync(0xffffffffu, longest);
+  if ((threadIdx.x & 31) == 0) atomicMax(&sh_longest, longest);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  int incl = local;
+  int2 incl = local;
 #pragma unroll
   for (int dd = 1; dd < 32; dd <<= 1) {
-    const int y = __shfl_up_sync(0xffffffffu, incl, dd);
-    if (lane >= dd) incl += y;
+    const int x = __shfl_up_sync(0xffffffffu, incl.x, dd);
+    const int y = __shfl_up_sync(0xffffffffu, incl.y, dd);
+    if (lane >= dd) {
+      incl.x += x;
+      incl.y += y;
+    }
   }
   if (lane == 31) sh[warp] = incl;
   __syncthreads();
-  int p = incl - local;
-  for (int k = 0; k < warp; ++k) p += sh[k];
-  for (int f = f0; f < f1; ++f) {
-    b.tile_start[f] = p;
-    const int64_t lo = b.off[f], hi = b.off[f + 1], n = hi - lo;
-    const bool ok = lo >= 0 && n >= 0 && hi <= b.max_n &&
-                    n <= kBatchMaxN;
-    p += ok ? static_cast<int>((n + kTile - 1) / kTile) : 0;
+  int2 p = make_int2(incl.x - local.x, incl.y - local.y);
+  for (int k = 0; k < warp; ++k) {
+    p.x += sh[k].x;
+    p.y += sh[k].y;
   }
-  if (f1 == F && f0 < F) b.tile_start[F] = p;
-  if (F == 0 && threadIdx.x == 0) b.tile_start[0] = 0;
+  for (int f = f0; f < f1; ++f) {
+    b.tile_start[f] = p.x;
+    b.seg_start[f] = p.y;
+    const int2 c = counts(f, false);
+    p.x += c.x;
+    p.y += c.y;
+  }
+  if (f1 == F && f0 < F) {
+    b.tile_start[F] = p.x;
+    b.seg_start[F] = p.y;
+  }
+  if (threadIdx.x == 0) b.seg_start[F + 1] = sh_longest;  // (complete: the barrier above)
 }
 
 // Locates batch tile t: its filter f, the filter's bounds and the tile's first particle.
@@ -332,53 +359,157 @@ batch_emit_kernel(const T* __restrict__ lw, Batch b, Keys base_keys,
 
 // ---------------------------------------------------------------------------------------
 // The max, sum, prefix and emission passes of all filters in one cooperative launch (after the
-// plan kernel): CTA c owns the contiguous batch tiles [c T / G, (c+1) T / G) of the T tiles of
-// all filters together, and the CTAs meet at one grid barrier (two for compensated binary32,
-// whose records follow the filter maxima):
-//   phase 1  per tile, the records of its segments (seg_record, each warp its own: the
-//            segment's maximum log-weight and its weights' sum relative to it), the maxima
-//            combined per filter by an atomic max of keys;
-//   phase 2  per tile, the exact sums of its filter's records scaled to the filter's maximum
-//            (those before each of its segments, and all), rounded once to the segment
-//            prefixes and W^N as seg_prefix_compute rounds them, then the emission.
+// plan kernel). The unit of work is the segment, and each warp of the grid owns a contiguous
+// range of the segments of all filters together (so filters of any sizes share the grid evenly);
+// all passes but the prefixes of very long filters are warp-level work, and a filter's bounds,
+// totals and uniform are looked up when a warp comes to a new filter. The phases meet at two
+// grid barriers (three for compensated binary32, whose records follow the filter maxima):
+//   phase 1  the records of the warp's segments (seg_record: the segment's maximum log-weight
+//            and its weights' sum relative to it), last to first, and the filter maxima (an
+//            atomic max of keys per warp and filter);
+//   phase 2  per filter, one warp (a CTA from kWarpPrefixSegs segments): the exact sums of its
+//            records scaled to its maximum, rounded once to the segment prefixes and W^N;
+//   phase 3  the emission of the warp's segments, first to last (those phase 1 read last).
 // Every segment goes through the same device functions and rounded prefixes as in the separate
 // batched kernels and the single-filter kernels, so filter f still equals rs_resample on its
 // slice with filter = f, bit for bit.
 // ---------------------------------------------------------------------------------------
+constexpr int kWarpPrefixSegs = 1024;
+constexpr int kOwnPrefixSegs = 64;
+
+// Position of a warp in the batch: filter f and its bounds, segments [s0, s1) of the batch.
+struct SegWalk {
+  int f, s0, s1;
+  int64_t lo, hi;
+};
+__device__ __forceinline__ void seg_enter(const Batch& b, int f, SegWalk& w) {
+  w.f = f;
+  w.s0 = __ldg(b.seg_start + f);
+  w.s1 = __ldg(b.seg_start + f + 1);
+  w.lo = __ldg(b.off + f);
+  w.hi = __ldg(b.off + f + 1);
+}
+
+// Prefixes, total and N / total of filter f by one warp (the sums and roundings of
+// seg_prefix_compute: exact in fixed point, each prefix rounded once).
+template <typename T, typename V>
+__device__ __forceinline__ void warp_prefix(const Batch& b, int f, int s0, int nseg, int64_t n,
+                                            T M, const float2* tab) {
+  const int lane = threadIdx.x & 31;
+  double2* const P = b.P_rec + s0 + f;
+  u128 carry = 0;
+  for (int k0 = 0; k0 < nseg; k0 += 32) {
+    const int k = k0 + lane;
+    const u128 v = k < nseg ? rec_fixed<T, V>(b.s_rec + s0 + k, M, tab) : static_cast<u128>(0);
+    u128 incl = v;
+#pragma unroll
+    for (int dd = 1; dd < 32; dd <<= 1) {
+      const u128 y = shfl_up_u128(incl, dd);
+      if (lane >= dd) incl += y;
+    }
+    if (k < nseg) store_v<V>(P + k, fixed_to(carry + (incl - v), V(), kFixFrac));
+    const uint64_t hi = __shfl_sync(0xffffffffu, static_cast<uint64_t>(incl >> 64), 31);
+    const uint64_t lo = __shfl_sync(0xffffffffu, static_cast<uint64_t>(incl), 31);
+    carry += (static_cast<u128>(hi) << 64) | lo;
+  }
+  if (lane == 0) {
+    const V S = fixed_to(carry, V(), kFixFrac);
+    const double Sd = vto_double(S);
+    store_v<V>(P + nseg, S);
+    store_v<V>(b.fS + f, S);
+    store_v<V>(b.fscale + f, vfrom_double(__ddiv_rn(static_cast<double>(n), Sd), V()));
+    b.fSd[f] = Sd;
+  }
+}
+
+// The same sums for one segment `own` of filter f, by the warp that emits it: its prefix Ps, the
+// next one Pn, the total S and N / S (every lane gets them); the warp of the filter's first
+// segment also stores the totals (for the search kernel).
+template <typename T, typename V>
+__device__ __forceinline__ void warp_own_prefix(const Batch& b, int f, int s0, int nseg, int own,
+                                                int64_t n, T M, const float2* tab, V& Ps, V& Pn,
+                                                V& S, V& scale) {
+  u128 upto = 0, all = 0, mine = 0;  // (mine: the segment's own sum, in lane own mod 32)
+  for (int k = threadIdx.x & 31; k < nseg; k += 32) {
+    const u128 v = rec_fixed<T, V>(b.s_rec + s0 + k, M, tab);
+    all += v;
+    if (k <= own) upto += v;
+    if (k == own) mine = v;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    upto += shfl_xor_u128(upto, o);
+    all += shfl_xor_u128(all, o);
+  }
+  const uint64_t mh = __shfl_sync(0xffffffffu, static_cast<uint64_t>(mine >> 64), own & 31);
+  const uint64_t ml = __shfl_sync(0xffffffffu, static_cast<uint64_t>(mine), own & 31);
+  const u128 before = upto - ((static_cast<u128>(mh) << 64) | ml);
+  // one rounding for the three: each in a lane of its own
+  const int lane = threadIdx.x & 31;
+  const V r = fixed_to(lane == 0 ? before : lane == 1 ? upto : all, V(), kFixFrac);
+  Ps = vshfl(r, 0);
+  Pn = vshfl(r, 1);
+  S = vshfl(r, 2);
+  const double Sd = vto_double(S);
+  scale = vfrom_double(__ddiv_rn(static_cast<double>(n), Sd), V());
+  if (own == 0 && lane == 0) {
+    store_v<V>(b.fS + f, S);
+    store_v<V>(b.fscale + f, scale);
+    b.fSd[f] = Sd;
+  }
+}
+
 template <typename T, typename V, int SCHEME>
-__global__ void __launch_bounds__(kBlock)
+__global__ void __launch_bounds__(kBlock, 3)
 batch_coop_kernel(const T* __restrict__ lw, Batch b, Keys base_keys, int32_t* __restrict__ a,
                   int32_t* __restrict__ d, V* __restrict__ W, GridBar* bar) {
   __shared__ SegSh sh;
   __shared__ float2 sh_tab[64];
-  __shared__ u128 sh_sum[2 * kWarps];
-  __shared__ u128 sh_f[kWarps];
-  __shared__ double2 sh_P[kWarps + 1], sh_S, sh_scale;
-  __shared__ double sh_Sd;
   unsigned int target = 0;
-  const int T_tiles = __ldcg(b.tile_start + b.F);
-  const int G = static_cast<int>(gridDim.x), c = static_cast<int>(blockIdx.x);
-  const int t0 = static_cast<int>(static_cast<int64_t>(c) * T_tiles / G);
-  const int t1 = static_cast<int>(static_cast<int64_t>(c + 1) * T_tiles / G);
-  const bool vec = (reinterpret_cast<uintptr_t>(lw) & 15u) == 0;
+  const int U = __ldcg(b.seg_start + b.F);  // segments of the batch
+  const int warps = static_cast<int>(gridDim.x) * kWarps;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int gw = static_cast<int>(blockIdx.x) * kWarps + warp;
+  const int u0 = static_cast<int>(static_cast<int64_t>(gw) * U / warps);
+  const int u1 = static_cast<int>(static_cast<int64_t>(gw + 1) * U / warps);
+  const bool vec = (reinterpret_cast<uintptr_t>(lw) & 15u) == 0;
   if (threadIdx.x < 64) sh_tab[threadIdx.x] = kExp2Frac64[threadIdx.x];
   __syncthreads();
 
   // ---- phase 1: segment records -> filter maxima (compensated binary32: the maxima only) ----
-  {
-    bool bad = false;
-    for (int t = t0; t < t1; ++t) {
-      TileLoc L;
-      if (!locate_tile(b, t, L) || !resampled(b.resample, L.f)) continue;  // uniform per CTA
-      const int64_t base = L.base + kSeg * warp;
+  const int f_last = u1 > u0 ? filter_of_warp(b.seg_start, b.F, u1 - 1) : 0;
+  auto records = [&](bool with_max) {
+    SegWalk w;
+    bool bad = false, on = false;
+    long long fm = LLONG_MIN;  // the running maximum of the current filter's segments
+    long long ref = kTileMaxRef;
+    for (int u = u1 - 1; u >= u0; --u) {
+      if (u == u1 - 1 || u < w.s0) {
+        if (u < u1 - 1) {
+          if (with_max && on && lane == 0) atomicMax(b.fmax + w.f, max_key(key_to_double(fm, T())));
+          int f = w.f - 1;
+          while (__ldg(b.seg_start + f) > u) --f;  // (empty filters)
+          seg_enter(b, f, w);
+        } else {
+          seg_enter(b, f_last, w);
+        }
+        on = resampled(b.resample, w.f);
+        fm = max_key(neg_inf<T>());
+        if (!with_max) {
+          const double M = filter_M(b, w.f);
+          ref = M > -DBL_MAX ? max_key(static_cast<T>(M)) : kTileMaxRef;
+        }
+      }
+      if (!on) continue;  // a filter that keeps its particles: no passes
+      const int64_t base = w.lo + static_cast<int64_t>(u - w.s0) * kSeg;
       long long k;
-      if constexpr (Path<T, V>::kTileRef) {
-        k = seg_record<T, V>(lw, L.lo, L.hi, base, sh_tab, vec,
-                             b.s_rec + kWarps * t + warp, bad);
+      if (Path<T, V>::kTileRef || !with_max) {
+        k = seg_record<T, V>(lw, w.lo, w.hi, base, sh_tab, vec, b.s_rec + u, bad, ref,
+                             L2Hint::kEvictLast);
       } else {
         T x[kPer];
-        load_per(lw, base + kPer * static_cast<int64_t>(lane), L.lo, L.hi, vec, x);
+        load_per(lw, base + kPer * static_cast<int64_t>(lane), w.lo, w.hi, vec, x,
+                 L2Hint::kEvictLast);
         k = max_key(neg_inf<T>());
 #pragma unroll
         for (int q = 0; q < kPer; ++q) {
@@ -393,102 +524,109 @@ batch_coop_kernel(const T* __restrict__ lw, Batch b, Keys base_keys, int32_t* __
           k = y > k ? y : k;
         }
       }
-      // stored as the key of the binary64 value, comparable across both input types
-      if (lane == 0) atomicMax(b.fmax + L.f, max_key(key_to_double(k, T())));
+      fm = k > fm ? k : fm;
     }
-    if (bad) flag_error(b.err, RS_ERR_NONFINITE);
-  }
+    // (stored as the key of the binary64 value, comparable across both input types)
+    if (with_max && on && lane == 0) atomicMax(b.fmax + w.f, max_key(key_to_double(fm, T())));
+    if (with_max && bad) flag_error(b.err, RS_ERR_NONFINITE);
+  };
+  records(true);
   grid_barrier(bar, target, b.err);
   if constexpr (!Path<T, V>::kTileRef) {
-    bool bad = false;
-    for (int t = t0; t < t1; ++t) {
-      TileLoc L;
-      if (!locate_tile(b, t, L) || !resampled(b.resample, L.f)) continue;
-      const double M = filter_M(b, L.f);
-      seg_record<T, V>(lw, L.lo, L.hi, L.base + kSeg * warp, sh_tab, vec,
-                       b.s_rec + kWarps * t + warp, bad,
-                       M > -DBL_MAX ? max_key(static_cast<T>(M)) : kTileMaxRef);
-    }
+    records(false);
     grid_barrier(bar, target, b.err);
   }
 
-  // ---- phase 2: prefixes of each segment from its filter's exact record sums, emission -------
-  for (int t = t0; t < t1; ++t) {
-    TileLoc L;
-    if (!locate_tile(b, t, L)) continue;
-    const int64_t n = L.hi - L.lo;
-    const double M = filter_M(b, L.f);
-    const bool active = resampled(b.resample, L.f) && M > -DBL_MAX;
-    if (resampled(b.resample, L.f) && !(M > -DBL_MAX) && L.t == 0 && threadIdx.x == 0) {
-      b.fSd[L.f] = 0.0;
-      flag_error(b.err, RS_ERR_ZERO_WEIGHT);
-    }
-    double Sd = 0.0;
-    V Ps = vzero(V()), Pn = vzero(V()), S = vzero(V()), scale = vzero(V());
-    if (active) {
-      const int first = kWarps * __ldg(b.tile_start + L.f);  // the filter's first segment
-      const int nseg = kWarps * __ldg(b.tile_start + L.f + 1) - first;
-      const int own = kWarps * L.t;                          // this tile's first, in the filter
-      const T Mt = static_cast<T>(M);  // (exact: M is one of the filter's log-weights)
-      u128 part = 0, tot = 0;
-      for (int k = threadIdx.x; k < nseg; k += kBlock) {
-        const u128 v = rec_fixed<T, V>(b.s_rec + first + k, Mt);
-        tot += v;
-        if (k < own) part += v;
-        if (k >= own && k < own + kWarps) sh_f[k - own] = v;
-      }
-      block_sum2_u128(part, tot, sh_sum);  // (its barriers also publish sh_f)
-      if (threadIdx.x <= kWarps) {  // the tile's segment prefixes, one per thread
-        u128 p = part;
-        for (int w = 0; w < static_cast<int>(threadIdx.x); ++w) p += sh_f[w];
-        store_v<V>(&sh_P[threadIdx.x], fixed_to(p, V(), kFixFrac));
-      }
-      if (threadIdx.x == 0) {
-        const V S0 = fixed_to(tot, V(), kFixFrac);
-        const double Sd0 = vto_double(S0);
-        const V sc0 = vfrom_double(__ddiv_rn(static_cast<double>(n), Sd0), V());
-        store_v<V>(&sh_S, S0);
-        store_v<V>(&sh_scale, sc0);
-        sh_Sd = Sd0;
-        if (L.t == 0) {  // the filter's totals, for the search kernel
-          store_v<V>(b.fS + L.f, S0);
-          store_v<V>(b.fscale + L.f, sc0);
-          b.fSd[L.f] = Sd0;
+  // ---- phase 2: per filter, the exact prefixes of its segments and its total -----------------
+  // Small batches (a segment per warp at most, no filter above kOwnPrefixSegs segments) skip it and
+  // its barrier: every warp sums its filter's records itself (64 filters of up to 4096: 22.5
+  // against 20.6 us a call).
+  const bool own_prefix = U <= warps && __ldcg(b.seg_start + b.F + 1) <= kOwnPrefixSegs;
+  for (int pass = 0; pass < 2 && !own_prefix; ++pass) {  // (by warps; then very long filters by CTAs)
+    for (int f = pass == 0 ? gw : static_cast<int>(blockIdx.x); f < b.F;
+         f += pass == 0 ? warps : static_cast<int>(gridDim.x)) {
+      const int s0 = __ldg(b.seg_start + f), nseg = __ldg(b.seg_start + f + 1) - s0;
+      if (nseg == 0 || (nseg >= kWarpPrefixSegs) != (pass == 1) || !resampled(b.resample, f)) continue;
+      const double M = filter_M(b, f);
+      if (!(M > -DBL_MAX)) {
+        if (pass == 0 ? lane == 0 : threadIdx.x == 0) {
+          b.fSd[f] = 0.0;
+          flag_error(b.err, RS_ERR_ZERO_WEIGHT);
         }
+        continue;
       }
-      __syncthreads();
-      Ps = load_v<V>(&sh_P[warp]);
-      Pn = load_v<V>(&sh_P[warp + 1]);
-      S = load_v<V>(&sh_S);
-      scale = load_v<V>(&sh_scale);
-      Sd = sh_Sd;
-      __syncthreads();  // the shared values are rewritten by the next tile
+      const int64_t n = __ldg(b.off + f + 1) - __ldg(b.off + f);
+      if (pass == 0)
+        warp_prefix<T, V>(b, f, s0, nseg, n, static_cast<T>(M), sh_tab);  // (exact: M is a log-weight)
+      else
+        seg_prefix_compute<T, V>(b.s_rec + s0, b.P_rec + s0 + f, nseg, n, static_cast<T>(M),
+                                 reinterpret_cast<V*>(b.fS + f),
+                                 reinterpret_cast<V*>(b.fscale + f), b.fSd + f);
     }
-    if (!active || !(Sd > 0.0)) {  // all weights zero (flagged) or not resampled: identity
-      for (int64_t e = L.base + threadIdx.x; e < L.hi && e < L.base + kTile; e += kBlock) {
-        a[e] = static_cast<int32_t>(e - L.lo);
-        if (d) d[e] = static_cast<int32_t>(e - L.lo);
+  }
+  if (!own_prefix) grid_barrier(bar, target, b.err);
+
+  // ---- phase 3: emission ---------------------------------------------------------------------
+  SegWalk w;
+  bool live = false;
+  WeightCtx wc;
+  V S = vzero(V()), scale = vzero(V()), Ps = vzero(V()), Pn = vzero(V());
+  typename Path<T, V>::U u_sys = typename Path<T, V>::U();
+  for (int u = u0; u < u1; ++u) {
+    if (u == u0 || u >= w.s1) {
+      int f = u == u0 ? filter_of_warp(b.seg_start, b.F, u0) : w.f + 1;
+      while (__ldg(b.seg_start + f + 1) <= u) ++f;  // (empty filters)
+      seg_enter(b, f, w);
+      const double M = filter_M(b, f);
+      // all weights zero (flagged), or a filter that is not resampled: the identity
+      live = resampled(b.resample, f);
+      if (own_prefix && live && !(M > -DBL_MAX) && u == w.s0 && lane == 0) {
+        b.fSd[f] = 0.0;
+        flag_error(b.err, RS_ERR_ZERO_WEIGHT);
+      }
+      live = live && M > -DBL_MAX;
+      if (live && own_prefix) {
+        warp_own_prefix<T, V>(b, f, w.s0, w.s1 - w.s0, u - w.s0, w.hi - w.lo, static_cast<T>(M),
+                              sh_tab, Ps, Pn, S, scale);
+      } else if (live) {
+        S = load_v_cg<V>(b.fS + f);
+        scale = load_v_cg<V>(b.fscale + f);
+      }
+      live = live && vto_double(S) > 0.0;
+      wc = ctx_staged<T, V>(live ? M : 0.0, sh_tab);  // (the table was staged at the start)
+      if (live) {
+        if constexpr (SCHEME == RS_SYSTEMATIC)
+          u_sys = Path<T, V>::draw_u(
+              draw(with_tag(base_keys, static_cast<uint32_t>(f), SCHEME), 0u, 0u));
+      }
+    }
+    const int64_t base = w.lo + static_cast<int64_t>(u - w.s0) * kSeg;
+    uint8_t* const cl = claimed_bits(b, w.f, w.lo);
+    if (!live) {
+      const int64_t end = min(w.hi, base + kSeg);
+      for (int64_t e = base + lane; e < end; e += 32) {
+        a[e] = static_cast<int32_t>(e - w.lo);
+        if (d) d[e] = static_cast<int32_t>(e - w.lo);
         if (W) W[e] = vzero(V());
       }
-      claim_all(claimed_bits(b, L.f, L.lo), L);
+      if (cl && base - w.lo + 8 * lane < end - w.lo) cl[((base - w.lo) >> 3) + lane] = 0xFFu;
       continue;
     }
-    const WeightCtx wc = ctx_staged<T, V>(M, sh_tab);  // (the table was staged at the start)
-    const int64_t base = L.base + kSeg * warp;
+    if (!own_prefix) {
+      Ps = load_v_cg<V>(b.P_rec + u + w.f);
+      Pn = load_v_cg<V>(b.P_rec + u + w.f + 1);
+    }
     if constexpr (SCHEME == RS_MULTINOMIAL) {
-      if (d)  // claims of the search kernel start from the sentinel n
-        for (int64_t e = L.base + threadIdx.x; e < L.hi && e < L.base + kTile; e += kBlock)
-          d[e] = static_cast<int32_t>(n);
-      emit_seg_W<T, V, V>(lw, L.lo, L.hi, base, wc, vec, Ps, Pn, W);
+      if (d) {  // claims of the search kernel start from the sentinel n
+        const int32_t n = static_cast<int32_t>(w.hi - w.lo);
+        for (int64_t e = base + lane; e < w.hi && e < base + kSeg; e += 32) d[e] = n;
+      }
+      emit_seg_W<T, V, V>(lw, w.lo, w.hi, base, wc, vec, Ps, Pn, W);
     } else {
-      const Keys keys = with_tag(base_keys, static_cast<uint32_t>(L.f), SCHEME);
-      // the filter's systematic uniform, drawn by every thread (no block synchronisation)
-      const typename Path<T, V>::U u_sys =
-          SCHEME == RS_STRATIFIED ? typename Path<T, V>::U()
-                                  : Path<T, V>::draw_u(draw(keys, 0u, 0u));
-      emit_seg_cumoff<T, V, SCHEME == RS_STRATIFIED>(lw, L.lo, L.hi, base, wc, vec, Ps, Pn, S,
-                                                      scale, u_sys, keys, a, d, sh.win[warp],
-                                                      claimed_bits(b, L.f, L.lo));
+      emit_seg_cumoff<T, V, SCHEME == RS_STRATIFIED>(
+          lw, w.lo, w.hi, base, wc, vec, Ps, Pn, S, scale, u_sys,
+          with_tag(base_keys, static_cast<uint32_t>(w.f), SCHEME), a, d, sh.win[warp], cl,
+          L2Hint::kEvictFirst);
     }
   }
   grid_exit(bar, target);
@@ -976,12 +1114,13 @@ const char* const kLblCoop[4] = {"batch_coop_f32", "batch_coop_f32c", "batch_coo
 // The cooperative form of the batched scan passes (batch_coop_kernel), sized to the resident
 // grid; false when the device cannot run it (then the separate kernels run).
 template <typename T, typename V, int SCHEME>
-bool launch_batched_coop(const Scratch& s, const T* lw, const Batch& b, int64_t cap_tiles,
-                         const Keys& keys, int32_t* a, int32_t* d, V* W, cudaStream_t st,
-                         cudaError_t& e) {
+bool launch_batched_coop(const Scratch& s, const T* lw, const Batch& b, const Keys& keys,
+                         int32_t* a, int32_t* d, V* W, cudaStream_t st, cudaError_t& e) {
   const int cap = coop_capacity(reinterpret_cast<const void*>(batch_coop_kernel<T, V, SCHEME>));
   if (cap < 1) return false;
-  const int grid = static_cast<int64_t>(cap) < cap_tiles ? cap : static_cast<int>(cap_tiles);
+  // a segment per warp at most: every filter adds at most one partial segment
+  const int64_t want = (s.max_n / kSeg + b.F + kWarps) / kWarps;
+  const int grid = static_cast<int64_t>(cap) < want ? cap : static_cast<int>(want);
   trace_mark(s.trace, kLblCoop[Path<T, V>::id], st);
   e = coop_launch(batch_coop_kernel<T, V, SCHEME>, grid, st, lw, b, keys, a, d, W, &s.glob->bar);
   return true;
@@ -999,7 +1138,7 @@ cudaError_t run_batched_scan(const Scratch& s, int scheme, const T* lw, const Ba
     bool done;
     switch (scheme) {
       case RS_MULTINOMIAL:
-        done = launch_batched_coop<T, V, RS_MULTINOMIAL>(s, lw, b, cap_tiles, keys, a, d, Wc, st, e);
+        done = launch_batched_coop<T, V, RS_MULTINOMIAL>(s, lw, b, keys, a, d, Wc, st, e);
         if (done && e == cudaSuccess) {
           trace_mark(s.trace, kLblSearch[ai], st);
           launch_pdl(batch_search_kernel<T, V>, grid_particles(s.max_n), kBlock, st, Wc, b,
@@ -1008,12 +1147,10 @@ cudaError_t run_batched_scan(const Scratch& s, int scheme, const T* lw, const Ba
         }
         break;
       case RS_STRATIFIED:
-        done = launch_batched_coop<T, V, RS_STRATIFIED>(s, lw, b, cap_tiles, keys, a, d, nullptr,
-                                                        st, e);
+        done = launch_batched_coop<T, V, RS_STRATIFIED>(s, lw, b, keys, a, d, nullptr, st, e);
         break;
       default:
-        done = launch_batched_coop<T, V, RS_SYSTEMATIC>(s, lw, b, cap_tiles, keys, a, d, nullptr,
-                                                        st, e);
+        done = launch_batched_coop<T, V, RS_SYSTEMATIC>(s, lw, b, keys, a, d, nullptr, st, e);
         break;
     }
     if (done) return e;
@@ -1110,6 +1247,7 @@ cudaError_t launch_batched(const Scratch& s, int scheme, Acc acc, const void* lo
     b.F = F;
     b.max_n = s.max_n;
     b.tile_start = s.batch_tile_start;
+    b.seg_start = s.batch_tile_start + s.max_filters + 1;  // (F + 2 entries)
     b.fmax = s.batch_fmax;
     b.fS = s.batch_fS;
     b.fscale = s.batch_fscale;

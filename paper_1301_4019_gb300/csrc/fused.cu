@@ -189,8 +189,8 @@ __device__ __forceinline__ void fused_body(const T* __restrict__ lw, const Fused
       const int g = gb + static_cast<int>(threadIdx.x);
       u128 f = 0;
       if (g < g1) {
-        if (kKept<T, V> && gb == g0) f = rec_fixed_of<T, V>(rec0, Mt);
-        else f = rec_fixed<T, V>(A.s_rec + g, Mt);
+        if (kKept<T, V> && gb == g0) f = rec_fixed_of<T, V>(rec0, Mt, sh_tab);
+        else f = rec_fixed<T, V>(A.s_rec + g, Mt, sh_tab);
       }
       u128 tot;
       const u128 ex = block_excl_scan_u128(f, sh_sum, tot);

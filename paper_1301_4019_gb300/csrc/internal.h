@@ -73,7 +73,7 @@ struct Scratch {
   ScanGlob* glob;
   int* err;          // device status word
   // batched resampling: per-filter and per-tile records
-  int32_t* batch_tile_start;  // max_filters + 1
+  int32_t* batch_tile_start;  // 2 max_filters + 3: first tile and first segment of each filter
   long long* batch_fmax;      // max_filters
   double2* batch_fS;          // max_filters
   double2* batch_fscale;      // max_filters

@@ -600,8 +600,10 @@ __device__ __forceinline__ void load_rec(const double2* p, T& m, V& s) {
 // accumulators by the two-float exp of the two-term difference, as their weights are formed.
 // M = +inf (flagged non-finite input) gives 0 for finite m_t and NaN for m_t = +inf, as the
 // weights exp(lw_i - M) themselves do.
+// tab: the exp table of the two-float accumulators (in shared memory where many lanes scale
+// records at once: lanes that read different entries of constant memory take turns).
 template <typename T, typename V>
-__device__ __forceinline__ V rec_scaled_of(const double2 r, T M) {
+__device__ __forceinline__ V rec_scaled_of(const double2 r, T M, const float2* tab = kExp2Frac64) {
   T m;
   V sv;
   from_bits(static_cast<unsigned long long>(__double_as_longlong(r.x)), m);
@@ -629,20 +631,20 @@ __device__ __forceinline__ V rec_scaled_of(const double2 r, T M) {
     float2 d;
     if constexpr (sizeof(T) == 4) d = two_sum(m, -M);
     else d = add22_accurate(split_f64(m), neg2(split_f64(M)));
-    return mul22(sv, exp_df(d, kExp2Frac64));
+    return mul22(sv, exp_df(d, tab));
   }
 }
 template <typename T, typename V>
-__device__ __forceinline__ V rec_scaled(const double2* p, T M) {
-  return rec_scaled_of<T, V>(__ldcg(p), M);  // (written by another CTA, or earlier, in this launch)
+__device__ __forceinline__ V rec_scaled(const double2* p, T M, const float2* tab = kExp2Frac64) {
+  return rec_scaled_of<T, V>(__ldcg(p), M, tab);  // (written by another CTA, or earlier, in this launch)
 }
 template <typename T, typename V>
-__device__ __forceinline__ u128 rec_fixed(const double2* p, T M) {
-  return to_fixed(rec_scaled<T, V>(p, M));
+__device__ __forceinline__ u128 rec_fixed(const double2* p, T M, const float2* tab = kExp2Frac64) {
+  return to_fixed(rec_scaled<T, V>(p, M, tab));
 }
 template <typename T, typename V>
-__device__ __forceinline__ u128 rec_fixed_of(const double2 r, T M) {
-  return to_fixed(rec_scaled_of<T, V>(r, M));
+__device__ __forceinline__ u128 rec_fixed_of(const double2 r, T M, const float2* tab = kExp2Frac64) {
+  return to_fixed(rec_scaled_of<T, V>(r, M, tab));
 }
 
 // Prefixes of one sequence of nt segment records, M the sequence's maximum log-weight

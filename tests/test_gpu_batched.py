@@ -332,3 +332,32 @@ def test_staged_chains_equal_one_thread_per_particle(rs, dtype, layout):
             rs.rs_resample_batched(hh, rs.METROPOLIS, t, off, B_per_filter=Bs - 1)
             assert rs.rs_last_error(hh) == (rs.RS_ERR_ARG if int((Bs.cpu() == 0).sum()) and any(
                 s and b == 0 for s, b in zip(sizes, Bs.cpu().tolist())) else rs.RS_OK)
+
+
+@pytest.mark.parametrize("dtype,prec", MODES)
+@pytest.mark.parametrize("layout", ["own", "long", "many"])
+def test_batched_scan_work_split(rs, dtype, prec, layout):
+    """The cooperative batched scan equals the single-filter calls however its segments fall on
+    the warps: every warp summing its filter's records itself (few segments, none above 64 in a
+    filter), filters whose prefixes a whole CTA forms (1024 segments and more), and several
+    filters per warp; with empty and all-zero filters in between."""
+    sizes = {"own": [1, 255, 0, 256, 257, 16384, 16383, 5000, 0, 2049],
+             "long": [262143, 0, 262145, 300, 300001, 1],
+             "many": [257, 3, 0, 511] * 3000}[layout]
+    offsets, lw = _batch(sizes, dtype, seed=23)
+    zero = 3
+    lw[offsets[zero]:offsets[zero + 1]] = -np.inf
+    t = torch.from_numpy(lw).to(DEV)
+    off = torch.from_numpy(offsets).to(DEV)
+    sample = range(len(sizes)) if len(sizes) < 20 else [0, 1, 2, 3, 4, 5, 7, 6001, 8000, 11996, 11999]
+    with rs.Handle(lw.size) as hh:
+        for scheme in (rs.MULTINOMIAL, rs.STRATIFIED, rs.SYSTEMATIC):
+            a = rs.rs_resample_batched(hh, scheme, t, off, seed=31, step=5, permute=True,
+                                       prec=prec).cpu().numpy()
+            assert rs.rs_last_error(hh) == rs.RS_ERR_ZERO_WEIGHT
+            for f in sample:
+                lo, hi = offsets[f], offsets[f + 1]
+                if hi > lo:
+                    want = _single(rs, hh, scheme, lw[lo:hi], f, True, prec)
+                    rs.rs_last_error(hh)
+                    assert np.array_equal(a[lo:hi], want), (scheme, f, hi - lo)
