@@ -114,9 +114,14 @@ __device__ __forceinline__ uint4 draw(const Keys& k, const DrawRow& row, uint32_
 __device__ __forceinline__ float u01_f32(uint4 x) {
   return __fmul_rn(__uint2float_rn(x.x >> 8), 0x1p-24f);
 }
+// (binary64 without the binary64 pipe: m 2^-53 has its leading bit at position 63 - lz of m, so
+// its exponent field is 1023 + 63 - lz - 53 and its fraction the bits below)
 __device__ __forceinline__ double u01_f64(uint4 x) {
   const uint64_t m = (static_cast<uint64_t>(x.x) << 21) | static_cast<uint64_t>(x.y >> 11);
-  return __dmul_rn(__ull2double_rn(m), 0x1p-53);
+  const int lz = __clzll(static_cast<long long>(m));  // (>= 11; 64 for m = 0)
+  const uint64_t e = static_cast<uint64_t>(1033 - lz);
+  const uint64_t frac = (m << (lz - 11)) & 0xfffffffffffffull;
+  return __longlong_as_double(m ? static_cast<long long>((e << 52) | frac) : 0LL);
 }
 template <typename T> __device__ __forceinline__ T u01(uint4 x);
 template <> __device__ __forceinline__ float u01<float>(uint4 x) { return u01_f32(x); }
@@ -172,10 +177,18 @@ __device__ __forceinline__ float exp_pinned(float x) {
   return __fmul_rn(p, scale);
 }
 
+// In binary64 everything but the arithmetic itself stays off the binary64 pipe (1/57 of the
+// binary32 rate): the tests are made on the bit pattern, rint(t) is t + 1.5 2^52 - 1.5 2^52 (round
+// to nearest even of |t| < 2^51, whose low word is then the integer), and the scaling by 2^k
+// (k >= -1020: the result is a normal number) an addition to the exponent. 18 operations.
 __device__ __forceinline__ double exp_pinned(double x) {
-  if (x != x) return x;
-  if (x < -707.0) return 0.0;
-  const double k = rint(__dmul_rn(x, 0x1.71547652b82fep+0));
+  const unsigned long long bits = static_cast<unsigned long long>(__double_as_longlong(x));
+  if ((bits << 1) > 0xffe0000000000000ull) return x;     // NaN
+  if (bits > 0xc086180000000000ull) return 0.0;          // x < -707
+  const double magic = 0x1.8p52;
+  const double t = __dadd_rn(__dmul_rn(x, 0x1.71547652b82fep+0), magic);
+  const int ki = __double2loint(t);
+  const double k = __dsub_rn(t, magic);
   double r = __fma_rn(-k, 0x1.62e42fefa39efp-1, x);
   r = __fma_rn(-k, 0x1.abc9e3b39803fp-56, r);
   double p = 0x1.6124613a86d09p-33;       // 1/13!
@@ -192,9 +205,7 @@ __device__ __forceinline__ double exp_pinned(double x) {
   p = __fma_rn(p, r, 0x1p-1);                 // 1/2!
   p = __fma_rn(p, r, 1.0);                    // 1/1!
   p = __fma_rn(p, r, 1.0);                    // 1/0!
-  const long long ki = static_cast<long long>(k);
-  const double scale = __longlong_as_double((ki + 1023LL) << 52);
-  return __dmul_rn(p, scale);
+  return __hiloint2double(__double2hiint(p) + (ki << 20), __double2loint(p));
 }
 
 // ---------------------------------------------------------------------------------------

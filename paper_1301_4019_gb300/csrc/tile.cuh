@@ -74,7 +74,7 @@ template <> struct Path<double, double> {
   static constexpr bool kTable = false;
   static constexpr bool kTileRef = true;
   __device__ static double weight(double x, const WeightCtx& c) {
-    return (x == neg_inf<double>()) ? 0.0 : exp_pinned(__dsub_rn(x, c.Md));
+    return is_neg_inf(x) ? 0.0 : exp_pinned(__dsub_rn(x, c.Md));
   }
   __device__ static U draw_u(uint4 x) { return u01_f64(x); }
 };
@@ -235,24 +235,39 @@ __device__ __forceinline__ int seg_count(int64_t base, int64_t N) {
   return c < kSeg ? static_cast<int>(c) : kSeg;
 }
 
-// Maximum and minimum of non-negative accumulator values (exact; one instruction for the
-// IEEE types, whose values here are never NaN).
+// Maximum and minimum of non-negative accumulator values (exact; binary32: one instruction;
+// binary64: by the bit pattern, which orders like the value, off the binary64 pipe). A NaN (from
+// flagged input) never survives tmin(tmax(., lo), hi) with numbers lo and hi.
 __device__ __forceinline__ float tmax(float a, float b) { return fmaxf(a, b); }
 __device__ __forceinline__ float tmin(float a, float b) { return fminf(a, b); }
-__device__ __forceinline__ double tmax(double a, double b) { return fmax(a, b); }
-__device__ __forceinline__ double tmin(double a, double b) { return fmin(a, b); }
+__device__ __forceinline__ double tmax(double a, double b) {
+  const long long x = __double_as_longlong(a), y = __double_as_longlong(b);
+  return __longlong_as_double(x > y ? x : y);
+}
+__device__ __forceinline__ double tmin(double a, double b) {
+  const long long x = __double_as_longlong(a), y = __double_as_longlong(b);
+  return __longlong_as_double(x < y ? x : y);
+}
 __device__ __forceinline__ float2 tmax(float2 a, float2 b) { return vmax(a, b); }
 __device__ __forceinline__ float2 tmin(float2 a, float2 b) { return vmin(a, b); }
 
 // Equality of two accumulator values (non-negative, never NaN here).
 __device__ __forceinline__ bool vsame(float a, float b) { return a == b; }
-__device__ __forceinline__ bool vsame(double a, double b) { return a == b; }
+__device__ __forceinline__ bool vsame(double a, double b) {
+  return __double_as_longlong(a) == __double_as_longlong(b);
+}
 __device__ __forceinline__ bool vsame(float2 a, float2 b) { return a.x == b.x && a.y == b.y; }
 
 // floor(x) as a 32-bit integer (x >= 0; values of 2^31 and above saturate, and every caller
 // clamps to n < 2^31 afterwards). floor of a two-float is floor(hi) unless hi is an integer.
 __device__ __forceinline__ int32_t floor_i32(float x) { return __float2int_rd(x); }
-__device__ __forceinline__ int32_t floor_i32(double x) { return __double2int_rd(x); }
+__device__ __forceinline__ int32_t floor_i32(double x) {  // (integer operations only)
+  const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(x));
+  const int e = static_cast<int>(b >> 52) - 1023;
+  if (e < 0) return 0;
+  if (e > 30) return INT32_MAX;
+  return static_cast<int32_t>(((b & 0xfffffffffffffull) | 0x10000000000000ull) >> (52 - e));
+}
 __device__ __forceinline__ int32_t floor_i32(float2 z) {
   const float f = floorf(z.x);
   if (!(f < 0x1p31f)) return INT32_MAX;
