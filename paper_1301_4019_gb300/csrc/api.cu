@@ -141,7 +141,9 @@ int rs_create(rs_handle** out, int64_t max_n, int device) {
   ok &= cudaMalloc(&s.guide, sizeof(int32_t) * (max_n + 1)) == cudaSuccess;
   ok &= cudaMalloc(&s.rec, sizeof(double2) * 2 * rsk::seg_cap(s.max_tiles)) == cudaSuccess;
   ok &= cudaMalloc(&s.blockmax, sizeof(double) * s.max_blocks) == cudaSuccess;
-  ok &= cudaMalloc(&s.irec, sizeof(long long) * 2 * (s.max_tiles + 2)) == cudaSuccess;
+  // (also the per-CTA totals of the cooperative scans, 16 bytes each for at most max_blocks CTAs)
+  const int64_t irecs = s.max_tiles + 2 > s.max_blocks ? s.max_tiles + 2 : s.max_blocks;
+  ok &= cudaMalloc(&s.irec, sizeof(long long) * 2 * irecs) == cudaSuccess;
   ok &= cudaMalloc(&s.glob, sizeof(rsk::ScanGlob)) == cudaSuccess;
   s.batch_tile_cap = max_n / rsk::kTile + s.max_filters + 1;
   const size_t mf = static_cast<size_t>(s.max_filters);

@@ -2,11 +2,11 @@
 // (maximum and segment records, segment prefixes, emission) as one persistent cooperative
 // kernel.
 //
-// Each CTA owns a contiguous range of tiles; the CTAs are all resident at once (cooperative
+// Each CTA owns a contiguous range of segments; the CTAs are all resident at once (cooperative
 // launch) and meet at grid-wide barriers between the phases (see fused_body). The segment
 // prefixes are exact fixed-point sums, so they can be assembled in parallel from per-CTA
 // totals instead of by one CTA, and each phase calls the same device functions as the
-// separate kernels on the same tiles: the results are identical. The latency-bound
+// separate kernels on the same segments: the results are identical. The latency-bound
 // particle-parallel steps that follow (the multinomial search, Permute) stay separate
 // full-occupancy kernels.
 // A barrier waits at most the handle's barrier timeout (then it records RS_ERR_TIMEOUT and proceeds;
@@ -57,9 +57,12 @@ struct FusedArgs {
   int* err;
 };
 
-// CTA c owns the contiguous tiles [c T / G, (c+1) T / G) of the T tiles (G = gridDim.x <= T):
-//   phase 1  the records (m_g, s_g) of its tiles' segments (seg_record, each warp its own:
-//            the segment's maximum and its weights' sum relative to it), last tile to first,
+// CTA c owns the contiguous segments [c T / G, (c+1) T / G) of the T segments of kSeg particles
+// (G = gridDim.x <= T), its warps taking them in turns of kWarps: cutting by segments, not by
+// tiles, gives every SM the same work to within a segment a CTA (2^20 particles: 4096 segments on
+// 608 CTAs; as 512 tiles some SMs had four, most three).
+//   phase 1  the records (m_g, s_g) of its segments (seg_record, each warp its own: the
+//            segment's maximum and its weights' sum relative to it), last turn to first,
 //            and its largest m_g -> barrier;
 //   phase 2  M = maximum over the CTAs; T_g = s_g exp(m_g - M) (rec_scaled) of its segments
 //            and their exact running sum in fixed point (the in-range prefix of each segment,
@@ -70,9 +73,9 @@ struct FusedArgs {
 //   phase 3  every CTA sums the exact CTA totals: those before it (CP) and all (the total);
 //            P_g = RN(CP + in-range prefix of g) for its segments and P_{g1} = RN(CP + its
 //            own total), which is the P_{g1} the next CTA computes; W^N = RN(total), N / W^N;
-//   phase 4  emission of its tiles, first to last (it starts on the tiles phase 1 read last,
-//            still in L2 when the log-weights exceed half of it), each warp its segments.
-// Phases 1 and 4 are warp-level work only: no block barrier per tile. The log-weights are read
+//   phase 4  emission of its segments, first to last (it starts on those phase 1 read last,
+//            still in L2 when the log-weights exceed half of it), each warp its own.
+// Phases 1 and 4 are warp-level work only: no block barrier per turn. The log-weights are read
 // twice (phases 1 and 4; three times for compensated binary32), the least the normaliser
 // allows. P_g is the exact sum of the T before g rounded once, as in seg_prefix_compute, so the
 // results equal
@@ -93,44 +96,47 @@ __device__ __forceinline__ void fused_body(const T* __restrict__ lw, const Fused
   __shared__ long long sh_key[kWarps];
   __shared__ u128 sh_sum[2 * kWarps];
   const int64_t N = A.N;
-  const int T_tiles = static_cast<int>((N + kTile - 1) / kTile);
+  const int T_segs = static_cast<int>((N + kSeg - 1) / kSeg);
   const int G = static_cast<int>(gridDim.x), c = static_cast<int>(blockIdx.x);
-  const int t0 = static_cast<int>(static_cast<int64_t>(c) * T_tiles / G);
-  const int t1 = static_cast<int>(static_cast<int64_t>(c + 1) * T_tiles / G);
-  const int g0 = kWarps * t0, g1 = kWarps * t1;  // this CTA's segments
-  const int warp = threadIdx.x >> 5;
-  const int64_t e0 = static_cast<int64_t>(t0) * kTile;
-  const int64_t e1 = min(static_cast<int64_t>(t1) * kTile, N);
-  const int64_t off = kPer * static_cast<int64_t>(threadIdx.x);  // (= kSeg warp + kPer lane)
+  const int g0 = static_cast<int>(static_cast<int64_t>(c) * T_segs / G);  // this CTA's segments
+  const int g1 = static_cast<int>(static_cast<int64_t>(c + 1) * T_segs / G);
+  const int turns = (g1 - g0 + kWarps - 1) / kWarps;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t e0 = static_cast<int64_t>(g0) * kSeg;
+  const int64_t e1 = min(static_cast<int64_t>(g1) * kSeg, N);
+  const int64_t off = kPer * static_cast<int64_t>(threadIdx.x);
   const bool vec = (reinterpret_cast<uintptr_t>(lw) & 15u) == 0;
   if (threadIdx.x < 64) sh_tab[threadIdx.x] = kExp2Frac64[threadIdx.x];
   __syncthreads();
 
-  // ---- phase 1: segment records, last tile to first (and the Prepermute sentinel of the
-  // multinomial claims); the next tile's log-weights are loaded while this one is reduced.
+  // ---- phase 1: segment records, last turn to first (and the Prepermute sentinel of the
+  // multinomial claims); the next segment's log-weights are loaded while this one is reduced.
   // Without kTileRef, the maximum only (the records follow once M is known) ----------------
   double2 rec0 = make_double2(0.0, 0.0);  // (kKept) the record of segment g0 + threadIdx.x
+  const int last_turn = turns - (g0 + kWarps * (turns - 1) + warp < g1 ? 1 : 2);  // (of this warp)
+  const int64_t lane0 = e0 + static_cast<int64_t>(kSeg) * warp + kPer * lane;  // (turn 0)
   {
     long long cm = max_key(neg_inf<T>());
     bool bad = false;
     if constexpr (Path<T, V>::kTileRef) {
       T xn[kPer];
-      if (t1 > t0)
-        load_per(lw, static_cast<int64_t>(t1 - 1) * kTile + off, 0, N, vec, xn, L2Hint::kEvictLast);
-      for (int t = t1 - 1; t >= t0; --t) {
+      if (last_turn >= 0)
+        load_per(lw, lane0 + static_cast<int64_t>(kTile) * last_turn, 0, N, vec, xn, L2Hint::kEvictLast);
+      for (int t = last_turn; t >= 0; --t) {
         T x[kPer];
 #pragma unroll
         for (int q = 0; q < kPer; ++q) x[q] = xn[q];
-        if (t > t0)
-          load_per(lw, static_cast<int64_t>(t - 1) * kTile + off, 0, N, vec, xn, L2Hint::kEvictLast);
-        const long long k = seg_record<T, V>(x, sh_tab, A.s_rec + kWarps * t + warp, bad);
+        if (t > 0)
+          load_per(lw, lane0 + static_cast<int64_t>(kTile) * (t - 1), 0, N, vec, xn,
+                   L2Hint::kEvictLast);
+        const long long k = seg_record<T, V>(x, sh_tab, A.s_rec + g0 + kWarps * t + warp, bad);
         cm = k > cm ? k : cm;
       }
     } else {
       float mf = -INFINITY;  // (binary32 inputs)
-      for (int t = t0; t < t1; ++t) {
+      for (int t = 0; t <= last_turn; ++t) {
         T x[kPer];
-        load_per(lw, static_cast<int64_t>(t) * kTile + off, 0, N, vec, x, L2Hint::kEvictLast);
+        load_per(lw, lane0 + static_cast<int64_t>(kTile) * t, 0, N, vec, x, L2Hint::kEvictLast);
 #pragma unroll
         for (int q = 0; q < kPer; ++q) {
           bad |= !(x[q] <= FLT_MAX);  // NaN or +inf
@@ -178,11 +184,13 @@ __device__ __forceinline__ void fused_body(const T* __restrict__ lw, const Fused
   u128 lp0 = 0;  // the exact in-range prefix of segment g0 + threadIdx.x (kept for phase 3)
   if (!zero) {
     const T Mt = static_cast<T>(M);  // (exact: M is one of the log-weights)
-    if constexpr (!Path<T, V>::kTileRef) {  // the records, relative to M, last tile to first
+    if constexpr (!Path<T, V>::kTileRef) {  // the records, relative to M, last turn to first
       bool bad = false;
-      for (int t = t1 - 1; t >= t0; --t)
-        seg_record<T, V>(lw, 0, N, static_cast<int64_t>(t) * kTile + kSeg * warp, sh_tab, vec,
-                         A.s_rec + kWarps * t + warp, bad, max_key(Mt), L2Hint::kEvictLast);
+      for (int t = last_turn; t >= 0; --t) {
+        const int g = g0 + kWarps * t + warp;
+        seg_record<T, V>(lw, 0, N, static_cast<int64_t>(g) * kSeg, sh_tab, vec, A.s_rec + g, bad,
+                         max_key(Mt), L2Hint::kEvictLast);
+      }
       __syncthreads();  // (lane 0 of each warp stored them; all threads read them below)
     }
     for (int gb = g0; gb < g1; gb += kBlock) {
@@ -285,7 +293,7 @@ __device__ __forceinline__ void fused_body(const T* __restrict__ lw, const Fused
   }
   __syncthreads();
 
-  // ---- phase 4: emission of this CTA's tiles, each warp its own segments (no block-level
+  // ---- phase 4: emission of this CTA's segments, each warp its own (no block-level
   // synchronisation) -------------------------------------------------------------------------
   typename Path<T, V>::U u_sys = typename Path<T, V>::U();
   Guide gd;
@@ -294,9 +302,8 @@ __device__ __forceinline__ void fused_body(const T* __restrict__ lw, const Fused
   } else if constexpr (SCHEME == RS_SYSTEMATIC) {
     u_sys = cta_uniform0<T, V>(A.keys);
   }
-  for (int t = t0; t < t1; ++t) {
-    const int g = kWarps * t + warp;
-    const int64_t base = static_cast<int64_t>(t) * kTile + kSeg * warp;
+  for (int g = g0 + warp; g < g1; g += kWarps) {
+    const int64_t base = static_cast<int64_t>(g) * kSeg;
     const V Ps = load_v_cg<V>(A.P_rec + g);
     const V Pn = (g + 1 < g1) ? load_v_cg<V>(A.P_rec + g + 1) : load_v<V>(&sh_pend);
     if constexpr (SCHEME == RS_MULTINOMIAL) {
@@ -310,10 +317,16 @@ __device__ __forceinline__ void fused_body(const T* __restrict__ lw, const Fused
   }
 }
 
-// (at most 64 registers a thread, so that four CTAs of kBlock threads share an SM: the
-// cooperative grid is four CTAs per SM)
+// CTAs of kBlock threads that share an SM (the cooperative grid holds so many on each): four for
+// binary32 log-weights (64 registers), three for binary64 ones, whose emission keeps more values in
+// flight (80 registers; 3000001 particles, double-float: 92.2 -> 90.2 us, IEEE 700001: 85.8 ->
+// 78.9; compensated binary32 at 2^20 is faster with four).
+template <typename T, typename V>
+constexpr int fused_ctas() {
+  return sizeof(T) == 4 ? 4 : 3;
+}
 template <typename T, typename V, int SCHEME>
-__global__ void __launch_bounds__(kBlock, 4) fused_scan_kernel(const T* __restrict__ lw, FusedArgs A) {
+__global__ void __launch_bounds__(kBlock, (fused_ctas<T, V>())) fused_scan_kernel(const T* __restrict__ lw, FusedArgs A) {
   unsigned int target = 0;
   fused_body<T, V, SCHEME>(lw, A, target);
   grid_exit(&A.g->bar, target);
@@ -338,8 +351,12 @@ template <typename T, typename V, int SCHEME>
 cudaError_t launch_fused(const Scratch& s, const T* lw, const FusedArgs& A, cudaStream_t st) {
   int64_t grid = fused_capacity<T, V, SCHEME>();
   if (grid > s.max_blocks) grid = s.max_blocks;
-  const int64_t tiles = (A.N + kTile - 1) / kTile;
-  if (grid > tiles) grid = tiles;
+  // a full turn of the warps each; half a turn for native binary64, which is bound by the
+  // binary64 pipes of the SMs it reaches (20000 particles: 51 -> 33 us), while the others lose by
+  // more CTAs at the barriers (2^20 binary32: 27.2 -> 29.0 us)
+  constexpr int64_t per = std::is_same_v<V, double> ? kWarps / 2 : kWarps;
+  const int64_t want = ((A.N + kSeg - 1) / kSeg + per - 1) / per;
+  if (grid > want) grid = want;
   if (grid < 1) return cudaErrorCooperativeLaunchTooLarge;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(static_cast<unsigned>(grid));
@@ -404,7 +421,7 @@ cudaError_t launch_fused_passes(const Scratch& s, int scheme, Acc acc, const voi
   A.guide = s.guide;
   A.s_rec = s.rec;
   A.P_rec = s.rec + seg_cap(s.max_tiles);
-  A.agg = reinterpret_cast<u128*>(s.irec);  // (max_tiles + 2) entries >= gridDim.x
+  A.agg = reinterpret_cast<u128*>(s.irec);  // at least max_blocks entries >= gridDim.x
   A.g = s.glob;
   A.blockmax = s.blockmax;
   A.err = s.err;

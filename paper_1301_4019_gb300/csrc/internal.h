@@ -69,7 +69,8 @@ struct Scratch {
   int32_t* guide;    // guide table of the multinomial search, max_n + 1
   double2* rec;      // per-segment records, then prefixes (two blocks of seg_cap(max_tiles))
   double* blockmax;  // per-CTA maxima of the max pass
-  long long* irec;   // per-tile records of the integer scan (2 * (max_tiles + 2))
+  long long* irec;   // per-tile records of the integer scan (2 * (max_tiles + 2), or 2 * max_blocks
+                     // if more: the per-CTA exact totals of the cooperative scan)
   ScanGlob* glob;
   int* err;          // device status word
   // batched resampling: per-filter and per-tile records
