@@ -276,6 +276,18 @@ int rs_lgssm_step(rs_handle* h, float* x_dev, int64_t N, int init, int accumulat
                   float sigma_x, float y, float sigma_y, uint64_t seed, uint64_t step,
                   uint32_t filter, float* logw_dev, void* stream);
 
+/* One step of the bootstrap filter around its resampling: rs_copy_ancestors of the states x_dev
+ * (D = 1) by c_dev (NULL: no copy; must be NULL with init = 1), rs_lgssm_step with accumulate = 0
+ * and rs_ess of the new log-weights (either of ess_dev, log_total_dev may be NULL, not both). The
+ * states, log-weights, arguments and errors are those of the three calls (the ESS sums are added
+ * in the same precision); up to about 2.4 million particles it is one cooperative launch that
+ * reads and writes every particle once. RS_ERR_CUDA where the device cannot launch
+ * cooperatively, as rs_ess; 1 <= N <= the handle's max_n. */
+int rs_lgssm_step_ess(rs_handle* h, float* x_dev, const int32_t* c_dev, int64_t N, int init,
+                      float phi, float sigma_x, float y, float sigma_y, uint64_t seed,
+                      uint64_t step, uint32_t filter, float* logw_dev, double* ess_dev,
+                      double* log_total_dev, void* stream);
+
 /* ---- resampling on demand inside a CUDA graph ------------------------------------------
  * The adaptive filter resamples only when the effective sample size falls below a threshold
  * (Section 4 mentions the practice). To keep that decision on the device -- the whole filter

@@ -41,6 +41,7 @@ EXPORTED = [
     "rs_prepermute", "rs_permute", "rs_metropolis_B", "rs_last_error", "rs_strerror",
     "rs_trace", "rs_trace_count", "rs_trace_label", "rs_systematic_noalloc",
     "rs_resample_batched", "rs_set_launch_mode", "rs_copy_ancestors", "rs_lgssm_step",
+    "rs_lgssm_step_ess",
     "rs_ess", "rs_resample_prc", "rs_copy_ancestors_batched", "rs_lgssm_step_batched",
     "rs_log_sum_weights_batched", "rs_ess_batched", "rs_metropolis_B_batched",
     "rs_resample_batched_masked", "rs_reset_weights_batched",
@@ -138,6 +139,8 @@ def _declare(lib):
                                 P]),
         "rs_resample_rejection_estimated": (I, [P, I, P, I64, I64, I64, U64, U64, C.c_uint32, P,
                                                 P, P, P, I, P]),
+        "rs_lgssm_step_ess": (I, [P, P, P, I64, I, C.c_float, C.c_float, C.c_float, C.c_float, U64,
+                                  U64, C.c_uint32, P, P, P, P]),
         "rs_lgssm_step": (I, [P, P, I64, I, I, C.c_float, C.c_float, C.c_float, C.c_float,
                               U64, U64, C.c_uint32, P, P]),
     }
@@ -473,6 +476,31 @@ def rs_lgssm_step(h: Handle, x: torch.Tensor, init: bool, phi: float, sigma_x: f
                                 int(seed), int(step), int(filter),
                                 _dev(logw, torch.float32, "logw", N, h), _stream(stream)),
            "rs_lgssm_step")
+    return logw
+
+
+def rs_lgssm_step_ess(h: Handle, x: torch.Tensor, c: torch.Tensor | None, init: bool, phi: float,
+                      sigma_x: float, y: float, sigma_y: float, seed: int = 0, step: int = 0,
+                      filter: int = 0, logw: torch.Tensor | None = None,
+                      ess: torch.Tensor | None = None, log_total: torch.Tensor | None = None,
+                      stream=None) -> torch.Tensor:
+    """One bootstrap step around the resampling: x by the ancestry c (None: no copy), propagated
+    and weighted in place, and the ESS and log weight total of the new log-weights (returned)."""
+    N = x.numel()
+    if c is not None and c.numel() != N:
+        raise ValueError("x and c disagree on N")
+    if logw is None:
+        logw = torch.empty(N, dtype=torch.float32, device=x.device)
+    if ess is None and log_total is None:
+        ess = torch.empty(1, dtype=torch.float64, device=x.device)
+    _check(load().rs_lgssm_step_ess(
+        h.ptr, _dev(x, torch.float32, "x", h=h),
+        _dev(c, torch.int32, "c", h=h) if c is not None else None, N, int(bool(init)),
+        float(phi), float(sigma_x), float(y), float(sigma_y), int(seed), int(step), int(filter),
+        _dev(logw, torch.float32, "logw", N, h),
+        _dev(ess, torch.float64, "ess", 1, h) if ess is not None else None,
+        _dev(log_total, torch.float64, "log_total", 1, h) if log_total is not None else None,
+        _stream(stream)), "rs_lgssm_step_ess")
     return logw
 
 

@@ -541,6 +541,25 @@ int rs_lgssm_step(rs_handle* h, float* x_dev, int64_t N, int init, int accumulat
   return cuda_status(e);
 }
 
+int rs_lgssm_step_ess(rs_handle* h, float* x_dev, const int32_t* c_dev, int64_t N, int init,
+                      float phi, float sigma_x, float y, float sigma_y, uint64_t seed,
+                      uint64_t step, uint32_t filter, float* logw_dev, double* ess_dev,
+                      double* log_total_dev, void* stream) {
+  if (!h || !x_dev || !logw_dev || (!ess_dev && !log_total_dev)) return RS_ERR_ARG;
+  int st = check_n(h, N);
+  if (st != RS_OK) return st;
+  if ((init != 0 && init != 1) || (init == 1 && c_dev)) return RS_ERR_ARG;
+  if (!(std::fabs(phi) < 1.0f) || !(sigma_x > 0.0f) || !(sigma_y > 0.0f) || !std::isfinite(y) ||
+      !std::isfinite(sigma_x) || !std::isfinite(sigma_y) || filter >= (1u << 29))
+    return RS_ERR_ARG;
+  if ((st = set_device(h)) != RS_OK) return st;
+  const cudaError_t e = rsk::launch_lgssm_step_ess(h->s, x_dev, c_dev, N, init, phi, sigma_x, y,
+                                                   sigma_y, seed, step, filter, logw_dev, ess_dev,
+                                                   log_total_dev, as_stream(stream));
+  end_mark(h, as_stream(stream));
+  return cuda_status(e);
+}
+
 int rs_copy_ancestors_batched(rs_handle* h, float* x_dev, int32_t D, const int32_t* c_dev,
                               const int64_t* offsets_dev, int32_t F, void* stream) {
   if (!h || !x_dev || !c_dev || !offsets_dev || D < 1 || F < 1) return RS_ERR_ARG;
@@ -836,8 +855,10 @@ int rs_last_error(rs_handle* h, void* stream) {
     return RS_ERR_CUDA;
   if (cudaMemcpy(h->s.err, &none, sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess)
     return RS_ERR_CUDA;
-  if (v == -RS_ERR_TIMEOUT) {  // a grid barrier gave up: its arrival counter may be stale
+  if (v == -RS_ERR_TIMEOUT) {  // a grid barrier gave up: the state it guards may be stale
     if (cudaMemset(&h->s.glob->bar.count, 0, sizeof(unsigned int)) != cudaSuccess ||
+        cudaMemset(&h->s.glob->ess_ticket, 0, sizeof(unsigned int)) != cudaSuccess ||
+        cudaMemset(&h->s.glob->ess_key, 0, sizeof(unsigned long long)) != cudaSuccess ||
         cudaDeviceSynchronize() != cudaSuccess)
       return RS_ERR_CUDA;
   }

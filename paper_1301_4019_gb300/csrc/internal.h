@@ -23,7 +23,8 @@ struct ScanGlob {
   unsigned int ticket_tile;
   unsigned int ticket_iscan;
   unsigned int batch_next;   // work counter of the batched kernel (self-resetting)
-  unsigned int batch_ticket;
+  unsigned int ess_ticket;   // CTAs of the ESS kernels that have finished (self-resetting)
+  unsigned long long ess_key;  // maximum log-weight of an ESS kernel, ordered key (self-resetting)
   GridBar bar;               // grid barrier of the cooperative kernels
   int all_zero;              // every weight of the call is zero (set with the total)
   float guide_step;          // W^N / N and N / W^N in binary32 (multinomial guide table),
@@ -176,6 +177,11 @@ cudaError_t launch_cumoff_to_ancestors(const Scratch& s, const int32_t* O, int64
                                        int32_t* a, cudaStream_t st);
 
 // ess.cu (cooperative; cudaErrorNotSupported without cooperative launches)
+// one bootstrap step: copy by c (or null), propagate and weight, ESS and log weight total
+cudaError_t launch_lgssm_step_ess(const Scratch& s, float* x, const int32_t* c, int64_t N,
+                                  int init, float phi, float sigma_x, float y, float sigma_y,
+                                  uint64_t seed, uint64_t step, uint32_t filter, float* logw,
+                                  double* ess, double* log_total, cudaStream_t st);
 cudaError_t launch_ess(const Scratch& s, bool f64, const void* logw, int64_t N, double* ess,
                        double* log_total, cudaStream_t st);
 

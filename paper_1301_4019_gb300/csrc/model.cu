@@ -8,6 +8,7 @@
 #include "common.cuh"
 #include "internal.h"
 #include "measure.h"
+#include "model.cuh"
 #include "values.cuh"
 
 namespace rsk {
@@ -29,15 +30,6 @@ copy_ancestors_kernel(float* __restrict__ x, int D, const int32_t* __restrict__ 
   }
   if (ci == i) return;
   for (int k = 0; k < D; ++k) x[i * D + k] = x[static_cast<int64_t>(ci) * D + k];
-}
-
-// One standard normal per particle by Box-Muller from the Philox words 0 and 1 of counter
-// (i, 0, step, filter * 8 + 5): u1 = 1 - U_0 in (0, 1], u2 = U_1 in [0, 1).
-__device__ __forceinline__ float normal_draw(const Keys& keys, int64_t i) {
-  const uint4 r = draw(keys, static_cast<uint32_t>(i), 0u);
-  const float u1 = 1.0f - __fmul_rn(__uint2float_rn(r.x >> 8), 0x1p-24f);
-  const float u2 = __fmul_rn(__uint2float_rn(r.y >> 8), 0x1p-24f);
-  return sqrtf(-2.0f * logf(u1)) * cospif(2.0f * u2);
 }
 
 __global__ void __launch_bounds__(kBlock)
@@ -336,11 +328,10 @@ cudaError_t launch_copy_ancestors(const Scratch& s, float* x, int D, const int32
 cudaError_t launch_lgssm_step(const Scratch& s, float* x, int64_t N, int init, int accumulate,
                               float phi, float sigma_x, float y, float sigma_y, uint64_t seed,
                               uint64_t step, uint32_t filter, float* logw, cudaStream_t st) {
-  const double s0 = static_cast<double>(sigma_x) / std::sqrt(1.0 - static_cast<double>(phi) * phi);
-  const float inv_2vy = static_cast<float>(0.5 / (static_cast<double>(sigma_y) * sigma_y));
+  const LgssmConsts k = lgssm_consts(phi, sigma_x, sigma_y);
   trace_mark(s.trace, "lgssm_step", st);
   launch_pdl(lgssm_step_kernel, grid_for(N), kBlock, st, x, N, init, accumulate, phi, sigma_x,
-                                                   static_cast<float>(s0), y, inv_2vy,
+                                                   k.sigma_0, y, k.inv_2vy,
                                                    make_keys(seed, step, filter, 5u), logw);
   return cudaGetLastError();
 }
@@ -358,11 +349,10 @@ cudaError_t launch_lgssm_step_batched(const Scratch& s, float* x, const int64_t*
                                       int init, int accumulate, float phi, float sigma_x,
                                       const float* y, float sigma_y, uint64_t seed,
                                       uint64_t step, float* logw, cudaStream_t st) {
-  const double s0 = static_cast<double>(sigma_x) / std::sqrt(1.0 - static_cast<double>(phi) * phi);
-  const float inv_2vy = static_cast<float>(0.5 / (static_cast<double>(sigma_y) * sigma_y));
+  const LgssmConsts k = lgssm_consts(phi, sigma_x, sigma_y);
   trace_mark(s.trace, "lgssm_step_batched", st);
   launch_pdl(lgssm_step_batched_kernel, grid_for(s.max_n), kBlock, st, x, offsets, F, s.max_n,
-             init, accumulate, phi, sigma_x, static_cast<float>(s0), y, inv_2vy,
+             init, accumulate, phi, sigma_x, k.sigma_0, y, k.inv_2vy,
              make_keys(seed, step, 0u, 5u), logw);
   return cudaGetLastError();
 }

@@ -16,7 +16,7 @@ import torch
 
 from . import (PREC_COMPENSATED, Handle, rs_capture_end_if, rs_capture_if_below,
                rs_copy_ancestors, rs_copy_ancestors_batched, rs_ess,
-               rs_lgssm_step, rs_lgssm_step_batched, rs_log_sum_weights_batched, rs_resample,
+               rs_lgssm_step, rs_lgssm_step_batched, rs_lgssm_step_ess, rs_log_sum_weights_batched, rs_resample,
                rs_resample_batched, rs_smc_loglik_step, rs_smc_mark_resampled, rs_ess_batched,
                rs_reset_weights_batched)
 
@@ -46,10 +46,9 @@ def lgssm_bootstrap_launch(h: Handle, y, N: int, scheme: int, phi: float, sigma_
         if t > 0:
             rs_resample(h, scheme, b.logw, B=B, seed=seed, step=t, out=b.c, permute=True,
                         prec=prec, log_wmax=0.0, filter=filter, stream=stream)
-            rs_copy_ancestors(h, b.x, b.c, stream=stream)
-        rs_lgssm_step(h, b.x, t == 0, phi, sigma_x, float(y[t]), sigma_y, seed=seed, step=t,
-                      filter=filter, logw=b.logw, stream=stream)
-        rs_ess(h, b.logw, out=b.ess, log_total=b.log_total[t:t + 1], stream=stream)
+        rs_lgssm_step_ess(h, b.x, b.c if t > 0 else None, t == 0, phi, sigma_x, float(y[t]),
+                          sigma_y, seed=seed, step=t, filter=filter, logw=b.logw, ess=b.ess,
+                          log_total=b.log_total[t:t + 1], stream=stream)
     return b
 
 

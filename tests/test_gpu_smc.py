@@ -366,3 +366,55 @@ def test_batched_adaptive_loglik_matches_kalman(rs, h, scheme):
     assert rs.rs_last_error(h) == rs.RS_OK
     assert bool(fa.all())
     assert torch.equal(a.x, e.x) and torch.equal(a.log_total, e.log_total)
+
+
+# one particle, partial quadruples, one and several quadruples per thread (608 CTAs of 256
+# threads hold 622592 particles at one each), more than the one-launch form takes
+@pytest.mark.parametrize("N", [1, 3, 4, 1021, 4099, 622592, 622593, 1245185, 2490368, 2490371])
+@pytest.mark.parametrize("shift", [0, 1])
+def test_step_ess_equals_the_three_calls(rs, N, shift):
+    """rs_lgssm_step_ess gives the states and log-weights of rs_copy_ancestors + rs_lgssm_step bit
+    for bit, and rs_ess's values to the precision of its sums (weights equal, two-float sums in
+    another order: 2^-40), on aligned and unaligned buffers; a row whose ancestor breaks Permute's
+    predicate stays and is reported."""
+    g = torch.Generator(device=DEV)
+    g.manual_seed(N + shift)
+
+    def buf(dtype):
+        return torch.empty(N + shift, dtype=dtype, device=DEV)[shift:]
+
+    with rs.Handle(N) as hh:
+        lw = torch.randn(N, generator=g, device=DEV, dtype=torch.float32)
+        c = buf(torch.int32)
+        c.copy_(rs.rs_resample(hh, rs.SYSTEMATIC, lw, seed=3, permute=True))
+        x0 = torch.randn(N, generator=g, device=DEV, dtype=torch.float32)
+        args = dict(phi=PHI, sigma_x=SX, y=0.7, sigma_y=SY, seed=5, step=2, filter=3)
+        for bad in (False, True):
+            if bad and N < 4:
+                continue
+            if bad:
+                loser = int((c != torch.arange(N, device=DEV, dtype=torch.int32)).nonzero()[0])
+                c[0 if loser else 1] = loser  # c[loser] != loser
+            for init in (False, True):
+                cc = None if init else c
+                xa, xb, la, lb = (buf(torch.float32) for _ in range(4))
+                xa.copy_(x0)
+                xb.copy_(x0)
+                ess = torch.empty(2, dtype=torch.float64, device=DEV)
+                lt = torch.empty(2, dtype=torch.float64, device=DEV)
+                if cc is not None:
+                    rs.rs_copy_ancestors(hh, xa, cc)
+                rs.rs_lgssm_step(hh, xa, init, logw=la, **args)
+                rs.rs_ess(hh, la, out=ess[:1], log_total=lt[:1])
+                st = rs.rs_last_error(hh)
+                assert st == (rs.RS_ERR_ARG if bad and not init else rs.RS_OK)
+                for _ in range(2):  # (the second finds the shared state reset)
+                    xb.copy_(x0)
+                    rs.rs_lgssm_step_ess(hh, xb, cc, init, logw=lb, ess=ess[1:],
+                                         log_total=lt[1:], **args)
+                    assert rs.rs_last_error(hh) == st
+                    assert torch.equal(xa, xb) and torch.equal(la, lb)
+                    e, t = ess.tolist(), lt.tolist()
+                    assert abs(e[1] - e[0]) <= 2.0 ** -40 * e[0] and abs(t[1] - t[0]) <= 2.0 ** -40
+        with pytest.raises(rs.RsError):
+            rs.rs_lgssm_step_ess(hh, xb, c, True, logw=lb, **args)
