@@ -127,7 +127,7 @@ __global__ void __launch_bounds__(kBlock)
 cumoff_to_ancestors_kernel(const int32_t* __restrict__ O, int64_t N, int32_t* __restrict__ a,
                            int* err) {
   pdl_wait();
-  __shared__ alignas(16) int32_t win[kWarps][kRunWin];
+  __shared__ SegSh sh;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t j0l = (static_cast<int64_t>(blockIdx.x) * kWarps + warp) * kSeg;
   if (j0l >= N) return;  // (warp-uniform: only warp-level synchronisation below)
@@ -177,7 +177,7 @@ cumoff_to_ancestors_kernel(const int32_t* __restrict__ O, int64_t N, int32_t* __
     }
   }
   if (__any_sync(0xffffffffu, bad) && lane == 0) flag_error(err, RS_ERR_ARG);
-  warp_runs(Oe, prev, i0, a, win[warp]);
+  warp_runs(Oe, prev, i0, a, sh.win[warp]);
 }
 
 // Integer inclusive prefix sum, reduce-then-scan over tiles of 4096 (exact in int64):

@@ -352,7 +352,7 @@ batch_emit_kernel(const T* __restrict__ lw, Batch b, Keys base_keys,
         SCHEME == RS_STRATIFIED ? typename Path<T, V>::U() : cta_uniform0<T, V>(keys);
     emit_seg_cumoff<T, V, SCHEME == RS_STRATIFIED>(
         lw, L.lo, L.hi, base, wc, vec, Ps, Pn, load_v_cg<V>(b.fS + L.f),
-        load_v_cg<V>(b.fscale + L.f), u_sys, keys, a, d, sh.win[warp],
+        load_v_cg<V>(b.fscale + L.f), u_sys, keys, a, sh.win[warp],
         claimed_bits(b, L.f, L.lo));
   }
 }
@@ -625,7 +625,7 @@ batch_coop_kernel(const T* __restrict__ lw, Batch b, Keys base_keys, int32_t* __
     } else {
       emit_seg_cumoff<T, V, SCHEME == RS_STRATIFIED>(
           lw, w.lo, w.hi, base, wc, vec, Ps, Pn, S, scale, u_sys,
-          with_tag(base_keys, static_cast<uint32_t>(w.f), SCHEME), a, d, sh.win[warp], cl,
+          with_tag(base_keys, static_cast<uint32_t>(w.f), SCHEME), a, sh.win[warp], cl,
           L2Hint::kEvictFirst);
     }
   }

@@ -13,7 +13,7 @@ namespace rsk {
 constexpr int kBlock = 256;          // threads per CTA of the streaming kernels
 constexpr int kPer = 8;              // consecutive particles per thread in a scan tile
 constexpr int kTile = kBlock * kPer; // particles per CTA tile of the scan kernels (2048)
-constexpr int kRunWin = 32 * kPer;  // positions a warp covers per round of Code 11 (warp_runs)
+constexpr int kRunWin = 32 * kPer;  // positions a warp covers at a time in Code 11 (warp_runs)
 constexpr int kWarps = kBlock / 32;  // 8 warps
 // Entries of each of the two record blocks of the scan scratch (records, then prefixes): one
 // per warp segment of kRunWin particles (kWarps per tile), plus the total's prefix and a spare.
@@ -223,8 +223,14 @@ __device__ __forceinline__ double exp_pinned(double x) {
 // 0, not NaN); every t < -87 gives 0 or a value below 2^-125. NaN stays NaN.
 // ---------------------------------------------------------------------------------------
 constexpr double kScanExpRelErr = 0x1p-21;
+// max(a, b), NaN if either is.
+__device__ __forceinline__ float max_nan(float a, float b) {
+  float r;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+  return r;
+}
 __device__ __forceinline__ float exp_scan_f32(float t) {
-  t = (t < -150.0f) ? -150.0f : t;
+  t = max_nan(t, -150.0f);
   const float a = __fmul_rn(t, 0x1.715476p+0f);
   float e = __fmaf_rn(t, 0x1.715476p+0f, -a);
   e = __fmaf_rn(t, 0x1.4ae0c0p-26f, e);

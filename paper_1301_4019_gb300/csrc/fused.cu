@@ -45,8 +45,8 @@ struct FusedArgs {
   int64_t N;
   Keys keys;
   int32_t* a;      // ancestors (systematic / stratified)
-  int32_t* d;      // Prepermute claims, or nullptr
-  uint8_t* cl;     // claimed bits of the particles (in place of d for the sorted Permute), or nullptr
+  int32_t* d;      // Prepermute claims of the multinomial (set to the sentinel), or nullptr
+  uint8_t* cl;     // claimed bits of the particles (systematic / stratified), or nullptr
   void* W;         // multinomial cumulative weights
   int32_t* guide;  // multinomial guide table
   double2* s_rec;  // segment records
@@ -221,7 +221,6 @@ __device__ __forceinline__ void fused_body(const T* __restrict__ lw, const Fused
     if constexpr (SCHEME != RS_MULTINOMIAL) {  // (the search kernel writes the identity)
       for (int64_t i = e0 + threadIdx.x; i < e1; i += kBlock) {
         A.a[i] = static_cast<int32_t>(i);
-        if (A.d) A.d[i] = static_cast<int32_t>(i);
       }
       if (A.cl)  // every slot claimed (e0 is a multiple of 8)
         for (int64_t b = (e0 >> 3) + threadIdx.x; b < ((e1 + 7) >> 3); b += kBlock) A.cl[b] = 0xFFu;
@@ -269,7 +268,6 @@ __device__ __forceinline__ void fused_body(const T* __restrict__ lw, const Fused
     if constexpr (SCHEME != RS_MULTINOMIAL) {
       for (int64_t i = e0 + threadIdx.x; i < e1; i += kBlock) {
         A.a[i] = static_cast<int32_t>(i);
-        if (A.d) A.d[i] = static_cast<int32_t>(i);
       }
       if (A.cl)
         for (int64_t b = (e0 >> 3) + threadIdx.x; b < ((e1 + 7) >> 3); b += kBlock) A.cl[b] = 0xFFu;
@@ -311,7 +309,7 @@ __device__ __forceinline__ void fused_body(const T* __restrict__ lw, const Fused
                              sh.win[warp], L2Hint::kEvictFirst);
     } else {
       emit_seg_cumoff<T, V, SCHEME == RS_STRATIFIED>(lw, 0, N, base, wc, vec, Ps, Pn, S, scale,
-                                                      u_sys, A.keys, A.a, A.d, sh.win[warp], A.cl,
+                                                      u_sys, A.keys, A.a, sh.win[warp], A.cl,
                                                       L2Hint::kEvictFirst);
     }
   }

@@ -251,6 +251,32 @@ __device__ __forceinline__ double tmin(double a, double b) {
 __device__ __forceinline__ float2 tmax(float2 a, float2 b) { return vmax(a, b); }
 __device__ __forceinline__ float2 tmin(float2 a, float2 b) { return vmin(a, b); }
 
+// One step of a scan over the lanes: y + v (the accumulator's addition) or max(y, v) with y the
+// value dd lanes below, v itself in the first dd lanes. Binary32 takes the predicate that the
+// shuffle returns.
+template <typename V> __device__ __forceinline__ V up_add(V v, int dd) {
+  const V y = vshfl_up(v, dd);
+  return (threadIdx.x & 31) >= dd ? vadd(y, v) : v;
+}
+template <typename V> __device__ __forceinline__ V up_max(V v, int dd) {
+  const V y = vshfl_up(v, dd);
+  return (threadIdx.x & 31) >= dd ? tmax(y, v) : v;
+}
+template <> __device__ __forceinline__ float up_add<float>(float v, int dd) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t.reg .f32 y;\n\t"
+      "shfl.sync.up.b32 y|p, %0, %1, 0, 0xffffffff;\n\t@p add.rn.f32 %0, y, %0;\n\t}"
+      : "+f"(v) : "r"(dd));
+  return v;
+}
+template <> __device__ __forceinline__ float up_max<float>(float v, int dd) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t.reg .f32 y;\n\t"
+      "shfl.sync.up.b32 y|p, %0, %1, 0, 0xffffffff;\n\t@p max.f32 %0, y, %0;\n\t}"
+      : "+f"(v) : "r"(dd));
+  return v;
+}
+
 // Equality of two accumulator values (non-negative, never NaN here).
 __device__ __forceinline__ bool vsame(float a, float b) { return a == b; }
 __device__ __forceinline__ bool vsame(double a, double b) {
@@ -726,66 +752,133 @@ __device__ void seg_prefix_compute(const double2* s_rec, double2* P_rec, int nt,
 }
 
 // Shared scratch of the segment emissions: one warp_runs window per warp.
+constexpr int kRunSpan = 2 * kRunWin;  // positions of a window
 struct SegSh {
-  alignas(16) int32_t win[kWarps][kRunWin];
+  alignas(16) int32_t win[kWarps][kRunSpan];
 };
+
+// Eight consecutive values to a 32-byte aligned address (one whole sector).
+__device__ __forceinline__ void st_global_v8(int32_t* p, const int32_t (&v)[kPer]) {
+  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(v[0]),
+               "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
+               : "memory");
+}
 
 // Code 11 for the particles of one warp: out[j] = the index of the particle whose run
 // [O_{i-1}, O_i) holds j, for every j of the warp's range [P0, P1) (P0 = the count before the
 // warp's first particle, P1 = after its last). Lane l holds the non-decreasing counts Oe[q] of
-// its kPer particles i0 + q and `prev`, the count before them. The range is written in
-// rounds of kRunWin positions through the warp's shared window: -1 everywhere, the first
-// position of each run receives its particle's index, a running maximum (in-lane, then a
-// max-scan over the lanes, then the last value of the previous round, which every lane takes
-// into account: a run can cover a whole round) fills the runs, and the window is stored with
-// consecutive lanes on consecutive positions. The first position P0 always starts a run, so
-// the carry of the first round can be -1. Same result as writing out[j] = i for j in
-// [O_{i-1}, O_i) particle by particle, without its divergent loops.
-__device__ __forceinline__ void warp_runs(const int32_t (&Oe)[kPer], int32_t prev, int32_t i0,
-                                          int32_t* __restrict__ out, int32_t* win) {
+// its kPer particles i0 + q and `prev`, the count before them. Returns the bits of this lane's
+// particles that have a run (bit q: particle i0 + q).
+//
+// The range is written through the warp's shared window of kRunSpan positions (nearly always
+// one: a segment's kSeg particles have about kSeg offspring): -1 everywhere, then the first
+// position of each run receives its particle's index; the window is read back, eight consecutive
+// positions per lane, and filled by a running maximum (in-lane; then the last head before the
+// lane, found by ballot; or the last value of the part before, which every lane takes into
+// account: a run can cover a whole part). Windows start at 32-byte boundaries of `out`, so a
+// lane's eight positions are one 256-bit store; the two groups of eight that the range's ends
+// cut are written back and stored by sixteen lanes. A short rest beyond the first 256 positions
+// (half of the segments have one, mostly under 32 positions) is read two positions per lane.
+// The first position P0 always starts a run, so the carry of the first part can be -1.
+//
+// Every head lies in [P0, P1): the counts are those of cumulative weights (or of checked counts)
+// that lie between the segment's two prefixes and are non-decreasing functions of them, so one
+// window holds all heads when P1 - base <= kRunSpan; longer ranges test every head.
+// Same result as writing out[j] = i for j in [O_{i-1}, O_i) particle by particle, without its
+// divergent loops.
+__device__ __forceinline__ uint32_t warp_runs(const int32_t (&Oe)[kPer], int32_t prev, int32_t i0,
+                                              int32_t* __restrict__ out, int32_t* win) {
+  static_assert(kPer == 8 && kRunWin == 256, "a lane's positions are one 32-byte sector");
   const int lane = threadIdx.x & 31;
+  const unsigned below = (1u << lane) - 1u;
   const int32_t P0 = __shfl_sync(0xffffffffu, prev, 0);
   const int32_t P1 = __shfl_sync(0xffffffffu, Oe[kPer - 1], 31);
+  const int32_t shift = static_cast<int32_t>((reinterpret_cast<uintptr_t>(out) >> 2) & 7u);
   int4* const w4 = reinterpret_cast<int4*>(win);
+  uint32_t bits = 0;
   int32_t carry = -1;
-  for (int32_t base = P0; base < P1; base += kRunWin) {  // warp-uniform
-    __syncwarp();
-    w4[2 * lane] = make_int4(-1, -1, -1, -1);
-    w4[2 * lane + 1] = make_int4(-1, -1, -1, -1);
-    __syncwarp();
-    int32_t p = prev;
-#pragma unroll
-    for (int q = 0; q < kPer; ++q) {
-      const int32_t pos = p - base;
-      if (Oe[q] > p && pos >= 0 && pos < kRunWin) win[pos] = i0 + q;
-      p = Oe[q];
-    }
-    __syncwarp();
-    const int4 u0 = w4[2 * lane], u1 = w4[2 * lane + 1];
+  // the last head at or before this lane's last position of a part (top: its in-lane maximum)
+  auto before_lane = [&](int32_t top) {
+    const unsigned heads = __ballot_sync(0xffffffffu, top >= 0);
+    const unsigned earlier = heads & below;
+    const int32_t m = __shfl_sync(0xffffffffu, top, 31 - __clz(earlier | 1u));
+    const int32_t em = earlier ? m : carry;
+    const int32_t last = __shfl_sync(0xffffffffu, top, 31 - __clz(heads | 1u));
+    carry = heads ? last : carry;
+    return em;
+  };
+  auto part8 = [&](int h, int32_t base) {  // 256 positions
+    const int4 u0 = w4[64 * h + 2 * lane], u1 = w4[64 * h + 2 * lane + 1];
     int32_t v[kPer] = {u0.x, u0.y, u0.z, u0.w, u1.x, u1.y, u1.z, u1.w};
 #pragma unroll
     for (int k = 1; k < kPer; ++k) v[k] = max(v[k], v[k - 1]);
-    int32_t m = v[kPer - 1];
-#pragma unroll
-    for (int dd = 1; dd < 32; dd <<= 1) {
-      const int32_t y = __shfl_up_sync(0xffffffffu, m, dd);
-      if (lane >= dd) m = max(m, y);
-    }
-    int32_t em = __shfl_up_sync(0xffffffffu, m, 1);  // the earlier lanes of this round
-    em = lane == 0 ? carry : max(em, carry);          // and the run carried into the round
+    const int32_t em = before_lane(v[kPer - 1]);
 #pragma unroll
     for (int k = 0; k < kPer; ++k) v[k] = max(v[k], em);
-    carry = __shfl_sync(0xffffffffu, v[kPer - 1], 31);
-    __syncwarp();
-    w4[2 * lane] = make_int4(v[0], v[1], v[2], v[3]);
-    w4[2 * lane + 1] = make_int4(v[4], v[5], v[6], v[7]);
-    __syncwarp();
-#pragma unroll
-    for (int k = 0; k < kPer; ++k) {
-      const int32_t j = base + 32 * k + lane;
-      if (j < P1) out[j] = win[32 * k + lane];
+    const int32_t j0 = base + kPer * lane;
+    if (j0 >= P0 && j0 + kPer <= P1) {
+      st_global_v8(out + j0, v);
+    } else if (j0 + kPer > P0 && j0 < P1) {  // cut by an end of the range
+      w4[64 * h + 2 * lane] = make_int4(v[0], v[1], v[2], v[3]);
+      w4[64 * h + 2 * lane + 1] = make_int4(v[4], v[5], v[6], v[7]);
     }
+  };
+  for (int32_t base = ((P0 + shift) & ~7) - shift; base < P1; base += kRunSpan) {  // warp-uniform
+    const int32_t len = P1 - base;
+    const int4 none = make_int4(-1, -1, -1, -1);
+    __syncwarp();
+    w4[lane] = none;
+    w4[32 + lane] = none;
+    if (len > kRunWin) {
+      w4[64 + lane] = none;
+      w4[96 + lane] = none;
+    }
+    __syncwarp();
+    int32_t p = prev;
+    if (len <= kRunSpan && base <= P0) {
+      int32_t* const wb = win - base;
+#pragma unroll
+      for (int q = 0; q < kPer; ++q) {
+        if (Oe[q] > p) {
+          bits |= 1u << q;
+          wb[p] = i0 + q;
+        }
+        p = Oe[q];
+      }
+    } else {
+#pragma unroll
+      for (int q = 0; q < kPer; ++q) {
+        if (Oe[q] > p) {
+          bits |= 1u << q;
+          const uint32_t pos = static_cast<uint32_t>(p - base);
+          if (pos < static_cast<uint32_t>(kRunSpan)) win[pos] = i0 + q;
+        }
+        p = Oe[q];
+      }
+    }
+    __syncwarp();
+    part8(0, base);
+    int32_t cut = len < kRunSpan ? (len & ~7) : kRunSpan;  // the group that the range's end cuts
+    if (len > kRunWin + 64) {
+      part8(1, base + kRunWin);
+    } else if (len > kRunWin) {  // a short rest: two positions per lane
+      const int2 u = reinterpret_cast<const int2*>(win + kRunWin)[lane];
+      const int32_t top = max(u.x, u.y);
+      const int32_t em = before_lane(top);
+      const int32_t j0 = base + kRunWin + 2 * lane;
+      if (j0 < P1) out[j0] = max(u.x, em);
+      if (j0 + 1 < P1) out[j0 + 1] = max(top, em);
+      cut = kRunSpan;  // (nothing left to store)
+    }
+    __syncwarp();
+    // the groups that the ends cut: the window's first (where it starts before P0), by the first
+    // eight lanes, and the one that holds P1, by the next eight
+    const int idx = lane < kPer ? lane : cut + lane - kPer;
+    if (lane < 2 * kPer && idx < len && idx < kRunSpan && base + idx >= P0 &&
+        (lane >= kPer ? (len & 7) != 0 : base < P0))
+      out[base + idx] = win[idx];
   }
+  return bits;
 }
 
 // The record of a segment (warp-level) from this lane's kPer log-weights x of it (-inf outside
@@ -810,11 +903,14 @@ __device__ __forceinline__ long long seg_record(const T (&x)[kPer], const float2
   if (ref != kTileMaxRef) {  // (uniform) a given reference replaces the segment's maximum
     m = ref;
   } else if constexpr (sizeof(T) == 4) {
-    float mf = -INFINITY;
+    float mf = x[0];
 #pragma unroll
-    for (int q = 0; q < kPer; ++q) {
-      bad |= !(x[q] <= FLT_MAX);  // NaN or +inf (-inf and finite values pass)
-      mf = fmaxf(mf, x[q]);       // fmaxf skips NaN
+    for (int q = 1; q < kPer; ++q) mf = max_nan(mf, x[q]);
+    if (!(mf <= FLT_MAX)) {  // a NaN or +inf among them (-inf and finite values pass)
+      bad = true;
+      mf = -INFINITY;
+#pragma unroll
+      for (int q = 0; q < kPer; ++q) mf = fmaxf(mf, x[q]);  // fmaxf skips NaN
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) mf = fmaxf(mf, __shfl_xor_sync(0xffffffffu, mf, o));
@@ -891,10 +987,7 @@ __device__ __forceinline__ void seg_cum_weights(const T* __restrict__ lw, int64_
   }
   V incl = W[kPer - 1];
 #pragma unroll
-  for (int dd = 1; dd < 32; dd <<= 1) {
-    const V y = vshfl_up(incl, dd);
-    if (lane >= dd) incl = vadd(y, incl);
-  }
+  for (int dd = 1; dd < 32; dd <<= 1) incl = up_add(incl, dd);
   V excl = vshfl_up(incl, 1);
   if (lane == 0) excl = vzero(V());
   const V b = vadd(Ps, excl);
@@ -902,17 +995,14 @@ __device__ __forceinline__ void seg_cum_weights(const T* __restrict__ lw, int64_
   for (int q = 0; q < kPer; ++q) W[q] = vadd(b, W[q]);
   V m = W[kPer - 1];
 #pragma unroll
-  for (int dd = 1; dd < 32; dd <<= 1) {
-    const V y = vshfl_up(m, dd);
-    if (lane >= dd) m = tmax(y, m);
-  }
+  for (int dd = 1; dd < 32; dd <<= 1) m = up_max(m, dd);
   V pm = vshfl_up(m, 1);
   if (lane == 0) pm = Ps;
 #pragma unroll
   for (int q = 0; q < kPer; ++q) W[q] = tmin(tmax(W[q], pm), Pn);
   if (lane == 31) W[kPer - 1] = Pn;
-  const int lq = seg_count(base, N) - 1 - kPer * lane;  // the segment's last valid particle here?
-  if (lq >= 0 && lq < kPer) {
+  if (base + kSeg > N) {  // (warp-uniform) the segment's last valid particle is an earlier one
+    const int lq = seg_count(base, N) - 1 - kPer * lane;
 #pragma unroll
     for (int q = 0; q < kPer; ++q)
       if (q == lq) W[q] = Pn;
@@ -945,14 +1035,11 @@ __device__ __forceinline__ void store_per(int32_t* __restrict__ p, const int32_t
 }
 
 // Systematic / stratified emission of one segment starting at `base` of the sequence [lo, N)
-// (warp-level): cumulative offspring O of every particle, the Code-11 scatter of local
-// ancestor indices into a[lo + j] through the warp's window `win` and, when d is given, the
-// Prepermute claims d[lo + i] = O_{i-1} if particle i has offspring, else n (for a
-// non-decreasing ancestry the lowest claimant of slot i is the first position of its run).
-// When cl is given (single sequence, lo = 0), one bit per particle instead: bit i % 8 of
-// cl[i / 8] is set when particle i has offspring (its slot is claimed), the only part of the
-// claims that the Permute of a non-decreasing ancestry cannot read off a itself
-// (permute_sorted_bits_kernel).
+// (warp-level): cumulative offspring O of every particle and the Code-11 scatter of local
+// ancestor indices into a[lo + j] through the warp's window `win`. When cl is given (the claimed
+// bits of the sequence), one bit per particle: bit i % 8 of cl[i / 8] is set when particle i has
+// offspring (its slot is claimed), the only part of the Prepermute claims that the Permute of a
+// non-decreasing ancestry cannot read off a itself (permute_sorted_slots).
 // Ps, Pn: prefixes of this segment and the next; u_sys: the systematic uniform (cta_uniform0;
 // unused when STRAT). Local indices are 32-bit (n < 2^31).
 template <typename T, typename V, bool STRAT>
@@ -961,13 +1048,13 @@ __device__ __forceinline__ void emit_seg_cumoff(const T* __restrict__ lw, int64_
                                                 V Ps, V Pn, V S, V scale,
                                                 typename Path<T, V>::U u_sys,
                                                 const Keys& keys, int32_t* __restrict__ a,
-                                                int32_t* __restrict__ d, int32_t* win,
-                                                uint8_t* __restrict__ cl = nullptr,
+                                                int32_t* win, uint8_t* __restrict__ cl = nullptr,
                                                 L2Hint hint = L2Hint::kNormal) {
   const int lane = threadIdx.x & 31;
   const int32_t n = static_cast<int32_t>(N - lo);
+  const int32_t b0 = static_cast<int32_t>(base - lo);
   const int cnt = seg_count(base, N) - kPer * lane;  // valid here
-  const int32_t i0 = static_cast<int32_t>(base - lo) + kPer * lane;
+  const int32_t i0 = b0 + kPer * lane;
   V W[kPer], Wb;
   seg_cum_weights<T, V>(lw, lo, N, base, wc, vec, Ps, Pn, W, Wb, hint);
   // O of this lane's particles; the last particle of the sequence gets n, and positions
@@ -978,39 +1065,34 @@ __device__ __forceinline__ void emit_seg_cumoff(const T* __restrict__ lw, int64_
   if constexpr (STRAT) {
     strat_offspring_warp<T, V>(W, Wb, S, scale, keys, n, cnt > 0, O, Ob);
   } else {
+    // (warp-uniform) where the count at Pn is below n no cumulative weight of the segment
+    // reaches the total or needs the clamp to n, O being monotone in W <= Pn
+    const int32_t on = vsame(Pn, S) ? n : floor_i32(vplus_u(vscale(Pn, scale), u_sys));
+    if (on < n) {
 #pragma unroll
-    for (int q = 0; q < kPer; ++q) O[q] = cum_offspring<T, V, STRAT>(W[q], S, scale, u_sys, keys, n);
+      for (int q = 0; q < kPer; ++q) O[q] = floor_i32(vplus_u(vscale(W[q], scale), u_sys));
+    } else {
+#pragma unroll
+      for (int q = 0; q < kPer; ++q)
+        O[q] = cum_offspring<T, V, STRAT>(W[q], S, scale, u_sys, keys, n);
+    }
     if (lane == 0 && cnt > 0) Ob = cum_offspring<T, V, STRAT>(Wb, S, scale, u_sys, keys, n);
   }
   const int32_t last = (cnt >= kPer && i0 + kPer - 1 != n - 1) ? O[kPer - 1] : n;
   int32_t prev = __shfl_up_sync(0xffffffffu, last, 1);
   if (lane == 0)  // (a segment wholly past the end follows the sequence's last particle: n)
     prev = Ob;
-  int32_t dv[kPer];
-  int32_t p = prev;
-  if (base + kSeg < N) {  // (warp-uniform) all kSeg particles valid, none the sequence's last
+  if (b0 + kSeg >= n) {  // (warp-uniform) the sequence's last particle, or positions past it
+    int32_t p = prev;
 #pragma unroll
     for (int q = 0; q < kPer; ++q) {
-      dv[q] = (O[q] > p) ? p : n;
+      O[q] = (q >= cnt) ? p : ((i0 + q == n - 1) ? n : O[q]);
       p = O[q];
     }
-  } else {
-#pragma unroll
-    for (int q = 0; q < kPer; ++q) {
-      const int32_t Oc = (q >= cnt) ? p : ((i0 + q == n - 1) ? n : O[q]);
-      dv[q] = (Oc > p) ? p : n;
-      O[q] = Oc;
-      p = Oc;
-    }
   }
-  warp_runs(O, prev, i0, a + lo, win);
-  if (d && cnt > 0) store_per(d + lo + i0, dv, cnt);
-  if (cl && cnt > 0) {  // (i0 is a multiple of kPer = 8: one byte per lane)
-    uint32_t bits = 0;
-#pragma unroll
-    for (int q = 0; q < kPer; ++q) bits |= static_cast<uint32_t>(dv[q] != n) << q;
-    cl[i0 >> 3] = static_cast<uint8_t>(bits);
-  }
+  const uint32_t bits = warp_runs(O, prev, i0, a + lo, win);
+  // (i0 is a multiple of kPer = 8: one byte per lane)
+  if (cl && cnt > 0) cl[i0 >> 3] = static_cast<uint8_t>(bits);
 }
 
 // Stored cumulative weights of one segment (warp-level): W[e] for e in [lo, N).
