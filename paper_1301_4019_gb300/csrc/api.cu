@@ -859,6 +859,7 @@ int rs_last_error(rs_handle* h, void* stream) {
     if (cudaMemset(&h->s.glob->bar.count, 0, sizeof(unsigned int)) != cudaSuccess ||
         cudaMemset(&h->s.glob->ess_ticket, 0, sizeof(unsigned int)) != cudaSuccess ||
         cudaMemset(&h->s.glob->ess_key, 0, sizeof(unsigned long long)) != cudaSuccess ||
+        cudaMemset(&h->s.glob->scan_key, 0, sizeof(unsigned long long)) != cudaSuccess ||
         cudaDeviceSynchronize() != cudaSuccess)
       return RS_ERR_CUDA;
   }

@@ -270,7 +270,7 @@ lgssm_step_ess_kernel(float* __restrict__ x, const int32_t* __restrict__ c, uint
     }
   }
   float2 s1 = make_float2(0.0f, 0.0f), s2 = make_float2(0.0f, 0.0f);
-  if (Mf > -FLT_MAX) {
+  if (!is_neg_inf(Mf)) {
 #pragma unroll
     for (int r = 0; r < K; ++r) {
 #pragma unroll

@@ -13,7 +13,6 @@
 // every phase stays bounds-checked, so the kernel still ends); the barrier counter returns
 // to 0 at the end of every launch.
 #include <cfloat>
-#include <climits>
 #include <type_traits>
 
 #include "common.cuh"
@@ -24,22 +23,6 @@
 
 namespace rsk {
 namespace {
-
-// Block-wide maximum of a key (every thread gets the result).
-__device__ __forceinline__ long long block_max_key(long long m, long long* sh) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const long long y = __shfl_xor_sync(0xffffffffu, m, o);
-    m = y > m ? y : m;
-  }
-  __syncthreads();
-  if (lane == 0) sh[warp] = m;
-  __syncthreads();
-  long long bm = sh[0];
-  for (int k = 1; k < kWarps; ++k) bm = sh[k] > bm ? sh[k] : bm;
-  return bm;
-}
 
 struct FusedArgs {
   int64_t N;
@@ -53,7 +36,6 @@ struct FusedArgs {
   double2* P_rec;  // segment prefixes: exact in-range prefixes (u128), then rounded P_g
   u128* agg;       // per-CTA exact totals (gridDim.x entries)
   ScanGlob* g;
-  double* blockmax;  // per-CTA maxima (gridDim.x entries)
   int* err;
 };
 
@@ -63,10 +45,10 @@ struct FusedArgs {
 // 608 CTAs; as 512 tiles some SMs had four, most three).
 //   phase 1  the records (m_g, s_g) of its segments (seg_record, each warp its own: the
 //            segment's maximum and its weights' sum relative to it), last turn to first,
-//            and its largest m_g -> barrier;
-//   phase 2  M = maximum over the CTAs; T_g = s_g exp(m_g - M) (rec_scaled) of its segments
-//            and their exact running sum in fixed point (the in-range prefix of each segment,
-//            and the CTA total) -> barrier;
+//            and its largest m_g
+//            (an atomic maximum of ordered keys per CTA) -> barrier;
+//   phase 2  T_g = s_g exp(m_g - M) (rec_scaled) of its segments and their exact running sum in
+//            fixed point (the in-range prefix of each segment, and the CTA total) -> barrier;
 //            (compensated binary32, whose records must sum the weights exp(lw - M) themselves:
 //            phase 1 forms the maximum only and phase 2 the records relative to M, which then
 //            scale by exactly 1);
@@ -78,47 +60,71 @@ struct FusedArgs {
 // Phases 1 and 4 are warp-level work only: no block barrier per turn. The log-weights are read
 // twice (phases 1 and 4; three times for compensated binary32), the least the normaliser
 // allows. P_g is the exact sum of the T before g rounded once, as in seg_prefix_compute, so the
-// results equal
-// those of the separate kernels. Two grid barriers per call.
+// results equal those of the separate kernels. Two grid barriers per call (none for one CTA).
+//
+// Phases 2 and 3 are a chain of short dependent steps that every CTA takes whatever N is (at 2^20
+// they were two thirds of the kernel's instructions and about 8 of its 20 us). So a CTA with
+// fewer than 32 segments scans them in one warp, records and prefixes of a CTA's segments stay
+// in shared memory (up to kCtaSegs of them), the totals before the CTA and the total with its
+// binary64 division are finished by two different warps, and the systematic uniform is drawn at
+// the start: 2^20 binary32 systematic 26.7 -> 24.7 us a call, 1000 particles 14.3 -> 10.3.
+constexpr int kCtaSegs = kBlock;  // segments of a CTA whose records and prefixes stay on chip
 
-// kKept: phase 2 takes this thread's first record from a load issued before the first grid
-// barrier, and phase 3 its first exact in-range prefix and the CTA total from registers (not
-// for the compensated binary32 path, whose records follow the maximum pass, nor for native
-// binary64, whose emission runs short of registers with them: both read them back from L2).
-template <typename T, typename V>
-constexpr bool kKept = Path<T, V>::kTileRef && !std::is_same_v<V, double>;
+// The order-preserving key of a log-weight as an unsigned number above 0, and back.
+template <typename T> __device__ __forceinline__ T from_key(unsigned long long k) {
+  if constexpr (sizeof(T) == 4) return from_ordered_key(static_cast<uint32_t>(k));
+  else return from_ordered_key(k);
+}
+
+// Inclusive sum over the lanes of a warp.
+__device__ __forceinline__ u128 warp_incl_scan_u128(u128 v) {
+#pragma unroll
+  for (int dd = 1; dd < 32; dd <<= 1) {
+    const u128 y = shfl_up_u128(v, dd);
+    if ((threadIdx.x & 31) >= dd) v += y;
+  }
+  return v;
+}
 
 template <typename T, typename V, int SCHEME>
 __device__ __forceinline__ void fused_body(const T* __restrict__ lw, const FusedArgs& A,
                                            unsigned int& target) {
   __shared__ SegSh sh;
   __shared__ float2 sh_tab[64];
-  __shared__ long long sh_key[kWarps];
+  __shared__ unsigned long long sh_key[kWarps];
   __shared__ u128 sh_sum[2 * kWarps];
+  __shared__ double2 sh_rp[kCtaSegs + 1];  // records, then rounded prefixes, of the CTA's segments
+  __shared__ typename Path<T, V>::U sh_u;
   const int64_t N = A.N;
   const int T_segs = static_cast<int>((N + kSeg - 1) / kSeg);
   const int G = static_cast<int>(gridDim.x), c = static_cast<int>(blockIdx.x);
   const int g0 = static_cast<int>(static_cast<int64_t>(c) * T_segs / G);  // this CTA's segments
   const int g1 = static_cast<int>(static_cast<int64_t>(c + 1) * T_segs / G);
-  const int turns = (g1 - g0 + kWarps - 1) / kWarps;
+  const int nseg = g1 - g0;
+  const bool on_chip = (T_segs + G - 1) / G <= kCtaSegs;  // (uniform over the grid)
+  const bool one_warp = nseg < 32;
+  const int turns = (nseg + kWarps - 1) / kWarps;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t e0 = static_cast<int64_t>(g0) * kSeg;
   const int64_t e1 = min(static_cast<int64_t>(g1) * kSeg, N);
   const int64_t off = kPer * static_cast<int64_t>(threadIdx.x);
   const bool vec = (reinterpret_cast<uintptr_t>(lw) & 15u) == 0;
+  double2* const recs = on_chip ? sh_rp : A.s_rec + g0;
   if (threadIdx.x < 64) sh_tab[threadIdx.x] = kExp2Frac64[threadIdx.x];
+  if constexpr (SCHEME == RS_SYSTEMATIC)
+    if (threadIdx.x == kBlock - 1) sh_u = Path<T, V>::draw_u(draw(A.keys, 0u, 0u));
   __syncthreads();
 
   // ---- phase 1: segment records, last turn to first (and the Prepermute sentinel of the
   // multinomial claims); the next segment's log-weights are loaded while this one is reduced.
   // Without kTileRef, the maximum only (the records follow once M is known) ----------------
-  double2 rec0 = make_double2(0.0, 0.0);  // (kKept) the record of segment g0 + threadIdx.x
-  const int last_turn = turns - (g0 + kWarps * (turns - 1) + warp < g1 ? 1 : 2);  // (of this warp)
+  const int last_turn = turns - (kWarps * (turns - 1) + warp < nseg ? 1 : 2);  // (of this warp)
   const int64_t lane0 = e0 + static_cast<int64_t>(kSeg) * warp + kPer * lane;  // (turn 0)
   {
-    long long cm = max_key(neg_inf<T>());
+    unsigned long long key;  // of this warp's largest log-weight
     bool bad = false;
     if constexpr (Path<T, V>::kTileRef) {
+      long long cm = max_key(neg_inf<T>());
       T xn[kPer];
       if (last_turn >= 0)
         load_per(lw, lane0 + static_cast<int64_t>(kTile) * last_turn, 0, N, vec, xn, L2Hint::kEvictLast);
@@ -129,9 +135,10 @@ __device__ __forceinline__ void fused_body(const T* __restrict__ lw, const Fused
         if (t > 0)
           load_per(lw, lane0 + static_cast<int64_t>(kTile) * (t - 1), 0, N, vec, xn,
                    L2Hint::kEvictLast);
-        const long long k = seg_record<T, V>(x, sh_tab, A.s_rec + g0 + kWarps * t + warp, bad);
+        const long long k = seg_record<T, V>(x, sh_tab, recs + kWarps * t + warp, bad);
         cm = k > cm ? k : cm;
       }
+      key = ordered_key(key_to<T>(cm));
     } else {
       float mf = -INFINITY;  // (binary32 inputs)
       for (int t = 0; t <= last_turn; ++t) {
@@ -143,7 +150,7 @@ __device__ __forceinline__ void fused_body(const T* __restrict__ lw, const Fused
           mf = fmaxf(mf, static_cast<float>(x[q]));
         }
       }
-      cm = max_key(mf);
+      key = __reduce_max_sync(0xffffffffu, ordered_key(mf));
     }
     if constexpr (SCHEME == RS_MULTINOMIAL) {
       if (A.d) {
@@ -155,60 +162,59 @@ __device__ __forceinline__ void fused_body(const T* __restrict__ lw, const Fused
       }
     }
     if (bad) flag_error(A.err, RS_ERR_NONFINITE);
-    cm = block_max_key(cm, sh_key);
-    if (threadIdx.x == 0) A.blockmax[c] = key_to_double(cm, T());
-    // this thread's record for phase 2, loaded before the grid barrier so that the load
-    // overlaps the wait (lane 0 of each warp stored the records before block_max_key's
-    // block barrier)
-    if constexpr (kKept<T, V>) {
-      const int g = g0 + static_cast<int>(threadIdx.x);
-      if (g < g1) rec0 = __ldcg(A.s_rec + g);
+    if (lane == 0) sh_key[warp] = key;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      for (int w = 1; w < kWarps; ++w) key = sh_key[w] > key ? sh_key[w] : key;
+      if (G > 1) atomicMax(&A.g->scan_key, key);
+      else sh_key[0] = key;
     }
   }
-  grid_barrier(&A.g->bar, target, A.err);
-  double M;
-  {
-    long long m = max_key(-static_cast<double>(INFINITY));
-    for (int b = threadIdx.x; b < G; b += kBlock) {
-      const long long y = max_key(__ldcg(A.blockmax + b));
-      m = y > m ? y : m;
-    }
-    M = key_to_double(block_max_key(m, sh_key), 0.0);
-  }
-  const bool zero = !(M > -DBL_MAX);
-  u128* LP = reinterpret_cast<u128*>(A.P_rec);  // in-range exact prefixes, then rounded P_g
+  if (G > 1) grid_barrier(&A.g->bar, target, A.err);
+  else __syncthreads();
+  const T Mt = from_key<T>(G > 1 ? __ldcg(&A.g->scan_key) : sh_key[0]);
+  const double M = static_cast<double>(Mt);
+  const bool zero = sizeof(T) == 4 ? is_neg_inf(Mt) : !(M > -DBL_MAX);  // (M > -DBL_MAX, in binary32)
+  u128* LP = reinterpret_cast<u128*>(A.P_rec);  // (not on_chip) in-range exact prefixes, then P_g
 
   // ---- phase 2: segment totals relative to M and their exact running sum -------------------
-  const WeightCtx wc = make_ctx<T, V>(zero ? 0.0 : M, sh_tab);
-  u128 run = 0;  // the running exact total of this CTA's segments (the same in every thread)
-  u128 lp0 = 0;  // the exact in-range prefix of segment g0 + threadIdx.x (kept for phase 3)
+  const WeightCtx wc = ctx_staged<T, V>(zero ? 0.0 : M, sh_tab);
+  u128 run = 0;  // the exact total of this CTA's segments (one_warp: in warp 0)
+  u128 lp0 = 0;  // the exact in-range prefix of segment g0 + threadIdx.x
   if (!zero) {
-    const T Mt = static_cast<T>(M);  // (exact: M is one of the log-weights)
     if constexpr (!Path<T, V>::kTileRef) {  // the records, relative to M, last turn to first
       bool bad = false;
       for (int t = last_turn; t >= 0; --t) {
         const int g = g0 + kWarps * t + warp;
-        seg_record<T, V>(lw, 0, N, static_cast<int64_t>(g) * kSeg, sh_tab, vec, A.s_rec + g, bad,
+        seg_record<T, V>(lw, 0, N, static_cast<int64_t>(g) * kSeg, sh_tab, vec, recs + (g - g0), bad,
                          max_key(Mt), L2Hint::kEvictLast);
       }
       __syncthreads();  // (lane 0 of each warp stored them; all threads read them below)
     }
-    for (int gb = g0; gb < g1; gb += kBlock) {
-      const int g = gb + static_cast<int>(threadIdx.x);
-      u128 f = 0;
-      if (g < g1) {
-        if (kKept<T, V> && gb == g0) f = rec_fixed_of<T, V>(rec0, Mt, sh_tab);
-        else f = rec_fixed<T, V>(A.s_rec + g, Mt, sh_tab);
+    if (one_warp) {
+      if (warp == 0) {
+        const u128 f = lane < nseg ? to_fixed(rec_scaled_of<T, V>(recs[lane], Mt, sh_tab)) : u128(0);
+        const u128 incl = warp_incl_scan_u128(f);
+        lp0 = incl - f;
+        run = (static_cast<u128>(__shfl_sync(0xffffffffu, static_cast<uint64_t>(incl >> 64), 31)) << 64) |
+              __shfl_sync(0xffffffffu, static_cast<uint64_t>(incl), 31);
       }
-      u128 tot;
-      const u128 ex = block_excl_scan_u128(f, sh_sum, tot);
-      if (g < g1) st_u128(LP + g, run + ex);
-      if (gb == g0) lp0 = ex;
-      run += tot;
+    } else {
+      for (int gb = 0; gb < nseg; gb += kBlock) {
+        const int g = gb + static_cast<int>(threadIdx.x);
+        u128 f = 0;
+        if (g < nseg) f = to_fixed(rec_scaled_of<T, V>(on_chip ? recs[g] : __ldcg(recs + g), Mt, sh_tab));
+        u128 tot;
+        const u128 ex = block_excl_scan_u128(f, sh_sum, tot);
+        if (!on_chip && g < nseg) st_u128(LP + g0 + g, run + ex);
+        if (gb == 0) lp0 = ex;
+        run += tot;
+      }
     }
     if (threadIdx.x == 0) st_u128(A.agg + c, run);
   }
-  grid_barrier(&A.g->bar, target, A.err);
+  if (G > 1) grid_barrier(&A.g->bar, target, A.err);
+  else __syncthreads();
 
   // ---- phase 3: the total and this CTA's segment prefixes ----------------------------------
   if (zero) {  // all weights zero (flagged): every particle keeps itself
@@ -219,91 +225,97 @@ __device__ __forceinline__ void fused_body(const T* __restrict__ lw, const Fused
       flag_error(A.err, RS_ERR_ZERO_WEIGHT);
     }
     if constexpr (SCHEME != RS_MULTINOMIAL) {  // (the search kernel writes the identity)
-      for (int64_t i = e0 + threadIdx.x; i < e1; i += kBlock) {
-        A.a[i] = static_cast<int32_t>(i);
-      }
+      for (int64_t i = e0 + threadIdx.x; i < e1; i += kBlock) A.a[i] = static_cast<int32_t>(i);
       if (A.cl)  // every slot claimed (e0 is a multiple of 8)
         for (int64_t b = (e0 >> 3) + threadIdx.x; b < ((e1 + 7) >> 3); b += kBlock) A.cl[b] = 0xFFu;
     }
     return;  // uniform over the grid
   }
-  u128 CP = 0, TOT = 0;
-  for (int k = threadIdx.x; k < G; k += kBlock) {
-    const u128 v = ld_u128_cg(A.agg + k);
-    TOT += v;
-    if (k < c) CP += v;
-  }
-  block_sum2_u128(CP, TOT, sh_sum);
-  // the total, N / total and the guide step: once per CTA (a binary64 division runs on the
-  // 1/57-rate pipe), then shared
-  __shared__ double2 sh_S, sh_scale;
-  __shared__ double sh_Sd;
+  __shared__ double2 sh_S, sh_scale, sh_pend;
+  __shared__ bool sh_zero;
   __shared__ Guide sh_gd;
-  if (threadIdx.x == 0) {
-    const V S0 = fixed_to(TOT, V(), kFixFrac);
-    const double Sd0 = vto_double(S0);
-    store_v<V>(&sh_S, S0);
-    store_v<V>(&sh_scale, vfrom_double(__ddiv_rn(static_cast<double>(N), Sd0), V()));
-    sh_Sd = Sd0;
-    if constexpr (SCHEME == RS_MULTINOMIAL) sh_gd = make_guide(Sd0, N);
+  {
+    u128 CP = 0, TOT = 0;  // this thread's, then this warp's, part of the sums over the CTAs
+    for (int k = threadIdx.x; k < G; k += kBlock) {
+      const u128 v = ld_u128_cg(A.agg + k);
+      TOT += v;
+      if (k < c) CP += v;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      CP += shfl_xor_u128(CP, o);
+      TOT += shfl_xor_u128(TOT, o);
+    }
+    if (lane == 0) {
+      sh_sum[warp] = CP;
+      sh_sum[kWarps + warp] = TOT;
+    }
+    __syncthreads();
+    // the prefixes: of segment g0 + threadIdx.x (one_warp: warp 0 has them all) and of g1
+    if (!one_warp || warp == 0) {
+      CP = 0;
+#pragma unroll
+      for (int k = 0; k < kWarps; ++k) CP += sh_sum[k];
+      for (int g = threadIdx.x; g <= nseg; g += kBlock) {
+        const u128 lp = g == nseg ? run : (on_chip || g < kBlock) ? lp0 : ld_u128_cg(LP + g0 + g);
+        const V P = fixed_to(CP + lp, V(), kFixFrac);
+        if (on_chip) store_v<V>(sh_rp + g, P);
+        else if (g < nseg || c == G - 1) store_v<V>(A.P_rec + g0 + g, P);
+        if (g == nseg) store_v<V>(&sh_pend, P);
+      }
+    }
+    // the total, N / total and the guide step (a binary64 division takes about a microsecond),
+    // in the last warp
+    if (threadIdx.x == kBlock - 32) {
+      TOT = 0;
+#pragma unroll
+      for (int k = 0; k < kWarps; ++k) TOT += sh_sum[kWarps + k];
+      const V S0 = fixed_to(TOT, V(), kFixFrac);
+      const double Sd0 = vto_double(S0);
+      const V scale0 = vfrom_double(__ddiv_rn(static_cast<double>(N), Sd0), V());
+      store_v<V>(&sh_S, S0);
+      store_v<V>(&sh_scale, scale0);
+      sh_zero = !(Sd0 > 0.0);
+      if constexpr (SCHEME == RS_MULTINOMIAL) sh_gd = make_guide(Sd0, N);
+      if (c == 0) {  // read by the search kernel and the host-side callers
+        store_v<V>(&A.g->S_raw, S0);
+        store_v<V>(&A.g->scale_raw, scale0);
+        A.g->S_d = Sd0;
+        A.g->M = M;
+        A.g->all_zero = !(Sd0 > 0.0);
+        if constexpr (SCHEME == RS_MULTINOMIAL) {
+          A.g->guide_step = sh_gd.step;
+          A.g->guide_inv_step = sh_gd.inv_step;
+        }
+        if (!(Sd0 > 0.0)) flag_error(A.err, RS_ERR_ZERO_WEIGHT);
+      }
+    }
+    __syncthreads();
   }
-  __syncthreads();
   const V S = load_v<V>(&sh_S), scale = load_v<V>(&sh_scale);
-  const double Sd = sh_Sd;
-  const bool all_zero = !(Sd > 0.0);
-  if (c == 0 && threadIdx.x == 0) {  // read by the search kernel and the host-side callers
-    store_v<V>(&A.g->S_raw, S);
-    store_v<V>(&A.g->scale_raw, scale);
-    A.g->S_d = Sd;
-    A.g->M = M;
-    A.g->all_zero = all_zero;
-    const Guide gd = make_guide(Sd, N);
-    A.g->guide_step = gd.step;
-    A.g->guide_inv_step = gd.inv_step;
-    if (all_zero) flag_error(A.err, RS_ERR_ZERO_WEIGHT);
-  }
+  const bool all_zero = sh_zero;
   // the kernels that follow (search, Permute) may launch now; they wait for this grid's end
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (all_zero) {  // the total rounds to zero: every particle keeps itself
     if constexpr (SCHEME != RS_MULTINOMIAL) {
-      for (int64_t i = e0 + threadIdx.x; i < e1; i += kBlock) {
-        A.a[i] = static_cast<int32_t>(i);
-      }
+      for (int64_t i = e0 + threadIdx.x; i < e1; i += kBlock) A.a[i] = static_cast<int32_t>(i);
       if (A.cl)
         for (int64_t b = (e0 >> 3) + threadIdx.x; b < ((e1 + 7) >> 3); b += kBlock) A.cl[b] = 0xFFu;
     }
     return;
   }
-  // rounded prefixes of this CTA's segments, in place of their exact in-range prefixes (each
-  // slot is read and then overwritten by the same thread), and of the next CTA's first
-  // segment, which that CTA owns: kept in shared memory (the last CTA also writes the total's
-  // slot)
-  __shared__ double2 sh_pend;
-  // (kKept: the exact in-range prefixes of the first kBlock segments and the CTA total are
-  // still in registers from phase 2)
-  const int gfirst = g0 + static_cast<int>(threadIdx.x);
-  for (int g = gfirst; g <= g1; g += kBlock) {
-    const u128 lp = (g == g1) ? (kKept<T, V> ? run : ld_u128_cg(A.agg + c))
-                              : (kKept<T, V> && g == gfirst) ? lp0 : ld_u128_cg(LP + g);
-    const V P = fixed_to(CP + lp, V(), kFixFrac);
-    if (g < g1 || c == G - 1) store_v<V>(A.P_rec + g, P);
-    if (g == g1) store_v<V>(&sh_pend, P);
-  }
-  __syncthreads();
 
   // ---- phase 4: emission of this CTA's segments, each warp its own (no block-level
   // synchronisation) -------------------------------------------------------------------------
   typename Path<T, V>::U u_sys = typename Path<T, V>::U();
   Guide gd;
-  if constexpr (SCHEME == RS_MULTINOMIAL) {
-    gd = sh_gd;
-  } else if constexpr (SCHEME == RS_SYSTEMATIC) {
-    u_sys = cta_uniform0<T, V>(A.keys);
-  }
+  if constexpr (SCHEME == RS_MULTINOMIAL) gd = sh_gd;
+  else if constexpr (SCHEME == RS_SYSTEMATIC) u_sys = sh_u;
   for (int g = g0 + warp; g < g1; g += kWarps) {
     const int64_t base = static_cast<int64_t>(g) * kSeg;
-    const V Ps = load_v_cg<V>(A.P_rec + g);
-    const V Pn = (g + 1 < g1) ? load_v_cg<V>(A.P_rec + g + 1) : load_v<V>(&sh_pend);
+    const V Ps = on_chip ? load_v<V>(sh_rp + (g - g0)) : load_v_cg<V>(A.P_rec + g);
+    const V Pn = g + 1 == g1 ? load_v<V>(&sh_pend)
+                             : on_chip ? load_v<V>(sh_rp + (g + 1 - g0)) : load_v_cg<V>(A.P_rec + g + 1);
     if constexpr (SCHEME == RS_MULTINOMIAL) {
       emit_seg_W_guide<T, V>(lw, 0, N, base, wc, vec, Ps, Pn, gd, static_cast<V*>(A.W), A.guide,
                              sh.win[warp], L2Hint::kEvictFirst);
@@ -327,7 +339,12 @@ template <typename T, typename V, int SCHEME>
 __global__ void __launch_bounds__(kBlock, (fused_ctas<T, V>())) fused_scan_kernel(const T* __restrict__ lw, FusedArgs A) {
   unsigned int target = 0;
   fused_body<T, V, SCHEME>(lw, A, target);
-  grid_exit(&A.g->bar, target);
+  // the last CTA to end returns the shared state to its start (every CTA has read the key)
+  if (gridDim.x > 1 && threadIdx.x == 0 &&
+      atomicAdd(&A.g->bar.count, 1u) == target + gridDim.x - 1) {
+    A.g->scan_key = 0ull;
+    atomicExch(&A.g->bar.count, 0u);
+  }
 }
 
 template <typename T, typename V, int SCHEME>
@@ -421,7 +438,6 @@ cudaError_t launch_fused_passes(const Scratch& s, int scheme, Acc acc, const voi
   A.P_rec = s.rec + seg_cap(s.max_tiles);
   A.agg = reinterpret_cast<u128*>(s.irec);  // at least max_blocks entries >= gridDim.x
   A.g = s.glob;
-  A.blockmax = s.blockmax;
   A.err = s.err;
   trace_mark(s.trace, kLblFused[static_cast<int>(acc)][scheme], st);
   switch (acc) {

@@ -25,6 +25,7 @@ struct ScanGlob {
   unsigned int batch_next;   // work counter of the batched kernel (self-resetting)
   unsigned int ess_ticket;   // CTAs of the ESS kernels that have finished (self-resetting)
   unsigned long long ess_key;  // maximum log-weight of an ESS kernel, ordered key (self-resetting)
+  unsigned long long scan_key;  // the same of a cooperative scan (self-resetting)
   GridBar bar;               // grid barrier of the cooperative kernels
   int all_zero;              // every weight of the call is zero (set with the total)
   float guide_step;          // W^N / N and N / W^N in binary32 (multinomial guide table),
@@ -69,7 +70,7 @@ struct Scratch {
   void* W;           // cumulative weights of the multinomial scheme, 8 * max_n bytes
   int32_t* guide;    // guide table of the multinomial search, max_n + 1
   double2* rec;      // per-segment records, then prefixes (two blocks of seg_cap(max_tiles))
-  double* blockmax;  // per-CTA maxima of the max pass
+  double* blockmax;  // per-CTA maxima of the max pass (separate kernels)
   long long* irec;   // per-tile records of the integer scan (2 * (max_tiles + 2), or 2 * max_blocks
                      // if more: the per-CTA exact totals of the cooperative scan)
   ScanGlob* glob;

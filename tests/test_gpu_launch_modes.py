@@ -159,3 +159,35 @@ def test_mcmc_and_conversions_equal_across_launch_modes(rs, h, N):
     assert np.array_equal(res[0][1], res[1][1]) and np.array_equal(res[0][2], res[1][2])
     assert np.array_equal(res[0][1], np.bincount(a.cpu().numpy(), minlength=N))
     assert np.array_equal(res[0][2], np.cumsum(res[0][1]))
+
+
+# one CTA (no barrier) and two; the most segments a CTA's first warp scans alone (31 of 256
+# particles, 608 or 456 CTAs), one more; records and prefixes on chip (256 segments) and beyond
+@pytest.mark.parametrize("N", [1, 2048, 2049, 31 * 256 * 608, 31 * 256 * 608 + 1, 31 * 256 * 456 + 257,
+                               256 * 256 * 608, 256 * 256 * 608 + 4099])
+@pytest.mark.parametrize("dtype,prec", [(torch.float32, 0), (torch.float32, 1), (torch.float64, 0)])
+def test_fused_segment_split(rs, N, dtype, prec):
+    """The cooperative kernel equals the separate ones however many segments a CTA owns, twice in
+    a row (its shared maximum is reset)."""
+    if N > (1 << 25) and dtype != torch.float32:
+        pytest.skip("the binary32 forms cover the largest split")
+    g = torch.Generator(device=DEV)
+    g.manual_seed(N % 1000)
+    lw = -0.5 * (torch.randn(N, generator=g, device=DEV, dtype=dtype) - 2.0) ** 2
+    with rs.Handle(N) as hh:
+        for scheme in (rs.SYSTEMATIC, rs.STRATIFIED, rs.MULTINOMIAL):
+            rs.rs_set_launch_mode(hh, rs.LAUNCH_SEPARATE)
+            want = rs.rs_resample(hh, scheme, lw, seed=9, step=4, prec=prec, permute=True)
+            rs.rs_set_launch_mode(hh, rs.LAUNCH_FUSED)
+            for _ in range(2):
+                got = rs.rs_resample(hh, scheme, lw, seed=9, step=4, prec=prec, permute=True)
+                assert rs.rs_last_error(hh) == rs.RS_OK
+                assert torch.equal(got, want), scheme
+        low = torch.full((N,), -float("inf"), dtype=dtype, device=DEV)
+        low[N // 2] = torch.finfo(dtype).min  # the type's lowest log-weight carries all the weight
+        st = []
+        for mode in (rs.LAUNCH_SEPARATE, rs.LAUNCH_FUSED):
+            rs.rs_set_launch_mode(hh, mode)
+            a = rs.rs_resample(hh, rs.SYSTEMATIC, low, seed=9, prec=prec)
+            st.append((rs.rs_last_error(hh), a))
+        assert st[0][0] == st[1][0] and torch.equal(st[0][1], st[1][1])
