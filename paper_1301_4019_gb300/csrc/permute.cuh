@@ -175,19 +175,19 @@ __device__ __forceinline__ void permute4_slots(const int32_t* __restrict__ a,
 // d is injective on the claimed slots and the walks end (Appendix C), so each backward chain
 // is one walk reversed and c is Code 10's exactly; the claims are never stored.
 //
-// The chain of one unclaimed run head whose ancestor is z, to its start: returns the value
+// The chain of one unclaimed run head whose ancestor is z < n, to its start: returns the value
 // that the head receives, or sets bad (only a corrupted a can do that).
 __device__ __forceinline__ int32_t sorted_chain(const int32_t* __restrict__ a, int32_t z,
-                                                int64_t n, bool& bad) {
-  const uint32_t un = static_cast<uint32_t>(n);
-  for (int64_t steps = 0;; ++steps) {
-    const int32_t y = a[z];
-    const bool zhead = z == 0 || a[z - 1] != y;
-    if (static_cast<uint32_t>(y) >= un || steps > n) {
+                                                int32_t n, bool& bad) {
+  for (int32_t left = n;; --left) {
+    const int32_t* const p = a + z;
+    const int32_t y = *p;
+    const int32_t before = z > 0 ? p[-1] : -1;
+    if (static_cast<uint32_t>(y) >= static_cast<uint32_t>(n) || left == 0) {
       bad = true;
       return 0;
     }
-    if (!zhead) return y;
+    if (before == y) return y;  // not the first of its run
     z = y;
   }
 }
@@ -205,65 +205,80 @@ __device__ __forceinline__ void permute_sorted_one(const int32_t* __restrict__ a
   int32_t v;
   if ((cl[i >> 3] >> (i & 7)) & 1) v = static_cast<int32_t>(i);
   else if (i > 0 && a[i - 1] == ai) v = ai;
-  else v = sorted_chain(a, ai, n, bad);
+  else v = sorted_chain(a, ai, static_cast<int32_t>(n), bad);
   if (bad) flag_error(err, RS_ERR_ARG);
   else c[i] = v;
 }
 
 // K consecutive slots i0 .. i0 + K - 1 of it per lane (lane l's follow lane l - 1's), called by
 // all 32 lanes of a warp; slots at n or beyond do nothing. The chains that go on past their
-// first step are queued per warp (pend: 32 K entries) and run one per lane; the warp's results
-// are gathered in cw (32 K entries, 16-byte aligned) and stored 128 bits at a time where the
-// addresses allow.
+// first step are queued per warp in slot order (pend: 32 K entries) and run one per lane; the
+// warp's results are gathered in cw (32 K entries, 16-byte aligned) and stored 128 bits at a time
+// where the addresses allow. A warp with all its slots below n and all its ancestors in range
+// (every warp but the last of a sequence) takes no tests per slot.
 template <int K>
 __device__ __forceinline__ void permute_sorted_slots(const int32_t* __restrict__ a,
-                                                     const uint8_t* __restrict__ cl, int64_t n,
-                                                     int32_t* __restrict__ c, int64_t i0,
+                                                     const uint8_t* __restrict__ cl, int64_t n64,
+                                                     int32_t* __restrict__ c, int64_t i064,
                                                      int32_t* cw, int2* pend, int* err) {
   static_assert(K == 1 || K == 4, "one or four slots per thread");
   const int lane = threadIdx.x & 31;
+  // (n < 2^31; slots past n only need to compare as such: i0 < n + 2^12 < 2^32)
+  const uint32_t n = static_cast<uint32_t>(n64), i0 = static_cast<uint32_t>(i064);
   const bool full = i0 + K <= n;
-  int32_t A[K];
+  uint32_t A[K];
   if (K == 4 && full && (reinterpret_cast<uintptr_t>(a + i0) & 15u) == 0) {
-    const int4 va = *reinterpret_cast<const int4*>(a + i0);
+    const uint4 va = *reinterpret_cast<const uint4*>(a + i0);
     A[0] = va.x; A[1] = va.y; A[2] = va.z; A[3] = va.w;
   } else {
 #pragma unroll
-    for (int q = 0; q < K; ++q) A[q] = i0 + q < n ? a[i0 + q] : 0;
+    for (int q = 0; q < K; ++q) A[q] = i0 + q < n ? static_cast<uint32_t>(a[i0 + q]) : 0u;
   }
-  // a_{i0-1}: the previous lane's last slot, loaded by lane 0 only
-  int32_t prev = __shfl_up_sync(0xffffffffu, A[K - 1], 1);
-  if (lane == 0) prev = (i0 > 0 && i0 - 1 < n) ? a[i0 - 1] : -1;
   uint32_t bits = 0u;
   if (i0 < n) {
-    const int sh = static_cast<int>(i0 & 7);
+    const int sh = static_cast<int>(i0 & 7u);
     bits = static_cast<uint32_t>(cl[i0 >> 3]) >> sh;
     if (K == 4 && sh > 4 && i0 + (8 - sh) < n)  // (the slots reach into the next byte)
       bits |= static_cast<uint32_t>(cl[(i0 >> 3) + 1]) << (8 - sh);
   }
-  const unsigned below = (1u << lane) - 1u;
-  int total = 0;
-  bool bad = false;
+  // a_{i0-1}: the previous lane's last slot, loaded by lane 0 only
+  uint32_t prev = __shfl_up_sync(0xffffffffu, A[K - 1], 1);
+  if (lane == 0) prev = (i0 > 0 && i0 - 1 < n) ? static_cast<uint32_t>(a[i0 - 1]) : ~0u;
+  // this lane's unclaimed run heads (bit q: slot i0 + q), and every other slot's result
+  uint32_t top = A[0], go = 0u;
   int32_t R[K];
 #pragma unroll
   for (int q = 0; q < K; ++q) {
-    const int64_t x = i0 + q;
-    bool go = false;
-    R[q] = 0;
-    const int32_t ax = A[q];
-    if (x < n) {
-      if (ax < 0 || ax >= n) bad = true;
-      else if ((bits >> q) & 1u) R[q] = static_cast<int32_t>(x);
-      else if (prev == ax) R[q] = ax;  // not the first of its run
-      else go = true;
-      prev = ax;
-    }
-    const unsigned m = __ballot_sync(0xffffffffu, go);
-    if (go) pend[total + __popc(m & below)] = make_int2(K * lane + q, ax);
-    total += __popc(m);
+    if (q > 0) top = max(top, A[q]);
+    const bool claimed = (bits >> q) & 1u;
+    go |= static_cast<uint32_t>(!claimed && A[q] != (q > 0 ? A[q > 0 ? q - 1 : 0] : prev)) << q;
+    R[q] = static_cast<int32_t>(claimed ? i0 + q : A[q]);
   }
+  bool bad = false;
+  if (!full || top >= n) {  // the sequence's end, or an ancestor out of range: slot by slot
+    go = 0u;
+#pragma unroll
+    for (int q = 0; q < K; ++q) {
+      if (i0 + q >= n) continue;
+      if (A[q] >= n) bad = true;
+      else if (!((bits >> q) & 1u) && A[q] != (q > 0 ? A[q > 0 ? q - 1 : 0] : prev)) go |= 1u << q;
+    }
+  }
+  // places in the queue: the heads of the lanes below (counts 0 .. 4, a ballot per bit of them)
+  const uint32_t cnt = __popc(go), below = (1u << lane) - 1u;
+  const uint32_t b0 = __ballot_sync(0xffffffffu, cnt & 1u);
+  int at = __popc(b0 & below), total = __popc(b0);
   if (K == 4) {
-    reinterpret_cast<int4*>(cw)[lane] = make_int4(R[0], R[1], R[2], R[3]);
+    const uint32_t b1 = __ballot_sync(0xffffffffu, cnt & 2u);
+    const uint32_t b2 = __ballot_sync(0xffffffffu, cnt & 4u);
+    at += 2 * __popc(b1 & below) + 4 * __popc(b2 & below);
+    total += 2 * __popc(b1) + 4 * __popc(b2);
+  }
+#pragma unroll
+  for (int q = 0; q < K; ++q)
+    if ((go >> q) & 1u) pend[at++] = make_int2(K * lane + q, static_cast<int32_t>(A[q]));
+  if (K == 4) {
+    reinterpret_cast<int4*>(cw)[lane] = make_int4(R[0], R[K > 1 ? 1 : 0], R[K > 2 ? 2 : 0], R[K - 1]);
   } else {
     cw[lane] = R[0];
   }
@@ -271,7 +286,7 @@ __device__ __forceinline__ void permute_sorted_slots(const int32_t* __restrict__
   for (int e = lane; e < total; e += 32) {
     const int2 w = pend[e];
     bool cbad = false;
-    const int32_t v = sorted_chain(a, w.y, n, cbad);
+    const int32_t v = sorted_chain(a, w.y, static_cast<int32_t>(n), cbad);
     if (cbad) bad = true;
     else cw[w.x] = v;
   }
