@@ -328,15 +328,15 @@ __device__ __forceinline__ void fused_body(const T* __restrict__ lw, const Fused
 }
 
 // CTAs of kBlock threads that share an SM (the cooperative grid holds so many on each): four for
-// binary32 log-weights (64 registers), three for binary64 ones, whose emission keeps more values in
-// flight (80 registers; 3000001 particles, double-float: 92.2 -> 90.2 us, IEEE 700001: 85.8 ->
+// binary32 log-weights and the multinomial (64 registers), three for the stratified and systematic
+// of binary64 log-weights, whose emission keeps more values in flight (80 registers; 3000001 particles, double-float: 92.2 -> 90.2 us, IEEE 700001: 85.8 ->
 // 78.9; compensated binary32 at 2^20 is faster with four).
-template <typename T, typename V>
+template <typename T, int SCHEME>
 constexpr int fused_ctas() {
-  return sizeof(T) == 4 ? 4 : 3;
+  return sizeof(T) == 4 || SCHEME == RS_MULTINOMIAL ? 4 : 3;
 }
 template <typename T, typename V, int SCHEME>
-__global__ void __launch_bounds__(kBlock, (fused_ctas<T, V>())) fused_scan_kernel(const T* __restrict__ lw, FusedArgs A) {
+__global__ void __launch_bounds__(kBlock, (fused_ctas<T, SCHEME>())) fused_scan_kernel(const T* __restrict__ lw, FusedArgs A) {
   unsigned int target = 0;
   fused_body<T, V, SCHEME>(lw, A, target);
   // the last CTA to end returns the shared state to its start (every CTA has read the key)

@@ -243,71 +243,54 @@ emit_W_guide_kernel(const T* __restrict__ lw, int64_t N, const ScanGlob* g, cons
 }
 
 // ---------------------------------------------------------------------------------------
-// Multinomial search (Code 5), one particle per thread, with the Prepermute claim
-// atomicMin(d[a_i], i) when d is given.
+// Multinomial search (Code 5), K consecutive outputs per thread (their loads in flight together;
+// K = 4: one 128-bit store of the four ancestors), with the Prepermute claim atomicMin(d[a_i], i)
+// when d is given. Bound by the latency of its dependent reads (the totals, the guide entries,
+// the cumulative weights). Four outputs from kSearch4MinN particles, where W and the guide table
+// leave L2 (measured at 2^24: 577 vs 656 us binary32, 668 vs 754 us double-float); at
+// 2^20-2^22, with the tables in L2, one output per thread keeps more loads in flight.
 // ---------------------------------------------------------------------------------------
-template <typename T, typename V>
+template <typename T, typename V, int K>
 __global__ void __launch_bounds__(kBlock)
 search_kernel(const V* __restrict__ W, const int32_t* __restrict__ G, int64_t N,
               const ScanGlob* g, Keys keys, int32_t* __restrict__ a, int32_t* __restrict__ d) {
   pdl_wait();
-  const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (i >= N) return;
-  if (g->all_zero) {
-    a[i] = static_cast<int32_t>(i);
-    if (d) atomicMin(d + i, static_cast<int32_t>(i));
-    return;
-  }
-  const Guide gd{g->guide_step, g->guide_inv_step};
-  const int32_t k = search_one_guided<T, V>(W, G, N, gd, keys, i);
-  a[i] = k;
-  if (d) atomicMin(d + k, static_cast<int32_t>(i));
-}
-
-// The same search, four consecutive outputs per thread (their loads in flight together) and
-// one 128-bit store of the four ancestors; used from kSearch4MinN particles, where W and the
-// guide table leave L2 (measured at 2^24: 577 vs 656 us binary32, 668 vs 754 us double-float;
-// at 2^20-2^22, with the tables in L2, one output per thread keeps more loads in flight:
-// 21 vs 27 us at 2^20).
-template <typename T, typename V>
-__global__ void __launch_bounds__(kBlock)
-search4_kernel(const V* __restrict__ W, const int32_t* __restrict__ G, int64_t N,
-               const ScanGlob* g, Keys keys, int32_t* __restrict__ a, int32_t* __restrict__ d) {
-  pdl_wait();
-  const int64_t i0 = 4 * (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x);
+  const int64_t i0 = K * (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x);
   if (i0 >= N) return;
-  int32_t k[4];
+  int32_t k[K];
   if (g->all_zero) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) k[q] = static_cast<int32_t>(i0 + q);
+    for (int q = 0; q < K; ++q) k[q] = static_cast<int32_t>(i0 + q);
   } else {
     const Guide gd{g->guide_step, g->guide_inv_step};
-    search_group_guided<T, V, 4>(W, G, N, gd, keys, i0, k);
+    search_guided<T, V, K>(W, G, static_cast<int32_t>(N), gd, keys, static_cast<int32_t>(i0), k);
   }
-  if (i0 + 3 < N && (reinterpret_cast<uintptr_t>(a + i0) & 15u) == 0) {
-    *reinterpret_cast<int4*>(a + i0) = make_int4(k[0], k[1], k[2], k[3]);
+  if (K == 4 && i0 + 3 < N && (reinterpret_cast<uintptr_t>(a + i0) & 15u) == 0) {
+    *reinterpret_cast<int4*>(a + i0) = make_int4(k[0], k[K > 1 ? 1 : 0], k[K > 2 ? 2 : 0], k[K - 1]);
   } else {
 #pragma unroll
-    for (int q = 0; q < 4; ++q)
+    for (int q = 0; q < K; ++q)
       if (i0 + q < N) a[i0 + q] = k[q];
   }
   if (d) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q)
+    for (int q = 0; q < K; ++q)
       if (i0 + q < N) atomicMin(d + k[q], static_cast<int32_t>(i0 + q));
   }
 }
 constexpr int64_t kSearch4MinN = int64_t{1} << 23;
 
+template <typename T, typename V, int K>
+void launch_search_k(const Scratch& s, const V* W, int64_t N, const Keys& keys, int32_t* a,
+                     int32_t* d, cudaStream_t st) {
+  launch_pdl(search_kernel<T, V, K>, static_cast<int>((N + K * kBlock - 1) / (K * kBlock)), kBlock,
+             st, W, s.guide, N, s.glob, keys, a, d);
+}
 template <typename T, typename V>
 void launch_search(const Scratch& s, const V* W, int64_t N, const Keys& keys, int32_t* a,
                    int32_t* d, cudaStream_t st) {
-  if (N >= kSearch4MinN)
-    launch_pdl(search4_kernel<T, V>, static_cast<int>((N + 4 * kBlock - 1) / (4 * kBlock)),
-               kBlock, st, W, s.guide, N, s.glob, keys, a, d);
-  else
-    launch_pdl(search_kernel<T, V>, static_cast<int>((N + kBlock - 1) / kBlock), kBlock, st, W,
-               s.guide, N, s.glob, keys, a, d);
+  if (N >= kSearch4MinN) launch_search_k<T, V, 4>(s, W, N, keys, a, d, st);
+  else launch_search_k<T, V, 1>(s, W, N, keys, a, d, st);
 }
 
 int max_grid(int64_t N, int max_blocks) {

@@ -1156,11 +1156,10 @@ __device__ __forceinline__ Guide make_guide(double Sd, int64_t n) {
   g.inv_step = __double2float_rn(__ddiv_rn(static_cast<double>(n), Sd));
   return g;
 }
-// (b < n < 2^31: a 32-bit conversion gives the same binary32 value as a 64-bit one; the 32-bit
-// conversions here measured 2-5 % faster multinomial calls)
-__device__ __forceinline__ float guide_edge(int64_t b, const Guide& g, int64_t n) {
+// (b <= n < 2^31: 32-bit indices and conversions)
+__device__ __forceinline__ float guide_edge(int32_t b, const Guide& g, int32_t n) {
   if (b >= n) return INFINITY;
-  return __fmul_rn(__int2float_rn(static_cast<int>(b)), g.step);
+  return __fmul_rn(__int2float_rn(b), g.step);
 }
 template <typename V> __device__ __forceinline__ V edge_as(float e);
 template <> __device__ __forceinline__ float edge_as<float>(float e) { return e; }
@@ -1169,22 +1168,32 @@ template <> __device__ __forceinline__ float2 edge_as<float2>(float e) { return 
 
 // C(W) = the first b in [0, n] with e_b >= W.
 template <typename V>
-__device__ __forceinline__ int64_t guide_count(V W, const Guide& g, int64_t n) {
+__device__ __forceinline__ int32_t guide_count(V W, const Guide& g, int32_t n) {
   const float est = ceilf(__fmul_rn(vhi(W), g.inv_step));
-  int64_t b = est > 0.0f ? (est < __int2float_rn(static_cast<int>(n)) ? __float2int_rz(est) : n)
-                         : 0;
+  int32_t b = est > 0.0f ? (est < __int2float_rn(n) ? __float2int_rz(est) : n) : 0;
   int steps = 0;
   while (b > 0 && vle(W, edge_as<V>(guide_edge(b - 1, g, n))) && ++steps < 64) --b;
   while (b < n && !vle(W, edge_as<V>(guide_edge(b, g, n))) && ++steps < 64) ++b;
   if (steps >= 64) {  // far from the estimate: bisect the edges
-    int64_t lo = 0, hi = n;
+    int32_t lo = 0, hi = n;
     while (lo < hi) {
-      const int64_t mid = lo + ((hi - lo) >> 1);
+      const int32_t mid = lo + ((hi - lo) >> 1);
       if (vle(W, edge_as<V>(guide_edge(mid, g, n)))) hi = mid; else lo = mid + 1;
     }
     b = lo;
   }
   return b;
+}
+
+// The bucket b in [0, n) with e_b <= u < e_{b+1}, or -1 when it is far from the estimate.
+template <typename V>
+__device__ __forceinline__ int32_t guide_bucket(V u, const Guide& g, int32_t n) {
+  const float est = floorf(__fmul_rn(vhi(u), g.inv_step));
+  int32_t b = est > 0.0f ? (est < __int2float_rn(n - 1) ? __float2int_rz(est) : n - 1) : 0;
+  int steps = 0;
+  while (b > 0 && !vle(edge_as<V>(guide_edge(b, g, n)), u) && ++steps < 64) --b;
+  while (b < n - 1 && vle(edge_as<V>(guide_edge(b + 1, g, n)), u) && ++steps < 64) ++b;
+  return steps < 64 ? b : -1;
 }
 
 // Stored cumulative weights of one segment plus the guide-table scatter of its particles
@@ -1207,13 +1216,13 @@ __device__ __forceinline__ void emit_seg_W_guide(const T* __restrict__ lw, int64
 #pragma unroll
   for (int q = 0; q < kPer; ++q) {
     if (q < cnt) p[q] = W[q];
-    C[q] = static_cast<int32_t>(guide_count<V>(W[q], gd, n));
+    C[q] = guide_count<V>(W[q], gd, n);
   }
   // the guide entries of a particle's buckets form runs like the ancestors of Code 11 (the
   // last particle's run ends at n, positions past the end add none)
   const int32_t last = (cnt >= kPer && j0 + kPer - 1 != n - 1) ? C[kPer - 1] : n;
   int32_t prev = __shfl_up_sync(0xffffffffu, last, 1);
-  if (lane == 0) prev = cnt > 0 ? static_cast<int32_t>(guide_count<V>(Wb, gd, n)) : n;
+  if (lane == 0) prev = cnt > 0 ? guide_count<V>(Wb, gd, n) : n;
   int32_t pc = prev;
 #pragma unroll
   for (int q = 0; q < kPer; ++q) {
@@ -1226,110 +1235,61 @@ __device__ __forceinline__ void emit_seg_W_guide(const T* __restrict__ lw, int64
   if (j0 <= n - 1 && n - 1 < j0 + kPer) Gl[n] = n - 1;
 }
 
-// Loads of W and G; kCoherent: written earlier in the same kernel launch, read through L2.
-template <bool kCoherent, typename X> __device__ __forceinline__ X ld_val(const X* p) {
-  if constexpr (kCoherent) return __ldcg(p); else return __ldg(p);
-}
-
-// Multinomial search of output i through the guide table (same result as search_one).
-template <typename T, typename V, bool kCoherent = false>
-__device__ __forceinline__ int32_t search_one_guided(const V* __restrict__ W,
-                                                     const int32_t* __restrict__ G, int64_t n,
-                                                     const Guide& gd, const Keys& keys,
-                                                     int64_t i) {
-  const V S = ld_val<kCoherent>(W + (n - 1));
-  const auto U = Path<T, V>::draw_u(draw(keys, static_cast<uint32_t>(i), 0u));
-  const V u = vtimes_u(S, U);
-  // bucket b with e_b <= u < e_{b+1}
-  const float est = floorf(__fmul_rn(vhi(u), gd.inv_step));
-  int64_t b = est > 0.0f
-                  ? (est < __int2float_rn(static_cast<int>(n - 1)) ? __float2int_rz(est) : n - 1)
-                  : 0;
-  int steps = 0;
-  while (b > 0 && !vle(edge_as<V>(guide_edge(b, gd, n)), u) && ++steps < 64) --b;
-  while (b < n - 1 && vle(edge_as<V>(guide_edge(b + 1, gd, n)), u) && ++steps < 64) ++b;
-  int64_t lo = 0, hi = n;
-  if (steps < 64) {
-    lo = ld_val<kCoherent>(G + b);
-    hi = static_cast<int64_t>(ld_val<kCoherent>(G + b + 1)) + 1;
-  }
-  if (hi - lo <= 8) {  // the usual case: count W_j <= u over the range, loads in parallel
-    const int64_t len = hi - lo;
-    int cnt = 0;
+// The first j of the non-decreasing W_lo .. W_{hi-1} with W_j > u, hi if none: four are read
+// together (a bucket of the guide table usually spans two or three particles), then four more,
+// the rest by a binary search.
+template <typename V>
+__device__ __forceinline__ int32_t search_range(const V* __restrict__ W, V u, int32_t lo, int32_t hi) {
 #pragma unroll
-    for (int q = 0; q < 8; ++q)
-      if (q < len && vle(ld_val<kCoherent>(W + lo + q), u)) ++cnt;
+  for (int part = 0; part < 2; ++part) {
+    const int32_t len = hi - lo;
+    int32_t cnt = 0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (q < len && vle(__ldg(W + lo + q), u)) ++cnt;
     lo += cnt;
-  } else {
-    while (lo < hi) {
-      const int64_t mid = lo + ((hi - lo) >> 1);
-      if (vle(ld_val<kCoherent>(W + mid), u)) lo = mid + 1; else hi = mid;
-    }
+    if (cnt < 4) return lo;
   }
-  return static_cast<int32_t>(lo < n ? lo : n - 1);
+  while (lo < hi) {
+    const int32_t mid = lo + ((hi - lo) >> 1);
+    if (vle(__ldg(W + mid), u)) lo = mid + 1; else hi = mid;
+  }
+  return lo;
 }
 
-// The same search for K outputs i0 .. i0 + K - 1 at once (the valid ones: i0 + q < n): the
-// bucket of every draw first, then the guide entries of all K issued together, then their
-// short W ranges (up to 8 entries each) together, so that K dependent chains of loads are in
-// flight per thread. Each result equals search_one_guided's for its output.
+// Multinomial search of the K outputs i0 .. i0 + K - 1 (those below n) through the guide table
+// (each the same result as search_one): the bucket of every draw first, then the guide entries of
+// all K together, then their short W ranges, so that K dependent chains of loads are in flight
+// per thread. 32-bit indices; the searches of one output took 255 instructions, half of them
+// 64-bit index arithmetic and eight predicated loads of W where two or three are needed.
 template <typename T, typename V, int K>
-__device__ __forceinline__ void search_group_guided(const V* __restrict__ W,
-                                                    const int32_t* __restrict__ G, int64_t n,
-                                                    const Guide& gd, const Keys& keys,
-                                                    int64_t i0, int32_t (&res)[K]) {
+__device__ __forceinline__ void search_guided(const V* __restrict__ W,
+                                              const int32_t* __restrict__ G, int32_t n,
+                                              const Guide& gd, const Keys& keys, int32_t i0,
+                                              int32_t (&res)[K]) {
   const V S = __ldg(W + (n - 1));
   V u[K];
-  int64_t lo[K], hi[K];
-  bool ok[K];
+  int32_t lo[K], hi[K];
 #pragma unroll
   for (int q = 0; q < K; ++q) {
-    ok[q] = i0 + q < n;
     const auto U = Path<T, V>::draw_u(draw(keys, static_cast<uint32_t>(i0 + q), 0u));
     u[q] = vtimes_u(S, U);
-    const float est = floorf(__fmul_rn(vhi(u[q]), gd.inv_step));
-    int64_t b = est > 0.0f
-                    ? (est < __int2float_rn(static_cast<int>(n - 1)) ? __float2int_rz(est) : n - 1)
-                    : 0;
-    int steps = 0;
-    while (b > 0 && !vle(edge_as<V>(guide_edge(b, gd, n)), u[q]) && ++steps < 64) --b;
-    while (b < n - 1 && vle(edge_as<V>(guide_edge(b + 1, gd, n)), u[q]) && ++steps < 64) ++b;
-    lo[q] = steps < 64 ? b : -1;  // (-1: search the whole range)
+    lo[q] = guide_bucket(u[q], gd, n);
   }
 #pragma unroll
   for (int q = 0; q < K; ++q) {
-    const int64_t b = lo[q];
-    if (ok[q] && b >= 0) {
+    const int32_t b = lo[q];
+    lo[q] = 0;
+    hi[q] = n - i0 > q ? n : 0;  // (no such output: an empty range)
+    if (n - i0 > q && b >= 0) {
       lo[q] = __ldg(G + b);
-      hi[q] = static_cast<int64_t>(__ldg(G + b + 1)) + 1;
-    } else {
-      lo[q] = 0;
-      hi[q] = ok[q] ? n : 0;  // (no output: an empty range)
-    }
-  }
-  int cnt[K];
-#pragma unroll
-  for (int q = 0; q < K; ++q) {
-    cnt[q] = 0;
-    const int64_t len = hi[q] - lo[q];
-    if (ok[q] && len <= 8) {
-#pragma unroll
-      for (int k = 0; k < 8; ++k)
-        if (k < len && vle(__ldg(W + lo[q] + k), u[q])) ++cnt[q];
+      hi[q] = __ldg(G + b + 1) + 1;
     }
   }
 #pragma unroll
   for (int q = 0; q < K; ++q) {
-    int64_t l = lo[q], h = hi[q];
-    if (h - l <= 8) {
-      l += cnt[q];
-    } else {
-      while (l < h) {
-        const int64_t mid = l + ((h - l) >> 1);
-        if (vle(__ldg(W + mid), u[q])) l = mid + 1; else h = mid;
-      }
-    }
-    res[q] = static_cast<int32_t>(l < n ? l : n - 1);
+    const int32_t j = search_range(W, u[q], lo[q], hi[q]);
+    res[q] = j < n ? j : n - 1;
   }
 }
 
