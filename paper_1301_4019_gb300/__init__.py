@@ -79,6 +79,8 @@ def library_path() -> str:
 def load(build: bool = True):
     """Build (if stale) and load the shared library; raises if either fails."""
     global _lib
+    if _lib is not None:  # (set once, under the lock)
+        return _lib
     with _lock:
         if _lib is None:
             path = _build.build() if build else _build.LIB_PATH
@@ -155,27 +157,56 @@ def _check(status: int, what: str):
         raise RsError(status, what)
 
 
-def _stream(stream) -> C.c_void_p:
+# The raw handle of the current stream without a Stream object (about a microsecond less a call);
+# both names are what torch.cuda.current_stream itself calls.
+try:
+    from torch._C import _cuda_getCurrentRawStream, _cuda_getDevice
+except ImportError:  # (a torch built without CUDA, or without these names)
+    _cuda_getCurrentRawStream = _cuda_getDevice = None
+
+
+def _stream(stream) -> int:
+    """The cudaStream_t of `stream` (None: the current stream) as an integer."""
     if stream is None:
+        if _cuda_getCurrentRawStream is not None and torch.cuda.is_initialized():
+            return _cuda_getCurrentRawStream(_cuda_getDevice())
         stream = torch.cuda.current_stream()
-    return C.c_void_p(stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream))
+    return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
-def _dev(t: torch.Tensor, dtype, name: str, n: int | None = None, h=None):
-    """Device pointer of a contiguous CUDA tensor; with `n`, the tensor must hold at least n
+def _dev(t: torch.Tensor, dtype, name: str, n: int | None = None, h=None) -> int:
+    """Device address of a contiguous CUDA tensor; with `n`, the tensor must hold at least n
     elements (the kernels read or write n of them); with `h`, it must live on the handle's
     device."""
     if not isinstance(t, torch.Tensor) or not t.is_cuda:
         raise TypeError(f"{name} must be a CUDA tensor")
-    if dtype is not None and t.dtype not in (dtype if isinstance(dtype, tuple) else (dtype,)):
-        raise TypeError(f"{name} has dtype {t.dtype}")
+    if dtype is not None:
+        d = t.dtype
+        if d is not dtype and not (isinstance(dtype, tuple) and d in dtype):
+            raise TypeError(f"{name} has dtype {d}")
     if not t.is_contiguous():
         raise ValueError(f"{name} must be contiguous")
     if n is not None and t.numel() < n:
         raise ValueError(f"{name} holds {t.numel()} elements, {n} needed")
-    if h is not None and t.device.index != h.device:
+    if h is not None and t.get_device() != h.device:
         raise ValueError(f"{name} is on {t.device}, the handle on cuda:{h.device}")
-    return C.c_void_p(t.data_ptr())
+    return t.data_ptr()
+
+
+_LOGW_TYPES = (torch.float32, torch.float64)
+_U64 = 0xFFFFFFFFFFFFFFFF
+_tls = threading.local()
+
+
+def _opts(prec, log_wmax, max_trials, filter):
+    """The options in a structure of this thread's, refilled by every call (the library copies
+    them before it returns)."""
+    o = getattr(_tls, "opts", None)
+    if o is None:
+        o = _tls.opts = _Opts()
+        _tls.opts_ref = C.byref(o)
+    o.prec, o.log_wmax, o.max_trials, o.filter = prec, float(log_wmax), int(max_trials), int(filter)
+    return _tls.opts_ref
 
 
 def _dtype_code(t: torch.Tensor) -> int:
@@ -230,13 +261,13 @@ def rs_resample(h: Handle, scheme: int, logw: torch.Tensor, B: int = 0, seed: in
     N = logw.numel()
     if out is None:
         out = torch.empty(N, dtype=torch.int32, device=logw.device)
-    opts = _Opts(prec, float(log_wmax), int(max_trials), int(filter))
-    _check(load().rs_resample(h.ptr, int(scheme), _dtype_code(logw),
-                              _dev(logw, (torch.float32, torch.float64), "logw", h=h), N,
-                              int(B), int(seed) & 0xFFFFFFFFFFFFFFFF,
-                              int(step) & 0xFFFFFFFFFFFFFFFF,
-                              _dev(out, torch.int32, "out", N, h), 1 if permute else 0,
-                              C.byref(opts), _stream(stream)), "rs_resample")
+    st = load().rs_resample(h.ptr, int(scheme), _dtype_code(logw),
+                            _dev(logw, _LOGW_TYPES, "logw", None, h), N, int(B),
+                            int(seed) & _U64, int(step) & _U64,
+                            _dev(out, torch.int32, "out", N, h), 1 if permute else 0,
+                            _opts(prec, log_wmax, max_trials, filter), _stream(stream))
+    if st != RS_OK:
+        raise RsError(st, "rs_resample")
     return out
 
 
@@ -297,15 +328,15 @@ def rs_resample_batched(h: Handle, scheme: int, logw: torch.Tensor, offsets: tor
     F = offsets.numel() - 1
     if out is None:
         out = torch.empty(logw.numel(), dtype=torch.int32, device=logw.device)
-    opts = _Opts(prec, float(log_wmax), int(max_trials), 0)
+    opts = _opts(prec, log_wmax, max_trials, 0)
     bptr = (_dev(B_per_filter, torch.int32, "B_per_filter", F, h)
             if B_per_filter is not None else None)
     head = (h.ptr, int(scheme), _dtype_code(logw),
             _dev(logw, (torch.float32, torch.float64), "logw", h=h),
             _dev(offsets, torch.int64, "offsets", F + 1, h), F, bptr, int(B),
             int(seed) & 0xFFFFFFFFFFFFFFFF, int(step) & 0xFFFFFFFFFFFFFFFF)
-    tail = (_dev(out, torch.int32, "out", logw.numel(), h), 1 if permute else 0,
-            C.byref(opts), _stream(stream))
+    tail = (_dev(out, torch.int32, "out", logw.numel(), h), 1 if permute else 0, opts,
+            _stream(stream))
     if resample is None:
         _check(load().rs_resample_batched(*head, *tail), "rs_resample_batched")
     else:

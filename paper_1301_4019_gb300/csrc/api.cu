@@ -133,9 +133,11 @@ int rs_create(rs_handle** out, int64_t max_n, int device) {
   // the allocation-free call's static scratch on this device: looked up now, so that calls
   // made later while a stream is captured find it ready
   bool ok = rsk::noalloc_prepare_current_device() == RS_OK;
-  // (the claims, or the claimed bits: of a batch, one extra byte per filter)
+  // the claims, or the claimed bits: of a batch, one extra byte per filter (more than the claims
+  // only for the smallest handles)
   s.max_filters = max_n / 16 > 1024 ? max_n / 16 : 1024;
-  ok &= cudaMalloc(&s.d, sizeof(int32_t) * max_n + s.max_filters) == cudaSuccess;
+  const int64_t claims = sizeof(int32_t) * max_n, claim_bits = max_n / 8 + s.max_filters + 1;
+  ok &= cudaMalloc(&s.d, claims > claim_bits ? claims : claim_bits) == cudaSuccess;
   ok &= cudaMalloc(&s.a_tmp, sizeof(int32_t) * max_n) == cudaSuccess;
   ok &= cudaMalloc(&s.W, 8 * static_cast<size_t>(max_n)) == cudaSuccess;
   ok &= cudaMalloc(&s.guide, sizeof(int32_t) * (max_n + 1)) == cudaSuccess;
