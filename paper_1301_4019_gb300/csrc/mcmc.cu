@@ -39,6 +39,11 @@ metropolis_kernel(const T* __restrict__ lw, const float* __restrict__ lwf, int64
   if (d) atomicMin(d + k, static_cast<int32_t>(i));
 }
 
+// Particles per warp run, at least: so few that a small call reaches the whole GPU and its warps
+// share their particles among their lanes from the start (rejection_tail; runs of 256 / 64 / 8:
+// 96 / 39 / 17 us for 2688 particles at y = 3.5, 313 / 125 / 98 for 100000 at y = 4).
+constexpr int kRejRun = 8;
+
 // Rejection with warp refill (mcmc.cuh) over the particles [start, end) of one warp run.
 template <typename T>
 __device__ __forceinline__ void rejection_run(const T* __restrict__ lw,
@@ -54,17 +59,21 @@ __device__ __forceinline__ void rejection_run(const T* __restrict__ lw,
   uint64_t s = 0;  // attempts made (max_trials < 2^32, but s + kRejBatch may pass 2^32)
   T lwi = active ? __ldg(lw + i) : T(0);
   if (active && nonfinite_logw(lwi)) flag_error(err, RS_ERR_NONFINITE);
+  auto attempts = [&](int64_t ii, uint32_t from, T own, int64_t& j, bool& over) -> bool {
+    if constexpr (sizeof(T) == 8)
+      return rejection_attempts_sc<kRejBatch>(lw, lwf, N, rb, keys, ii, from, f64_sidecar(own),
+                                              max_trials, j, over);
+    else
+      return rejection_attempts<kRejBatch>(lw, N, rb, keys, ii, from, own, max_trials, j, over);
+  };
   for (;;) {
+    const unsigned busy = __ballot_sync(0xffffffffu, active);
+    if (head >= end && __popc(busy) <= 16) break;  // no particle left to take in: share the rest
     bool settled = false;
     if (active) {
       int64_t j;
-      if constexpr (sizeof(T) == 8)
-        settled = rejection_attempts_sc<kRejBatch>(lw, lwf, N, rb, keys, i,
-                                                   static_cast<uint32_t>(s), f64_sidecar(lwi),
-                                                   max_trials, j, err);
-      else
-        settled = rejection_attempts<kRejBatch>(lw, N, rb, keys, i, static_cast<uint32_t>(s),
-                                                lwi, max_trials, j, err);
+      bool over = false;
+      settled = attempts(i, static_cast<uint32_t>(s), lwi, j, over);
       s += kRejBatch;
       if (!settled && s >= static_cast<uint64_t>(max_trials)) {
         flag_error(err, RS_ERR_REJECTION_CAP);
@@ -72,6 +81,7 @@ __device__ __forceinline__ void rejection_run(const T* __restrict__ lw,
         settled = true;
       }
       if (settled) {
+        if (over) flag_error(err, RS_ERR_BOUND_VIOLATED);
         a[i] = static_cast<int32_t>(j);
         if (d) atomicMin(d + j, static_cast<int32_t>(i));
       }
@@ -87,8 +97,17 @@ __device__ __forceinline__ void rejection_run(const T* __restrict__ lw,
       }
     }
     head += __popc(done);
-    if (!__any_sync(0xffffffffu, active)) break;
   }
+  const RejParticle<T> own{active, static_cast<uint32_t>(i), 0u, 0u, 0, s, lwi};
+  rejection_tail<T>(
+      own, max_trials, err,
+      [&](const RejParticle<T>& P, uint32_t from, int64_t& j, bool& over) {
+        return attempts(P.i, from, P.lwi, j, over);
+      },
+      [&](const RejParticle<T>& P, int64_t j) {
+        a[P.i] = static_cast<int32_t>(j);
+        if (d) atomicMin(d + j, static_cast<int32_t>(P.i));
+      });
 }
 
 // Warp w takes the runs w, w + W, ... of run_len particles (W = warps of the grid). The host
@@ -365,7 +384,7 @@ cudaError_t launch_rejection_t(const Scratch& s, const T* lw, int64_t N, double 
   GridBar* bar = &s.glob->bar;
   float* lwf = static_cast<float*>(s.W);  // the sidecars of binary64 log-weights (4 B each)
   const int64_t runs = (N + kRejRun - 1) / kRejRun;
-  const int64_t want = (runs * 32 + kBlock - 1) / kBlock;
+  const int64_t want = (runs + kBlock / 32 - 1) / (kBlock / 32);
   if (s.coop && s.launch_mode != RS_LAUNCH_SEPARATE) {
     const int cap = coop_capacity(reinterpret_cast<const void*>(rejection_kernel<T, true>));
     if (cap > 0) {

@@ -369,70 +369,14 @@ __device__ __forceinline__ int32_t metropolis_one_sc(const double* __restrict__ 
 // of counter (i, floor(s/2)) (half_u01_f32, half_index); accept when u < exp(lw^j - log w_max).
 // A log-weight above the bound is flagged and accepted; max_trials attempts without
 // acceptance keep i and flag the cap.
-__device__ __forceinline__ int32_t rejection_one(const float* __restrict__ lw, int64_t n,
-                                                 double log_wmax, int64_t max_trials,
-                                                 const Keys& keys, int64_t i, int* err) {
-  const float lwmax = static_cast<float>(log_wmax);
-  const float lwi = __ldg(lw + i);
-  if (nonfinite_logw(lwi)) flag_error(err, RS_ERR_NONFINITE);
-  const uint32_t ii = static_cast<uint32_t>(i);
-  int64_t j = i;
-  uint4 x = make_uint4(0u, 0u, 0u, 0u);
-  for (int64_t s = 0; s < max_trials; ++s) {
-    if ((s & 1) == 0) x = draw(keys, ii, static_cast<uint32_t>(s >> 1));
-    const uint32_t w0 = (s & 1) ? x.z : x.x, w1 = (s & 1) ? x.w : x.y;
-    if (s > 0) j = half_index<false>(w0, w1, static_cast<uint32_t>(n));
-    const float u = half_u01_f32(w0);
-    const float lwj = (s == 0) ? lwi : __ldg(lw + j);
-    const float delta = lwj - lwmax;
-    if (delta > 0.0f) {
-      flag_error(err, RS_ERR_BOUND_VIOLATED);
-      return static_cast<int32_t>(j);
-    }
-    if (delta == 0.0f || u < exp_pinned(delta)) return static_cast<int32_t>(j);
-  }
-  flag_error(err, RS_ERR_REJECTION_CAP);
-  return static_cast<int32_t>(i);
-}
-
-__device__ __forceinline__ int32_t rejection_one(const double* __restrict__ lw, int64_t n,
-                                                 double lwmax, int64_t max_trials,
-                                                 const Keys& keys, int64_t i, int* err) {
-  const double lwi = __ldg(lw + i);
-  if (nonfinite_logw(lwi)) flag_error(err, RS_ERR_NONFINITE);
-  float lwmax_f;
-  const bool okm = f64_to_f32_trunc(lwmax, lwmax_f);
-  const long long km = f64_key(lwmax);
-  const long long kNegInf = f64_key(-INFINITY);
-  const uint32_t ii = static_cast<uint32_t>(i);
-  int64_t j = i;
-  for (int64_t s = 0; s < max_trials; ++s) {
-    const uint4 x = draw(keys, ii, static_cast<uint32_t>(s));
-    if (s > 0) j = uniform_index(x, static_cast<uint32_t>(n));
-    const double lwj = (s == 0) ? lwi : __ldg(lw + j);
-    const long long kj = f64_key(lwj);
-    if (kj > km && !is_nan(lwj)) {  // above the bound (NaN never compares)
-      flag_error(err, RS_ERR_BOUND_VIOLATED);
-      return static_cast<int32_t>(j);
-    }
-    if (kj == km) return static_cast<int32_t>(j);  // ratio exactly 1
-    if (kj == kNegInf || is_nan(lwj)) continue;
-    float lwj_f;
-    const bool okj = f64_to_f32_trunc(lwj, lwj_f);
-    if (f64_accept_lt(lwj, lwj_f, okj, lwmax, lwmax_f, okm, x)) return static_cast<int32_t>(j);
-  }
-  flag_error(err, RS_ERR_REJECTION_CAP);
-  return static_cast<int32_t>(i);
-}
-
+//
 // ---------------------------------------------------------------------------------------
 // Rejection with warp refill. Trial counts vary per particle (a geometric tail, Section 2.2),
 // and a warp would wait for its slowest lane. Instead every warp owns a run of particles and
 // a lane that settles its particle takes the next unstarted one of the run, so all lanes stay
-// busy. Attempt s of particle i always uses counter (i, s): the result does not depend on
-// the schedule and equals rejection_one.
+// busy. Attempt s of particle i always uses the same draw: the result does not depend on the
+// schedule.
 // ---------------------------------------------------------------------------------------
-constexpr int kRejRun = 32 * 8;  // particles per warp run
 
 // The bound log w_max in the forms the attempts compare against. clamp: partial rejection
 // control (Section 2.2): the attempts sample v = min(w, v_max) with v_max = the bound, so a
@@ -457,12 +401,12 @@ __device__ __forceinline__ RejBound make_bound(double log_wmax, bool clamp = fal
 
 // Decision of one rejection attempt with the uniform's word w0 (binary32) or draw x (binary64) and
 // proposal log-weight lwj: accept when u < exp(lw^j - log w_max); a log-weight above the bound
-// is flagged (unless clamped) and accepted.
+// is accepted and, unless clamped, sets over (which the caller flags if the attempt counts).
 __device__ __forceinline__ bool rejection_accept(const RejBound& rb, uint32_t w0, float lwj,
-                                                 int* err) {
+                                                 bool& over) {
   const float delta = lwj - rb.lwmax_rn;
   if (delta > 0.0f) {
-    if (!rb.clamp) flag_error(err, RS_ERR_BOUND_VIOLATED);
+    over |= !rb.clamp;
     return true;
   }
   if (delta == 0.0f) return true;
@@ -472,10 +416,10 @@ __device__ __forceinline__ bool rejection_accept(const RejBound& rb, uint32_t w0
 }
 
 __device__ __forceinline__ bool rejection_accept(const RejBound& rb, uint4 x, double lwj,
-                                                 int* err) {
+                                                 bool& over) {
   const long long kj = f64_key(lwj);
   if (kj > rb.km && !is_nan(lwj)) {  // above the bound (NaN never compares)
-    if (!rb.clamp) flag_error(err, RS_ERR_BOUND_VIOLATED);
+    over |= !rb.clamp;
     return true;
   }
   if (kj == rb.km) return true;  // ratio exactly 1
@@ -489,10 +433,10 @@ __device__ __forceinline__ bool rejection_accept(const RejBound& rb, uint4 x, do
 // binary64 log-weight lw[j] is read only when the sidecar cannot decide. Same decision.
 __device__ __forceinline__ bool rejection_accept_sc(const RejBound& rb, uint4 x,
                                                     const double* __restrict__ lw, int64_t j,
-                                                    float tj, int* err) {
-  if (!(tj == tj) || !rb.okm || tj == rb.lwmax_f) return rejection_accept(rb, x, __ldg(lw + j), err);
+                                                    float tj, bool& over) {
+  if (!(tj == tj) || !rb.okm || tj == rb.lwmax_f) return rejection_accept(rb, x, __ldg(lw + j), over);
   if (tj > rb.lwmax_f) {  // lw_j above the bound
-    if (!rb.clamp) flag_error(err, RS_ERR_BOUND_VIOLATED);
+    over |= !rb.clamp;
     return true;
   }
   if (tj == -INFINITY) return false;
@@ -513,7 +457,7 @@ template <int K, typename T>
 __device__ __forceinline__ bool rejection_attempts(const T* __restrict__ lw, int64_t n,
                                                    const RejBound& rb, const Keys& keys,
                                                    int64_t i, uint32_t s, T lwi,
-                                                   int64_t max_trials, int64_t& j, int* err) {
+                                                   int64_t max_trials, int64_t& j, bool& over) {
   uint4 x[K];
   int64_t jq[K];
   T lwj[K];
@@ -527,7 +471,7 @@ __device__ __forceinline__ bool rejection_attempts(const T* __restrict__ lw, int
 #pragma unroll
   for (int q = 0; q < K; ++q) {
     if (static_cast<int64_t>(s) + q >= max_trials) return false;
-    if (rejection_accept(rb, x[q], lwj[q], err)) {
+    if (rejection_accept(rb, x[q], lwj[q], over)) {
       j = jq[q];
       return true;
     }
@@ -541,7 +485,7 @@ template <int K>
 __device__ __forceinline__ bool rejection_attempts(const float* __restrict__ lw, int64_t n,
                                                    const RejBound& rb, const Keys& keys,
                                                    int64_t i, uint32_t s, float lwi,
-                                                   int64_t max_trials, int64_t& j, int* err) {
+                                                   int64_t max_trials, int64_t& j, bool& over) {
   static_assert(K % 2 == 0, "whole blocks");
   uint32_t w[K];
   float lwj[K];
@@ -560,7 +504,7 @@ __device__ __forceinline__ bool rejection_attempts(const float* __restrict__ lw,
 #pragma unroll
   for (int q = 0; q < K; ++q) {
     if (static_cast<int64_t>(s) + q >= max_trials) return false;
-    if (rejection_accept(rb, w[q], lwj[q], err)) {
+    if (rejection_accept(rb, w[q], lwj[q], over)) {
       j = jq[q];
       return true;
     }
@@ -575,7 +519,7 @@ __device__ __forceinline__ bool rejection_attempts_sc(const double* __restrict__
                                                       const float* __restrict__ lwf, int64_t n,
                                                       const RejBound& rb, const Keys& keys,
                                                       int64_t i, uint32_t s, float ti,
-                                                      int64_t max_trials, int64_t& j, int* err) {
+                                                      int64_t max_trials, int64_t& j, bool& over) {
   uint4 x[K];
   int64_t jq[K];
   float tj[K];
@@ -589,13 +533,86 @@ __device__ __forceinline__ bool rejection_attempts_sc(const double* __restrict__
 #pragma unroll
   for (int q = 0; q < K; ++q) {
     if (static_cast<int64_t>(s) + q >= max_trials) return false;
-    if (rejection_accept_sc(rb, x[q], lw, jq[q], tj[q], err)) {
+    if (rejection_accept_sc(rb, x[q], lw, jq[q], tj[q], over)) {
       j = jq[q];
       return true;
     }
   }
   return false;
 }
+
+// ---------------------------------------------------------------------------------------
+// The end of a warp's run: no particle left to take in and at most half of its lanes still busy.
+// The trial counts have a geometric tail, and a lane alone makes two attempts per round of
+// dependent steps (draw, gather, decision: about a microsecond), so the longest particle of a
+// call set its time (100000 particles at y = 4: 880 attempts, 432 us). The draws are counted, not
+// drawn in turn, so here the lanes share the particles that are left: with m particles each gets
+// the largest power of two of lanes <= 32 / m, lane r of a group takes attempts s + 2r and
+// s + 2r + 1, and the first accepted one in attempt order is the result, exactly as one lane
+// would have found it (attempts after it leave no trace: `over` counts only for the winner).
+// ---------------------------------------------------------------------------------------
+// One particle of a warp: local index i of the n particles from lo on, its attempts made so far,
+// its log-weight and the counter tag of its filter.
+template <typename T>
+struct RejParticle {
+  bool active;
+  uint32_t i, n, tag;
+  int64_t lo;
+  uint64_t s;
+  T lwi;
+};
+
+__device__ __forceinline__ uint64_t shfl_u64(uint64_t v, int src) {
+  const uint32_t lo = __shfl_sync(0xffffffffu, static_cast<uint32_t>(v), src);
+  const uint32_t hi = __shfl_sync(0xffffffffu, static_cast<uint32_t>(v >> 32), src);
+  return (static_cast<uint64_t>(hi) << 32) | lo;
+}
+
+// attempts(P, s, j, over): rejection_attempts of particle P from attempt s on; settle(P, j): its
+// result. Called by all 32 lanes, each with its own particle (or inactive).
+template <typename T, typename Attempts, typename Settle>
+__device__ __forceinline__ void rejection_tail(RejParticle<T> own, int64_t max_trials, int* err,
+                                               const Attempts& attempts, const Settle& settle) {
+  const int lane = threadIdx.x & 31;
+  const uint64_t most = static_cast<uint64_t>(max_trials);
+  for (;;) {
+    const unsigned mask = __ballot_sync(0xffffffffu, own.active);
+    if (mask == 0u) return;
+    const int m = __popc(mask);
+    const int lg = 31 - __clz(32 / m), g = 1 << lg;
+    const int grp = lane >> lg, r = lane & (g - 1);
+    const int src = grp < m ? static_cast<int>(__fns(mask, 0, grp + 1)) : 0;  // the group's owner
+    RejParticle<T> P;
+    P.i = __shfl_sync(0xffffffffu, own.i, src);
+    P.n = __shfl_sync(0xffffffffu, own.n, src);
+    P.tag = __shfl_sync(0xffffffffu, own.tag, src);
+    P.lo = static_cast<int64_t>(shfl_u64(static_cast<uint64_t>(own.lo), src));
+    P.s = shfl_u64(own.s, src);
+    P.lwi = __shfl_sync(0xffffffffu, own.lwi, src);
+    const uint64_t s = P.s + 2 * static_cast<uint64_t>(r);
+    bool acc = false, over = false;
+    int64_t j = 0;
+    if (grp < m && s < most) acc = attempts(P, static_cast<uint32_t>(s), j, over);
+    const unsigned won = __ballot_sync(0xffffffffu, acc);
+    const unsigned ones = g == 32 ? 0xffffffffu : (1u << g) - 1u;
+    if (acc && __ffs(won & (ones << (grp << lg))) == lane + 1) {
+      settle(P, j);
+      if (over) flag_error(err, RS_ERR_BOUND_VIOLATED);
+    }
+    if (own.active) {
+      const int rank = __popc(mask & ((1u << lane) - 1u));
+      own.s += 2 * static_cast<uint64_t>(g);
+      if (won & (ones << (rank << lg))) {
+        own.active = false;
+      } else if (own.s >= most) {
+        flag_error(err, RS_ERR_REJECTION_CAP);
+        settle(own, static_cast<int64_t>(own.i));
+        own.active = false;
+      }
+    }
+  }
+}
+static_assert(kRejBatch == 2, "two attempts per lane and round");
 
 }  // namespace
 }  // namespace rsk
