@@ -288,7 +288,7 @@ __device__ __forceinline__ uint4 words_of_u(uint64_t m) {
                     0u, 0u);
 }
 
-// Binary64 decisions on the binary32 pipes (f64_accept_lt) against the binary64 definition
+// Binary64 decisions on the binary32 pipes (f64_accept_lt, band_accept_sc) against the binary64 definition
 // u < exp_pinned(lwj - lwk), on n log-weight pairs: lwk from four magnitudes (0, -2.75,
 // -1234.5678, 30000.5: the last two push the filter to its exact fallback), lwj = lwk + d with
 // d spread over [-90, 0) (plus hashed low bits, so that many bit patterns occur), and per pair
@@ -330,6 +330,9 @@ check_f64_decisions_kernel(int64_t n, unsigned long long* out) {
         const bool got = f64_accept_lt(lwj, lwj_f, okj, lwk, lwk_f, okk, x);
         const bool want = u01_f64(x) < p;
         if (got != want) ++bad;
+        bool amb = false;  // the branch-free band of the Metropolis steps, from the sidecars
+        const bool quick = band_accept_sc(x.x, f64_sidecar(lwj), f64_sidecar(lwk), amb);
+        if (!amb && quick != want) ++bad;
       }
     }
   }

@@ -242,59 +242,6 @@ __device__ __forceinline__ bool f64_step_accept(double lwk, float lwk_f, bool ok
   return f64_accept_lt(lwj, lwj_f, okj, lwk, lwk_f, okk, x);
 }
 
-__device__ __forceinline__ int32_t metropolis_one(const double* __restrict__ lw, int64_t n,
-                                                  int32_t B, const Keys& keys, int64_t i,
-                                                  int* err) {
-  double lwk = __ldg(lw + i);
-  if (nonfinite_logw(lwk)) flag_error(err, RS_ERR_NONFINITE);
-  float lwk_f;
-  bool okk = f64_to_f32_trunc(lwk, lwk_f);
-  long long kk = f64_key(lwk);
-  int64_t k = i;
-  const uint32_t ii = static_cast<uint32_t>(i);
-  int32_t s = 0;
-  for (; s + kUnroll64 <= B; s += kUnroll64) {
-    uint4 x[kUnroll64];
-    double lwj[kUnroll64];
-    int64_t j[kUnroll64];
-#pragma unroll
-    for (int q = 0; q < kUnroll64; ++q) {
-      x[q] = draw(keys, ii, static_cast<uint32_t>(s + q));
-      j[q] = uniform_index(x[q], static_cast<uint32_t>(n));
-      lwj[q] = __ldg(lw + j[q]);
-    }
-#pragma unroll
-    for (int q = 0; q < kUnroll64; ++q) {
-      const long long kj = f64_key(lwj[q]);
-      float lwj_f;
-      const bool okj = f64_to_f32_trunc(lwj[q], lwj_f);
-      if (f64_step_accept(lwk, lwk_f, okk, kk, lwj[q], lwj_f, okj, kj, x[q])) {
-        k = j[q];
-        lwk = lwj[q];
-        lwk_f = lwj_f;
-        okk = okj;
-        kk = kj;
-      }
-    }
-  }
-  for (; s < B; ++s) {
-    const uint4 x = draw(keys, ii, static_cast<uint32_t>(s));
-    const int64_t j = uniform_index(x, static_cast<uint32_t>(n));
-    const double lwj = __ldg(lw + j);
-    const long long kj = f64_key(lwj);
-    float lwj_f;
-    const bool okj = f64_to_f32_trunc(lwj, lwj_f);
-    if (f64_step_accept(lwk, lwk_f, okk, kk, lwj, lwj_f, okj, kj, x)) {
-      k = j;
-      lwk = lwj;
-      lwk_f = lwj_f;
-      okk = okj;
-      kk = kj;
-    }
-  }
-  return static_cast<int32_t>(k);
-}
-
 // A Metropolis step of a binary64 chain decided from sidecars (f64_sidecar): state k with
 // sidecar tk, proposal j with tj; the binary64 log-weights lw[k], lw[j] are read only when the
 // sidecars cannot decide. Same decision as f64_step_accept on the binary64 values.
@@ -313,44 +260,84 @@ __device__ __forceinline__ bool sc_step_accept(const double* __restrict__ lw, in
                        [&] { return exact_f64_less_exp(__ldg(lw + j), __ldg(lw + k), x); });
 }
 
+// The same decision from the band alone in almost every case, without branches: with
+// e = 2^32 exp(tj - tk), v = x0 rounded towards zero to binary32 (2^32 u lies in [v, v + 257)) and
+// m the filter's relative margin (f64_filter_lt), the step accepts iff v < e wherever
+// |v - e| > e m + 257 and the truncations' bound E is below 0.01; elsewhere `amb` is set (and
+// stays set): a zero-weight state, a NaN, wide bounds, u next to the ratio. Equal sidecars and
+// ratios above 1 are covered by the same inequality. A zero-weight proposal is e = 0, rejected,
+// from any state of non-zero weight. (The chain of tests took about 45 instructions, this 16.)
+__device__ __forceinline__ bool band_accept_sc(uint32_t x0, float tj, float tk, bool& amb) {
+  const float df = __fsub_rn(tj, tk);
+  const float E = __fmaf_ru(fabsf(tj) + fabsf(tk), 0x1p-23f,
+                            __fmaf_ru(fabsf(df), 0x1p-24f, 0x1p-124f));
+  const float e = exp_band_estimate32(df);
+  const float d = __fsub_rn(__uint2float_rz(x0), e);
+  const float w = __fmaf_ru(e, __fmaf_ru(E, 1.02f, kExpBand), 257.0f);
+  amb |= !(fabsf(d) > w && E < 0.01f) && !(is_neg_inf(tj) && tk > -INFINITY);
+  return d < 0.0f;
+}
+
 // metropolis_chain for n < 2^31 binary64 log-weights lw from the state i with sidecar tk:
-// gather(j) reads the sidecar of proposal j (4 bytes instead of 8). Same ancestor as
-// metropolis_one on the binary64 values.
+// gather(j) reads the sidecar of proposal j (4 bytes instead of 8). Steps kUnroll64 at a time
+// from the band; if any of them was undecided they are taken again by sc_step_accept. The
+// decisions, and so the ancestor, are those of the binary64 definition.
 template <typename Gather>
 __device__ __forceinline__ int32_t metropolis_chain_sc(const double* __restrict__ lw, float tk,
                                                        const Gather& gather, uint32_t n,
                                                        int32_t B, const Keys& keys, uint32_t i) {
   uint32_t k = i;
   const DrawRow row = draw_row(keys, i);
-  int32_t s = 0;
-  for (; s + kUnroll64 <= B; s += kUnroll64) {
-    uint4 x[kUnroll64];
-    uint32_t j[kUnroll64];
+  for (int32_t s = 0; s < B; s += kUnroll64) {
+    uint32_t x0[kUnroll64], j[kUnroll64];
     float tj[kUnroll64];
 #pragma unroll
     for (int q = 0; q < kUnroll64; ++q) {
-      x[q] = draw(keys, row, static_cast<uint32_t>(s + q));
-      j[q] = uniform_index(x[q], n);
-      tj[q] = gather(j[q]);
+      if (s + q < B) {
+        const uint4 x = draw(keys, row, static_cast<uint32_t>(s + q));
+        x0[q] = x.x;
+        j[q] = uniform_index(x, n);
+        tj[q] = gather(j[q]);
+      }
     }
+    const uint32_t k0 = k;
+    const float tk0 = tk;
+    bool amb = false;
 #pragma unroll
     for (int q = 0; q < kUnroll64; ++q) {
-      if (sc_step_accept(lw, k, tk, j[q], tj[q], x[q])) {
+      if (s + q < B && band_accept_sc(x0[q], tj[q], tk, amb)) {
         k = j[q];
         tk = tj[q];
       }
     }
-  }
-  for (; s < B; ++s) {
-    const uint4 x = draw(keys, row, static_cast<uint32_t>(s));
-    const uint32_t j = uniform_index(x, n);
-    const float tj = gather(j);
-    if (sc_step_accept(lw, k, tk, j, tj, x)) {
-      k = j;
-      tk = tj;
+    if (amb) {
+      k = k0;
+      tk = tk0;
+#pragma unroll 1
+      for (int32_t t = s; t < s + kUnroll64 && t < B; ++t) {
+        const uint4 x = draw(keys, row, static_cast<uint32_t>(t));
+        const uint32_t jt = uniform_index(x, n);
+        const float tt = gather(jt);
+        if (sc_step_accept(lw, k, tk, jt, tt, x)) {
+          k = jt;
+          tk = tt;
+        }
+      }
     }
   }
   return static_cast<int32_t>(k);
+}
+
+// The chain of particle i with its proposals gathered from the binary64 log-weights (batched
+// chains, which have no sidecars in memory).
+__device__ __forceinline__ int32_t metropolis_one(const double* __restrict__ lw, int64_t n,
+                                                  int32_t B, const Keys& keys, int64_t i,
+                                                  int* err) {
+  const double lwi = __ldg(lw + i);
+  if (nonfinite_logw(lwi)) flag_error(err, RS_ERR_NONFINITE);
+  return metropolis_chain_sc(lw, f64_sidecar(lwi),
+                             [&](uint32_t j) { return f64_sidecar(__ldg(lw + j)); },
+                             static_cast<uint32_t>(n), B, keys, static_cast<uint32_t>(i));
 }
 
 // The chain of particle i with its proposals gathered from the sidecars lwf in memory.
