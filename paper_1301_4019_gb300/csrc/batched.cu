@@ -772,6 +772,7 @@ batch_chain_plan_kernel(const int64_t* __restrict__ off, int F, int64_t total,
 static_assert(kBatchMaxN < (1 << 24), "half_index<true>");
 constexpr int kChainCap = 57344;                            // staged log-weights
 constexpr size_t kChainSmem = sizeof(float) * (kChainCap + 4);  // (+ the alignment shift)
+constexpr int kChainBlocks = 2;                             // blocks of a chain drawn together
 constexpr int kChainChunks = 16;                            // chunks per CTA, at most
 
 __global__ void __launch_bounds__(kChainBlock, 1)
@@ -883,8 +884,8 @@ batch_chain_kernel(const float* __restrict__ lw, const int64_t* __restrict__ off
               auto part = [&](uint32_t j) {
                 return j < static_cast<uint32_t>(kChainCap) ? sw[j] : __ldg(lf + j);
               };
-              k = whole ? metropolis_chain<true>(lwi, all, un, Bv, keys, ui)
-                        : metropolis_chain<true>(lwi, part, un, Bv, keys, ui);
+              k = whole ? metropolis_chain<true, kChainBlocks>(lwi, all, un, Bv, keys, ui)
+                        : metropolis_chain<true, kChainBlocks>(lwi, part, un, Bv, keys, ui);
             }
             a[g] = k;
             if (d) atomicMin(d + P.lo + k, static_cast<int32_t>(P.i));
@@ -931,7 +932,7 @@ batch_mcmc_kernel(const T* __restrict__ lw, const int64_t* __restrict__ off, int
         Bv = 0;
       }
       const Keys keys = with_tag(base_keys, static_cast<uint32_t>(P.f), RS_METROPOLIS);
-      if constexpr (sizeof(T) == 4) k = metropolis_one<true>(lw + P.lo, P.n, Bv, keys, P.i, err);
+      if constexpr (sizeof(T) == 4) k = metropolis_one<true, 2>(lw + P.lo, P.n, Bv, keys, P.i, err);
       else k = metropolis_one(lw + P.lo, P.n, Bv, keys, P.i, err);
     }
     a[g] = k;

@@ -22,10 +22,15 @@ namespace {
 // slower: their four proposals in flight need them).
 template <typename T> constexpr int metropolis_min_ctas() { return sizeof(T) == 4 ? 6 : 1; }
 
+// Binary32 chains draw two blocks (four proposals) together below this size and one from it on,
+// where the gathers leave L1 and are bound by the L2's rate, not by their latency (2^20: 74.3
+// against 76.1 us with Permute; 2^18 at B = 60: 60.6 against 58.9).
+constexpr int64_t kMetropolisOneBlockMinN = int64_t{1} << 19;
+
 // One thread per particle (the claims d, when given, were set to the sentinel N before). SMALL:
-// N < 2^24. Binary64 log-weights come with their sidecars lwf (f64_sidecar; sidecar_kernel),
+// N < 2^24; P: blocks drawn together (binary32). Binary64 log-weights come with their sidecars lwf (f64_sidecar; sidecar_kernel),
 // which the chains gather instead of the binary64 values.
-template <typename T, bool SMALL>
+template <typename T, bool SMALL, int P>
 __global__ void __launch_bounds__(kBlock, metropolis_min_ctas<T>())
 metropolis_kernel(const T* __restrict__ lw, const float* __restrict__ lwf, int64_t N, int32_t B,
                   Keys keys, int32_t* __restrict__ a, int32_t* __restrict__ d, int* err) {
@@ -34,7 +39,7 @@ metropolis_kernel(const T* __restrict__ lw, const float* __restrict__ lwf, int64
   if (i >= N) return;
   int32_t k;
   if constexpr (sizeof(T) == 8) k = metropolis_one_sc(lw, lwf, N, B, keys, i, err);
-  else k = metropolis_one<SMALL>(lw, N, B, keys, i, err);
+  else k = metropolis_one<SMALL, P>(lw, N, B, keys, i, err);
   a[i] = k;
   if (d) atomicMin(d + k, static_cast<int32_t>(i));
 }
@@ -371,11 +376,11 @@ cudaError_t launch_metropolis_t(const Scratch& s, const T* lw, int64_t N, int32_
   }
   trace_mark(s.trace, f64 ? "metropolis_f64" : "metropolis_f32", st);
   const int grid = static_cast<int>((N + kBlock - 1) / kBlock);
-  if (sizeof(T) == 4 && N < (int64_t{1} << 24))
-    launch_pdl(metropolis_kernel<T, sizeof(T) == 4>, grid, kBlock, st, lw, lwf, N, B, keys, a_out,
-               d, s.err);
-  else
-    launch_pdl(metropolis_kernel<T, false>, grid, kBlock, st, lw, lwf, N, B, keys, a_out, d, s.err);
+  const auto kernel = sizeof(T) == 8                 ? metropolis_kernel<T, false, 2>
+                      : N < kMetropolisOneBlockMinN  ? metropolis_kernel<T, true, 2>
+                      : N < (int64_t{1} << 24)       ? metropolis_kernel<T, true, 1>
+                                                     : metropolis_kernel<T, false, 1>;
+  launch_pdl(kernel, grid, kBlock, st, lw, lwf, N, B, keys, a_out, d, s.err);
   return cudaGetLastError();
 }
 

@@ -152,7 +152,6 @@ __device__ __forceinline__ float f64_sidecar(double x) {
   return is_neg_inf(x) ? -INFINITY : __int_as_float(0x7fffffff);
 }
 
-constexpr int kUnroll = 4;    // binary32 chains: proposals issued together
 constexpr int kUnroll64 = 4;  // binary64 chains (2 measured slower)
 
 // 2 P consecutive steps (s even) of a binary32 chain in state (k, lwk), those below B: the P
@@ -206,30 +205,31 @@ __device__ __forceinline__ void metropolis_steps(uint32_t& k, float& lwk, const 
 // Metropolis chain of particle i over n < 2^31 (SMALL: n < 2^24) binary32 log-weights (Code 2),
 // from the state i with log-weight lwk; gather(j) reads the log-weight of proposal j. B steps;
 // steps 2m and 2m + 1 take the two halves of the block of counter (i, m) (half_u01_f32,
-// half_index), so a chain draws ceil(B / 2) blocks. Returns the ancestor.
-template <bool SMALL, typename Gather>
+// half_index), so a chain draws ceil(B / 2) blocks. P blocks (2 P proposals) are issued together.
+// Returns the ancestor.
+template <bool SMALL, int P, typename Gather>
 __device__ __forceinline__ int32_t metropolis_chain(float lwk, const Gather& gather, uint32_t n,
                                                     int32_t B, const Keys& keys, uint32_t i) {
-  static_assert(kUnroll % 2 == 0, "whole blocks per round");
   uint32_t k = i;
   const DrawRow row = draw_row(keys, i);
   int32_t s = 0;
-  for (; s + kUnroll <= B; s += kUnroll)  // (s even)
-    metropolis_steps<kUnroll / 2, SMALL>(k, lwk, gather, n, s, B, keys, row);
-  for (; s < B; s += 2)  // the last B mod kUnroll steps, a block per two
+  if constexpr (P > 1)
+    for (; s + 2 * P <= B; s += 2 * P)  // (s even)
+      metropolis_steps<P, SMALL>(k, lwk, gather, n, s, B, keys, row);
+  for (; s < B; s += 2)  // the last B mod 2 P steps, a block per two
     metropolis_steps<1, SMALL>(k, lwk, gather, n, s, B, keys, row);
   return static_cast<int32_t>(k);
 }
 
 // The chain of particle i with its proposals gathered from the log-weights themselves.
-template <bool SMALL>
+template <bool SMALL, int P>
 __device__ __forceinline__ int32_t metropolis_one(const float* __restrict__ lw, int64_t n,
                                                   int32_t B, const Keys& keys, int64_t i,
                                                   int* err) {
   const float lwi = __ldg(lw + i);
   if (nonfinite_logw(lwi)) flag_error(err, RS_ERR_NONFINITE);
   const auto gather = [&](uint32_t j) { return __ldg(lw + j); };
-  return metropolis_chain<SMALL>(lwi, gather, static_cast<uint32_t>(n), B, keys,
+  return metropolis_chain<SMALL, P>(lwi, gather, static_cast<uint32_t>(n), B, keys,
                                  static_cast<uint32_t>(i));
 }
 
