@@ -10,13 +10,16 @@
 //   max     : per tile, maximum log-weight, combined per filter by an atomic max of keys
 //   sums    : per tile, the tile scan total                               (tile-parallel)
 //   prefix  : per filter, tile prefixes, W^N and N / W^N                  (CTA per filter)
-//   emit    : per tile, cumulative offspring + Code-11 scatter + claims, or stored W
-//   search / Metropolis / rejection / Permute: one thread per particle, its filter found by a
-//             binary search of the offsets.
+//   emit    : per tile, cumulative offspring + Code-11 scatter + claimed bits, or stored W
+//   search  : one thread per particle, its filter found by a binary search of the offsets
+//   chains  : binary32 Metropolis from shared memory, chunks of equal work per CTA
+//             (batch_chain_kernel); binary64 one thread per particle
+//   rejection : a warp per run of particles, its lanes sharing the last ones
+//   Permute : a warp per 32 or 128 consecutive slots, its filter looked up once.
 // With cooperative launches (the default), max, sums, prefixes and emission run as one
-// persistent launch over the tiles of all filters (batch_coop_kernel) after the plan, so a
+// persistent launch over the segments of all filters (batch_coop_kernel) after the plan, so a
 // scan-based scheme is plan + one launch (+ the search for the multinomial) + Permute.
-// Every unit runs the same device functions as the single-filter kernels on the same tile
+// Every unit runs the same device functions as the single-filter kernels on the same segment
 // structure (relative to the filter's first particle), with the filter index in the
 // random-number counter: filter f of a batched call equals rs_resample on that filter's slice
 // with filter = f, bit for bit.

@@ -420,9 +420,13 @@ cudaError_t launch_rejection_t(const Scratch& s, const T* lw, int64_t N, double 
     if (e != cudaSuccess) return e;
   }
   trace_mark(s.trace, f64 ? "rejection_f64" : "rejection_f32", st);
-  launch_pdl(rejection_kernel<T, false>, static_cast<int>(want), kBlock, st, lw, lwf, N,
-             log_wmax, lwmax_dev, clamp, max_trials, keys, a_out, d,
-             static_cast<int64_t>(kRejRun), bar, s.err);
+  // (about the resident warps' number of runs, of at most 256 particles)
+  int64_t run_len = N / (static_cast<int64_t>(device_sm_count()) * 40);
+  run_len = run_len < kRejRun ? kRejRun : run_len > 256 ? 256 : run_len;
+  const int64_t warps = (N + run_len - 1) / run_len;
+  launch_pdl(rejection_kernel<T, false>,
+             static_cast<int>((warps + kBlock / 32 - 1) / (kBlock / 32)), kBlock, st, lw, lwf, N,
+             log_wmax, lwmax_dev, clamp, max_trials, keys, a_out, d, run_len, bar, s.err);
   return cudaGetLastError();
 }
 

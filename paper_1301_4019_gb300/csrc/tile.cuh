@@ -1,7 +1,7 @@
-// tile.cuh -- the tile scan shared by the single-filter and batched scan-based resamplers:
-// weights per (input type, accumulator type), the kTile-particle tile prefix sum made
-// monotone (tile_cum_weights), the exact tile prefixes, and the cumulative offspring of Codes
-// 7 and 8 with the Code-11 scatter.
+// tile.cuh -- the segment scan shared by the single-filter and batched scan-based resamplers:
+// weights per (input type, accumulator type), the segment records and their exact prefixes, the
+// monotone prefix sum of a segment (seg_cum_weights), and the cumulative offspring of Codes 7 and
+// 8 with the Code-11 scatter.
 #pragma once
 
 #include <cfloat>
@@ -221,14 +221,9 @@ template <> __device__ __forceinline__ float2 load_v_cg<float2>(const double2* p
 
 // Particles of a tile: thread t holds the kPer consecutive offsets kPer t .. kPer t + kPer - 1,
 // so warp w holds 32 kPer consecutive particles and the tile kTile = kBlock kPer.
-// Valid elements of the tile starting at `base` of a sequence ending at N (tiles start at or
-// after the sequence start): offsets 0 .. count-1.
-__device__ __forceinline__ int tile_count(int64_t base, int64_t N) {
-  const int64_t c = N - base;
-  return c < kTile ? static_cast<int>(c) : kTile;
-}
-// The same for a segment: the kSeg = 32 kPer particles of one warp (lane l holds kPer l ..
-// kPer l + kPer - 1); zero or negative past the end.
+// A segment is the kSeg = 32 kPer particles of one warp (lane l holds kPer l .. kPer l + kPer - 1).
+// Its valid particles in a sequence ending at N: offsets 0 .. count - 1 (zero or negative past
+// the end).
 constexpr int kSeg = 32 * kPer;
 __device__ __forceinline__ int seg_count(int64_t base, int64_t N) {
   const int64_t c = N - base;
@@ -551,18 +546,6 @@ __device__ __forceinline__ void st_u128(u128* p, u128 v) {
       make_ulonglong2(static_cast<uint64_t>(v), static_cast<uint64_t>(v >> 64));
 }
 
-__device__ __forceinline__ u128 block_sum_u128(u128 v, u128* sh) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += shfl_xor_u128(v, o);
-  __syncthreads();
-  if (lane == 0) sh[warp] = v;
-  __syncthreads();
-  u128 t = 0;
-  for (int k = 0; k < kWarps; ++k) t += sh[k];
-  return t;
-}
-
 // Block-wide exclusive scan of u128 values in thread order; `total` gets the block's sum
 // (every thread). sh: kWarps entries.
 __device__ __forceinline__ u128 block_excl_scan_u128(u128 v, u128* sh, u128& total) {
@@ -683,11 +666,6 @@ template <typename T, typename V>
 __device__ __forceinline__ u128 rec_fixed(const double2* p, T M, const float2* tab = kExp2Frac64) {
   return to_fixed(rec_scaled<T, V>(p, M, tab));
 }
-template <typename T, typename V>
-__device__ __forceinline__ u128 rec_fixed_of(const double2 r, T M, const float2* tab = kExp2Frac64) {
-  return to_fixed(rec_scaled_of<T, V>(r, M, tab));
-}
-
 // Prefixes of one sequence of nt segment records, M the sequence's maximum log-weight
 // (block-level, every thread of the CTA calls it): with T_g = rec_scaled(record g), P_g =
 // RN(T_0 + ... + T_{g-1}) for g = 0..nt, the exact sums taken in fixed point (each thread a

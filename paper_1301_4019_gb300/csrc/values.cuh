@@ -98,10 +98,6 @@ __device__ __forceinline__ float2 add21(float2 a, float b) {
 // ---- generic ----------------------------------------------------------------------------
 template <typename V> __device__ __forceinline__ V vmax(V a, V b) { return vle(a, b) ? b : a; }
 template <typename V> __device__ __forceinline__ V vmin(V a, V b) { return vle(a, b) ? a : b; }
-template <typename V> __device__ __forceinline__ V vclamp(V x, V lo, V hi) {
-  return vmin(vmax(x, lo), hi);
-}
-template <typename V> __device__ __forceinline__ bool veq(V a, V b) { return vle(a, b) && vle(b, a); }
 
 // ---- cumulative offspring from a cumulative weight W --------------------------------------
 // r = W * (N / W^N); O = floor(r + u) clamped to N; W equal to the total gives O = N (all
