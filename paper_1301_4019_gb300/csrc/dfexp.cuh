@@ -90,6 +90,16 @@ __constant__ float2 kExp2Frac64[64] = {
 // the next 29 bits rounded to 24), with integer operations only: |x - (hi + lo)| <= 2^-48 |x|.
 // Infinities and NaN give hi = x (as binary32), lo = 0; |x| >= 2^128 gives +-inf.
 __device__ __forceinline__ float2 split_f64(double x) {
+  const unsigned int xh = static_cast<unsigned int>(__double2hiint(x));
+  const unsigned int xl = static_cast<unsigned int>(__double2loint(x));
+  const unsigned int ex = (xh >> 20) & 0x7ffu;
+  if (ex - 950u <= 200u) {  // 2^-73 <= |x| < 2^128: both parts normal (or lo = 0), ten operations
+    const unsigned int mag = (__funnelshift_r(xl, xh, 29) - (896u << 23)) & 0x7fffffffu;
+    const float lo = __fmul_rn(__uint2float_rn(xl & 0x1fffffffu),
+                               __uint_as_float((mag & 0x7f800000u) - (52u << 23)));
+    const unsigned int sg = xh & 0x80000000u;
+    return make_float2(__uint_as_float(mag | sg), __uint_as_float(__float_as_uint(lo) ^ sg));
+  }
   const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(x));
   const unsigned int sign = static_cast<unsigned int>(b >> 32) & 0x80000000u;
   const int e = static_cast<int>((b >> 52) & 0x7ffu);
