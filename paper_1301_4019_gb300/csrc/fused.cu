@@ -338,14 +338,15 @@ __device__ __forceinline__ void fused_body(const T* __restrict__ lw, const Fused
 
 // CTAs of kBlock threads that share an SM (the cooperative grid holds so many on each): four for
 // binary32 log-weights and the multinomial (64 registers), three for the stratified and systematic
-// of binary64 log-weights, whose emission keeps more values in flight (80 registers; 3000001 particles, double-float: 92.2 -> 90.2 us, IEEE 700001: 85.8 ->
-// 78.9; compensated binary32 at 2^20 is faster with four).
+// of binary64 log-weights, whose emission keeps more values in flight (80 registers; 3000001
+// particles, double-float: 92.2 -> 90.2 us, IEEE 700001: 85.8 -> 78.9; see launch_fused for the
+// sizes where four take one turn; compensated binary32 at 2^20 is faster with four).
 template <typename T, int SCHEME>
 constexpr int fused_ctas() {
   return sizeof(T) == 4 || SCHEME == RS_MULTINOMIAL ? 4 : 3;
 }
-template <typename T, typename V, int SCHEME>
-__global__ void __launch_bounds__(kBlock, (fused_ctas<T, SCHEME>())) fused_scan_kernel(const T* __restrict__ lw, FusedArgs A) {
+template <typename T, typename V, int SCHEME, int CTAS>
+__global__ void __launch_bounds__(kBlock, CTAS) fused_scan_kernel(const T* __restrict__ lw, FusedArgs A) {
   unsigned int target = 0;
   fused_body<T, V, SCHEME>(lw, A, target);
   // the last CTA to end returns the shared state to its start (every CTA has read the key)
@@ -356,14 +357,14 @@ __global__ void __launch_bounds__(kBlock, (fused_ctas<T, SCHEME>())) fused_scan_
   }
 }
 
-template <typename T, typename V, int SCHEME>
+template <typename T, typename V, int SCHEME, int CTAS = fused_ctas<T, SCHEME>()>
 int fused_capacity() {
   static int cap = -1;  // identical devices assumed
   if (cap < 0) {
     int dev = 0, sms = 0, per_sm = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fused_scan_kernel<T, V, SCHEME>,
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fused_scan_kernel<T, V, SCHEME, CTAS>,
                                                       kBlock, 0) != cudaSuccess)
       return 0;
     cap = per_sm * sms;
@@ -371,15 +372,24 @@ int fused_capacity() {
   return cap;
 }
 
-template <typename T, typename V, int SCHEME>
+template <typename T, typename V, int SCHEME, int CTAS = fused_ctas<T, SCHEME>()>
 cudaError_t launch_fused(const Scratch& s, const T* lw, const FusedArgs& A, cudaStream_t st) {
-  int64_t grid = fused_capacity<T, V, SCHEME>();
+  int64_t grid = fused_capacity<T, V, SCHEME, CTAS>();
   if (grid > s.max_blocks) grid = s.max_blocks;
   // a full turn of the warps each; half a turn for native binary64, which is bound by the
   // binary64 pipes of the SMs it reaches (20000 particles: 51 -> 33 us), while the others lose by
   // more CTAs at the barriers (2^20 binary32: 27.2 -> 29.0 us)
   constexpr int64_t per = std::is_same_v<V, double> ? kWarps / 2 : kWarps;
   const int64_t want = ((A.N + kSeg - 1) / kSeg + per - 1) / per;
+  if constexpr (CTAS == 3 && per == kWarps) {
+    // a fourth CTA on an SM (64 registers) where it makes one turn of the warps of two: double-float
+    // at 2^20 (4096 segments, 456 x 8 warps) systematic 42.7 -> 39.0 us with Permute, stratified
+    // 47.3 -> 43.9; from two turns on the registers win (stratified 3600000: 92.7 against 95.3)
+    int64_t more = fused_capacity<T, V, SCHEME, 4>();
+    if (more > s.max_blocks) more = s.max_blocks;
+    if (grid >= 1 && want > grid && want <= more)
+      return launch_fused<T, V, SCHEME, 4>(s, lw, A, st);
+  }
   if (grid > want) grid = want;
   if (grid < 1) return cudaErrorCooperativeLaunchTooLarge;
   cudaLaunchConfig_t cfg = {};
@@ -392,7 +402,7 @@ cudaError_t launch_fused(const Scratch& s, const T* lw, const FusedArgs& A, cuda
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, fused_scan_kernel<T, V, SCHEME>, lw, A);
+  return cudaLaunchKernelEx(&cfg, fused_scan_kernel<T, V, SCHEME, CTAS>, lw, A);
 }
 
 template <typename T, typename V>

@@ -164,7 +164,8 @@ def test_mcmc_and_conversions_equal_across_launch_modes(rs, h, N):
 # one CTA (no barrier) and two; the most segments a CTA's first warp scans alone (31 of 256
 # particles, 608 or 456 CTAs), one more; records and prefixes on chip (256 segments) and beyond
 @pytest.mark.parametrize("N", [1, 2048, 2049, 31 * 256 * 608, 31 * 256 * 608 + 1, 31 * 256 * 456 + 257,
-                               256 * 256 * 608, 256 * 256 * 608 + 4099])
+                               256 * 256 * 608, 256 * 256 * 608 + 4099,
+                               2048 * 456, 2048 * 456 + 1, 2048 * 608, 2048 * 608 + 1])
 @pytest.mark.parametrize("dtype,prec", [(torch.float32, 0), (torch.float32, 1), (torch.float64, 0)])
 def test_fused_segment_split(rs, N, dtype, prec):
     """The cooperative kernel equals the separate ones however many segments a CTA owns, twice in
