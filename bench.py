@@ -227,26 +227,26 @@ class ClockSampler:
 # headers it includes, hashed; `traffic` is null once any of them has changed.
 # ---------------------------------------------------------------------------------------
 NCU_TRAFFIC = {  # label: (bytes per launch, source hash)
-    "permute": (8397926, "e733186968d7e6df"),
-    "metropolis_f64": (16800695, "c46523a1c822c284"),
-    "metropolis_f32": (8404544, "c46523a1c822c284"),
-    "fused_multinomial_f64": (8527008, "97e0f268cecd64bc"),
-    "rejection_f64": (8419657, "c46523a1c822c284"),
-    "rejection_f32": (4212192, "c46523a1c822c284"),
-    "fused_stratified_f64": (8512987, "97e0f268cecd64bc"),
-    "permute_sorted": (4333500, "e733186968d7e6df"),
-    "fused_systematic_f64": (8506295, "97e0f268cecd64bc"),
-    "fused_multinomial_f32": (4351392, "97e0f268cecd64bc"),
-    "fused_stratified_f32": (4331552, "97e0f268cecd64bc"),
-    "iscan": (4214240, "e733186968d7e6df"),
-    "fused_systematic_f32": (4326752, "97e0f268cecd64bc"),
-    "search_f32": (12592032, "88475038523181d3"),
-    "search_f64": (16783872, "88475038523181d3"),
-    "cumoff_to_ancestors": (4204688, "e733186968d7e6df"),
-    "offspring": (8391520, "e733186968d7e6df"),
-    "fill": (8437, "e733186968d7e6df"),
-    "adjacent_difference": (4198432, "e733186968d7e6df"),
-    "sidecar": (8394167, "c46523a1c822c284")}
+    "permute": (8398575, "51b550508569d7d7"),
+    "metropolis_f32": (8398176, "84cbf3f6b0dd19a7"),
+    "metropolis_f64": (16797184, "84cbf3f6b0dd19a7"),
+    "fused_multinomial_f64": (8528384, "7f0f7fee292ba9e8"),
+    "rejection_f64": (8428434, "84cbf3f6b0dd19a7"),
+    "fused_stratified_f64": (8517193, "7f0f7fee292ba9e8"),
+    "permute_sorted": (4332877, "51b550508569d7d7"),
+    "rejection_f32": (4220768, "84cbf3f6b0dd19a7"),
+    "fused_systematic_f64": (8511195, "7f0f7fee292ba9e8"),
+    "fused_multinomial_f32": (4280256, "7f0f7fee292ba9e8"),
+    "iscan": (4214672, "51b550508569d7d7"),
+    "fused_stratified_f32": (4265664, "7f0f7fee292ba9e8"),
+    "search_f32": (12589152, "76b91365ace2aac1"),
+    "fused_systematic_f32": (4261824, "7f0f7fee292ba9e8"),
+    "search_f64": (16782043, "76b91365ace2aac1"),
+    "offspring": (8391440, "51b550508569d7d7"),
+    "cumoff_to_ancestors": (4206880, "51b550508569d7d7"),
+    "fill": (8682, "51b550508569d7d7"),
+    "adjacent_difference": (4198368, "51b550508569d7d7"),
+    "sidecar": (8394167, "84cbf3f6b0dd19a7")}
 
 _LABEL_FILES = (("fused_", "fused.cu"), ("permute", "aux.cu"), ("iscan", "aux.cu"),
                 ("fill", "aux.cu"), ("offspring", "aux.cu"), ("adjacent", "aux.cu"),
