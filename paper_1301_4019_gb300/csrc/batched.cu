@@ -31,39 +31,18 @@
 #include "internal.h"
 #include "mcmc.cuh"
 #include "permute.cuh"
+#include "ragged.cuh"
 #include "tile.cuh"
 #include "values.cuh"
 
 namespace rsk {
 namespace {
 
-// Particle g of the batch -> (filter f, its first particle lo, its size n, local index i).
-// Returns false for positions past offsets[F] and for filters the plan rejected.
-struct PartLoc {
-  int f;
-  int64_t lo, n, i;
-};
-__device__ __forceinline__ int filter_of(const int64_t* __restrict__ off, int F, int64_t g);
+// locate_in with the filter of position g looked up; false for positions past offsets[F].
 __device__ __forceinline__ bool locate_particle(const int64_t* __restrict__ off, int F,
                                                 int64_t max_n, int64_t g, PartLoc& P) {
   if (g >= __ldg(off + F)) return false;
-  P.f = filter_of(off, F, g);
-  P.lo = __ldg(off + P.f);
-  const int64_t hi = __ldg(off + P.f + 1);
-  P.n = hi - P.lo;
-  P.i = g - P.lo;
-  return P.lo >= 0 && hi <= max_n && P.n > 0 &&
-         P.n <= kBatchMaxN && P.i >= 0 && P.i < P.n;
-}
-
-// Filter holding global position g: the last f with off[f] <= g (off has F + 1 entries).
-__device__ __forceinline__ int filter_of(const int64_t* __restrict__ off, int F, int64_t g) {
-  int lo = 0, hi = F;  // invariant: off[lo] <= g < off[hi]
-  while (hi - lo > 1) {
-    const int mid = (lo + hi) >> 1;
-    if (__ldg(off + mid) <= g) lo = mid; else hi = mid;
-  }
-  return lo;
+  return locate_in(off, filter_of(off, F, g), max_n, g, P);
 }
 
 // filter_of for one position g, by a whole warp (every lane calls it with the same g): 32
@@ -92,18 +71,6 @@ __device__ __forceinline__ int advance_filter(const int64_t* __restrict__ off, i
     ++f;
   }
   return (f + 1 < F && __ldg(off + f + 1) <= g) ? filter_of(off, F, g) : f;
-}
-
-// locate_particle for position g < off[F] once its filter f is known.
-__device__ __forceinline__ bool locate_in(const int64_t* __restrict__ off, int f, int64_t max_n,
-                                          int64_t g, PartLoc& P) {
-  P.f = f;
-  P.lo = __ldg(off + f);
-  const int64_t hi = __ldg(off + f + 1);
-  P.n = hi - P.lo;
-  P.i = g - P.lo;
-  return P.lo >= 0 && hi <= max_n && P.n > 0 &&
-         P.n <= kBatchMaxN && P.i >= 0 && P.i < P.n;
 }
 
 // Tile t of the batch -> its filter (the last f with tile_start[f] <= t).
@@ -827,25 +794,14 @@ batch_chain_kernel(const float* __restrict__ lw, const int64_t* __restrict__ off
     int f = sh_f[0], i = sh_i[0];
     const int fe = sh_f[1], ie = sh_i[1];
     while (f < fe || (f == fe && i < ie)) {  // one window of filters (uniform over the CTA)
-      const int64_t lo = __ldg(off + f), n = __ldg(off + f + 1) - lo;
       if (__ldg(work + f + 1) == __ldg(work + f)) {  // empty or malformed: no particles
         ++f;
         i = 0;
         continue;
       }
-      // the last filter f1 of the window: whole filters while they fit, up to the chunk's end
-      int f1 = f;
-      {
-        int hi = ie > 0 ? fe : fe - 1;  // (the last filter with particles of this chunk)
-        while (f1 < hi) {
-          const int mid = (f1 + hi + 1) >> 1;
-          const int64_t e = __ldg(off + mid + 1), len = e - lo;
-          if (len <= kChainCap && len >= n && e <= total) f1 = mid; else hi = mid - 1;
-        }
-      }
-      const int64_t len = __ldg(off + f1 + 1) - lo;
-      const bool whole = len <= kChainCap;
-      const int staged = static_cast<int>(whole ? len : kChainCap);
+      const ChainWindow w = chain_window(off, total, f, i, fe, ie, kChainCap);
+      const int64_t lo = w.lo;
+      const int f1 = w.f1, staged = w.staged;
       const int pad = static_cast<int>(lo & 3);  // shared index = particle - lo + pad
       __syncthreads();  // (the previous window has been read)
       if (threadIdx.x == 0) sh_group = 0u;
@@ -861,7 +817,7 @@ batch_chain_kernel(const float* __restrict__ lw, const int64_t* __restrict__ off
         for (int e = threadIdx.x; e < staged; e += kChainBlock) sh_lw[e + pad] = __ldg(lw + lo + e);
       }
       __syncthreads();
-      const int64_t ps = lo + i, pe = f1 == fe ? __ldg(off + fe) + ie : lo + len;
+      const int64_t ps = w.ps, pe = w.pe;
       for (;;) {
         unsigned int grp = 0;
         if (lane == 0) grp = atomicAdd(&sh_group, 1u);
@@ -877,7 +833,7 @@ batch_chain_kernel(const float* __restrict__ lw, const int64_t* __restrict__ off
             const uint32_t un = static_cast<uint32_t>(P.n), ui = static_cast<uint32_t>(P.i);
             const float* const sw = sh_lw + (pad + static_cast<int>(P.lo - lo));
             int32_t k = static_cast<int32_t>(P.i);  // (not resampled: keeps its particle)
-            if (resampled(flags, ff)) {
+            if (resampled(flags, ff) && in_window(w, P)) {
               const int32_t Bv = filter_steps(Bf, B, ff);
               const Keys keys = with_tag(base_keys, static_cast<uint32_t>(ff), RS_METROPOLIS);
               const float lwi = __ldg(lw + g);
@@ -887,8 +843,8 @@ batch_chain_kernel(const float* __restrict__ lw, const int64_t* __restrict__ off
               auto part = [&](uint32_t j) {
                 return j < static_cast<uint32_t>(kChainCap) ? sw[j] : __ldg(lf + j);
               };
-              k = whole ? metropolis_chain<true, kChainBlocks>(lwi, all, un, Bv, keys, ui)
-                        : metropolis_chain<true, kChainBlocks>(lwi, part, un, Bv, keys, ui);
+              k = w.whole ? metropolis_chain<true, kChainBlocks>(lwi, all, un, Bv, keys, ui)
+                          : metropolis_chain<true, kChainBlocks>(lwi, part, un, Bv, keys, ui);
             }
             a[g] = k;
             if (d) atomicMin(d + P.lo + k, static_cast<int32_t>(P.i));

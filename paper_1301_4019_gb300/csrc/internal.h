@@ -51,7 +51,6 @@ inline void trace_mark(Trace* t, const char* label, cudaStream_t st) {
   }
 }
 
-constexpr int64_t kBatchMaxN = 1 << 20;  // particles of one filter of a batched call, at most
 
 // Launch shape of a particle-parallel batched kernel: threads per CTA and particles per thread
 // (rs_set_batched_launch / rs_tune_batched). The results never depend on it.
