@@ -167,7 +167,9 @@ int rs_resample_rejection_estimated(rs_handle* h, int dtype, const void* logw_de
 /* Many independent filters in one launch. F filters in CSR layout: offsets_dev holds F + 1
  * int64 offsets (device), filter f owning the particles offsets[f] .. offsets[f+1]-1 of
  * logw_dev and ancestors_dev; every filter has at most 2^20 particles (empty filters are
- * skipped) and offsets[F] <= the handle's max_n (violations: RS_ERR_ARG via rs_last_error).
+ * skipped), offsets ascend and offsets[F] <= the handle's max_n (violations: RS_ERR_ARG via
+ * rs_last_error; a batch whose offsets descend is left without valid ancestors, and nothing beyond
+ * offsets[F] is read or written).
  * ancestors_dev receives, for each filter, local ancestor indices 0..N_f-1. B_dev: NULL
  * (every filter uses B) or F int32 Metropolis step counts. The filter index f is the filter
  * of the random-number counter, so filter f equals rs_resample on its slice with

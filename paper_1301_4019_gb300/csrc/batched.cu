@@ -38,11 +38,19 @@
 namespace rsk {
 namespace {
 
-// locate_in with the filter of position g looked up; false for positions past offsets[F].
+// locate_in with the filter of position g looked up; false for positions past the batch's end.
 __device__ __forceinline__ bool locate_particle(const int64_t* __restrict__ off, int F,
                                                 int64_t max_n, int64_t g, PartLoc& P) {
-  if (g >= __ldg(off + F)) return false;
-  return locate_in(off, filter_of(off, F, g), max_n, g, P);
+  const int64_t end = batch_end(off, F, max_n);
+  return g < end && locate_in(off, filter_of(off, F, g), end, g, P);
+}
+
+// Flags descending offsets (the per-particle schemes, whose kernels look every particle's filter
+// up themselves and stay inside it).
+__device__ __forceinline__ void flag_descending(const int64_t* __restrict__ off, int F, int* err) {
+  const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
+  for (int64_t f = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; f < F; f += stride)
+    if (descends(off, static_cast<int>(f))) flag_error(err, RS_ERR_ARG);
 }
 
 // filter_of for one position g, by a whole warp (every lane calls it with the same g): 32
@@ -98,6 +106,7 @@ struct Batch {
   double2* P_rec;        // tile prefixes, filter f at tile_start[f] + f
   const uint8_t* resample;  // F flags (0: the filter keeps its particles), or null = all
   uint8_t* cl;           // claimed bits (filter f's bytes at (off[f] >> 3) + f), or null
+  int32_t* limit;        // set by the plan: the batch's end, 0 if its offsets descend
   int* err;
 };
 
@@ -120,27 +129,31 @@ __global__ void __launch_bounds__(1024) batch_plan_kernel(Batch b) {
   const int F = b.F;
   const int chunk = (F + blockDim.x - 1) / blockDim.x;
   const int f0 = min(F, static_cast<int>(threadIdx.x) * chunk), f1 = min(F, f0 + chunk);
-  auto counts = [&](int f, bool flag) -> int2 {  // (tiles, segments) of filter f
-    const int64_t lo = __ldg(b.off + f), hi = __ldg(b.off + f + 1), n = hi - lo;
-    if (!(lo >= 0 && n >= 0 && hi <= b.max_n && n <= kBatchMaxN)) {
-      if (flag) flag_error(b.err, RS_ERR_ARG);
-      return make_int2(0, 0);
-    }
+  const int64_t end = batch_end(b.off, F, b.max_n);
+  auto counts = [&](int f) -> int2 {  // (tiles, segments) of filter f
+    const int64_t n = filter_size(b.off, f, end);
+    if (n < 0) return make_int2(0, 0);
     return make_int2(static_cast<int>((n + kTile - 1) / kTile),
                      static_cast<int>((n + kSeg - 1) / kSeg));
   };
   int2 local = make_int2(0, 0);
   int longest = 0;
+  bool rejected = false, down = false;
   for (int f = f0; f < f1; ++f) {
-    const int2 c = counts(f, true);
+    const int2 c = counts(f);
     local.x += c.x;
     local.y += c.y;
     longest = max(longest, c.y);
     b.fmax[f] = LLONG_MIN;
+    rejected |= filter_size(b.off, f, end) < 0;
+    down |= descends(b.off, f);
   }
+  if (rejected) flag_error(b.err, RS_ERR_ARG);
   __shared__ int sh_longest;
   if (threadIdx.x == 0) sh_longest = 0;
-  __syncthreads();
+  down = __syncthreads_or(down);
+  if (down) local = make_int2(0, 0);
+  if (threadIdx.x == 0) *b.limit = down ? 0 : static_cast<int32_t>(end);
   longest = __reduce_max_sync(0xffffffffu, longest);
   if ((threadIdx.x & 31) == 0) atomicMax(&sh_longest, longest);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -164,7 +177,8 @@ __global__ void __launch_bounds__(1024) batch_plan_kernel(Batch b) {
   for (int f = f0; f < f1; ++f) {
     b.tile_start[f] = p.x;
     b.seg_start[f] = p.y;
-    const int2 c = counts(f, false);
+    if (down) continue;
+    const int2 c = counts(f);
     p.x += c.x;
     p.y += c.y;
   }
@@ -625,13 +639,13 @@ batch_search_kernel(const V* __restrict__ W, Batch b, int64_t total, Keys base_k
 // locate_in rejects get nothing.
 constexpr int kFillPer = 8;
 __device__ __forceinline__ void fill_sentinels_warp(const int64_t* __restrict__ off, int F,
-                                                    int64_t total, int64_t end, int64_t gw,
+                                                    int64_t end, int64_t gw,
                                                     int32_t* __restrict__ d) {
   if (gw >= end) return;  // (uniform over the warp)
   int f = filter_of_warp(off, F, gw);
   const int64_t g0 = gw + kFillPer * static_cast<int64_t>(threadIdx.x & 31);
   PartLoc P;
-  if (locate_in(off, f, total, gw, P) && P.i + 32 * kFillPer <= P.n && gw + 32 * kFillPer <= end &&
+  if (locate_in(off, f, end, gw, P) && P.i + 32 * kFillPer <= P.n && gw + 32 * kFillPer <= end &&
       (reinterpret_cast<uintptr_t>(d + g0) & 15u) == 0) {
     const int32_t n = static_cast<int32_t>(P.n);
     int4* const p4 = reinterpret_cast<int4*>(d + g0);
@@ -643,7 +657,7 @@ __device__ __forceinline__ void fill_sentinels_warp(const int64_t* __restrict__ 
     const int64_t g = g0 + q;
     if (g >= end) break;
     f = advance_filter(off, F, g, f);
-    if (locate_in(off, f, total, g, P)) d[g] = static_cast<int32_t>(P.n);
+    if (locate_in(off, f, end, g, P)) d[g] = static_cast<int32_t>(P.n);
   }
 }
 
@@ -663,43 +677,47 @@ __device__ __forceinline__ unsigned long long particle_work(const uint8_t* flags
                              : 2ull;
 }
 
-// Plan of the batched chains (CTA 0): the exclusive prefix over the filters of their work,
-// work[0 .. F], and the chunk counter reset; malformed filters and negative B are flagged and
-// get no work. The other CTAs (every CTA when work is null) write the claims' sentinels (d given).
+// Plan of the per-particle schemes (CTA 0): the batch's end (limit: 0 if its offsets descend) and, with work
+// given (the staged chains), the exclusive prefix over the filters of their work, work[0 .. F], and
+// the chunk counter reset; rejected filters and negative B are flagged and get no work. The other
+// CTAs write the claims' sentinels (d given).
 constexpr int kChainBlock = 1024;
 __global__ void __launch_bounds__(kChainBlock)
 batch_chain_plan_kernel(const int64_t* __restrict__ off, int F, int64_t total,
                         const int32_t* __restrict__ Bf, int32_t B,
                         const uint8_t* __restrict__ flags, unsigned long long* work,
-                        unsigned int* counter, int32_t* __restrict__ d, int* err) {
+                        unsigned int* counter, int32_t* __restrict__ d, int32_t* limit, int* err) {
   pdl_wait();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int planners = work ? 1 : 0;
-  if (static_cast<int>(blockIdx.x) >= planners) {
-    const int64_t offF = __ldg(off + F);
-    const int64_t end = offF < total ? offF : total;
-    const int64_t warps = static_cast<int64_t>(gridDim.x - planners) * (kChainBlock / 32);
-    for (int64_t w = static_cast<int64_t>(blockIdx.x - planners) * (kChainBlock / 32) + warp;
+  const int64_t end = batch_end(off, F, total);
+  if (blockIdx.x > 0) {
+    const int64_t warps = static_cast<int64_t>(gridDim.x - 1) * (kChainBlock / 32);
+    for (int64_t w = static_cast<int64_t>(blockIdx.x - 1) * (kChainBlock / 32) + warp;
          w * (32 * kFillPer) < end; w += warps)
-      fill_sentinels_warp(off, F, total, end, w * (32 * kFillPer), d);
+      fill_sentinels_warp(off, F, end, w * (32 * kFillPer), d);
     return;
   }
   __shared__ unsigned long long sh[kChainBlock / 32];
   const int chunk = (F + kChainBlock - 1) / kChainBlock;
   const int f0 = min(F, static_cast<int>(threadIdx.x) * chunk), f1 = min(F, f0 + chunk);
-  auto filter_work = [&](int f) -> unsigned long long {
-    const int64_t lo = __ldg(off + f), hi = __ldg(off + f + 1), n = hi - lo;
-    if (!(lo >= 0 && n >= 0 && hi <= total && n <= kBatchMaxN)) return ~0ull;
-    return static_cast<unsigned long long>(n) * particle_work(flags, Bf, B, f);
+  auto filter_work = [&](int f) -> unsigned long long {  // (~0: rejected)
+    const int64_t n = filter_size(off, f, end);
+    return n < 0 ? ~0ull : static_cast<unsigned long long>(n) * particle_work(flags, Bf, B, f);
   };
   unsigned long long local = 0;
+  bool down = false, rejected = false;
   for (int f = f0; f < f1; ++f) {
+    down |= descends(off, f);
+    if (!work) continue;  // (the other kernels check the filter of each of their particles)
     const unsigned long long w = filter_work(f);
-    if (w == ~0ull) flag_error(err, RS_ERR_ARG);
-    else local += w;
-    if (resampled(flags, f) && (Bf ? __ldg(Bf + f) : B) < 0 && w != ~0ull && w > 0)
-      flag_error(err, RS_ERR_ARG);
+    if (w != ~0ull) local += w;
+    rejected |= w == ~0ull || (w > 0 && resampled(flags, f) && (Bf ? __ldg(Bf + f) : B) < 0);
   }
+  if (rejected) flag_error(err, RS_ERR_ARG);
+  down = __syncthreads_or(down);
+  if (threadIdx.x == 0) *limit = down ? 0 : static_cast<int32_t>(end);
+  if (!work) return;
+  if (down) local = 0;
   unsigned long long incl = local;
 #pragma unroll
   for (int dd = 1; dd < 32; dd <<= 1) {
@@ -713,7 +731,7 @@ batch_chain_plan_kernel(const int64_t* __restrict__ off, int F, int64_t total,
   for (int f = f0; f < f1; ++f) {
     work[f] = p;
     const unsigned long long w = filter_work(f);
-    if (w != ~0ull) p += w;
+    if (w != ~0ull && !down) p += w;
   }
   if (f1 == F && f0 < F) work[F] = p;
   if (threadIdx.x == 0) *counter = 0u;
@@ -761,9 +779,8 @@ batch_chain_kernel(const float* __restrict__ lw, const int64_t* __restrict__ off
   // chunks: four turns of the CTA's threads each where there are (one turn: 243 against 175 us for
   // 150 filters of 256 .. 65536, the chunks of the highest B too few chains for the CTA), at
   // least one per CTA
-  const int64_t offF = __ldg(off + F);
   const unsigned long long G = gridDim.x;
-  unsigned long long K = static_cast<unsigned long long>(offF < total ? offF : total) / (4 * kChainBlock);
+  unsigned long long K = static_cast<unsigned long long>(batch_end(off, F, total)) / (4 * kChainBlock);
   K = K < G ? G : K > kChainChunks * G ? kChainChunks * G : K;
   const bool tapered = K >= 8 * G;  // (fewer chunks: all alike)
   const unsigned long long K1 = tapered ? K / 2 : K, W1 = tapered ? W / 10 * 9 : W;
@@ -873,6 +890,7 @@ batch_mcmc_kernel(const T* __restrict__ lw, const int64_t* __restrict__ off, int
                   const uint8_t* __restrict__ flags, int32_t* __restrict__ a,
                   int32_t* __restrict__ d, int ipt, int* err) {
   pdl_wait();
+  flag_descending(off, F, err);
   for (int q = 0; q < ipt; ++q) {
     const int64_t g = item_index(ipt, q);
     if (g >= total) return;
@@ -911,7 +929,8 @@ batch_rejection_kernel(const T* __restrict__ lw, const int64_t* __restrict__ off
   const int lane = threadIdx.x & 31;
   const int64_t run = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
   const int64_t start = run * run_len;
-  const int64_t limit = __ldg(off + F) < total ? __ldg(off + F) : total;
+  const int64_t limit = batch_end(off, F, total);
+  flag_descending(off, F, err);
   if (start >= limit) return;  // uniform across the warp
   const int64_t end = start + run_len < limit ? start + run_len : limit;
   const RejBound rb = make_bound(log_wmax);
@@ -1014,14 +1033,14 @@ template <bool SORTED, int K>
 __global__ void __launch_bounds__(kMaxTunedBlock)
 batch_permute_kernel(const int64_t* __restrict__ off, int F, int64_t total,
                      const int32_t* __restrict__ a, const int32_t* __restrict__ d,
-                     const uint8_t* __restrict__ cl, int32_t* __restrict__ c, int ipt, int* err) {
+                     const uint8_t* __restrict__ cl, int32_t* __restrict__ c, int ipt,
+                     const int32_t* limit, int* err) {
   pdl_wait();
   extern __shared__ __align__(16) unsigned char sh_perm[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   int32_t* const cw = reinterpret_cast<int32_t*>(sh_perm + warp * perm_smem_per_warp<K>());
   int2* const pend = reinterpret_cast<int2*>(cw + 32 * K);
-  const int64_t offF = __ldg(off + F);
-  const int64_t end = offF < total ? offF : total;
+  const int64_t end = __ldg(limit);  // (0: the offsets descend, no ancestors were formed)
   for (int q = 0; q < ipt; ++q) {
     // first slot of this warp (of this lane: K * lane further)
     const int64_t gw = K * ((static_cast<int64_t>(blockIdx.x) * ipt + q) * blockDim.x +
@@ -1197,9 +1216,9 @@ cudaError_t launch_batched(const Scratch& s, int scheme, Acc acc, const void* lo
     auto* work = reinterpret_cast<unsigned long long*>(s.batch_fS);  // F + 1 <= 2 max_filters
     if (d || staged) {
       trace_mark(s.trace, "batch_fill", st);
-      launch_pdl(batch_chain_plan_kernel, (staged ? 1 : 0) + (d ? fill_grid(total) : 0),
-                 kChainBlock, st, offsets, F, total, Bf, B, flags, staged ? work : nullptr,
-                 &s.glob->batch_next, d, s.err);
+      launch_pdl(batch_chain_plan_kernel, 1 + (d ? fill_grid(total) : 0), kChainBlock, st, offsets,
+                 F, total, Bf, B, flags, staged ? work : nullptr, &s.glob->batch_next, d,
+                 &s.glob->batch_limit, s.err);
     }
     trace_mark(s.trace, scheme == RS_METROPOLIS ? (f64 ? "batch_metropolis_f64" : "batch_metropolis_f32")
                                                 : (f64 ? "batch_rejection_f64" : "batch_rejection_f32"),
@@ -1247,6 +1266,7 @@ cudaError_t launch_batched(const Scratch& s, int scheme, Acc acc, const void* lo
     b.P_rec = s.batch_P_rec;
     b.resample = flags;
     b.cl = cl;
+    b.limit = &s.glob->batch_limit;
     b.err = s.err;
     trace_mark(s.trace, "batch_plan", st);
     launch_pdl(batch_plan_kernel, 1, 1024, st, b);
@@ -1280,7 +1300,8 @@ cudaError_t launch_batched(const Scratch& s, int scheme, Acc acc, const void* lo
     const size_t smem = (four ? perm_smem_per_warp<4>() : perm_smem_per_warp<1>()) * (c.block / 32);
     launch_pdl_smem(cl ? (four ? batch_permute_kernel<true, 4> : batch_permute_kernel<true, 1>)
                        : (four ? batch_permute_kernel<false, 4> : batch_permute_kernel<false, 1>),
-                    grid, c.block, smem, st, offsets, F, total, s.a_tmp, s.d, cl, out, c.ipt, s.err);
+                    grid, c.block, smem, st, offsets, F, total, s.a_tmp, s.d, cl, out, c.ipt,
+                    &s.glob->batch_limit, s.err);
     e = cudaGetLastError();
   }
   return e;

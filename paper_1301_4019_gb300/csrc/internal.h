@@ -22,7 +22,7 @@ struct ScanGlob {
   unsigned int ticket_max;   // last-CTA counters (self-resetting)
   unsigned int ticket_tile;
   unsigned int ticket_iscan;
-  unsigned int batch_next;   // work counter of the batched kernel (self-resetting)
+  unsigned int batch_next;   // work counter of the batched chains (set by their plan)
   unsigned int ess_ticket;   // CTAs of the ESS kernels that have finished (self-resetting)
   unsigned long long ess_key;  // maximum log-weight of an ESS kernel, ordered key (self-resetting)
   unsigned long long scan_key;  // the same of a cooperative scan (self-resetting)
@@ -30,7 +30,9 @@ struct ScanGlob {
   int all_zero;              // every weight of the call is zero (set with the total)
   float guide_step;          // W^N / N and N / W^N in binary32 (multinomial guide table),
   float guide_inv_step;      //   set with the total so that no later kernel divides
-  unsigned int pad[3];
+  int32_t batch_limit;       // end of the batch's particles, 0 if its offsets descend (set by the
+                             //   batch's plan, read by its Permute)
+  unsigned int pad[2];
   double2 S_raw;             // total, in the accumulator type of the call
   double2 scale_raw;         // N / total, in the accumulator type of the call
 };

@@ -41,15 +41,35 @@ RSK_BOTH int filter_of(const int64_t* __restrict__ off, int F, int64_t g) {
   return lo;
 }
 
-// Position g in filter f; false for filters that the plan rejects and positions outside them.
-RSK_BOTH bool locate_in(const int64_t* __restrict__ off, int f, int64_t max_n, int64_t g,
+// One past the last position that a filter may hold: off[F], at most the handle's max_n.
+RSK_BOTH int64_t batch_end(const int64_t* __restrict__ off, int F, int64_t max_n) {
+  const int64_t e = ld_ro(off + F);
+  return e < max_n ? e : max_n;
+}
+
+// Particles of filter f, -1 for one that is rejected (RS_ERR_ARG): it begins before 0, ends past
+// the batch's end or is too long. (No two accepted filters share a position, and together they hold
+// at most `end` particles, exactly if no offset is below the one before it: see descends.)
+RSK_BOTH int64_t filter_size(const int64_t* __restrict__ off, int f, int64_t end) {
+  const int64_t lo = ld_ro(off + f), hi = ld_ro(off + f + 1), n = hi - lo;
+  return lo >= 0 && n >= 0 && hi <= end && n <= kBatchMaxN ? n : -1;
+}
+
+// An offset below the one before it: the filters then overlap, and their tiles and segments can
+// outnumber the scratch. The plans give such a batch no work.
+RSK_BOTH bool descends(const int64_t* __restrict__ off, int f) {
+  return ld_ro(off + f + 1) < ld_ro(off + f);
+}
+
+// Position g in filter f; false for filters that are rejected and positions outside them.
+RSK_BOTH bool locate_in(const int64_t* __restrict__ off, int f, int64_t end, int64_t g,
                         PartLoc& P) {
   P.f = f;
   P.lo = ld_ro(off + f);
   const int64_t hi = ld_ro(off + f + 1);
   P.n = hi - P.lo;
   P.i = g - P.lo;
-  return P.lo >= 0 && hi <= max_n && P.n > 0 && P.n <= kBatchMaxN && P.i >= 0 && P.i < P.n;
+  return P.lo >= 0 && hi <= end && P.n > 0 && P.n <= kBatchMaxN && P.i >= 0 && P.i < P.n;
 }
 
 // Window of the staged chains (batch_chain_kernel): from position i of filter f, the filters
@@ -62,7 +82,7 @@ struct ChainWindow {
   int staged;
   int64_t lo, len, ps, pe;
 };
-RSK_BOTH ChainWindow chain_window(const int64_t* __restrict__ off, int64_t total, int f, int i,
+RSK_BOTH ChainWindow chain_window(const int64_t* __restrict__ off, int64_t end, int f, int i,
                                   int fe, int ie, int cap) {
   ChainWindow w;
   w.lo = ld_ro(off + f);
@@ -72,7 +92,7 @@ RSK_BOTH ChainWindow chain_window(const int64_t* __restrict__ off, int64_t total
   while (w.f1 < hi) {
     const int mid = (w.f1 + hi + 1) >> 1;
     const int64_t e = ld_ro(off + mid + 1), len = e - w.lo;
-    if (len <= cap && len >= n && e <= total) w.f1 = mid; else hi = mid - 1;
+    if (len <= cap && len >= n && e <= end) w.f1 = mid; else hi = mid - 1;
   }
   w.len = ld_ro(off + w.f1 + 1) - w.lo;
   w.whole = w.len <= cap;

@@ -1,6 +1,7 @@
-// The staged chains' index arithmetic (csrc/ragged.cuh) on the host: the windows of one chunk of
-// a batch are taken as a CTA of the batched Metropolis kernel takes them, and every index that
-// its chains may form is checked against the staged and the global range.
+// The ragged batches' index arithmetic (csrc/ragged.cuh) on the host. chain_chunk: the windows of one
+// chunk of a batch are taken as a CTA of the batched Metropolis kernel takes them, and every index
+// that its chains may form is checked against the staged and the global range. batch_sizes: the
+// filters' sizes as the plans accept them.
 #include "ragged.cuh"
 
 using namespace rsk;
@@ -41,4 +42,20 @@ extern "C" int chain_chunk(const int64_t* off, int F, int64_t total, const int64
     i = 0;
   }
   return 0;
+}
+
+// n[f]: particles of filter f that the plan gives work, 0 for a rejected one or a void batch;
+// returns 1 if the call is to be reported, +2 if the batch is void.
+extern "C" int batch_sizes(const int64_t* off, int F, int64_t max_n, int64_t* n) {
+  const int64_t end = batch_end(off, F, max_n);
+  bool down = false, rejected = false;
+  for (int f = 0; f < F; ++f) {
+    n[f] = filter_size(off, f, end);
+    rejected |= n[f] < 0;
+    down |= descends(off, f);
+    if (n[f] < 0) n[f] = 0;
+  }
+  if (down)
+    for (int f = 0; f < F; ++f) n[f] = 0;
+  return (rejected ? 1 : 0) + (down ? 2 : 0);
 }

@@ -30,3 +30,29 @@ def test_one_wrong_offset_is_reported(rs, shift):
         again = rs.rs_resample_batched(h, rs.METROPOLIS, t, good, B=16, seed=3)
         assert rs.rs_last_error(h) == rs.RS_OK
         assert torch.equal(want, again)
+
+
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+@pytest.mark.parametrize("scheme", range(5))
+def test_descending_offsets_write_nothing_past_the_last(rs, scheme, dtype):
+    """Offsets that run ahead of offsets[F] and fall back, and ones that give every second filter
+    the whole batch (more tiles than the scratch holds): RS_ERR_ARG with and without Permute and in
+    both launch modes, nothing written past offsets[F], and the next call is right."""
+    n = 20000
+    good = torch.tensor([0, 300, 9000, n], dtype=torch.int64, device=DEV)
+    ahead = torch.tensor([0, 300, 19000, 9000, 12000], dtype=torch.int64, device=DEV)
+    many = torch.tensor([0, n] * 500 + [0, 12000], dtype=torch.int64, device=DEV)
+    t = torch.from_numpy(workload.synthetic_logw(n, 2.0, seed=1, dtype=dtype)).to(DEV)
+    with rs.Handle(n) as h:
+        for mode in (rs.LAUNCH_AUTO, rs.LAUNCH_SEPARATE):
+            rs.rs_set_launch_mode(h, mode)
+            for permute in (False, True):
+                want = rs.rs_resample_batched(h, scheme, t, good, B=5, seed=1, permute=permute)
+                assert rs.rs_last_error(h) == rs.RS_OK
+                for off in (ahead, many):
+                    out = torch.full((n,), -7, dtype=torch.int32, device=DEV)
+                    rs.rs_resample_batched(h, scheme, t, off, B=5, seed=1, permute=permute, out=out)
+                    assert rs.rs_last_error(h) == rs.RS_ERR_ARG
+                    assert bool((out[12000:] == -7).all())
+                got = rs.rs_resample_batched(h, scheme, t, good, B=5, seed=1, permute=permute)
+                assert rs.rs_last_error(h) == rs.RS_OK and torch.equal(got, want)

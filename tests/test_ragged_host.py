@@ -1,7 +1,9 @@
-"""CPU test of the batched Metropolis kernel's staged windows (csrc/ragged.cuh): with ascending
-offsets every particle is run once, from staged values where its filter fits; with offsets that
-descend, overlap or leave the batch (which the call reports as RS_ERR_ARG) no index that a chain
-may form leaves the staged values or the log-weights."""
+"""CPU test of the ragged batches' index arithmetic (csrc/ragged.cuh). The staged windows of the
+batched Metropolis kernel: with ascending offsets every particle is run once, from staged values
+where its filter fits; with offsets that descend, overlap or leave the batch (which the call
+reports as RS_ERR_ARG) no index that a chain may form leaves the staged values or the log-weights.
+The plans: whatever the offsets, the accepted filters hold no more than the handle's particles and
+none beyond offsets[F], so tiles and segments fit the scratch."""
 import ctypes as C
 
 import numpy as np
@@ -77,3 +79,27 @@ def test_wide_wrong_offsets_stay_in_range(lib):
         st, _, _ = _run(lib, off, total, rng.integers(0, 60, F), int(rng.integers(1, 20)),
                         cap=int(rng.choice([64, 1000, CAP])))
         assert st == 0, (k, off.tolist())
+
+
+@pytest.mark.parametrize("max_n", [1, 4096, 300000])
+def test_accepted_filters_fit_the_scratch(lib, max_n):
+    rng = np.random.default_rng(max_n)
+    F_max = max(1024, max_n // 16)
+    cases = [np.tile([0, max_n], 600)[:1025],                     # every other filter holds all
+             np.array([0, max_n, max_n // 2]),                     # past offsets[F]
+             np.array([0, 1, max_n + 1, max_n + 2]), np.array([-1, 1, max_n])]
+    cases += [rng.integers(-2, max_n + 3, rng.integers(2, F_max + 1)) for _ in range(50)]
+    cases += [np.sort(rng.integers(0, max_n + 1, rng.integers(2, F_max + 1))) for _ in range(50)]
+    for off in cases:
+        off = off.astype(np.int64)
+        F = off.size - 1
+        n = np.empty(F, np.int64)
+        st = lib.batch_sizes(_ptr(off), F, C.c_int64(max_n), _ptr(n))
+        d = np.diff(off)
+        good = off[0] >= 0 and np.all(d >= 0) and off[-1] <= max_n and np.all(d <= MAX_FILTER)
+        assert (st == 0) == bool(good)
+        assert np.array_equal(n, d) or not good
+        # the scratch holds max_n / 2048 + max_filters + 1 tiles of 8 segments of 256 particles
+        tiles, segs = (n + 2047) // 2048, (n + 255) // 256
+        assert tiles.sum() <= max_n // 2048 + F_max + 1 and segs.sum() <= 8 * (max_n // 2048 + F_max + 1)
+        assert np.all((n == 0) | ((off[:-1] >= 0) & (off[:-1] + n <= min(max_n, off[-1]))))
