@@ -713,6 +713,8 @@ batch_chain_plan_kernel(const int64_t* __restrict__ off, int F, int64_t total,
     if (w != ~0ull) local += w;
     rejected |= w == ~0ull || (w > 0 && resampled(flags, f) && (Bf ? __ldg(Bf + f) : B) < 0);
   }
+  // (positions before the first filter belong to none: the other kernels report them too)
+  if (work && threadIdx.x == 0) rejected |= end > 0 && __ldg(off) > 0;
   if (rejected) flag_error(err, RS_ERR_ARG);
   down = __syncthreads_or(down);
   if (threadIdx.x == 0) *limit = down ? 0 : static_cast<int32_t>(end);

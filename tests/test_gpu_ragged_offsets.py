@@ -56,3 +56,22 @@ def test_descending_offsets_write_nothing_past_the_last(rs, scheme, dtype):
                     assert bool((out[12000:] == -7).all())
                 got = rs.rs_resample_batched(h, scheme, t, good, B=5, seed=1, permute=permute)
                 assert rs.rs_last_error(h) == rs.RS_OK and torch.equal(got, want)
+
+
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+def test_first_offset_above_zero(rs, dtype):
+    """Positions before offsets[0] belong to no filter: the per-particle schemes report them,
+    binary32 Metropolis from either of its kernels; the filters' own results are not affected."""
+    n = 5000
+    t = torch.from_numpy(workload.synthetic_logw(n, 2.0, seed=1, dtype=dtype)).to(DEV)
+    off = torch.tensor([3, 1200, n], dtype=torch.int64, device=DEV)
+    kernel = rs.BATCHED_METROPOLIS_F64 if dtype == np.float64 else rs.BATCHED_METROPOLIS_F32
+    with rs.Handle(n) as h:
+        got = []
+        for shape in ((256, 1), (128, 2)):
+            rs.rs_set_batched_launch(h, kernel, *shape)
+            got.append(rs.rs_resample_batched(h, rs.METROPOLIS, t, off, B=9, seed=1))
+            assert rs.rs_last_error(h) == rs.RS_ERR_ARG
+        assert torch.equal(got[0][3:], got[1][3:])
+        rs.rs_resample_batched(h, rs.REJECTION, t, off, seed=1)
+        assert rs.rs_last_error(h) == rs.RS_ERR_ARG
