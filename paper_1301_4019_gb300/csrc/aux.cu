@@ -133,16 +133,18 @@ cumoff_to_ancestors_kernel(const int32_t* __restrict__ O, int64_t N, int32_t* __
   if (j0l >= N) return;  // (warp-uniform: only warp-level synchronisation below)
   const int32_t n = static_cast<int32_t>(N);
   const int32_t j0 = static_cast<int32_t>(j0l);
-  const int32_t i0 = j0 + kPer * lane;
+  const int32_t i0 = at_i32(j0, kPer * lane);
+  const int cnt = seg_count(j0l, N) - kPer * lane;  // valid particles here
+  const bool tail = n - j0 <= kSeg;  // (the sequence's last particle is one of the warp's)
   int32_t Oe[kPer];
-  if (i0 + kPer <= n && (reinterpret_cast<uintptr_t>(O) & 15u) == 0) {
+  if (cnt >= kPer && (reinterpret_cast<uintptr_t>(O) & 15u) == 0) {
     const int4 u0 = __ldg(reinterpret_cast<const int4*>(O + i0));
     const int4 u1 = __ldg(reinterpret_cast<const int4*>(O + i0 + 4));
     Oe[0] = u0.x; Oe[1] = u0.y; Oe[2] = u0.z; Oe[3] = u0.w;
     Oe[4] = u1.x; Oe[5] = u1.y; Oe[6] = u1.z; Oe[7] = u1.w;
   } else {
 #pragma unroll
-    for (int q = 0; q < kPer; ++q) Oe[q] = i0 + q < n ? __ldg(O + i0 + q) : n;
+    for (int q = 0; q < kPer; ++q) Oe[q] = q < cnt ? __ldg(O + i0 + q) : n;
   }
   int32_t prev = __shfl_up_sync(0xffffffffu, Oe[kPer - 1], 1);
   if (lane == 0) prev = j0 > 0 ? __ldg(O + j0 - 1) : 0;
@@ -151,8 +153,8 @@ cumoff_to_ancestors_kernel(const int32_t* __restrict__ O, int64_t N, int32_t* __
     int32_t p = prev;
 #pragma unroll
     for (int q = 0; q < kPer; ++q) {
-      if (i0 + q < n)
-        bad |= p < 0 || Oe[q] < p || Oe[q] > n || (i0 + q == n - 1 && Oe[q] != n);
+      if (q < cnt)
+        bad |= p < 0 || Oe[q] < p || Oe[q] > n || (tail && q + 1 == cnt && Oe[q] != n);
       p = Oe[q];
     }
     // clamped into [0, n] and made non-decreasing within the lane, then across the warp

@@ -11,6 +11,7 @@
 
 #include "common.cuh"
 #include "dfexp.cuh"
+#include "runs.cuh"
 #include "values.cuh"
 
 namespace rsk {
@@ -221,14 +222,7 @@ template <> __device__ __forceinline__ float2 load_v_cg<float2>(const double2* p
 
 // Particles of a tile: thread t holds the kPer consecutive offsets kPer t .. kPer t + kPer - 1,
 // so warp w holds 32 kPer consecutive particles and the tile kTile = kBlock kPer.
-// A segment is the kSeg = 32 kPer particles of one warp (lane l holds kPer l .. kPer l + kPer - 1).
-// Its valid particles in a sequence ending at N: offsets 0 .. count - 1 (zero or negative past
-// the end).
-constexpr int kSeg = 32 * kPer;
-__device__ __forceinline__ int seg_count(int64_t base, int64_t N) {
-  const int64_t c = N - base;
-  return c < kSeg ? static_cast<int>(c) : kSeg;
-}
+// (segments of kSeg = 32 kPer particles: see runs.cuh).
 
 // Maximum and minimum of non-negative accumulator values (exact; binary32: one instruction;
 // binary64: by the bit pattern, which orders like the value, off the binary64 pipe). A NaN (from
@@ -730,134 +724,9 @@ __device__ void seg_prefix_compute(const double2* s_rec, double2* P_rec, int nt,
 }
 
 // Shared scratch of the segment emissions: one warp_runs window per warp.
-constexpr int kRunSpan = 2 * kRunWin;  // positions of a window
 struct SegSh {
   alignas(16) int32_t win[kWarps][kRunSpan];
 };
-
-// Eight consecutive values to a 32-byte aligned address (one whole sector).
-__device__ __forceinline__ void st_global_v8(int32_t* p, const int32_t (&v)[kPer]) {
-  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(v[0]),
-               "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
-               : "memory");
-}
-
-// Code 11 for the particles of one warp: out[j] = the index of the particle whose run
-// [O_{i-1}, O_i) holds j, for every j of the warp's range [P0, P1) (P0 = the count before the
-// warp's first particle, P1 = after its last). Lane l holds the non-decreasing counts Oe[q] of
-// its kPer particles i0 + q and `prev`, the count before them. Returns the bits of this lane's
-// particles that have a run (bit q: particle i0 + q).
-//
-// The range is written through the warp's shared window of kRunSpan positions (nearly always
-// one: a segment's kSeg particles have about kSeg offspring): -1 everywhere, then the first
-// position of each run receives its particle's index; the window is read back, eight consecutive
-// positions per lane, and filled by a running maximum (in-lane; then the last head before the
-// lane, found by ballot; or the last value of the part before, which every lane takes into
-// account: a run can cover a whole part). Windows start at 32-byte boundaries of `out`, so a
-// lane's eight positions are one 256-bit store; the two groups of eight that the range's ends
-// cut are written back and stored by sixteen lanes. A short rest beyond the first 256 positions
-// (half of the segments have one, mostly under 32 positions) is read two positions per lane.
-// The first position P0 always starts a run, so the carry of the first part can be -1.
-//
-// Every head lies in [P0, P1): the counts are those of cumulative weights (or of checked counts)
-// that lie between the segment's two prefixes and are non-decreasing functions of them, so one
-// window holds all heads when P1 - base <= kRunSpan; longer ranges test every head.
-// Same result as writing out[j] = i for j in [O_{i-1}, O_i) particle by particle, without its
-// divergent loops.
-__device__ __forceinline__ uint32_t warp_runs(const int32_t (&Oe)[kPer], int32_t prev, int32_t i0,
-                                              int32_t* __restrict__ out, int32_t* win) {
-  static_assert(kPer == 8 && kRunWin == 256, "a lane's positions are one 32-byte sector");
-  const int lane = threadIdx.x & 31;
-  const unsigned below = (1u << lane) - 1u;
-  const int32_t P0 = __shfl_sync(0xffffffffu, prev, 0);
-  const int32_t P1 = __shfl_sync(0xffffffffu, Oe[kPer - 1], 31);
-  const int32_t shift = static_cast<int32_t>((reinterpret_cast<uintptr_t>(out) >> 2) & 7u);
-  int4* const w4 = reinterpret_cast<int4*>(win);
-  uint32_t bits = 0;
-  int32_t carry = -1;
-  // the last head at or before this lane's last position of a part (top: its in-lane maximum)
-  auto before_lane = [&](int32_t top) {
-    const unsigned heads = __ballot_sync(0xffffffffu, top >= 0);
-    const unsigned earlier = heads & below;
-    const int32_t m = __shfl_sync(0xffffffffu, top, 31 - __clz(earlier | 1u));
-    const int32_t em = earlier ? m : carry;
-    const int32_t last = __shfl_sync(0xffffffffu, top, 31 - __clz(heads | 1u));
-    carry = heads ? last : carry;
-    return em;
-  };
-  auto part8 = [&](int h, int32_t base) {  // 256 positions
-    const int4 u0 = w4[64 * h + 2 * lane], u1 = w4[64 * h + 2 * lane + 1];
-    int32_t v[kPer] = {u0.x, u0.y, u0.z, u0.w, u1.x, u1.y, u1.z, u1.w};
-#pragma unroll
-    for (int k = 1; k < kPer; ++k) v[k] = max(v[k], v[k - 1]);
-    const int32_t em = before_lane(v[kPer - 1]);
-#pragma unroll
-    for (int k = 0; k < kPer; ++k) v[k] = max(v[k], em);
-    const int32_t j0 = base + kPer * lane;
-    if (j0 >= P0 && j0 + kPer <= P1) {
-      st_global_v8(out + j0, v);
-    } else if (j0 + kPer > P0 && j0 < P1) {  // cut by an end of the range
-      w4[64 * h + 2 * lane] = make_int4(v[0], v[1], v[2], v[3]);
-      w4[64 * h + 2 * lane + 1] = make_int4(v[4], v[5], v[6], v[7]);
-    }
-  };
-  for (int32_t base = ((P0 + shift) & ~7) - shift; base < P1; base += kRunSpan) {  // warp-uniform
-    const int32_t len = P1 - base;
-    const int4 none = make_int4(-1, -1, -1, -1);
-    __syncwarp();
-    w4[lane] = none;
-    w4[32 + lane] = none;
-    if (len > kRunWin) {
-      w4[64 + lane] = none;
-      w4[96 + lane] = none;
-    }
-    __syncwarp();
-    int32_t p = prev;
-    if (len <= kRunSpan && base <= P0) {
-      int32_t* const wb = win - base;
-#pragma unroll
-      for (int q = 0; q < kPer; ++q) {
-        if (Oe[q] > p) {
-          bits |= 1u << q;
-          wb[p] = i0 + q;
-        }
-        p = Oe[q];
-      }
-    } else {
-#pragma unroll
-      for (int q = 0; q < kPer; ++q) {
-        if (Oe[q] > p) {
-          bits |= 1u << q;
-          const uint32_t pos = static_cast<uint32_t>(p - base);
-          if (pos < static_cast<uint32_t>(kRunSpan)) win[pos] = i0 + q;
-        }
-        p = Oe[q];
-      }
-    }
-    __syncwarp();
-    part8(0, base);
-    int32_t cut = len < kRunSpan ? (len & ~7) : kRunSpan;  // the group that the range's end cuts
-    if (len > kRunWin + 64) {
-      part8(1, base + kRunWin);
-    } else if (len > kRunWin) {  // a short rest: two positions per lane
-      const int2 u = reinterpret_cast<const int2*>(win + kRunWin)[lane];
-      const int32_t top = max(u.x, u.y);
-      const int32_t em = before_lane(top);
-      const int32_t j0 = base + kRunWin + 2 * lane;
-      if (j0 < P1) out[j0] = max(u.x, em);
-      if (j0 + 1 < P1) out[j0 + 1] = max(top, em);
-      cut = kRunSpan;  // (nothing left to store)
-    }
-    __syncwarp();
-    // the groups that the ends cut: the window's first (where it starts before P0), by the first
-    // eight lanes, and the one that holds P1, by the next eight
-    const int idx = lane < kPer ? lane : cut + lane - kPer;
-    if (lane < 2 * kPer && idx < len && idx < kRunSpan && base + idx >= P0 &&
-        (lane >= kPer ? (len & 7) != 0 : base < P0))
-      out[base + idx] = win[idx];
-  }
-  return bits;
-}
 
 // The record of a segment (warp-level) from this lane's kPer log-weights x of it (-inf outside
 // the sequence): m_t = the segment's largest log-weight (NaN skipped; NaN and +inf set `bad`)
@@ -1031,8 +900,9 @@ __device__ __forceinline__ void emit_seg_cumoff(const T* __restrict__ lw, int64_
   const int lane = threadIdx.x & 31;
   const int32_t n = static_cast<int32_t>(N - lo);
   const int32_t b0 = static_cast<int32_t>(base - lo);
+  const bool tail = n - b0 <= kSeg;  // (the sequence's last particle, or positions past it)
   const int cnt = seg_count(base, N) - kPer * lane;  // valid here
-  const int32_t i0 = b0 + kPer * lane;
+  const int32_t i0 = at_i32(b0, kPer * lane);
   V W[kPer], Wb;
   seg_cum_weights<T, V>(lw, lo, N, base, wc, vec, Ps, Pn, W, Wb, hint);
   // O of this lane's particles; the last particle of the sequence gets n, and positions
@@ -1056,18 +926,10 @@ __device__ __forceinline__ void emit_seg_cumoff(const T* __restrict__ lw, int64_
     }
     if (lane == 0 && cnt > 0) Ob = cum_offspring<T, V, STRAT>(Wb, S, scale, u_sys, keys, n);
   }
-  const int32_t last = (cnt >= kPer && i0 + kPer - 1 != n - 1) ? O[kPer - 1] : n;
-  int32_t prev = __shfl_up_sync(0xffffffffu, last, 1);
+  int32_t prev = __shfl_up_sync(0xffffffffu, last_count(O, cnt, tail, n), 1);
   if (lane == 0)  // (a segment wholly past the end follows the sequence's last particle: n)
     prev = Ob;
-  if (b0 + kSeg >= n) {  // (warp-uniform) the sequence's last particle, or positions past it
-    int32_t p = prev;
-#pragma unroll
-    for (int q = 0; q < kPer; ++q) {
-      O[q] = (q >= cnt) ? p : ((i0 + q == n - 1) ? n : O[q]);
-      p = O[q];
-    }
-  }
+  if (tail) end_counts(O, prev, cnt, n);  // (warp-uniform)
   const uint32_t bits = warp_runs(O, prev, i0, a + lo, win);
   // (i0 is a multiple of kPer = 8: one byte per lane)
   if (cl && cnt > 0) cl[i0 >> 3] = static_cast<uint8_t>(bits);
@@ -1185,8 +1047,10 @@ __device__ __forceinline__ void emit_seg_W_guide(const T* __restrict__ lw, int64
                                                  L2Hint hint = L2Hint::kNormal) {
   const int lane = threadIdx.x & 31;
   const int32_t n = static_cast<int32_t>(N - lo);
+  const int32_t b0 = static_cast<int32_t>(base - lo);
+  const bool tail = n - b0 <= kSeg;  // (the sequence's last particle, or positions past it)
   const int cnt = seg_count(base, N) - kPer * lane;
-  const int32_t j0 = static_cast<int32_t>(base - lo) + kPer * lane;
+  const int32_t j0 = at_i32(b0, kPer * lane);
   V W[kPer], Wb;
   seg_cum_weights<T, V>(lw, lo, N, base, wc, vec, Ps, Pn, W, Wb, hint);
   V* const p = Wout + base + kPer * static_cast<int64_t>(lane);
@@ -1198,19 +1062,12 @@ __device__ __forceinline__ void emit_seg_W_guide(const T* __restrict__ lw, int64
   }
   // the guide entries of a particle's buckets form runs like the ancestors of Code 11 (the
   // last particle's run ends at n, positions past the end add none)
-  const int32_t last = (cnt >= kPer && j0 + kPer - 1 != n - 1) ? C[kPer - 1] : n;
-  int32_t prev = __shfl_up_sync(0xffffffffu, last, 1);
+  int32_t prev = __shfl_up_sync(0xffffffffu, last_count(C, cnt, tail, n), 1);
   if (lane == 0) prev = cnt > 0 ? guide_count<V>(Wb, gd, n) : n;
-  int32_t pc = prev;
-#pragma unroll
-  for (int q = 0; q < kPer; ++q) {
-    const int32_t Cc = (q >= cnt) ? pc : ((j0 + q == n - 1) ? n : C[q]);
-    C[q] = Cc;
-    pc = Cc;
-  }
+  if (tail) end_counts(C, prev, cnt, n);  // (warp-uniform)
   int32_t* const Gl = G + lo;
   warp_runs(C, prev, j0, Gl, win);
-  if (j0 <= n - 1 && n - 1 < j0 + kPer) Gl[n] = n - 1;
+  if (tail && cnt >= 1 && cnt <= kPer) Gl[n] = n - 1;  // (the last particle's lane)
 }
 
 // The first j of the non-decreasing W_lo .. W_{hi-1} with W_j > u, hi if none: four are read
