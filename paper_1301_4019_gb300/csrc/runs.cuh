@@ -46,6 +46,37 @@ __device__ __forceinline__ void end_counts(int32_t (&O)[kPer], int32_t prev, int
   }
 }
 
+// Counts of a warp's segment in non-decreasing order between those of its two ends: a count below
+// one before it is raised to it, and none exceeds the last lane's last count. For accumulators
+// whose scaling does not preserve order: two-float products rise and fall by up to 2^-46 relative
+// across a step of the high word, so that W_i < W_j can give r_i > r_j and, with an integer between
+// them, a count one lower. Nearly always the test finds nothing to do.
+__device__ __forceinline__ void order_counts(int32_t (&O)[kPer], int32_t& prev) {
+  bool down = false;
+  int32_t p = prev;
+#pragma unroll
+  for (int q = 0; q < kPer; ++q) {
+    down |= O[q] < p;
+    p = O[q];
+  }
+  if (!__any_sync(0xffffffffu, down)) return;
+  const int lane = threadIdx.x & 31;
+  const int32_t P0 = __shfl_sync(0xffffffffu, prev, 0);
+  const int32_t P1 = max(P0, __shfl_sync(0xffffffffu, O[kPer - 1], 31));
+#pragma unroll
+  for (int q = 1; q < kPer; ++q) O[q] = max(O[q], O[q - 1]);
+  int32_t m = O[kPer - 1];
+#pragma unroll
+  for (int dd = 1; dd < 32; dd <<= 1) {
+    const int32_t y = __shfl_up_sync(0xffffffffu, m, dd);
+    if (lane >= dd) m = max(m, y);
+  }
+  const int32_t before = __shfl_up_sync(0xffffffffu, m, 1);
+  prev = lane == 0 ? P0 : min(max(before, P0), P1);
+#pragma unroll
+  for (int q = 0; q < kPer; ++q) O[q] = min(max(O[q], prev), P1);
+}
+
 // Eight consecutive values to a 32-byte aligned address (one whole sector).
 __device__ __forceinline__ void st_global_v8(int32_t* p, const int32_t (&v)[kPer]) {
 #ifdef __CUDACC__
@@ -74,8 +105,10 @@ __device__ __forceinline__ void st_global_v8(int32_t* p, const int32_t (&v)[kPer
 // (half of the segments have one, mostly under 32 positions) is read two positions per lane.
 // The first position P0 always starts a run, so the carry of the first part can be -1.
 //
-// The counts are non-decreasing from P0 to P1 over the warp, so every head lies in [P0, P1) and
-// one window holds them all when P1 - base <= kRunSpan; longer ranges test every head.
+// The counts are non-decreasing from P0 to P1 over the warp (monotone functions of the cumulative
+// weights for binary32 and binary64 sums, order_counts for two-float sums, checked counts from a
+// caller), so every head lies in [P0, P1) and one window holds them all when P1 - base <= kRunSpan;
+// longer ranges test every head.
 // Same result as writing out[j] = i for j in [O_{i-1}, O_i) particle by particle, without its
 // divergent loops.
 __device__ __forceinline__ uint32_t warp_runs(const int32_t (&Oe)[kPer], int32_t prev, int32_t i0,

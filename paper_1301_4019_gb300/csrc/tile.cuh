@@ -930,6 +930,7 @@ __device__ __forceinline__ void emit_seg_cumoff(const T* __restrict__ lw, int64_
   if (lane == 0)  // (a segment wholly past the end follows the sequence's last particle: n)
     prev = Ob;
   if (tail) end_counts(O, prev, cnt, n);  // (warp-uniform)
+  if constexpr (std::is_same_v<V, float2>) order_counts(O, prev);
   const uint32_t bits = warp_runs(O, prev, i0, a + lo, win);
   // (i0 is a multiple of kPer = 8: one byte per lane)
   if (cl && cnt > 0) cl[i0 >> 3] = static_cast<uint8_t>(bits);
