@@ -862,8 +862,9 @@ batch_chain_kernel(const float* __restrict__ lw, const int64_t* __restrict__ off
               auto part = [&](uint32_t j) {
                 return j < static_cast<uint32_t>(kChainCap) ? sw[j] : __ldg(lf + j);
               };
-              k = w.whole ? metropolis_chain<true, kChainBlocks>(lwi, all, un, Bv, keys, ui)
-                          : metropolis_chain<true, kChainBlocks>(lwi, part, un, Bv, keys, ui);
+              k = w.whole
+                      ? metropolis_chain<true, kChainBlocks, false>(lwi, all, un, Bv, keys, ui)
+                      : metropolis_chain<true, kChainBlocks, false>(lwi, part, un, Bv, keys, ui);
             }
             a[g] = k;
             if (d) atomicMin(d + P.lo + k, static_cast<int32_t>(P.i));
@@ -886,7 +887,7 @@ __device__ __forceinline__ int64_t item_index(int ipt, int q) {
 // Metropolis over the particles of all filters, ipt particles per thread, one thread per particle
 // (the launch shape is tunable; every particle's chain and claim are the same for any shape).
 template <typename T>
-__global__ void __launch_bounds__(kMaxTunedBlock)
+__global__ void __launch_bounds__(kMaxTunedBlock, 2)
 batch_mcmc_kernel(const T* __restrict__ lw, const int64_t* __restrict__ off, int F,
                   int64_t total, const int32_t* __restrict__ Bf, int32_t B, Keys base_keys,
                   const uint8_t* __restrict__ flags, int32_t* __restrict__ a,

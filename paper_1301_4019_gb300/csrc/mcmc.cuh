@@ -41,14 +41,19 @@ __device__ __forceinline__ float exp_band_estimate32(float delta) {
 
 // The binary32 acceptance test u < exp_pinned(delta), u = (w0 >> 8) 2^-24, from the band: with
 // e = 2^32 exp(delta) and v = w0 rounded towards zero to binary32, which is at most 256 above
-// 2^32 u, the test is v < e wherever |v - e| > e 2^-15 + 256. Where that does not hold `amb` is
-// set (and stays set): probability about 6e-5 e / 2^32 a test, and every test of a NaN, of an
-// infinite e (a ratio above 2^95, or a zero-weight current state) and of u = 0 against
-// exp(delta) < 2^-24. Four operations after the exponential, no branch.
+// 2^32 u, the test is v < e wherever |v - e| > v b + 256, b = 2^-15 / (1 - 2^-15) rounded up: then
+// e (1 - 2^-15) > v, or e (1 + 2^-15) < v - 256. Where that does not hold `amb` is set (and stays
+// set): probability about 6e-5 v / 2^32 a test, and every test of a NaN and of u = 0 against
+// exp(delta) < 2^-24. A rise of any size, an infinite e included, is decided; with the margin taken
+// from e instead of v, e = inf was not, and steps of chains that rise by more than 66 were taken
+// twice (64 filters of 4096 log-weights spread over +-100, B = 29: 53 -> 26 us). Four operations
+// after the exponential, no branch.
+constexpr float kExpBandOfV = 0x1.0004p-15f;
 __device__ __forceinline__ bool band_accept(uint32_t w0, float delta, bool& amb) {
   const float e = exp_band_estimate32(delta);
-  const float d = __fsub_rn(__uint2float_rz(w0), e);
-  amb |= !(fabsf(d) > __fmaf_rn(e, kExpBand, 256.0f));
+  const float v = __uint2float_rz(w0);
+  const float d = __fsub_rn(v, e);
+  amb |= !(fabsf(d) > __fmaf_rn(v, kExpBandOfV, 256.0f));
   return d < 0.0f;
 }
 
@@ -153,12 +158,18 @@ __device__ __forceinline__ float f64_sidecar(double x) {
 }
 
 constexpr int kUnroll64 = 4;  // binary64 chains (2 measured slower)
+// Log-weights of which two of this size put the filter's bound past 0.01 (2 * 41943 * 2^-23).
+constexpr float kWide64 = 41000.0f;
 
 // 2 P consecutive steps (s even) of a binary32 chain in state (k, lwk), those below B: the P
 // blocks drawn and their proposals gathered together, then the decisions from the band
 // (band_accept: a ratio >= 1 is e >= 2^32 (1 - 1e-5), never rejected by it). If any of them was
-// undecided the steps are taken again by definition: one branch for 2 P steps.
-template <int P, bool SMALL, typename Gather>
+// undecided they are taken again by definition: one branch for 2 P steps. With ZEROS a state of zero
+// weight accepts without that branch, which is taken from the proposals at hand (200003 particles, 99
+// of 100 of weight zero, B = 29: 46 -> 30 us). Without, such a state is decided there where the
+// proposal's weight is zero too, and undecided steps are drawn and gathered again: the staged chains
+// take that form, which the operation a step and the registers held for the branch cost 4 %.
+template <int P, bool SMALL, bool ZEROS, typename Gather>
 __device__ __forceinline__ void metropolis_steps(uint32_t& k, float& lwk, const Gather& gather,
                                                  uint32_t n, int32_t s, int32_t B,
                                                  const Keys& keys, const DrawRow& row) {
@@ -179,7 +190,15 @@ __device__ __forceinline__ void metropolis_steps(uint32_t& k, float& lwk, const 
   bool amb = false;
 #pragma unroll
   for (int q = 0; q < 2 * P; ++q) {
-    const bool yes = band_accept(w[q], __fsub_rn(lwj[q], lwk), amb);
+    bool yes;
+    if constexpr (ZEROS) {
+      const bool none = lwk == -INFINITY;
+      bool open = false;
+      yes = band_accept(w[q], __fsub_rn(lwj[q], lwk), open) || none;
+      amb |= open && !none;
+    } else {
+      yes = band_accept(w[q], __fsub_rn(lwj[q], lwk), amb);
+    }
     if (yes && (P > 1 || q == 0 || s + 1 < B)) {  // (P > 1: called for whole rounds only)
       k = j[q];
       lwk = lwj[q];
@@ -190,10 +209,24 @@ __device__ __forceinline__ void metropolis_steps(uint32_t& k, float& lwk, const 
     lwk = lwk0;
 #pragma unroll 1
     for (int32_t t = s; t < s + 2 * P && t < B; ++t) {
-      const uint4 x = draw(keys, row, static_cast<uint32_t>(t >> 1));
-      const uint32_t w0 = (t & 1) ? x.z : x.x, w1 = (t & 1) ? x.w : x.y;
-      const uint32_t jt = half_index<SMALL>(w0, w1, n);
-      const float lwt = gather(jt);
+      uint32_t w0, jt;
+      float lwt;
+      if constexpr (ZEROS) {
+        w0 = w[0];
+        jt = j[0];
+        lwt = lwj[0];
+#pragma unroll
+        for (int q = 1; q < 2 * P; ++q) {  // (the next step's to the front: no indexing)
+          w[q - 1] = w[q];
+          j[q - 1] = j[q];
+          lwj[q - 1] = lwj[q];
+        }
+      } else {
+        const uint4 x = draw(keys, row, static_cast<uint32_t>(t >> 1));
+        w0 = (t & 1) ? x.z : x.x;
+        jt = half_index<SMALL>(w0, (t & 1) ? x.w : x.y, n);
+        lwt = gather(jt);
+      }
       if (metropolis_accept_exact(lwk, lwt, w0)) {
         k = jt;
         lwk = lwt;
@@ -207,7 +240,7 @@ __device__ __forceinline__ void metropolis_steps(uint32_t& k, float& lwk, const 
 // steps 2m and 2m + 1 take the two halves of the block of counter (i, m) (half_u01_f32,
 // half_index), so a chain draws ceil(B / 2) blocks. P blocks (2 P proposals) are issued together.
 // Returns the ancestor.
-template <bool SMALL, int P, typename Gather>
+template <bool SMALL, int P, bool ZEROS, typename Gather>
 __device__ __forceinline__ int32_t metropolis_chain(float lwk, const Gather& gather, uint32_t n,
                                                     int32_t B, const Keys& keys, uint32_t i) {
   uint32_t k = i;
@@ -215,9 +248,9 @@ __device__ __forceinline__ int32_t metropolis_chain(float lwk, const Gather& gat
   int32_t s = 0;
   if constexpr (P > 1)
     for (; s + 2 * P <= B; s += 2 * P)  // (s even)
-      metropolis_steps<P, SMALL>(k, lwk, gather, n, s, B, keys, row);
+      metropolis_steps<P, SMALL, ZEROS>(k, lwk, gather, n, s, B, keys, row);
   for (; s < B; s += 2)  // the last B mod 2 P steps, a block per two
-    metropolis_steps<1, SMALL>(k, lwk, gather, n, s, B, keys, row);
+    metropolis_steps<1, SMALL, ZEROS>(k, lwk, gather, n, s, B, keys, row);
   return static_cast<int32_t>(k);
 }
 
@@ -229,59 +262,62 @@ __device__ __forceinline__ int32_t metropolis_one(const float* __restrict__ lw, 
   const float lwi = __ldg(lw + i);
   if (nonfinite_logw(lwi)) flag_error(err, RS_ERR_NONFINITE);
   const auto gather = [&](uint32_t j) { return __ldg(lw + j); };
-  return metropolis_chain<SMALL, P>(lwi, gather, static_cast<uint32_t>(n), B, keys,
-                                 static_cast<uint32_t>(i));
+  return metropolis_chain<SMALL, P, true>(lwi, gather, static_cast<uint32_t>(n), B, keys,
+                                          static_cast<uint32_t>(i));
 }
 
-__device__ __forceinline__ bool f64_step_accept(double lwk, float lwk_f, bool okk, long long kk,
-                                                double lwj, float lwj_f, bool okj, long long kj,
-                                                uint4 x) {
-  const long long kNegInf = f64_key(-INFINITY);
-  if (kk == kNegInf || kj >= kk) return true;  // zero-weight state, or ratio >= 1
-  if (kj == kNegInf) return false;             // zero-weight proposal
-  return f64_accept_lt(lwj, lwj_f, okj, lwk, lwk_f, okk, x);
+// A Metropolis step of a binary64 chain, by definition: state lwk, proposal lwj, u from the words x.
+__device__ __forceinline__ bool f64_step_accept(double lwk, double lwj, uint2 x) {
+  const long long kk = f64_key(lwk), kj = f64_key(lwj), none = f64_key(-INFINITY);
+  if (kk == none || kj >= kk) return true;  // zero-weight state, or ratio >= 1
+  return kj != none && exact_f64_less_exp(lwj, lwk, make_uint4(x.x, x.y, 0u, 0u));
 }
 
 // A Metropolis step of a binary64 chain decided from sidecars (f64_sidecar): state k with
-// sidecar tk, proposal j with tj; the binary64 log-weights lw[k], lw[j] are read only when the
-// sidecars cannot decide. Same decision as f64_step_accept on the binary64 values.
-__device__ __forceinline__ bool sc_step_accept(const double* __restrict__ lw, int64_t k, float tk,
-                                               int64_t j, float tj, uint4 x) {
-  if (tk == -INFINITY) return true;              // zero-weight state (tk = -inf iff lw_k = -inf)
-  if (!(tj == tj) || !(tk == tk) || tj == tk) {  // undecided by the truncations
-    const double lwk = __ldg(lw + k), lwj = __ldg(lw + j);
-    float fk, fj;
-    const bool okk = f64_to_f32_trunc(lwk, fk), okj = f64_to_f32_trunc(lwj, fj);
-    return f64_step_accept(lwk, fk, okk, f64_key(lwk), lwj, fj, okj, f64_key(lwj), x);
+// sidecar tk, proposal j with tj, u from the words x; the binary64 log-weights lw[k], lw[j] are read
+// only when the sidecars cannot decide.
+__device__ __forceinline__ bool sc_step_accept(const double* __restrict__ lw, uint32_t k, float tk,
+                                               uint32_t j, float tj, uint2 x) {
+  if (tk == -INFINITY) return true;     // zero-weight state (tk = -inf iff lw_k = -inf)
+  if (tj > tk) return true;             // lw_j > lw_k: ratio above 1
+  const uint4 x4 = make_uint4(x.x, x.y, 0u, 0u);
+  bool open = true, yes = false;        // (equal sidecars or a NaN: undecided)
+  if (tj < tk) {
+    if (tj == -INFINITY) return false;  // zero-weight proposal
+    open = false;
+    yes = f64_filter_lt(tj, tk, x4, [&] { open = true; return false; });
   }
-  if (tj > tk) return true;                      // lw_j > lw_k: ratio above 1
-  if (tj == -INFINITY) return false;             // zero-weight proposal
-  return f64_filter_lt(tj, tk, x,
-                       [&] { return exact_f64_less_exp(__ldg(lw + j), __ldg(lw + k), x); });
+  return open ? f64_step_accept(__ldg(lw + k), __ldg(lw + j), x) : yes;
 }
 
-// The same decision from the band alone in almost every case, without branches: with
-// e = 2^32 exp(tj - tk), v = x0 rounded towards zero to binary32 (2^32 u lies in [v, v + 257)) and
-// m the filter's relative margin (f64_filter_lt), the step accepts iff v < e wherever
-// |v - e| > e m + 257 and the truncations' bound E is below 0.01; elsewhere `amb` is set (and
-// stays set): a zero-weight state, a NaN, wide bounds, u next to the ratio. Equal sidecars and
-// ratios above 1 are covered by the same inequality. A zero-weight proposal is e = 0, rejected,
-// from any state of non-zero weight. (The chain of tests took about 45 instructions, this 16.)
+// The same decision from the sidecars tj, tk and the band alone in almost every case, without
+// branches: with e = 2^32 exp(tj - tk), v = x0 rounded towards zero to binary32 (2^32 u lies in
+// [v, v + 257)) and m the filter's relative margin (f64_filter_lt), the step accepts iff v < e wherever
+// |v - e| > v m' + 260, m' >= m / (1 - m), and the truncations' bound E is below 0.01 (so m below
+// 0.0103): then e (1 - m) > v + 257, or e (1 + m) < v. Elsewhere `amb` is set (and stays set): a
+// zero-weight state, a NaN, wide bounds, u next to the ratio. Equal sidecars and ratios above 1, of
+// any size, are covered by the same inequality. A zero-weight proposal is e = 0, rejected, from any
+// state of non-zero weight. (The chain of tests took about 45 instructions, this 16.)
 __device__ __forceinline__ bool band_accept_sc(uint32_t x0, float tj, float tk, bool& amb) {
   const float df = __fsub_rn(tj, tk);
   const float E = __fmaf_ru(fabsf(tj) + fabsf(tk), 0x1p-23f,
                             __fmaf_ru(fabsf(df), 0x1p-24f, 0x1p-124f));
   const float e = exp_band_estimate32(df);
-  const float d = __fsub_rn(__uint2float_rz(x0), e);
-  const float w = __fmaf_ru(e, __fmaf_ru(E, 1.02f, kExpBand), 257.0f);
+  const float v = __uint2float_rz(x0);
+  const float d = __fsub_rn(v, e);
+  const float w = __fmaf_ru(v, __fmaf_ru(E, 1.04f, 1.02f * kExpBand), 260.0f);
   amb |= !(fabsf(d) > w && E < 0.01f) && !(is_neg_inf(tj) && tk > -INFINITY);
   return d < 0.0f;
 }
 
 // metropolis_chain for n < 2^31 binary64 log-weights lw from the state i with sidecar tk:
 // gather(j) reads the sidecar of proposal j (4 bytes instead of 8). Steps kUnroll64 at a time
-// from the band; if any of them was undecided they are taken again by sc_step_accept. The
-// decisions, and so the ancestor, are those of the binary64 definition.
+// from the band; if any of them was undecided their decisions are taken again from the proposals at
+// hand: by sc_step_accept, or, from a state so large that the filter cannot hold (unnormalised
+// log-likelihoods: every step is decided so), by definition on the binary64 log-weights, read
+// together. The decisions, and so the ancestor, are those of the binary64 definition. 200003
+// particles near -10^6, B = 29: 343 -> 268 us; log-weights spread over +-100: 51 -> 28 (rises above
+// 66 were undecided, and undecided steps were drawn and gathered again one by one).
 template <typename Gather>
 __device__ __forceinline__ int32_t metropolis_chain_sc(const double* __restrict__ lw, float tk,
                                                        const Gather& gather, uint32_t n,
@@ -289,14 +325,15 @@ __device__ __forceinline__ int32_t metropolis_chain_sc(const double* __restrict_
   uint32_t k = i;
   const DrawRow row = draw_row(keys, i);
   for (int32_t s = 0; s < B; s += kUnroll64) {
-    uint32_t x0[kUnroll64], j[kUnroll64];
+    uint2 x[kUnroll64];  // (the words of u)
+    uint32_t j[kUnroll64];
     float tj[kUnroll64];
 #pragma unroll
     for (int q = 0; q < kUnroll64; ++q) {
       if (s + q < B) {
-        const uint4 x = draw(keys, row, static_cast<uint32_t>(s + q));
-        x0[q] = x.x;
-        j[q] = uniform_index(x, n);
+        const uint4 r = draw(keys, row, static_cast<uint32_t>(s + q));
+        x[q] = make_uint2(r.x, r.y);
+        j[q] = uniform_index(r, n);
         tj[q] = gather(j[q]);
       }
     }
@@ -305,7 +342,7 @@ __device__ __forceinline__ int32_t metropolis_chain_sc(const double* __restrict_
     bool amb = false;
 #pragma unroll
     for (int q = 0; q < kUnroll64; ++q) {
-      if (s + q < B && band_accept_sc(x0[q], tj[q], tk, amb)) {
+      if (s + q < B && band_accept_sc(x[q].x, tj[q], tk, amb)) {
         k = j[q];
         tk = tj[q];
       }
@@ -313,14 +350,25 @@ __device__ __forceinline__ int32_t metropolis_chain_sc(const double* __restrict_
     if (amb) {
       k = k0;
       tk = tk0;
-#pragma unroll 1
-      for (int32_t t = s; t < s + kUnroll64 && t < B; ++t) {
-        const uint4 x = draw(keys, row, static_cast<uint32_t>(t));
-        const uint32_t jt = uniform_index(x, n);
-        const float tt = gather(jt);
-        if (sc_step_accept(lw, k, tk, jt, tt, x)) {
-          k = jt;
-          tk = tt;
+      if (fabsf(tk) > kWide64 && tk != -INFINITY) {
+        double lwk = __ldg(lw + k), lwj[kUnroll64];
+#pragma unroll
+        for (int q = 0; q < kUnroll64; ++q) lwj[q] = s + q < B ? __ldg(lw + j[q]) : 0.0;
+#pragma unroll
+        for (int q = 0; q < kUnroll64; ++q) {
+          if (s + q < B && f64_step_accept(lwk, lwj[q], x[q])) {
+            k = j[q];
+            tk = tj[q];
+            lwk = lwj[q];
+          }
+        }
+      } else {
+#pragma unroll
+        for (int q = 0; q < kUnroll64; ++q) {
+          if (s + q < B && sc_step_accept(lw, k, tk, j[q], tj[q], x[q])) {
+            k = j[q];
+            tk = tj[q];
+          }
         }
       }
     }
