@@ -28,8 +28,8 @@ template <typename T> constexpr int metropolis_min_ctas() { return sizeof(T) == 
 constexpr int64_t kMetropolisOneBlockMinN = int64_t{1} << 19;
 
 // One thread per particle (the claims d, when given, were set to the sentinel N before). SMALL:
-// N < 2^24; P: blocks drawn together (binary32). Binary64 log-weights come with their sidecars lwf (f64_sidecar; sidecar_kernel),
-// which the chains gather instead of the binary64 values.
+// N < 2^24; P: blocks drawn together (binary32). Binary64 log-weights come with their sidecars lwf
+// (f64_sidecar; sidecar_kernel), which the chains gather instead of the binary64 values.
 template <typename T, bool SMALL, int P>
 __global__ void __launch_bounds__(kBlock, metropolis_min_ctas<T>())
 metropolis_kernel(const T* __restrict__ lw, const float* __restrict__ lwf, int64_t N, int32_t B,

@@ -161,35 +161,38 @@ constexpr int kUnroll64 = 4;  // binary64 chains (2 measured slower)
 // Log-weights of which two of this size put the filter's bound past 0.01 (2 * 41943 * 2^-23).
 constexpr float kWide64 = 41000.0f;
 
-// 2 P consecutive steps (s even) of a binary32 chain in state (k, lwk), those below B: the P
-// blocks drawn and their proposals gathered together, then the decisions from the band
-// (band_accept: a ratio >= 1 is e >= 2^32 (1 - 1e-5), never rejected by it). If any of them was
-// undecided they are taken again by definition: one branch for 2 P steps. With ZEROS a state of zero
-// weight accepts without that branch, which is taken from the proposals at hand (200003 particles, 99
-// of 100 of weight zero, B = 29: 46 -> 30 us). Without, such a state is decided there where the
-// proposal's weight is zero too, and undecided steps are drawn and gathered again: the staged chains
-// take that form, which the operation a step and the registers held for the branch cost 4 %.
-template <int P, bool SMALL, bool ZEROS, typename Gather>
+// S consecutive steps (S = 1 or even, s even) of a binary32 chain of e steps in state (k, lwk), with
+// S = 2 and without ZEROS those of them below e: the blocks drawn and their proposals gathered
+// together, then the decisions from the band (band_accept: a ratio >= 1 is e >= 2^32 (1 - 1e-5),
+// never rejected by it). If any of them was undecided they are taken again by definition: one branch
+// for S steps. With ZEROS a state of zero weight accepts without that branch, which is taken from
+// the proposals at hand (200003 particles, 99 of 100 of weight zero, B = 29: 46 -> 30 us). Without,
+// such a state is decided there where the proposal's weight is zero too, and undecided steps are
+// drawn and gathered again: the staged chains take that form, which the operation a step and the
+// registers held for the branch cost 4 %.
+template <int S, bool SMALL, bool ZEROS, typename Gather>
 __device__ __forceinline__ void metropolis_steps(uint32_t& k, float& lwk, const Gather& gather,
-                                                 uint32_t n, int32_t s, int32_t B,
-                                                 const Keys& keys, const DrawRow& row) {
-  uint32_t w[2 * P], j[2 * P];
-  float lwj[2 * P];
+                                                 uint32_t n, int32_t s, int32_t e, const Keys& keys,
+                                                 const DrawRow& row) {
+  uint32_t w[S], j[S];
+  float lwj[S];
 #pragma unroll
-  for (int p = 0; p < P; ++p) {
-    const uint4 x = draw(keys, row, static_cast<uint32_t>(s / 2 + p));
-    w[2 * p] = x.x;
-    w[2 * p + 1] = x.z;
-    j[2 * p] = half_index<SMALL>(x.x, x.y, n);
-    j[2 * p + 1] = half_index<SMALL>(x.z, x.w, n);
-    lwj[2 * p] = gather(j[2 * p]);
-    lwj[2 * p + 1] = gather(j[2 * p + 1]);
+  for (int q = 0; q < S; q += 2) {
+    const uint4 x = draw(keys, row, (static_cast<uint32_t>(s) >> 1) + q / 2);
+    w[q] = x.x;
+    j[q] = half_index<SMALL>(x.x, x.y, n);
+    lwj[q] = gather(j[q]);
+    if constexpr (S > 1) {
+      w[q + 1] = x.z;
+      j[q + 1] = half_index<SMALL>(x.z, x.w, n);
+      lwj[q + 1] = gather(j[q + 1]);
+    }
   }
   const uint32_t k0 = k;
   const float lwk0 = lwk;
   bool amb = false;
 #pragma unroll
-  for (int q = 0; q < 2 * P; ++q) {
+  for (int q = 0; q < S; ++q) {
     bool yes;
     if constexpr (ZEROS) {
       const bool none = lwk == -INFINITY;
@@ -199,7 +202,7 @@ __device__ __forceinline__ void metropolis_steps(uint32_t& k, float& lwk, const 
     } else {
       yes = band_accept(w[q], __fsub_rn(lwj[q], lwk), amb);
     }
-    if (yes && (P > 1 || q == 0 || s + 1 < B)) {  // (P > 1: called for whole rounds only)
+    if (yes && (S != 2 || ZEROS || q == 0 || s + 1 < e)) {
       k = j[q];
       lwk = lwj[q];
     }
@@ -208,7 +211,7 @@ __device__ __forceinline__ void metropolis_steps(uint32_t& k, float& lwk, const 
     k = k0;
     lwk = lwk0;
 #pragma unroll 1
-    for (int32_t t = s; t < s + 2 * P && t < B; ++t) {
+    for (int32_t t = s; t < s + S && t < e; ++t) {
       uint32_t w0, jt;
       float lwt;
       if constexpr (ZEROS) {
@@ -216,7 +219,7 @@ __device__ __forceinline__ void metropolis_steps(uint32_t& k, float& lwk, const 
         jt = j[0];
         lwt = lwj[0];
 #pragma unroll
-        for (int q = 1; q < 2 * P; ++q) {  // (the next step's to the front: no indexing)
+        for (int q = 1; q < S; ++q) {  // (the next step's to the front: no indexing)
           w[q - 1] = w[q];
           j[q - 1] = j[q];
           lwj[q - 1] = lwj[q];
@@ -246,11 +249,18 @@ __device__ __forceinline__ int32_t metropolis_chain(float lwk, const Gather& gat
   uint32_t k = i;
   const DrawRow row = draw_row(keys, i);
   int32_t s = 0;
-  if constexpr (P > 1)
-    for (; s + 2 * P <= B; s += 2 * P)  // (s even)
-      metropolis_steps<P, SMALL, ZEROS>(k, lwk, gather, n, s, B, keys, row);
-  for (; s < B; s += 2)  // the last B mod 2 P steps, a block per two
-    metropolis_steps<1, SMALL, ZEROS>(k, lwk, gather, n, s, B, keys, row);
+  for (; s + 2 * P <= B; s += 2 * P)
+    metropolis_steps<2 * P, SMALL, ZEROS>(k, lwk, gather, n, s, B, keys, row);
+  if constexpr (ZEROS) {
+    if constexpr (P > 1)
+      for (; s + 2 <= B; s += 2)
+        metropolis_steps<2, SMALL, ZEROS>(k, lwk, gather, n, s, B, keys, row);
+    // an odd last step gathers one proposal from memory (with the block's other one 10^6 particles
+    // took 9.6 instead of 6.4 us at B = 1, 39.8 instead of 36.8 with Permute at B = 5)
+    if (s < B) metropolis_steps<1, SMALL, ZEROS>(k, lwk, gather, n, s, B, keys, row);
+  } else {  // (from shared memory it costs less than the code for it)
+    for (; s < B; s += 2) metropolis_steps<2, SMALL, ZEROS>(k, lwk, gather, n, s, B, keys, row);
+  }
   return static_cast<int32_t>(k);
 }
 
