@@ -23,6 +23,7 @@
 // structure (relative to the filter's first particle), with the filter index in the
 // random-number counter: filter f of a batched call equals rs_resample on that filter's slice
 // with filter = f, bit for bit.
+#include <algorithm>
 #include <climits>
 #include <mutex>
 
@@ -920,56 +921,60 @@ batch_mcmc_kernel(const T* __restrict__ lw, const int64_t* __restrict__ off, int
   }
 }
 
-// Rejection with warp refill over the particles of all filters (mcmc.cuh); a lane looks up
-// the filter of every particle it takes.
+// Rejection over the particles of all filters (mcmc.cuh), a warp per run of consecutive particles,
+// run_len of them (at most 32: a lane each), every lane looking up the filter of its particle; the
+// lanes make attempts of their own while more than half of them are busy and share the rest
+// (rejection_tail). Runs of 32; of 8 where the batch has fewer than kRejSmallBatch particles, whose
+// warps share them among their lanes from the start (64 filters of 256 .. 4096: 40 against 61 us;
+// 2000 of 256 .. 40000: 2398 against 1451; runs of 64 and 256 before the lanes share: 134 and 288
+// us against 108 for 200 filters of up to 20000). The batch's size is known on the device only: the
+// grid has at most kRejCtas CTAs per SM, which take the runs in turns, so that a small batch on a
+// large handle gets the short runs too and few idle CTAs (64 filters of up to 4096 on a handle of
+// 2^24: 71.9 -> 45.3 us with Permute; on one of their own size 39.2 -> 39.1). Five CTAs an SM
+// resident for binary32 (47 registers; 55 registers cost 4 % on 2000 filters).
+constexpr int64_t kRejSmallBatch = int64_t{1} << 18;
+constexpr int kRejCtas = 64;
 template <typename T>
-__global__ void __launch_bounds__(kBlock)
+__global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? 5 : 4)
 batch_rejection_kernel(const T* __restrict__ lw, const int64_t* __restrict__ off, int F,
                        int64_t total, Keys base_keys, double log_wmax, int64_t max_trials,
                        const uint8_t* __restrict__ flags, int32_t* __restrict__ a,
-                       int32_t* __restrict__ d, int run_len, int* err) {
+                       int32_t* __restrict__ d, int* err) {
   pdl_wait();
   const int lane = threadIdx.x & 31;
-  const int64_t run = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
-  const int64_t start = run * run_len;
   const int64_t limit = batch_end(off, F, total);
+  const int run_len = limit < kRejSmallBatch ? 8 : 32;
+  const int64_t stride = ((static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5) * run_len;
   flag_descending(off, F, err);
-  if (start >= limit) return;  // uniform across the warp
-  const int64_t end = start + run_len < limit ? start + run_len : limit;
   const RejBound rb = make_bound(log_wmax);
-  int64_t g = start + lane;
-  bool active = false;
-  PartLoc P;
-  Keys keys = base_keys;
-  T lwi = T(0);
-  bool keep = false;  // the particle's filter is not resampled: it settles on itself
-  auto take = [&](int64_t gg) {
-    g = gg;
-    active = false;
-    if (gg >= end) return;
-    if (!locate_particle(off, F, total, gg, P)) {
+  for (int64_t start = ((static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5) * run_len;
+       start < limit; start += stride) {  // uniform across the warp
+    const int64_t g = start + lane;
+    PartLoc P;
+    Keys keys = base_keys;
+    T lwi = T(0);
+    bool active = lane < run_len && g < limit;
+    if (active && !locate_particle(off, F, total, g, P)) {
       flag_error(err, RS_ERR_ARG);
-      return;
+      active = false;
     }
-    active = true;
-    keep = !resampled(flags, P.f);
-    keys = with_tag(base_keys, static_cast<uint32_t>(P.f), RS_REJECTION);
-    lwi = __ldg(lw + gg);
-    if (nonfinite_logw(lwi)) flag_error(err, RS_ERR_NONFINITE);
-  };
-  take(g);
-  int64_t head = start + 32;
-  uint64_t s = 0;  // attempts made (max_trials < 2^32, but s + kRejBatch may pass 2^32)
-  for (;;) {
-    const unsigned busy = __ballot_sync(0xffffffffu, active);
-    if (head >= end && __popc(busy) <= 16) break;  // no particle left to take in: share the rest
-    bool settled = false;
     if (active) {
+      keys = with_tag(base_keys, static_cast<uint32_t>(P.f), RS_REJECTION);
+      lwi = __ldg(lw + g);
+      if (nonfinite_logw(lwi)) flag_error(err, RS_ERR_NONFINITE);
+      if (!resampled(flags, P.f)) {  // the particle's filter is not resampled: it keeps its place
+        a[g] = static_cast<int32_t>(P.i);
+        if (d) atomicMin(d + g, static_cast<int32_t>(P.i));
+        active = false;
+      }
+    }
+    uint64_t s = 0;  // attempts made (max_trials < 2^32, but s + kRejBatch may pass 2^32)
+    while (__popc(__ballot_sync(0xffffffffu, active)) > 16) {
+      if (!active) continue;
       int64_t j = P.i;
       bool over = false;
-      settled = keep || rejection_attempts<kRejBatch>(lw + P.lo, P.n, rb, keys, P.i,
-                                                      static_cast<uint32_t>(s), lwi, max_trials,
-                                                      j, over);
+      bool settled = rejection_attempts<kRejBatch>(lw + P.lo, P.n, rb, keys, P.i,
+                                                   static_cast<uint32_t>(s), lwi, max_trials, j, over);
       s += kRejBatch;
       if (!settled && s >= static_cast<uint64_t>(max_trials)) {
         flag_error(err, RS_ERR_REJECTION_CAP);
@@ -980,39 +985,29 @@ batch_rejection_kernel(const T* __restrict__ lw, const int64_t* __restrict__ off
         if (over) flag_error(err, RS_ERR_BOUND_VIOLATED);
         a[g] = static_cast<int32_t>(j);
         if (d) atomicMin(d + P.lo + j, static_cast<int32_t>(P.i));
+        active = false;
       }
     }
-    const unsigned done = __ballot_sync(0xffffffffu, settled);
-    if (settled) {
-      take(head + __popc(done & ((1u << lane) - 1u)));
-      s = 0;
+    RejParticle<T> own{active, 0u, 1u, 0u, 0, s, lwi};
+    if (active) {
+      own.i = static_cast<uint32_t>(P.i);
+      own.n = static_cast<uint32_t>(P.n);
+      own.tag = keys.tag;
+      own.lo = P.lo;
     }
-    head += __popc(done);
+    rejection_tail<T>(
+        own, max_trials, err,
+        [&](const RejParticle<T>& R, uint32_t from, int64_t& j, bool& over) {
+          Keys rk = base_keys;
+          rk.tag = R.tag;
+          return rejection_attempts<kRejBatch>(lw + R.lo, R.n, rb, rk, R.i, from, R.lwi, max_trials, j,
+                                               over);
+        },
+        [&](const RejParticle<T>& R, int64_t j) {
+          a[R.lo + R.i] = static_cast<int32_t>(j);
+          if (d) atomicMin(d + R.lo + j, static_cast<int32_t>(R.i));
+        });
   }
-  if (active && keep) {  // (a particle that keeps its place takes no attempts)
-    a[g] = static_cast<int32_t>(P.i);
-    if (d) atomicMin(d + g, static_cast<int32_t>(P.i));
-    active = false;
-  }
-  RejParticle<T> own{active, 0u, 1u, 0u, 0, s, lwi};
-  if (active) {
-    own.i = static_cast<uint32_t>(P.i);
-    own.n = static_cast<uint32_t>(P.n);
-    own.tag = keys.tag;
-    own.lo = P.lo;
-  }
-  rejection_tail<T>(
-      own, max_trials, err,
-      [&](const RejParticle<T>& R, uint32_t from, int64_t& j, bool& over) {
-        Keys rk = base_keys;
-        rk.tag = R.tag;
-        return rejection_attempts<kRejBatch>(lw + R.lo, R.n, rb, rk, R.i, from, R.lwi, max_trials, j,
-                                             over);
-      },
-      [&](const RejParticle<T>& R, int64_t j) {
-        a[R.lo + R.i] = static_cast<int32_t>(j);
-        if (d) atomicMin(d + R.lo + j, static_cast<int32_t>(R.i));
-      });
 }
 
 // Permute of every filter: each warp takes 32 K consecutive slots of the batch, ipt times
@@ -1025,25 +1020,26 @@ batch_rejection_kernel(const T* __restrict__ lw, const int64_t* __restrict__ off
 // search of the offsets each) took 350 instructions per slot.
 //
 // K slots per lane: four for large batches; one for small ones, where it keeps more threads in
-// flight (50 filters of up to 5000: 30.8 against 34.9 us a call).
+// flight (50 filters of up to 5000: 30.8 against 34.9 us a call). The batch's size is known on the
+// device only, where the form is chosen; the grid covers the handle's capacity in either form. (By
+// the capacity, multinomial over 64 filters of up to 4096 took 26.8 us on a handle of 2^20 instead
+// of 24.7; two forms in one kernel cost multinomial over 2000 filters 1 %, 350.6 -> 354.2.) LARGE:
+// the handle holds batches of the size for four slots.
 constexpr int64_t kBatchSorted4MinN = int64_t{1} << 18;
 constexpr int64_t kBatchPermute4MinN = int64_t{1} << 20;
-template <int K>
-constexpr size_t perm_smem_per_warp() {
-  return 32 * K * (sizeof(int2) + sizeof(int32_t));
+template <bool SORTED> constexpr int64_t permute4_min_n() {
+  return SORTED ? kBatchSorted4MinN : kBatchPermute4MinN;
 }
+constexpr size_t kPermSmemPerWarp = 128 * (sizeof(int2) + sizeof(int32_t));
 template <bool SORTED, int K>
-__global__ void __launch_bounds__(kMaxTunedBlock)
-batch_permute_kernel(const int64_t* __restrict__ off, int F, int64_t total,
-                     const int32_t* __restrict__ a, const int32_t* __restrict__ d,
-                     const uint8_t* __restrict__ cl, int32_t* __restrict__ c, int ipt,
-                     const int32_t* limit, int* err) {
-  pdl_wait();
-  extern __shared__ __align__(16) unsigned char sh_perm[];
+__device__ __forceinline__ void batch_permute_slots(const int64_t* __restrict__ off, int F,
+                                                    int64_t total, int64_t end,
+                                                    const int32_t* __restrict__ a,
+                                                    const int32_t* __restrict__ d,
+                                                    const uint8_t* __restrict__ cl,
+                                                    int32_t* __restrict__ c, int ipt, int32_t* cw,
+                                                    int2* pend, int* err) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  int32_t* const cw = reinterpret_cast<int32_t*>(sh_perm + warp * perm_smem_per_warp<K>());
-  int2* const pend = reinterpret_cast<int2*>(cw + 32 * K);
-  const int64_t end = __ldg(limit);  // (0: the offsets descend, no ancestors were formed)
   for (int q = 0; q < ipt; ++q) {
     // first slot of this warp (of this lane: K * lane further)
     const int64_t gw = K * ((static_cast<int64_t>(blockIdx.x) * ipt + q) * blockDim.x +
@@ -1076,6 +1072,22 @@ batch_permute_kernel(const int64_t* __restrict__ off, int F, int64_t total,
         permute_one(a + P.lo, d + P.lo, P.n, c + P.lo, P.i, err);
     }
   }
+}
+template <bool SORTED, bool LARGE>
+__global__ void __launch_bounds__(kMaxTunedBlock)
+batch_permute_kernel(const int64_t* __restrict__ off, int F, int64_t total,
+                     const int32_t* __restrict__ a, const int32_t* __restrict__ d,
+                     const uint8_t* __restrict__ cl, int32_t* __restrict__ c, int ipt,
+                     const int32_t* limit, int* err) {
+  pdl_wait();
+  extern __shared__ __align__(16) unsigned char sh_perm[];
+  int32_t* const cw = reinterpret_cast<int32_t*>(sh_perm + (threadIdx.x >> 5) * kPermSmemPerWarp);
+  int2* const pend = reinterpret_cast<int2*>(cw + 128);
+  const int64_t end = __ldg(limit);  // (0: the offsets descend, no ancestors were formed)
+  if (LARGE && end >= permute4_min_n<SORTED>())
+    batch_permute_slots<SORTED, 4>(off, F, total, end, a, d, cl, c, ipt, cw, pend, err);
+  else
+    batch_permute_slots<SORTED, 1>(off, F, total, end, a, d, cl, c, ipt, cw, pend, err);
 }
 
 // Total number of particles of the batch (offsets[F]) is not known on the host without a
@@ -1226,21 +1238,19 @@ cudaError_t launch_batched(const Scratch& s, int scheme, Acc acc, const void* lo
     trace_mark(s.trace, scheme == RS_METROPOLIS ? (f64 ? "batch_metropolis_f64" : "batch_metropolis_f32")
                                                 : (f64 ? "batch_rejection_f64" : "batch_rejection_f32"),
                st);
-    // particles per warp of the rejection: 32; 8 in small batches, whose warps share them among
-    // their lanes from the start (64 filters of 256 .. 4096: 40 against 61 us; 2000 of 256 ..
-    // 40000: 2398 against 1451; runs of 64 and 256 before the lanes share: 134 and 288 us against
-    // 108 for 200 filters of up to 20000)
-    const int run_len = total < (int64_t{1} << 18) ? 8 : 32;
-    const int grid_runs = static_cast<int>(((total + run_len - 1) / run_len * 32 + kBlock - 1) / kBlock);
+    const int64_t runs = total < kRejSmallBatch ? (total + 7) / 8
+                                                : std::max((total + 31) / 32, kRejSmallBatch / 8);
+    const int grid_runs = static_cast<int>(std::min<int64_t>((32 * runs + kBlock - 1) / kBlock,
+                                                             kRejCtas * device_sm_count()));
     if (scheme == RS_REJECTION) {
       if (f64)
         launch_pdl(batch_rejection_kernel<double>, grid_runs, kBlock, st,
             static_cast<const double*>(logw), offsets, F, total, keys, log_wmax, max_trials,
-            flags, a, d, run_len, s.err);
+            flags, a, d, s.err);
       else
         launch_pdl(batch_rejection_kernel<float>, grid_runs, kBlock, st,
             static_cast<const float*>(logw), offsets, F, total, keys, log_wmax, max_trials,
-            flags, a, d, run_len, s.err);
+            flags, a, d, s.err);
     } else if (staged) {
       launch_pdl_smem(batch_chain_kernel, device_sm_count(), kChainBlock, kChainSmem, st,
                       static_cast<const float*>(logw), offsets, F, total, Bf, B, keys, flags, work,
@@ -1298,13 +1308,13 @@ cudaError_t launch_batched(const Scratch& s, int scheme, Acc acc, const void* lo
   if (e == cudaSuccess && permute) {
     trace_mark(s.trace, "batch_permute", st);
     const LaunchCfg& c = s.batch_cfg[kCfgPermute];
-    const bool four = total >= (cl ? kBatchSorted4MinN : kBatchPermute4MinN);
-    const int grid = grid_shaped(four ? (total + 3) / 4 : total, c);
-    const size_t smem = (four ? perm_smem_per_warp<4>() : perm_smem_per_warp<1>()) * (c.block / 32);
-    launch_pdl_smem(cl ? (four ? batch_permute_kernel<true, 4> : batch_permute_kernel<true, 1>)
-                       : (four ? batch_permute_kernel<false, 4> : batch_permute_kernel<false, 1>),
-                    grid, c.block, smem, st, offsets, F, total, s.a_tmp, s.d, cl, out, c.ipt,
-                    &s.glob->batch_limit, s.err);
+    const int64_t min4 = cl ? permute4_min_n<true>() : permute4_min_n<false>();
+    const int grid = grid_shaped(total < min4 ? total : std::max((total + 3) / 4, min4), c);
+    const bool large = total >= min4;
+    launch_pdl_smem(cl ? (large ? batch_permute_kernel<true, true> : batch_permute_kernel<true, false>)
+                       : (large ? batch_permute_kernel<false, true> : batch_permute_kernel<false, false>),
+                    grid, c.block, kPermSmemPerWarp * (c.block / 32), st, offsets, F, total, s.a_tmp,
+                    s.d, cl, out, c.ipt, &s.glob->batch_limit, s.err);
     e = cudaGetLastError();
   }
   return e;
