@@ -126,7 +126,7 @@ __device__ __forceinline__ bool resampled(const uint8_t* flags, int f) {
 // offsets checked.
 __global__ void __launch_bounds__(1024) batch_plan_kernel(Batch b) {
   pdl_wait();
-  __shared__ int2 sh[32];
+  __shared__ int3 sh[32];  // (all 32 warps write theirs)
   const int F = b.F;
   const int chunk = (F + blockDim.x - 1) / blockDim.x;
   const int f0 = min(F, static_cast<int>(threadIdx.x) * chunk), f1 = min(F, f0 + chunk);
@@ -150,14 +150,8 @@ __global__ void __launch_bounds__(1024) batch_plan_kernel(Batch b) {
     down |= descends(b.off, f);
   }
   if (rejected) flag_error(b.err, RS_ERR_ARG);
-  __shared__ int sh_longest;
-  if (threadIdx.x == 0) sh_longest = 0;
-  down = __syncthreads_or(down);
-  if (down) local = make_int2(0, 0);
-  if (threadIdx.x == 0) *b.limit = down ? 0 : static_cast<int32_t>(end);
-  longest = __reduce_max_sync(0xffffffffu, longest);
-  if ((threadIdx.x & 31) == 0) atomicMax(&sh_longest, longest);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  longest = __reduce_max_sync(0xffffffffu, longest);
   int2 incl = local;
 #pragma unroll
   for (int dd = 1; dd < 32; dd <<= 1) {
@@ -168,18 +162,19 @@ __global__ void __launch_bounds__(1024) batch_plan_kernel(Batch b) {
       incl.y += y;
     }
   }
-  if (lane == 31) sh[warp] = incl;
-  __syncthreads();
-  int2 p = make_int2(incl.x - local.x, incl.y - local.y);
-  for (int k = 0; k < warp; ++k) {
-    p.x += sh[k].x;
-    p.y += sh[k].y;
-  }
+  if (lane == 31) sh[warp] = make_int3(incl.x, incl.y, longest);
+  down = __syncthreads_or(down);
+  // (the sums of the warps before this one; the longest filter of all)
+  const int3 w = sh[lane];
+  int2 p = make_int2(__reduce_add_sync(0xffffffffu, lane < warp ? w.x : 0) + incl.x - local.x,
+                     __reduce_add_sync(0xffffffffu, lane < warp ? w.y : 0) + incl.y - local.y);
+  longest = __reduce_max_sync(0xffffffffu, w.z);
+  if (down) p = make_int2(0, 0);
   for (int f = f0; f < f1; ++f) {
     b.tile_start[f] = p.x;
     b.seg_start[f] = p.y;
     if (down) continue;
-    const int2 c = counts(f);
+    const int2 c = chunk == 1 ? local : counts(f);
     p.x += c.x;
     p.y += c.y;
   }
@@ -187,7 +182,10 @@ __global__ void __launch_bounds__(1024) batch_plan_kernel(Batch b) {
     b.tile_start[F] = p.x;
     b.seg_start[F] = p.y;
   }
-  if (threadIdx.x == 0) b.seg_start[F + 1] = sh_longest;  // (complete: the barrier above)
+  if (threadIdx.x == 0) {
+    b.seg_start[F + 1] = longest;
+    *b.limit = down ? 0 : static_cast<int32_t>(end);
+  }
 }
 
 // Locates batch tile t: its filter f, the filter's bounds and the tile's first particle.
@@ -352,15 +350,24 @@ batch_emit_kernel(const T* __restrict__ lw, Batch b, Keys base_keys,
 //   phase 1  the records of the warp's segments (seg_record: the segment's maximum log-weight
 //            and its weights' sum relative to it), last to first, and the filter maxima (an
 //            atomic max of keys per warp and filter);
-//   phase 2  per filter, one warp (a CTA from kWarpPrefixSegs segments): the exact sums of its
-//            records scaled to its maximum, rounded once to the segment prefixes and W^N;
+//   phase 2  per filter, one warp or, for a long one, a CTA: the exact sums of its records scaled to
+//            its maximum, rounded once to the segment prefixes and W^N;
 //   phase 3  the emission of the warp's segments, first to last (those phase 1 read last).
 // Every segment goes through the same device functions and rounded prefixes as in the separate
 // batched kernels and the single-filter kernels, so filter f still equals rs_resample on its
 // slice with filter = f, bit for bit.
 // ---------------------------------------------------------------------------------------
+//
+// The prefixes of one filter by one warp are a chain of steps of 32 records, which sets the length of
+// phase 2 where the filters are few and long. So a CTA takes a filter from kFewPrefixSegs segments
+// on where there are at most half as many filters as CTAs, from kSomePrefixSegs up to twice as many
+// (20 filters of 30000 .. 100000: binary32 32.9 -> 22.7 us, binary64 61.4 -> 47.3; stratified
+// binary64 over 256 of 16384 .. 262144: 525 -> 485; from 64 segments 500 of up to 20000 lost 2 of 25
+// us), and many filters keep all warps busy.
 constexpr int kWarpPrefixSegs = 1024;
-constexpr int kOwnPrefixSegs = 64;
+constexpr int kSomePrefixSegs = 256;
+constexpr int kFewPrefixSegs = 64;
+constexpr int kOwnPrefixSegs = 512;
 
 // Position of a warp in the batch: filter f and its bounds, segments [s0, s1) of the batch.
 struct SegWalk {
@@ -524,14 +531,16 @@ batch_coop_kernel(const T* __restrict__ lw, Batch b, Keys base_keys, int32_t* __
 
   // ---- phase 2: per filter, the exact prefixes of its segments and its total -----------------
   // Small batches (a segment per warp at most, no filter above kOwnPrefixSegs segments) skip it and
-  // its barrier: every warp sums its filter's records itself (64 filters of up to 4096: 22.5
-  // against 20.6 us a call).
+  // its barrier: every warp sums its filter's records itself (without Permute, 78 filters of up to
+  // 23655: 18.6 -> 16.2 us, 64 of up to 65536: 24.7 -> 19.9, with 64 segments as the most before).
   const bool own_prefix = U <= warps && __ldcg(b.seg_start + b.F + 1) <= kOwnPrefixSegs;
-  for (int pass = 0; pass < 2 && !own_prefix; ++pass) {  // (by warps; then very long filters by CTAs)
+  const int G = static_cast<int>(gridDim.x);
+  const int cta_segs = 2 * b.F <= G ? kFewPrefixSegs : b.F <= 2 * G ? kSomePrefixSegs : kWarpPrefixSegs;
+  for (int pass = 0; pass < 2 && !own_prefix; ++pass) {  // (by warps; then the longer filters by CTAs)
     for (int f = pass == 0 ? gw : static_cast<int>(blockIdx.x); f < b.F;
          f += pass == 0 ? warps : static_cast<int>(gridDim.x)) {
       const int s0 = __ldg(b.seg_start + f), nseg = __ldg(b.seg_start + f + 1) - s0;
-      if (nseg == 0 || (nseg >= kWarpPrefixSegs) != (pass == 1) || !resampled(b.resample, f)) continue;
+      if (nseg == 0 || (nseg >= cta_segs) != (pass == 1) || !resampled(b.resample, f)) continue;
       const double M = filter_M(b, f);
       if (!(M > -DBL_MAX)) {
         if (pass == 0 ? lane == 0 : threadIdx.x == 0) {
@@ -717,10 +726,6 @@ batch_chain_plan_kernel(const int64_t* __restrict__ off, int F, int64_t total,
   // (positions before the first filter belong to none: the other kernels report them too)
   if (work && threadIdx.x == 0) rejected |= end > 0 && __ldg(off) > 0;
   if (rejected) flag_error(err, RS_ERR_ARG);
-  down = __syncthreads_or(down);
-  if (threadIdx.x == 0) *limit = down ? 0 : static_cast<int32_t>(end);
-  if (!work) return;
-  if (down) local = 0;
   unsigned long long incl = local;
 #pragma unroll
   for (int dd = 1; dd < 32; dd <<= 1) {
@@ -728,9 +733,12 @@ batch_chain_plan_kernel(const int64_t* __restrict__ off, int F, int64_t total,
     if (lane >= dd) incl += y;
   }
   if (lane == 31) sh[warp] = incl;
-  __syncthreads();
+  down = __syncthreads_or(down);
+  if (threadIdx.x == 0) *limit = down ? 0 : static_cast<int32_t>(end);
+  if (!work) return;
   unsigned long long p = incl - local;
   for (int k = 0; k < warp; ++k) p += sh[k];
+  if (down) p = 0;
   for (int f = f0; f < f1; ++f) {
     work[f] = p;
     const unsigned long long w = filter_work(f);

@@ -667,7 +667,9 @@ __device__ __forceinline__ u128 rec_fixed(const double2* p, T M, const float2* t
 // order does not matter). P is non-decreasing because the exact prefixes are and rounding is
 // monotone. The total S is P_nt, the cumulative weight the emission gives the last particle
 // (seg_cum_weights), so that particle receives O = N.
-// Thread 0 writes S, N / S and S (binary64) to the given pointers, then the CTA synchronises.
+// The thread of the last record writes S, N / S and S (binary64) to the given pointers (it has the
+// total; read back through memory by thread 0 it came two microseconds later), then the CTA
+// synchronises.
 template <typename T, typename V>
 __device__ void seg_prefix_compute(const double2* s_rec, double2* P_rec, int nt, int64_t N,
                                    T M, V* S_out, V* scale_out, double* Sd_out) {
@@ -711,11 +713,10 @@ __device__ void seg_prefix_compute(const double2* s_rec, double2* P_rec, int nt,
       }
     }
   }
-  if (t1 == nt && t0 < nt) store_v<V>(P_rec + nt, fixed_to(p, V(), kFixFrac));
-  __syncthreads();
-  if (tid == 0) {
-    const V S = load_v_cg<V>(P_rec + nt);
+  if (t1 == nt && t0 < nt) {  // the thread of the last record has the total
+    const V S = fixed_to(p, V(), kFixFrac);
     const double Sd = vto_double(S);
+    store_v<V>(P_rec + nt, S);
     *S_out = S;
     *scale_out = vfrom_double(__ddiv_rn(static_cast<double>(N), Sd), V());
     *Sd_out = Sd;
