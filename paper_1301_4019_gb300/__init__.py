@@ -514,9 +514,11 @@ def rs_lgssm_step_ess(h: Handle, x: torch.Tensor, c: torch.Tensor | None, init: 
                       sigma_x: float, y: float, sigma_y: float, seed: int = 0, step: int = 0,
                       filter: int = 0, logw: torch.Tensor | None = None,
                       ess: torch.Tensor | None = None, log_total: torch.Tensor | None = None,
-                      stream=None) -> torch.Tensor:
+                      stream=None):
     """One bootstrap step around the resampling: x by the ancestry c (None: no copy), propagated
-    and weighted in place, and the ESS and log weight total of the new log-weights (returned)."""
+    and weighted in place, and the ESS and log weight total of the new log-weights. Returns
+    (logw, ess, log_total): the tensors given, or new ones for logw and, where neither of the other
+    two is given, ess; None for an output not asked for."""
     N = x.numel()
     if c is not None and c.numel() != N:
         raise ValueError("x and c disagree on N")
@@ -532,7 +534,7 @@ def rs_lgssm_step_ess(h: Handle, x: torch.Tensor, c: torch.Tensor | None, init: 
         _dev(ess, torch.float64, "ess", 1, h) if ess is not None else None,
         _dev(log_total, torch.float64, "log_total", 1, h) if log_total is not None else None,
         _stream(stream)), "rs_lgssm_step_ess")
-    return logw
+    return logw, ess, log_total
 
 
 def rs_copy_ancestors_batched(h: Handle, x: torch.Tensor, c: torch.Tensor,
