@@ -47,8 +47,8 @@ __device__ __forceinline__ bool locate_particle(const int64_t* __restrict__ off,
 }
 
 // Flags descending offsets (the per-particle schemes, whose kernels look every particle's filter
-// up themselves and stay inside it).
-__device__ __forceinline__ void flag_descending(const int64_t* __restrict__ off, int F, int* err) {
+// up themselves and stay inside it). Not inlined: in line it cost the rejection 10 %.
+__device__ __noinline__ void flag_descending(const int64_t* __restrict__ off, int F, int* err) {
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
   for (int64_t f = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; f < F; f += stride)
     if (descends(off, static_cast<int>(f))) flag_error(err, RS_ERR_ARG);
@@ -929,21 +929,22 @@ batch_mcmc_kernel(const T* __restrict__ lw, const int64_t* __restrict__ off, int
   }
 }
 
-// Rejection over the particles of all filters (mcmc.cuh), a warp per run of consecutive particles,
-// run_len of them (at most 32: a lane each), every lane looking up the filter of its particle; the
-// lanes make attempts of their own while more than half of them are busy and share the rest
-// (rejection_tail). Runs of 32; of 8 where the batch has fewer than kRejSmallBatch particles, whose
-// warps share them among their lanes from the start (64 filters of 256 .. 4096: 40 against 61 us;
-// 2000 of 256 .. 40000: 2398 against 1451; runs of 64 and 256 before the lanes share: 134 and 288
-// us against 108 for 200 filters of up to 20000). The batch's size is known on the device only: the
-// grid has at most kRejCtas CTAs per SM, which take the runs in turns, so that a small batch on a
-// large handle gets the short runs too and few idle CTAs (64 filters of up to 4096 on a handle of
-// 2^24: 71.9 -> 45.3 us with Permute; on one of their own size 39.2 -> 39.1). Five CTAs an SM
-// resident for binary32 (47 registers; 55 registers cost 4 % on 2000 filters).
+// Rejection over the particles of all filters (mcmc.cuh), a warp per run of consecutive particles (at
+// most 32: a lane each), every lane looking up the filter of its particle; the lanes make attempts
+// of their own while more than half of them are busy and share the rest (rejection_tail). Runs of
+// 32; of 8 where the batch has fewer than kRejSmallBatch particles, whose warps share them among
+// their lanes from the start (64 filters of 256 .. 4096: 40 against 61 us; 2000 of 256 .. 40000: 2398
+// against 1451; runs of 64 and 256 before the lanes share: 134 and 288 us against 108 for 200
+// filters of up to 20000). The batch's size is known on the device only: the grid covers the
+// handle's capacity up to kRejCtas CTAs per SM; larger handles get kRejTurnCtas per SM that take the
+// runs in turns (TURNS), so that a small batch on them gets few idle CTAs (64 filters of up to 4096
+// on a handle of 2^24: 71.9 -> 45.3 us with Permute). Bound by the latency of the longest particles
+// and the gathers of the others.
 constexpr int64_t kRejSmallBatch = int64_t{1} << 18;
-constexpr int kRejCtas = 64;
-template <typename T>
-__global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? 5 : 4)
+constexpr int kRejCtas = 256;
+constexpr int kRejTurnCtas = 64;
+template <typename T, bool TURNS>
+__global__ void __launch_bounds__(kBlock, sizeof(T) == 8 ? 4 : 5)
 batch_rejection_kernel(const T* __restrict__ lw, const int64_t* __restrict__ off, int F,
                        int64_t total, Keys base_keys, double log_wmax, int64_t max_trials,
                        const uint8_t* __restrict__ flags, int32_t* __restrict__ a,
@@ -951,18 +952,18 @@ batch_rejection_kernel(const T* __restrict__ lw, const int64_t* __restrict__ off
   pdl_wait();
   const int lane = threadIdx.x & 31;
   const int64_t limit = batch_end(off, F, total);
-  const int run_len = limit < kRejSmallBatch ? 8 : 32;
-  const int64_t stride = ((static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5) * run_len;
+  const int lg = limit < kRejSmallBatch ? 3 : 5;  // (log2 of the run length)
+  const int runs = static_cast<int>((limit + (1 << lg) - 1) >> lg);
   flag_descending(off, F, err);
   const RejBound rb = make_bound(log_wmax);
-  for (int64_t start = ((static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5) * run_len;
-       start < limit; start += stride) {  // uniform across the warp
-    const int64_t g = start + lane;
+  for (int run = static_cast<int>((blockIdx.x * blockDim.x + threadIdx.x) >> 5); run < runs;
+       run += TURNS ? static_cast<int>((gridDim.x * blockDim.x) >> 5) : runs) {  // uniform over the warp
+    const int64_t g = (static_cast<int64_t>(run) << lg) + lane;
     PartLoc P;
     Keys keys = base_keys;
     T lwi = T(0);
-    bool active = lane < run_len && g < limit;
-    if (active && !locate_particle(off, F, total, g, P)) {
+    bool active = lane < (1 << lg) && g < limit;
+    if (active && !locate_in(off, filter_of(off, F, g), limit, g, P)) {
       flag_error(err, RS_ERR_ARG);
       active = false;
     }
@@ -1246,19 +1247,20 @@ cudaError_t launch_batched(const Scratch& s, int scheme, Acc acc, const void* lo
     trace_mark(s.trace, scheme == RS_METROPOLIS ? (f64 ? "batch_metropolis_f64" : "batch_metropolis_f32")
                                                 : (f64 ? "batch_rejection_f64" : "batch_rejection_f32"),
                st);
-    const int64_t runs = total < kRejSmallBatch ? (total + 7) / 8
-                                                : std::max((total + 31) / 32, kRejSmallBatch / 8);
-    const int grid_runs = static_cast<int>(std::min<int64_t>((32 * runs + kBlock - 1) / kBlock,
-                                                             kRejCtas * device_sm_count()));
     if (scheme == RS_REJECTION) {
+      const int64_t runs = total < kRejSmallBatch ? (total + 7) / 8
+                                                  : std::max((total + 31) / 32, kRejSmallBatch / 8);
+      const int64_t ctas = (32 * runs + kBlock - 1) / kBlock;
+      const bool turns = ctas > kRejCtas * device_sm_count();
+      const int grid = turns ? kRejTurnCtas * device_sm_count() : static_cast<int>(ctas);
       if (f64)
-        launch_pdl(batch_rejection_kernel<double>, grid_runs, kBlock, st,
-            static_cast<const double*>(logw), offsets, F, total, keys, log_wmax, max_trials,
-            flags, a, d, s.err);
+        launch_pdl(turns ? batch_rejection_kernel<double, true> : batch_rejection_kernel<double, false>,
+                   grid, kBlock, st, static_cast<const double*>(logw), offsets, F, total, keys,
+                   log_wmax, max_trials, flags, a, d, s.err);
       else
-        launch_pdl(batch_rejection_kernel<float>, grid_runs, kBlock, st,
-            static_cast<const float*>(logw), offsets, F, total, keys, log_wmax, max_trials,
-            flags, a, d, s.err);
+        launch_pdl(turns ? batch_rejection_kernel<float, true> : batch_rejection_kernel<float, false>,
+                   grid, kBlock, st, static_cast<const float*>(logw), offsets, F, total, keys,
+                   log_wmax, max_trials, flags, a, d, s.err);
     } else if (staged) {
       launch_pdl_smem(batch_chain_kernel, device_sm_count(), kChainBlock, kChainSmem, st,
                       static_cast<const float*>(logw), offsets, F, total, Bf, B, keys, flags, work,

@@ -22,9 +22,10 @@ namespace {
 // slower: their four proposals in flight need them).
 template <typename T> constexpr int metropolis_min_ctas() { return sizeof(T) == 4 ? 6 : 1; }
 
-// Binary32 chains draw two blocks (four proposals) together below this size and one from it on,
-// where the gathers leave L1 and are bound by the L2's rate, not by their latency (2^20: 74.3
-// against 76.1 us with Permute; 2^18 at B = 60: 60.6 against 58.9).
+// Binary32 chains draw two blocks (four proposals) together, and one from this size to 2^24, where the
+// gathers leave L1 and are bound by the L2's rate, not by their latency (2^20: 74.3 against 76.1 us
+// with Permute; 2^18 at B = 60: 60.6 against 58.9; from 2^24 on part of them leaves L2: 1309 against
+// 1233 us at y = 2).
 constexpr int64_t kMetropolisOneBlockMinN = int64_t{1} << 19;
 
 // One thread per particle (the claims d, when given, were set to the sentinel N before). SMALL:
@@ -115,13 +116,23 @@ __device__ __forceinline__ void rejection_run(const T* __restrict__ lw,
       });
 }
 
+// CTAs that share an SM, at least (0: no demand; five of binary32 fit with 44 registers,
+// four of binary64 with 56), and one more from rejection_many_min_n particles on, where the gathers leave
+// L1 and L2 and want more warps in flight (2^24, y = 2, binary64 with Permute 892 -> 828 us, binary32
+// at y = 3 1559 -> 1490; below the line the registers are worth more: binary32 at 2^22 139.9 against
+// 143.2, binary64 at 2^20 53.7 against 55.7).
+template <typename T> constexpr int rejection_many() { return sizeof(T) == 4 ? 6 : 5; }
+template <typename T> constexpr int64_t rejection_many_min_n() {
+  return int64_t{1} << (sizeof(T) == 4 ? 24 : 22);
+}
+
 // Warp w takes the runs w, w + W, ... of run_len particles (W = warps of the grid). The host
 // sizes run_len so that every warp gets exactly one run (a warp that took an extra run
 // would set the kernel's length).
 // Binary64 log-weights come with their sidecars lwf, written by the cooperative grid before
 // its barrier, else beforehand by sidecar_kernel.
-template <typename T, bool COOP>
-__global__ void __launch_bounds__(kBlock)
+template <typename T, bool COOP, int CTAS>
+__global__ void __launch_bounds__(kBlock, CTAS)
 rejection_kernel(const T* __restrict__ lw, float* __restrict__ lwf, int64_t N, double log_wmax,
                  const double* lwmax_dev, bool clamp, int64_t max_trials, Keys keys,
                  int32_t* __restrict__ a, int32_t* __restrict__ d, int64_t run_len,
@@ -379,7 +390,7 @@ cudaError_t launch_metropolis_t(const Scratch& s, const T* lw, int64_t N, int32_
   const auto kernel = sizeof(T) == 8                 ? metropolis_kernel<T, false, 2>
                       : N < kMetropolisOneBlockMinN  ? metropolis_kernel<T, true, 2>
                       : N < (int64_t{1} << 24)       ? metropolis_kernel<T, true, 1>
-                                                     : metropolis_kernel<T, false, 1>;
+                                                     : metropolis_kernel<T, false, 2>;
   launch_pdl(kernel, grid, kBlock, st, lw, lwf, N, B, keys, a_out, d, s.err);
   return cudaGetLastError();
 }
@@ -394,7 +405,9 @@ cudaError_t launch_rejection_t(const Scratch& s, const T* lw, int64_t N, double 
   const int64_t runs = (N + kRejRun - 1) / kRejRun;
   const int64_t want = (runs + kBlock / 32 - 1) / (kBlock / 32);
   if (s.coop && s.launch_mode != RS_LAUNCH_SEPARATE) {
-    const int cap = coop_capacity(reinterpret_cast<const void*>(rejection_kernel<T, true>));
+    const auto kernel = N < rejection_many_min_n<T>() ? rejection_kernel<T, true, 0>
+                                                      : rejection_kernel<T, true, rejection_many<T>()>;
+    const int cap = coop_capacity(reinterpret_cast<const void*>(kernel));
     if (cap > 0) {
       // runs of at least kRejRun particles, one per warp of a grid of at most `cap` CTAs
       // (with more runs than warps some warps take two and the kernel waits for them:
@@ -404,7 +417,7 @@ cudaError_t launch_rejection_t(const Scratch& s, const T* lw, int64_t N, double 
       int64_t run_len = (N + warps - 1) / warps;
       run_len = run_len > kRejRun ? run_len : kRejRun;
       trace_mark(s.trace, f64 ? "rejection_f64" : "rejection_f32", st);
-      return coop_launch(rejection_kernel<T, true>, grid, st, lw, lwf, N, log_wmax, lwmax_dev,
+      return coop_launch(kernel, grid, st, lw, lwf, N, log_wmax, lwmax_dev,
                          clamp, max_trials, keys, a_out, d, run_len, bar, s.err);
     }
   }
@@ -424,7 +437,7 @@ cudaError_t launch_rejection_t(const Scratch& s, const T* lw, int64_t N, double 
   int64_t run_len = N / (static_cast<int64_t>(device_sm_count()) * 40);
   run_len = run_len < kRejRun ? kRejRun : run_len > 256 ? 256 : run_len;
   const int64_t warps = (N + run_len - 1) / run_len;
-  launch_pdl(rejection_kernel<T, false>,
+  launch_pdl(rejection_kernel<T, false, 0>,
              static_cast<int>((warps + kBlock / 32 - 1) / (kBlock / 32)), kBlock, st, lw, lwf, N,
              log_wmax, lwmax_dev, clamp, max_trials, keys, a_out, d, run_len, bar, s.err);
   return cudaGetLastError();
