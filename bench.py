@@ -227,26 +227,26 @@ class ClockSampler:
 # headers it includes, hashed; `traffic` is null once any of them has changed.
 # ---------------------------------------------------------------------------------------
 NCU_TRAFFIC = {  # label: (bytes per launch, source hash)
-    "permute": (8398575, "51b550508569d7d7"),
-    "metropolis_f32": (8398176, "84cbf3f6b0dd19a7"),
-    "metropolis_f64": (16797184, "84cbf3f6b0dd19a7"),
-    "fused_multinomial_f64": (8528384, "7f0f7fee292ba9e8"),
-    "rejection_f64": (8428434, "84cbf3f6b0dd19a7"),
-    "fused_stratified_f64": (8517193, "7f0f7fee292ba9e8"),
-    "permute_sorted": (4332877, "51b550508569d7d7"),
-    "rejection_f32": (4220768, "84cbf3f6b0dd19a7"),
-    "fused_systematic_f64": (8511195, "7f0f7fee292ba9e8"),
-    "fused_multinomial_f32": (4280256, "7f0f7fee292ba9e8"),
-    "iscan": (4214672, "51b550508569d7d7"),
-    "fused_stratified_f32": (4265664, "7f0f7fee292ba9e8"),
-    "search_f32": (12589152, "76b91365ace2aac1"),
-    "fused_systematic_f32": (4261824, "7f0f7fee292ba9e8"),
-    "search_f64": (16782043, "76b91365ace2aac1"),
-    "offspring": (8391440, "51b550508569d7d7"),
-    "cumoff_to_ancestors": (4206880, "51b550508569d7d7"),
-    "fill": (8682, "51b550508569d7d7"),
-    "adjacent_difference": (4198368, "51b550508569d7d7"),
-    "sidecar": (8394167, "84cbf3f6b0dd19a7")}
+    "permute": (8397699, "a98d0d2089b668f1"),
+    "metropolis_f32": (8394400, "8cc2115b47374442"),
+    "metropolis_f64": (16794295, "8cc2115b47374442"),
+    "fused_multinomial_f64": (8529216, "65ecdfca451709e7"),
+    "rejection_f64": (8428288, "8cc2115b47374442"),
+    "fused_stratified_f64": (8516571, "65ecdfca451709e7"),
+    "permute_sorted": (4332851, "a98d0d2089b668f1"),
+    "rejection_f32": (4220960, "8cc2115b47374442"),
+    "fused_systematic_f64": (8516718, "65ecdfca451709e7"),
+    "fused_multinomial_f32": (4279776, "65ecdfca451709e7"),
+    "iscan": (4214624, "a98d0d2089b668f1"),
+    "fused_stratified_f32": (4265344, "65ecdfca451709e7"),
+    "search_f32": (12590176, "542e24bb1620c007"),
+    "fused_systematic_f32": (4262144, "65ecdfca451709e7"),
+    "search_f64": (16782629, "542e24bb1620c007"),
+    "offspring": (8391376, "a98d0d2089b668f1"),
+    "cumoff_to_ancestors": (4206656, "a98d0d2089b668f1"),
+    "fill": (8804, "a98d0d2089b668f1"),
+    "adjacent_difference": (4198416, "a98d0d2089b668f1"),
+    "sidecar": (8394167, "8cc2115b47374442")}
 
 _LABEL_FILES = (("fused_", "fused.cu"), ("permute", "aux.cu"), ("iscan", "aux.cu"),
                 ("fill", "aux.cu"), ("offspring", "aux.cu"), ("adjacent", "aux.cu"),

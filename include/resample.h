@@ -407,8 +407,8 @@ int rs_metropolis_B_batched(rs_handle* h, int dtype, const void* logw_dev,
  * RS_BATCHED_PERMUTE (Code 10 per filter); block = threads per CTA (a multiple of 32, 32 to
  * 512), items_per_thread = particles per thread (Permute: turns of one slot, or of four in large
  * batches; 1 to 16). The handle starts at 256 x 1; binary32 Metropolis at that shape runs its
- * chains from shared memory, one CTA of 1024 threads per SM. Only the speed depends on the shape: every particle's draws, chain, claim and slot are the same
- * for any shape. RS_ERR_ARG for an unknown kernel or shape. Host-only. */
+ * chains from shared memory, one CTA of 1024 threads per SM. Only the speed depends on the shape:
+ * every particle's draws, chain, claim and slot are the same for any shape. RS_ERR_ARG for an unknown kernel or shape. Host-only. */
 #define RS_BATCHED_METROPOLIS_F32 0
 #define RS_BATCHED_METROPOLIS_F64 1
 #define RS_BATCHED_PERMUTE 2

@@ -535,7 +535,9 @@ batch_coop_kernel(const T* __restrict__ lw, Batch b, Keys base_keys, int32_t* __
   // 23655: 18.6 -> 16.2 us, 64 of up to 65536: 24.7 -> 19.9, with 64 segments as the most before).
   const bool own_prefix = U <= warps && __ldcg(b.seg_start + b.F + 1) <= kOwnPrefixSegs;
   const int G = static_cast<int>(gridDim.x);
-  const int cta_segs = 2 * b.F <= G ? kFewPrefixSegs : b.F <= 2 * G ? kSomePrefixSegs : kWarpPrefixSegs;
+  const int cta_segs = 2 * b.F <= G   ? kFewPrefixSegs
+                       : b.F <= 2 * G ? kSomePrefixSegs
+                                      : kWarpPrefixSegs;
   for (int pass = 0; pass < 2 && !own_prefix; ++pass) {  // (by warps; then the longer filters by CTAs)
     for (int f = pass == 0 ? gw : static_cast<int>(blockIdx.x); f < b.F;
          f += pass == 0 ? warps : static_cast<int>(gridDim.x)) {
@@ -687,10 +689,10 @@ __device__ __forceinline__ unsigned long long particle_work(const uint8_t* flags
                              : 2ull;
 }
 
-// Plan of the per-particle schemes (CTA 0): the batch's end (limit: 0 if its offsets descend) and, with work
-// given (the staged chains), the exclusive prefix over the filters of their work, work[0 .. F], and
-// the chunk counter reset; rejected filters and negative B are flagged and get no work. The other
-// CTAs write the claims' sentinels (d given).
+// Plan of the per-particle schemes (CTA 0): the batch's end (limit: 0 if its offsets descend) and,
+// with work given (the staged chains), the exclusive prefix over the filters of their work,
+// work[0 .. F], and the chunk counter reset; rejected filters and negative B are flagged and get no
+// work. The other CTAs write the claims' sentinels (d given).
 constexpr int kChainBlock = 1024;
 __global__ void __launch_bounds__(kChainBlock)
 batch_chain_plan_kernel(const int64_t* __restrict__ off, int F, int64_t total,
@@ -764,9 +766,9 @@ batch_chain_plan_kernel(const int64_t* __restrict__ off, int F, int64_t total,
 // particle, batch_chain_plan_kernel), taken in order from a counter: the first half of the
 // chunks covers 9/10 of the work, the second half the rest, so that the last one to end is
 // short. A chunk holds whole turns of the CTA's 1024 chains where it can: the end of a window
-// waits for its slowest warp (32 chunks per CTA instead of 16: 4.65 against 4.51 ms a call). Inside a window every warp takes the next 32 particles from a shared
-// counter (filters of one window may differ in B). Every particle's chain and claim are those of
-// batch_mcmc_kernel.
+// waits for its slowest warp (32 chunks per CTA instead of 16: 4.65 against 4.51 ms a call). Inside
+// a window every warp takes the next 32 particles from a shared counter (filters of one window may
+// differ in B). Every particle's chain and claim are those of batch_mcmc_kernel.
 // ---------------------------------------------------------------------------------------
 static_assert(kBatchMaxN < (1 << 24), "half_index<true>");
 constexpr int kChainCap = 57344;                            // staged log-weights

@@ -223,8 +223,8 @@ lgssm_step_ess_kernel(float* __restrict__ x, const int32_t* __restrict__ c, uint
       xn[r][q] = 0.0f;
       if (i < N && !init) {
         int32_t s = src[r][q];
-        if (static_cast<uint32_t>(s) >= N || (s != static_cast<int32_t>(i) && __ldg(c + s) != s)) {  // not from Permute: left alone
-          bad_c = true;
+        if (static_cast<uint32_t>(s) >= N || (s != static_cast<int32_t>(i) && __ldg(c + s) != s)) {
+          bad_c = true;  // not from Permute: left alone
           s = static_cast<int32_t>(i);
         }
         xn[r][q] = x[s];

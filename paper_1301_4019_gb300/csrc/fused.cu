@@ -67,7 +67,8 @@ struct FusedArgs {
 // fewer than 32 segments scans them in one warp, records and prefixes of a CTA's segments stay
 // in shared memory (up to kCtaSegs of them), the totals before the CTA and the total with its
 // binary64 division are finished by two different warps, and the systematic uniform is drawn at
-// the start: 2^20 binary32 systematic 26.7 -> 24.7 us a call, 1000 particles 14.3 -> 10.3.
+// the start: 2^20 binary32 systematic 26.7 -> 24.7 us a call, 1000 particles 14.4 -> 10.3 with the
+// launches queued ahead (alone, such a call was bound by its 14 us on the host then).
 constexpr int kCtaSegs = kBlock;  // segments of a CTA whose records and prefixes stay on chip
 
 // The order-preserving key of a log-weight as an unsigned number above 0, and back.

@@ -116,10 +116,10 @@ __device__ __forceinline__ void rejection_run(const T* __restrict__ lw,
       });
 }
 
-// CTAs that share an SM, at least (0: no demand; five of binary32 fit with 44 registers,
-// four of binary64 with 56), and one more from rejection_many_min_n particles on, where the gathers leave
-// L1 and L2 and want more warps in flight (2^24, y = 2, binary64 with Permute 892 -> 828 us, binary32
-// at y = 3 1559 -> 1490; below the line the registers are worth more: binary32 at 2^22 139.9 against
+// CTAs that share an SM, at least (0: no demand; five of binary32 fit with 44 registers, four of
+// binary64 with 56), and one more from rejection_many_min_n particles on, where the gathers leave L1
+// and L2 and want more warps in flight (2^24 with Permute, binary64 at y = 2 871 -> 807 us, binary32
+// at y = 0 365 -> 350; below the line the registers are worth more: binary32 at 2^22 139.9 against
 // 143.2, binary64 at 2^20 53.7 against 55.7).
 template <typename T> constexpr int rejection_many() { return sizeof(T) == 4 ? 6 : 5; }
 template <typename T> constexpr int64_t rejection_many_min_n() {
@@ -304,8 +304,8 @@ __device__ __forceinline__ uint4 words_of_u(uint64_t m) {
                     0u, 0u);
 }
 
-// Binary64 decisions on the binary32 pipes (f64_accept_lt, band_accept_sc) against the binary64 definition
-// u < exp_pinned(lwj - lwk), on n log-weight pairs: lwk from four magnitudes (0, -2.75,
+// Binary64 decisions on the binary32 pipes (f64_accept_lt, band_accept_sc) against the binary64
+// definition u < exp_pinned(lwj - lwk), on n log-weight pairs: lwk from four magnitudes (0, -2.75,
 // -1234.5678, 30000.5: the last two push the filter to its exact fallback), lwj = lwk + d with
 // d spread over [-90, 0) (plus hashed low bits, so that many bit patterns occur), and per pair
 // uniforms on the 53-bit grid at and next to p = exp_pinned(lwj - lwk), next to p (1 +- 2^-20),

@@ -302,9 +302,9 @@ __device__ __forceinline__ bool sc_step_accept(const double* __restrict__ lw, ui
 
 // The same decision from the sidecars tj, tk and the band alone in almost every case, without
 // branches: with e = 2^32 exp(tj - tk), v = x0 rounded towards zero to binary32 (2^32 u lies in
-// [v, v + 257)) and m the filter's relative margin (f64_filter_lt), the step accepts iff v < e wherever
-// |v - e| > v m' + 260, m' >= m / (1 - m), and the truncations' bound E is below 0.01 (so m below
-// 0.0103): then e (1 - m) > v + 257, or e (1 + m) < v. Elsewhere `amb` is set (and stays set): a
+// [v, v + 257)) and m the filter's relative margin (f64_filter_lt), the step accepts iff v < e
+// wherever |v - e| > v m' + 260, m' >= m / (1 - m), and the truncations' bound E is below 0.01 (so m
+// below 0.0103): then e (1 - m) > v + 257, or e (1 + m) < v. Elsewhere `amb` is set (and stays set): a
 // zero-weight state, a NaN, wide bounds, u next to the ratio. Equal sidecars and ratios above 1, of
 // any size, are covered by the same inequality. A zero-weight proposal is e = 0, rejected, from any
 // state of non-zero weight. (The chain of tests took about 45 instructions, this 16.)

@@ -103,8 +103,9 @@ RSK_BOTH ChainWindow chain_window(const int64_t* __restrict__ off, int64_t end, 
 }
 
 // Whether filter P lies inside the window, lo .. lo + len - 1, so that its value j is the window's
-// value P.lo - lo + j. Offsets that do not ascend can bring a window filters that begin before it
-// or end after it; nothing outside the staged values may be read for them.
+// value P.lo - lo + j. Offsets that do not ascend could bring a window filters that begin before it
+// or end after it; nothing outside the staged values is read for them. (Their plan gives such a
+// batch no work; this does not rely on it.)
 RSK_BOTH bool in_window(const ChainWindow& w, const PartLoc& P) {
   return P.lo >= w.lo && P.lo + P.n <= w.lo + w.len;
 }
